@@ -17,8 +17,11 @@ CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(BUILD, "libhfx.so")
 INCLUDE = os.path.join(ROOT, "include")
-SOURCES = ["hfx_api.cu", "hfx_eri.cu", "hfx_setup.cu", "hfx_batch.cu", "hfx_noalloc.cu", "hfx_nao.cu"]
-HEADERS = ["hfx_internal.cuh", "eri_engine.cuh", "eri_tables.inc", "hfx_eri.h", "hfx_setup.h", "hfx_ctx.h"]
+SOURCES = ["hfx_api.cu", "hfx_eri.cu", "hfx_setup.cu", "hfx_batch.cu", "hfx_noalloc.cu", "hfx_nao.cu",
+           "hfx_md_api.cu"]
+MD_SOURCE = "hfx_md.cu"  # compiled once per total angular momentum 0..8 (the slowest first)
+HEADERS = ["hfx_internal.cuh", "eri_engine.cuh", "eri_tables.inc", "eri_quartets.cuh", "hfx_md.cuh",
+           "gen_md_tables.py", "hfx_eri.h", "hfx_setup.h", "hfx_ctx.h"]
 ARCH = "-gencode=arch=compute_103a,code=sm_103a"
 
 
@@ -35,9 +38,7 @@ def _tables_current() -> bool:
     return os.path.exists(inc) and os.path.getmtime(inc) >= os.path.getmtime(gen)
 
 
-def generate_tables() -> None:
-    gen = os.path.join(CSRC, "gen_eri_tables.py")
-    inc = os.path.join(CSRC, "eri_tables.inc")
+def generate_tables(gen: str, inc: str) -> None:
     out = subprocess.run([sys.executable, gen], check=True, capture_output=True, text=True).stdout
     tmp = inc + f".tmp{os.getpid()}"
     with open(tmp, "w") as f:
@@ -55,28 +56,32 @@ def build(force: bool = False, verbose: bool = False, ptxas_verbose: bool = Fals
     lib_path = os.path.join(out_dir, "libhfx.so")
     os.makedirs(out_dir, exist_ok=True)
     if not _tables_current():
-        generate_tables()
+        generate_tables(os.path.join(CSRC, "gen_eri_tables.py"), os.path.join(CSRC, "eri_tables.inc"))
     deps = [os.path.join(CSRC, h) for h in HEADERS] + [os.path.join(INCLUDE, "hfx.h"), __file__]
-    srcs = [os.path.join(CSRC, s) for s in SOURCES]
+    srcs = [os.path.join(CSRC, s) for s in SOURCES + [MD_SOURCE]]
     if not force and os.path.exists(lib_path) and os.path.getmtime(lib_path) >= _newest(deps + srcs):
         return lib_path
+    generate_tables(os.path.join(CSRC, "gen_md_tables.py"), os.path.join(out_dir, "md_tables.inc"))
     nv = nvcc()
-    flags = [ARCH, "-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-I", INCLUDE, "-I", CSRC,
+    flags = [ARCH, "-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-I", INCLUDE, "-I", CSRC, "-I", out_dir,
              "--expt-relaxed-constexpr"]
     if ptxas_verbose:
         flags += ["-Xptxas", "-v"]
     flags += list(extra_flags)
 
-    def compile_one(src):
-        obj = os.path.join(out_dir, os.path.basename(src).replace(".cu", ".o"))
-        cmd = [nv] + flags + ["-c", src, "-o", obj]
+    units = [(MD_SOURCE, f"_l{k}", [f"-DHFX_MD_L={k}"]) for k in range(8, -1, -1)] + [(s, "", []) for s in SOURCES]
+
+    def compile_one(unit):
+        src, tag, more = unit
+        obj = os.path.join(out_dir, src.replace(".cu", tag + ".o"))
+        cmd = [nv] + flags + more + ["-c", os.path.join(CSRC, src), "-o", obj]
         r = subprocess.run(cmd, capture_output=True, text=True)
         if r.returncode != 0:
             raise RuntimeError(f"nvcc failed for {src}:\n{r.stderr}")
         return obj, r.stderr
 
-    with cf.ThreadPoolExecutor(max_workers=len(srcs)) as ex:
-        results = list(ex.map(compile_one, srcs))
+    with cf.ThreadPoolExecutor(max_workers=len(units)) as ex:
+        results = list(ex.map(compile_one, units))
     if verbose or ptxas_verbose:
         for obj, err in results:
             if err:

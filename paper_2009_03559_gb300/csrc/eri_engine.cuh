@@ -503,39 +503,4 @@ __device__ __forceinline__ double diag_max(const EriClassInfo& ci, const double*
   return mx;
 }
 
-// Locate the row of quartet q (global index) in [rlo, rhi): qoff[r] <= q < qoff[r+1].
-__device__ __forceinline__ int find_row(const long long* qoff, int rlo, int rhi, long long q) {
-  int lo = rlo, hi = rhi - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (__ldg(qoff + mid) <= q) lo = mid; else hi = mid - 1;
-  }
-  return lo;
-}
-
-__device__ __forceinline__ unsigned long long globaltimer_ns() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
-  return t;
-}
-
-// The quartet range [q0, q1) handled by group gid of ngroups.
-__device__ __forceinline__ void group_range(const EriLaunch& L, long long gid, long long ngroups,
-                                            long long& q0, long long& q1) {
-  if (L.schedule == 1) {
-    // parallel-pair split (paper Algorithm 2): an even share of the bra pairs, whatever
-    // the number of quartets they carry
-    const long long nr = L.row_end - L.row_begin;
-    const int r0 = L.row_begin + (int)(nr * gid / ngroups);
-    const int r1 = L.row_begin + (int)(nr * (gid + 1) / ngroups);
-    q0 = __ldg(L.qoff + r0);
-    q1 = __ldg(L.qoff + r1);
-  } else {
-    // parallel-quartet split (paper Algorithm 3 without the replicated screening): an
-    // even share of the screened quartet list
-    q0 = L.q_begin + L.q_count * gid / ngroups;
-    q1 = L.q_begin + L.q_count * (gid + 1) / ngroups;
-  }
-}
-
 }  // namespace hfx

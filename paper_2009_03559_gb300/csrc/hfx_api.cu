@@ -212,6 +212,8 @@ EriLaunch hfx::base_launch(hfx_ctx* ctx) {
   L.pa.prim_n = ctx->d_pp_n;
   L.pa.AB = ctx->d_AB;
   L.pa.prim = ctx->d_pp;
+  L.pa.md_off = ctx->d_md_off;
+  L.pa.md = ctx->d_md;
   L.sh.bf_off = ctx->d_bf_off;
   L.sh.atom = ctx->d_atom;
   L.boys = ctx->d_boys;
@@ -293,7 +295,15 @@ extern "C" int hfx_build_pairs(hfx_ctx* ctx) {
   }
   tb = tmp_bytes;
   CK(scan_int(tmp, tb, d_cap, ctx->d_pp_off, n_cand, s));
+  // offsets of the pairs' Hermite data
+  RK(ctx->alloc(&ctx->d_md_off, (size_t)n_cand + 1, true));
+  CK(cudaMemsetAsync(ctx->d_md_off, 0, sizeof(long long), s));
+  CK(launch_md_size(n_cand, ctx->d_pcls, d_cap, d_cand_t, s));  // d_cand_t has served
+  tb = tmp_bytes;
+  CK(scan_ll_inclusive(tmp, tb, d_cand_t, ctx->d_md_off + 1, n_cand, s));
   int last[2];
+  long long n_md = 0;
+  CK(cudaMemcpyAsync(&n_md, ctx->d_md_off + n_cand, sizeof(n_md), cudaMemcpyDeviceToHost, s));
   CK(cudaMemcpyAsync(&last[0], ctx->d_pp_off + n_cand - 1, sizeof(int), cudaMemcpyDeviceToHost, s));
   CK(cudaMemcpyAsync(&last[1], d_cap + n_cand - 1, sizeof(int), cudaMemcpyDeviceToHost, s));
   CK(cudaStreamSynchronize(s));
@@ -301,6 +311,9 @@ extern "C" int hfx_build_pairs(hfx_ctx* ctx) {
   RK(ctx->alloc(&ctx->d_pp, n_pp, true));
   CK(launch_prim_fill(n_cand, ctx->d_sa, ctx->d_sb, ctx->d_nprim, ctx->d_prim_off, ctx->d_atom, ctx->d_xyz,
                       ctx->d_alpha, ctx->d_w, ctx->d_pp_off, ctx->opt.prim_tau, ctx->d_pp, ctx->d_pp_n, s));
+  RK(ctx->alloc(&ctx->d_md, (size_t)n_md, true));
+  CK(launch_md_fill(n_cand, ctx->d_pcls, ctx->d_AB, ctx->d_pp_off, ctx->d_pp_n, ctx->d_pp, ctx->d_md_off, ctx->d_md,
+                    s));
   // 3. group candidates by pair class, Schwarz diagonal per class
   int *d_iota, *d_ckey, *d_cidx, *d_cnt;
   RK(ctx->alloc(&d_iota, n_cand, true));
@@ -325,7 +338,7 @@ extern "C" int hfx_build_pairs(hfx_ctx* ctx) {
         L.diag_list = d_cidx + start;
         L.diag_n = cnt[pc];
         L.diag_Q = ctx->d_Q;
-        const int gs = eri_group_size(cls);
+        const int gs = eri_group_size();
         CK(eri_launch(L, cls, 1, grid_for(ctx, cls, 1, cnt[pc], gs), s, gs, 0, false));
       }
       start += cnt[pc];
@@ -619,8 +632,9 @@ extern "C" int hfx_build_K_periodic(hfx_ctx* ctx, int n_R, const int* R_cells, c
       L.ket_bin_start = ctx->rt.bin_start[lo];
       L.q_begin = ctx->cls_qbegin[cp];
       L.q_count = ctx->cls_q[cp];
-      const int gs = eri_group_size(cp);
-      L.chunk = gs == 1 ? 256 : 8;
+      const int gs = eri_group_size();
+      const int grid = grid_for(ctx, cp, 0, L.q_count, gs, 3);
+      L.chunk = eri_chunk(gs, L.q_count, (long long)grid * eri_groups_per_block(gs));
       // forward: (p | q + G L) for bra class hi >= ket class lo; reverse (hi > lo): the
       // quartets (p | q + G L) with class(p) = lo < class(q) = hi, evaluated as (q | p - G L)
       for (int rev = 0; rev < (hi > lo ? 2 : 1); ++rev) {
@@ -630,7 +644,7 @@ extern "C" int hfx_build_K_periodic(hfx_ctx* ctx, int n_R, const int* R_cells, c
           L.shift[i] = rev ? -sh[i] : sh[i];
         }
         L.work = ctx->d_work + cp + 21 * rev;
-        CK(eri_launch(L, cp, 0, grid_for(ctx, cp, 0, L.q_count, gs, 3), s, gs, 3, false));
+        CK(eri_launch(L, cp, 0, grid, s, gs, 3, false));
       }
     }
   }
@@ -724,11 +738,10 @@ static int build_K_impl(hfx_ctx* ctx, const double* P, double* K, int ld, int pa
     // quartets that stay FP64 then those whose recurrences run in FP32, each with a kernel
     // compiled for its precision alone (registers, hence resident warps, of its own)
     L.fp32_ok = mixed && ((ctx->opt.fp32_class_mask >> cp) & 1);
-    const int gs = ctx->gs_override[cp] ? ctx->gs_override[cp] : eri_group_size(cp);
+    const int gs = ctx->gs_override[cp] ? ctx->gs_override[cp] : eri_group_size();
     ctx->gs_used[cp] = gs;
     const int streams = ctx->streams_override[cp];
     ctx->streams_used[cp] = gs == 32 ? eri_streams(cp, streams) : 0;
-    L.chunk = gs == 1 ? 256 : 8;
     const long long items = ctx->opt.schedule == HFX_SCHED_PAIR ? (L.row_end - L.row_begin) : L.q_count;
     if (ctx->timing) CK(cudaEventRecord(ctx->ev[2 + 2 * cp], s));
     for (int pass = 0; pass < (L.fp32_ok ? 2 : 1); ++pass) {
@@ -736,9 +749,10 @@ static int build_K_impl(hfx_ctx* ctx, const double* P, double* K, int ld, int pa
       // the FP32 pass runs on whole warps in every class (packed FP32 recurrences after an
       // FP32 set-up), unless the caller fixed the class's group size
       const int gsp = (prec == 2 && !ctx->gs_override[cp]) ? 32 : gs;
-      L.chunk = gsp == 1 ? 256 : 8;
+      const int grid = grid_for(ctx, cp, 0, items, gsp, prec, false, streams);
+      L.chunk = eri_chunk(gsp, L.q_count, (long long)grid * eri_groups_per_block(gsp));
       L.work = ctx->d_work + cp + 21 * pass;
-      CK(eri_launch(L, cp, 0, grid_for(ctx, cp, 0, items, gsp, prec, false, streams), s, gsp, prec, false, streams));
+      CK(eri_launch(L, cp, 0, grid, s, gsp, prec, false, streams));
     }
     if (ctx->timing) CK(cudaEventRecord(ctx->ev[3 + 2 * cp], s));
     ctx->class_launched[cp] = true;
@@ -797,7 +811,7 @@ extern "C" int hfx_get_stats(hfx_ctx* ctx, hfx_stats* out) {
   CK(cudaStreamSynchronize(ctx->stream));
   hfx_stats& st = ctx->stats;
   for (int cp = 0; cp < 21; ++cp) {
-    st.group_size_class[cp] = ctx->gs_used[cp] ? ctx->gs_used[cp] : eri_group_size(cp);
+    st.group_size_class[cp] = ctx->gs_used[cp] ? ctx->gs_used[cp] : eri_group_size();
     st.streams_class[cp] = ctx->streams_used[cp];
   }
   CK(cudaMemcpy(&st.energy, ctx->d_energy, sizeof(double), cudaMemcpyDeviceToHost));

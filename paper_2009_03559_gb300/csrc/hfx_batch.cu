@@ -39,7 +39,7 @@ struct BatchWork {
   bool mixed = false, pmax = false;
   bool fp32_class[21] = {};  // some system may run this class with FP32 recurrences
   long long total[21] = {};
-  int gs[21] = {}, chunk[21] = {};  // lanes per quartet and dynamic chunk per class
+  int gs[21] = {}, chunk[21] = {};  // lanes per quartet and dynamic chunk per class (0 = eri_chunk)
   int streams[21] = {};             // warp kernel: primitive quartets at a time (0 = default)
   EriLaunch *d_launch = nullptr, *h_launch = nullptr;
   BatchSys *d_sys = nullptr, *h_sys = nullptr;
@@ -83,8 +83,8 @@ cudaError_t bw_alloc(BatchWork& w, int cap, int n_sm) {
 // the default per-class choices (those of a single-system build)
 void bw_default_choices(BatchWork& w) {
   for (int cp = 0; cp < 21; ++cp) {
-    w.gs[cp] = eri_group_size(cp);
-    w.chunk[cp] = w.gs[cp] == 1 ? 256 : 8;
+    w.gs[cp] = eri_group_size();
+    w.chunk[cp] = 0;
     w.streams[cp] = 0;
   }
 }
@@ -179,6 +179,21 @@ int bw_prec(const BatchWork& w, int cp, int pass) { return w.fp32_class[cp] ? 1 
 // warps in every class (packed FP32 recurrences after an FP32 set-up)
 int bw_gs(const BatchWork& w, int cp, int prec) { return prec == 2 ? 32 : w.gs[cp]; }
 
+int bw_grid(const BatchWork& w, int cp, long long items, int prec) {
+  const int gs = bw_gs(w, cp, prec);
+  const long long groups_per_block = eri_groups_per_block(gs);
+  const long long need = (items + groups_per_block - 1) / groups_per_block;
+  const long long cap = (long long)eri_blocks_per_sm(cp, 0, gs, prec, true, w.streams[cp]) * w.n_sm;
+  return (int)std::max(1LL, std::min(need, cap));
+}
+
+// quartets per claim of a pass: the class's choice for its own lanes per quartet, else the rule's
+int bw_chunk(const BatchWork& w, int cp, int prec) {
+  const int gs = bw_gs(w, cp, prec);
+  if (gs == w.gs[cp] && w.chunk[cp]) return w.chunk[cp];
+  return eri_chunk(gs, w.total[cp], (long long)bw_grid(w, cp, w.total[cp], prec) * eri_groups_per_block(gs));
+}
+
 EriLaunch bw_class_launch(const BatchWork& w, int cp, int pass = 0) {
   EriLaunch L;
   std::memset(&L, 0, sizeof(L));
@@ -186,19 +201,11 @@ EriLaunch bw_class_launch(const BatchWork& w, int cp, int pass = 0) {
   L.schedule = HFX_SCHED_DYNAMIC;
   L.q_count = w.total[cp];
   L.work = w.d_work + cp + 21 * pass;
-  L.chunk = bw_gs(w, cp, bw_prec(w, cp, pass)) == w.gs[cp] ? w.chunk[cp] : 8;
+  L.chunk = bw_chunk(w, cp, bw_prec(w, cp, pass));
   L.n_sys = w.n;
   L.seg = w.d_seg + (size_t)cp * (w.cap + 1);
   L.batch = w.d_launch + (size_t)cp * w.cap;
   return L;
-}
-
-int bw_grid(const BatchWork& w, int cp, long long items, int prec) {
-  const int gs = bw_gs(w, cp, prec);
-  const long long groups_per_block = eri_groups_per_block(gs);
-  const long long need = (items + groups_per_block - 1) / groups_per_block;
-  const long long cap = (long long)eri_blocks_per_sm(cp, 0, gs, prec, true, w.streams[cp]) * w.n_sm;
-  return (int)std::max(1LL, std::min(need, cap));
 }
 
 cudaError_t bw_upload(const BatchWork& w, cudaStream_t s) {
@@ -514,11 +521,10 @@ extern "C" int hfx_batch_tune(hfx_batch* b, const double* const* P, double* cons
       int gs, streams, chunk;
     };
     std::vector<Cand> cands;
+    // streams are the FP32 pass's alone
     for (int k : {1, 2, 4})
-      if (eri_streams_valid(cp, k))
-        for (int c : {4, 8, 16}) cands.push_back({32, k, c});
-    if (eri_group_size(cp) == 1)
-      for (int c : {128, 256, 512}) cands.push_back({1, 0, c});
+      if (w.fp32_class[cp] ? eri_streams_valid(cp, k) : k == 1)
+        for (int c : {2, 8, 32}) cands.push_back({32, w.fp32_class[cp] ? k : 0, c});
     // window size: grow from 16k quartets until the incumbent takes the target, and at
     // least two claims for every resident warp of every candidate, so that a large chunk
     // is not timed on a window that leaves most of the GPU idle
@@ -603,7 +609,7 @@ extern "C" int hfx_batch_get_stats(hfx_batch* b, hfx_batch_stats* out) {
   for (int cp = 0; cp < 21; ++cp) {
     out->n_quartets += b->w.total[cp];
     out->group_size_class[cp] = b->w.gs[cp];
-    out->chunk_class[cp] = b->w.chunk[cp];
+    out->chunk_class[cp] = bw_chunk(b->w, cp, bw_prec(b->w, cp, 0));
     out->streams_class[cp] = b->w.gs[cp] == 32 ? eri_streams(cp, b->w.streams[cp]) : 0;
     out->tune_ms_class[cp] = b->tune_ms[cp];
     out->tune_window_class[cp] = b->tune_window[cp];

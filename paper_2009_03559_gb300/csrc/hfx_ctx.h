@@ -31,6 +31,8 @@ struct hfx_ctx {
   double *d_AB = nullptr, *d_Q = nullptr, *d_Qs = nullptr;
   double* d_dist = nullptr;  // distance-aware test data per sorted pair (5 doubles)
   hfx::PrimPair* d_pp = nullptr;
+  long long* d_md_off = nullptr;  // Hermite data of each candidate pair (PairArrays)
+  double* d_md = nullptr;
   int* d_sorted = nullptr;
   hfx::RowTable rt{};
   int n_rows = 0;

@@ -6,6 +6,7 @@
 #include <cstdio>
 #include <type_traits>
 #include "eri_engine.cuh"
+#include "eri_quartets.cuh"
 #include "hfx_eri.h"
 
 namespace hfx {
@@ -21,7 +22,7 @@ const EriClassInfo* class_info_host() { return kClassInfo; }
 // of the thread's own FP64 slot k (so no other lane's slots are ever touched); the
 // accumulated block is then widened in place into the FP64 slots Sd, where the horizontal
 // recurrences and the spherical step run.  R = double: the FP64 slots themselves.
-template <typename R, bool PER = false>
+template <typename R>
 __device__ __forceinline__ int contract_g1(const EriClassInfo& ci, const EriLaunch& L, int bra, int ket, double* Sd,
                                            int st) {
   R* S = reinterpret_cast<R*>(Sd);
@@ -39,7 +40,6 @@ __device__ __forceinline__ int contract_g1(const EriClassInfo& ci, const EriLaun
   // (the queue groups them so) run the same number of iterations
   const int npq = nb * nk;
   if constexpr (sizeof(R) == 4) {
-    static_assert(!PER, "the periodic build runs in FP64");
     // vertical recurrences and contraction on FP32 slots for one primitive quartet
     auto vrr = [&](const CoefRgT<float>& cf, const float* Gf) {
       for (int m = 0; m <= ci.Lt; ++m) V[m * sts] = Gf[m];
@@ -124,20 +124,11 @@ __device__ __forceinline__ int contract_g1(const EriClassInfo& ci, const EriLaun
         S[(w & 0xFFFF) * sts] += V[(w >> 16) * sts];
       }
     };
-    auto ket_of = [&](int ik) {
-      PrimPair k = pk[ik];
-      if constexpr (PER) {  // the ket pair's image in cell G (its centre moves, P - C does not)
-        k.P[0] += L.shift[0];
-        k.P[1] += L.shift[1];
-        k.P[2] += L.shift[2];
-      }
-      return k;
-    };
     for (int t = 0; t < npq; ++t) {
       const int ib = t / nk, ik = t - ib * nk;
       CoefRg c;
       double Gm[kMaxLt + 1];
-      if (!prim_setup(pb[ib], ket_of(ik), ci.E, ci.F, ci.Lt, omega, omega2, boys, c, Gm)) continue;
+      if (!prim_setup(pb[ib], pk[ik], ci.E, ci.F, ci.Lt, omega, omega2, boys, c, Gm)) continue;
       ++any;
       vrr(c, Gm);
     }
@@ -158,12 +149,6 @@ __device__ __forceinline__ int contract_g1(const EriClassInfo& ci, const EriLaun
   return any;
 }
 
-// ---------------------------------------------------------------------------
-// Contracted quartet, one warp: lanes set up 32 primitive quartets at a time (coefficient
-// sets in group scratch, compacted so that negligible ones take no place), then the warp
-// runs the class's schedule over k of them at a time (k streams, each with its own region
-// of accumulators and VRR slots), and finally sums the streams' accumulators.
-// ---------------------------------------------------------------------------
 // HRR and Cartesian -> spherical stages on the group scratch S (lanes share each stage)
 template <typename R>
 __device__ __forceinline__ void post_stages(const EriClassInfo& ci, const PairArrays& pa, int bra, int ket, R* S,
@@ -185,87 +170,12 @@ __device__ __forceinline__ void post_stages(const EriClassInfo& ci, const PairAr
 #define HFX_FP32_PACK 4
 #endif
 
-// Group scratch of one warp (in doubles): k stream regions, 33 coefficient sets (the last
-// one all zeros), one spare double.
-__host__ __device__ __forceinline__ int g32_stride(const SchedVariant& sv, int prec = 0) {
-  // the packed FP32 pass holds two primitive quartets per set (16 sets and the zero set), or
-  // four (stream regions of twice the size, 8 sets and the zero set, in doubles twice 9 x NCOEF)
-  if (prec != 2) return sv.group + 33 * HFX_NCOEF + 1;
+// Group scratch of one warp (in doubles): k stream regions, the coefficient sets (two
+// primitive quartets per set: 16 and the zero set; four: stream regions of twice the size,
+// 8 sets and the zero set, in doubles twice 9 x NCOEF), spare doubles.
+__host__ __device__ __forceinline__ int g32_stride(const SchedVariant& sv) {
   // float4 slots need 16-byte alignment: an even stride keeps every warp's region aligned
   return HFX_FP32_PACK == 4 ? 2 * sv.group + 9 * HFX_NCOEF * 2 + 2 : sv.group + 17 * HFX_NCOEF + 1;
-}
-
-template <bool PER = false>
-__device__ __forceinline__ int contract_g32(const EriClassInfo& ci, const SchedVariant& sv, const EriLaunch& L,
-                                            int bra, int ket, double* S, double* CF, int lane) {
-  const PairArrays pa = L.pa;
-  const double omega = L.omega, omega2 = L.omega2;
-  const double* boys = L.boys;
-  const int nb = __ldg(pa.prim_n + bra), nk = __ldg(pa.prim_n + ket);
-  const PrimPair* pb = pa.prim + __ldg(pa.prim_off + bra);
-  const PrimPair* pk = pa.prim + __ldg(pa.prim_off + ket);
-  const int k = sv.k, rsz = sv.rsz, nacc = ci.n_acc, nbase = ci.Lt + 1;
-  for (int i = lane; i < k * nacc; i += 32) {
-    const int u = i / nacc;
-    S[u * rsz + (i - u * nacc)] = 0.0;
-  }
-  if (lane < k) S[lane * rsz + sv.zero] = 0.0;
-  // coefficient set 32: all zeros, for streams past the chunk's last primitive quartet
-  for (int i = lane; i < HFX_NCOEF; i += 32) CF[32 * HFX_NCOEF + i] = 0.0;
-  const uint4* sched = reinterpret_cast<const uint4*>(kSched) + sv.off;
-  const int npq = nb * nk;
-  int any = 0;
-  for (int base = 0; base < npq; base += 32) {
-    const int t = base + lane;
-    double G[kMaxLt + 1];
-    PrimScalars ps;
-    int ib = 0, ik = 0;
-    bool ok = false;
-    if (t < npq) {
-      ib = t / nk;
-      ik = t - ib * nk;
-      PrimPair k = pk[ik];
-      if constexpr (PER) {  // the ket pair's image in cell G
-        k.P[0] += L.shift[0];
-        k.P[1] += L.shift[1];
-        k.P[2] += L.shift[2];
-      }
-      ok = prim_core(pb[ib], k, ci.Lt, omega, omega2, boys, G, ps);
-    }
-    const unsigned okm = __ballot_sync(0xffffffffu, ok);
-    if (ok)
-      write_set<double>(pb[ib], pk[ik], ci.E, ci.F, ci.Lt, G, ps, CF + __popc(okm & ((1u << lane) - 1u)) * HFX_NCOEF);
-    const int nv = __popc(okm);
-    any += nv;
-    __syncwarp();
-    for (int j = 0; j < nv; j += k) {
-      for (int i = lane; i < k * nbase; i += 32) {
-        const int u = i / nbase, m = i - u * nbase;
-        S[u * rsz + nacc + m] = (j + u < nv) ? CF[(j + u) * HFX_NCOEF + HFX_CF_G + m] : 0.0;
-      }
-      __syncwarp();
-      uint4 e = __ldg(sched + lane);
-      for (int it = 1; it <= sv.n_iter; ++it) {
-        // the next entry is fetched before this one runs (the last fetch reads one
-        // iteration past the variant's table: the tables end with a padding iteration)
-        const uint4 en = __ldg(sched + it * 32 + lane);
-        sched_op<double>(e, S, rsz, sv.zero, CF, j, nv);
-        __syncwarp();
-        e = en;
-      }
-    }
-  }
-  if (!any) return 0;
-  if (k > 1) {
-    for (int a = lane; a < nacc; a += 32) {
-      double sum = S[a];
-      for (int u = 1; u < k; ++u) sum += S[u * rsz + a];
-      S[a] = sum;
-    }
-    __syncwarp();
-  }
-  post_stages<double>(ci, pa, bra, ket, S, lane);
-  return any;
 }
 
 // Position of set bit number n (0-based, from the least significant) of m; -1 if m has fewer.
@@ -450,158 +360,12 @@ __device__ __forceinline__ int contract_g32_xw(const EriClassInfo& ci, const Sch
 #define HFX_G32F_MINB 8
 #endif
 
-// Precision passes of a class launch: 0 every quartet in FP64; 1 (mixed precision, first
-// pass) the quartets that must stay FP64; 2 (second pass) those whose recurrences run in FP32.
-// PREC_PERIODIC: the FP64 periodic instance (quartets of the lattice sums, see per_quartet).
-enum { PREC_FP64 = 0, PREC_MIXED64 = 1, PREC_MIXED32 = 2, PREC_PERIODIC = 3 };
-
-// The digest reads P_bd, P_bc, P_ad, P_ac.  max of their max|P| (or 1 without the table):
-// 0 means the quartet contributes exactly nothing; the mixed-precision and the
-// density-weighted screening tests use it too.
-__device__ __forceinline__ double pmax4(const EriLaunch& L, int sa, int sb, int sc, int sd) {
-  if (!L.pmax) return 1.0;
-  const double* pm = L.pmax;
-  const size_t ns = L.ns;
-  return fmax(fmax(__ldg(pm + sb * ns + sd), __ldg(pm + sb * ns + sc)),
-              fmax(__ldg(pm + sa * ns + sd), __ldg(pm + sa * ns + sc)));
-}
-
-// Distance-aware test: Q_IJ Q_KL exp(-kappa rho R^2) >= dist_tau (see hfx_options.dist_tau).
-__device__ __forceinline__ bool dist_keeps(const EriLaunch& Ls, int bra_s, int ket_s) {
-  if (!(Ls.dist_tau > 0.0)) return true;
-  const double* a = Ls.dist + 5 * (size_t)bra_s;
-  const double* b = Ls.dist + 5 * (size_t)ket_s;
-  const double dx = __ldg(a) - __ldg(b), dy = __ldg(a + 1) - __ldg(b + 1), dz = __ldg(a + 2) - __ldg(b + 2);
-  double r = sqrt(dx * dx + dy * dy + dz * dz) - __ldg(a + 3) - __ldg(b + 3);
-  if (r < 0.0) r = 0.0;
-  const double p = __ldg(a + 4), q = __ldg(b + 4);
-  const double rho = p * q / (p + q);
-  const double lam = Ls.omega2 * rho / (Ls.omega2 + rho);
-  return __ldg(Ls.Qs + bra_s) * __ldg(Ls.Qs + ket_s) * exp(-lam * r * r) >= Ls.dist_tau;
-}
-
-// Mixed precision: FP32 recurrences for the quartet when the class allows it and its
-// Schwarz bound times the largest density element it touches (or the largest of all of P)
-// is below fp32_tau.
-__device__ __forceinline__ bool fp32_eligible(const EriLaunch& Ls, int bra_s, int ket_s, double pm) {
-  if (!Ls.fp32_ok) return false;
-  const double pf = Ls.pglob ? __ldg(Ls.pglob) : pm;
-  return __ldg(Ls.Qs + bra_s) * __ldg(Ls.Qs + ket_s) * pf < Ls.fp32_tau;
-}
-
-// whether pass PREC takes the quartet
-template <int PREC>
-__device__ __forceinline__ bool pass_takes(const EriLaunch& Ls, int bra_s, int ket_s, double pm) {
-  if constexpr (PREC == PREC_FP64) return true;
-  const bool f32 = fp32_eligible(Ls, bra_s, ket_s, pm);
-  return PREC == PREC_MIXED32 ? f32 : !f32;
-}
-
-__device__ __forceinline__ void record_busy(const EriLaunch& L, unsigned long long t0) {
-  if (L.busy && threadIdx.x == 0) {
-    unsigned smid;
-    asm volatile("mov.u32 %0, %%smid;" : "=r"(smid));
-    atomicAdd(L.busy + smid, globaltimer_ns() - t0);
-  }
-}
-
-// ---------------------------------------------------------------------------
-// Periodic quartets (Eq. vx with lattice images): the launch for cell G evaluates
-// (X | Y + shift) for bra pair X and ket pair Y of the home-anchored pair list and adds
-//   K^G_{ab} += sum_{c,d} (a c | b d) P^{R}_{cd},   R = cell(d) - cell(c),
-// where a is the home-cell shell of the pair holding the row function (X for a forward
-// launch, Y for a reverse one), c its partner, b the home-cell shell of the other pair
-// (in cell G) and d its partner.  Every ordered pair of pairs is one quartet (no
-// permutational symmetry is used across cells), so the degeneracy factor is 1.
-// ---------------------------------------------------------------------------
-struct PerQuartet {
-  int pa, pb, pc, pd;        // positions of shells a, b, c, d in the quartet block (x1 x2 y1 y2)
-  int bfa, bfb, bfc, bfd;    // their first functions (home-cell numbering)
-  const double* PR;          // density block P^R
-};
-
-__device__ __forceinline__ bool per_quartet(const EriLaunch& L, int bra, int ket, PerQuartet& q) {
-  const PeriodicInfo& pi = L.per;
-  const int sax = __ldg(L.pa.sa + bra), sbx = __ldg(L.pa.sb + bra);
-  const int say = __ldg(L.pa.sa + ket), sby = __ldg(L.pa.sb + ket);
-  const bool hx = __ldg(pi.home_first + bra), hy = __ldg(pi.home_first + ket);
-  const int hxs = hx ? sax : sbx, oxs = hx ? sbx : sax;
-  const int hys = hy ? say : sby, oys = hy ? sby : say;
-  const int* cx = pi.cell_xyz + 3 * __ldg(pi.shell_cell + oxs);
-  const int* cy = pi.cell_xyz + 3 * __ldg(pi.shell_cell + oys);
-  const int w = 2 * pi.rb + 1;
-  int idx = 0;
-  for (int i = 0; i < 3; ++i) {
-    const int d = __ldg(cy + i) - __ldg(cx + i);
-    const int R = L.gcell[i] + (L.reverse ? -d : d);
-    if (R < -pi.rb || R > pi.rb) return false;
-    idx = idx * w + (R + pi.rb);
-  }
-  const int blk = __ldg(pi.rmap + idx);
-  if (blk < 0) return false;
-  // an exactly zero density block P^R_{cd} makes the quartet's contribution exactly zero
-  {
-    const int c = L.reverse ? oys : oxs, d = L.reverse ? oxs : oys;
-    if (__ldg(pi.pmax + ((size_t)blk * pi.nsh + c % pi.nsh) * pi.nsh + d % pi.nsh) == 0.0) return false;
-  }
-  q.PR = pi.P + (size_t)blk * pi.nbf * pi.nbf;
-  const int phx = hx ? 0 : 1, pox = 1 - phx, phy = hy ? 2 : 3, poy = 5 - phy;
-  if (!L.reverse) {
-    q.pa = phx; q.pc = pox; q.pb = phy; q.pd = poy;
-    q.bfa = __ldg(pi.shell_bf + hxs); q.bfc = __ldg(pi.shell_bf + oxs);
-    q.bfb = __ldg(pi.shell_bf + hys); q.bfd = __ldg(pi.shell_bf + oys);
-  } else {
-    q.pa = phy; q.pc = poy; q.pb = phx; q.pd = pox;
-    q.bfa = __ldg(pi.shell_bf + hys); q.bfc = __ldg(pi.shell_bf + oys);
-    q.bfb = __ldg(pi.shell_bf + hxs); q.bfd = __ldg(pi.shell_bf + oxs);
-  }
-  return true;
-}
-
-// K^G_{ab} += sum_{cd} v P^R_{cd} for the final block v (stride st); outputs o0, o0 + ostep, ...
-__device__ __forceinline__ void digest_per(const EriClassInfo& ci, const double* v, int st, const PerQuartet& q,
-                                           double* KG, int nbf, int o0, int ostep) {
-  int str[4];
-  str[3] = 1;
-  str[2] = ci.dims[3];
-  str[1] = ci.dims[2] * str[2];
-  str[0] = ci.dims[1] * str[1];
-  const int na = ci.dims[q.pa], nb = ci.dims[q.pb], nc = ci.dims[q.pc], nd = ci.dims[q.pd];
-  const int sa = str[q.pa], sb = str[q.pb], sc = str[q.pc], sd = str[q.pd];
-  for (int o = o0; o < na * nb; o += ostep) {
-    const int ia = o / nb, ib = o - ia * nb;
-    double acc = 0.0;
-    for (int ic = 0; ic < nc; ++ic)
-      for (int id = 0; id < nd; ++id)
-        acc = fma(v[(ia * sa + ib * sb + ic * sc + id * sd) * st], __ldg(q.PR + (size_t)(q.bfc + ic) * nbf + q.bfd + id),
-                  acc);
-    atomicAdd(KG + (size_t)(q.bfa + ia) * nbf + q.bfb + ib, acc);
-  }
-}
-
-// Per-thread tallies of one kernel, added to the launch's counters once at the end.
-struct Tally {
-  unsigned long long prim = 0, quart = 0, skip = 0, q32 = 0, p32 = 0;
-};
-
 // One quartet evaluated and digested by one lane (one quartet per thread), recurrences in
 // precision R; Sd: the thread's FP64 slots.
-template <typename R, bool PER = false>
+template <typename R>
 __device__ __forceinline__ void g1_quartet(const EriClassInfo& ci, const EriLaunch& Ls, int bra_s, int ket_s,
                                            double* Sd, int st, Tally& t) {
   const int bra = __ldg(Ls.sorted + bra_s), ket = __ldg(Ls.sorted + ket_s);
-  if constexpr (PER) {
-    PerQuartet pq;
-    if (!per_quartet(Ls, bra, ket, pq)) return;
-    const int npq = __ldg(Ls.pa.prim_n + bra) * __ldg(Ls.pa.prim_n + ket);
-    const int ne = contract_g1<double, true>(ci, Ls, bra, ket, Sd, st);
-    t.prim += ne;
-    t.skip += npq - ne;
-    if (!ne) return;
-    ++t.quart;
-    digest_per(ci, Sd + ci.out_base * st, st, pq, Ls.KG, Ls.per.nbf, 0, 1);
-    return;
-  }
   const int sa = __ldg(Ls.pa.sa + bra), sb = __ldg(Ls.pa.sb + bra);
   const int sc = __ldg(Ls.pa.sa + ket), sd = __ldg(Ls.pa.sb + ket);
   const int npq = __ldg(Ls.pa.prim_n + bra) * __ldg(Ls.pa.prim_n + ket);
@@ -656,7 +420,7 @@ __device__ __forceinline__ void sort64_desc(int& k0, int& k1, int lane) {
   }
 }
 
-template <bool BATCH, typename R, bool PER = false>
+template <bool BATCH, typename R>
 __device__ __forceinline__ void g1_drain(const EriLaunch& L, const EriClassInfo& ci, G1Queue& Q, int lane,
                                          double* Sd, int st, Tally& t, bool all) {
   while (Q.n >= 32 || (all && Q.n > 0)) {
@@ -679,13 +443,13 @@ __device__ __forceinline__ void g1_drain(const EriLaunch& L, const EriClassInfo&
     }
     __syncwarp();
     Q.n -= take;
-    if (lane < take) g1_quartet<R, PER>(ci, BATCH ? L.batch[e.x] : L, e.y, e.z, Sd, st, t);
+    if (lane < take) g1_quartet<R>(ci, BATCH ? L.batch[e.x] : L, e.y, e.z, Sd, st, t);
   }
 }
 
 // Quartets [q0, q1) of the launch record Ls (system sys), one quartet per thread: the warp
 // tests 32 consecutive quartets at a time and queues the survivors.
-template <bool BATCH, int PREC, typename R, bool PER = false>
+template <bool BATCH, int PREC, typename R>
 __device__ __forceinline__ void g1_range(const EriLaunch& L, const EriClassInfo& ci, const EriLaunch& Ls, int sys,
                                          long long q0, long long q1, double* Sd, int st, int lane, G1Queue& Q,
                                          Tally& t) {
@@ -704,30 +468,24 @@ __device__ __forceinline__ void g1_range(const EriLaunch& L, const EriClassInfo&
       bra_s = bra0 + (r - row_begin);
       ket_s = ket0 + (int)(q - __ldg(qoff + r));
       const int bra = __ldg(Ls.sorted + bra_s), ket = __ldg(Ls.sorted + ket_s);
-      if constexpr (PER) {
-        PerQuartet pq;
-        keep = per_quartet(Ls, bra, ket, pq);  // a density block exists for its cell offset
-      } else {
-        const double pm = pmax4(Ls, __ldg(Ls.pa.sa + bra), __ldg(Ls.pa.sb + bra), __ldg(Ls.pa.sa + ket),
-                                __ldg(Ls.pa.sb + ket));
-        keep = !(skip && pm == 0.0) && !(dens > 0.0 && __ldg(Ls.Qs + bra_s) * __ldg(Ls.Qs + ket_s) * pm < dens) &&
-               dist_keeps(Ls, bra_s, ket_s) && pass_takes<PREC>(Ls, bra_s, ket_s, pm);
-      }
+      const double pm = pmax4(Ls, __ldg(Ls.pa.sa + bra), __ldg(Ls.pa.sb + bra), __ldg(Ls.pa.sa + ket),
+                              __ldg(Ls.pa.sb + ket));
+      keep = !(skip && pm == 0.0) && !(dens > 0.0 && __ldg(Ls.Qs + bra_s) * __ldg(Ls.Qs + ket_s) * pm < dens) &&
+             dist_keeps(Ls, bra_s, ket_s) && pass_takes<PREC>(Ls, bra_s, ket_s, pm);
       npq = __ldg(Ls.pa.prim_n + bra) * __ldg(Ls.pa.prim_n + ket);
     }
     const unsigned m = __ballot_sync(0xffffffffu, keep);
     if (keep) Q.q[Q.n + __popc(m & ((1u << lane) - 1u))] = make_int4(sys, bra_s, ket_s, npq);
     Q.n += __popc(m);
     __syncwarp();
-    g1_drain<BATCH, R, PER>(L, ci, Q, lane, Sd, st, t, false);
+    g1_drain<BATCH, R>(L, ci, Q, lane, Sd, st, t, false);
   }
 }
 
-// Quartets [q0, q1) of the launch record Ls, one warp: the warp takes them one by one.
-// ci and sv: the launch's class record and schedule variant.
-template <int PREC>
+// Quartets [q0, q1) of the launch record Ls that qualify for FP32, one warp: the warp takes
+// them one by one.  ci and sv: the launch's class record and schedule variant.
 __device__ __forceinline__ void g32_range(const EriClassInfo& ci, const SchedVariant& sv, const EriLaunch& Ls,
-                                          long long q0, long long q1, double* S, double* CF, int lane, Tally& t) {
+                                          long long q0, long long q1, double* S, int lane, Tally& t) {
   if (q0 >= q1) return;
   int r = find_row(Ls.qoff, Ls.row_begin, Ls.row_end, q0);
   for (long long q = q0; q < q1; ++q) {
@@ -743,107 +501,29 @@ __device__ __forceinline__ void g32_range(const EriClassInfo& ci, const SchedVar
     if (Ls.dens_tau > 0.0 && __ldg(Ls.Qs + bra_s) * __ldg(Ls.Qs + ket_s) * pm < Ls.dens_tau) continue;
     // distance-aware screening (off when dist_tau = 0)
     if (!dist_keeps(Ls, bra_s, ket_s)) continue;
-    // mixed precision: this pass's share of the quartets (warp-uniform decision)
-    if (!pass_takes<PREC>(Ls, bra_s, ket_s, pm)) continue;
+    if (!fp32_eligible(Ls, bra_s, ket_s, pm)) continue;  // warp-uniform
     const int npq = __ldg(Ls.pa.prim_n + bra) * __ldg(Ls.pa.prim_n + ket);
-    const bool f32 = PREC == PREC_MIXED32;
-    int ne;
-    if (f32)
-      ne = contract_g32_xw<HFX_FP32_PACK>(ci, sv, Ls, bra, ket, S, S + (HFX_FP32_PACK / 2) * sv.group, lane);
-    else
-      ne = contract_g32<false>(ci, sv, Ls, bra, ket, S, CF, lane);
+    const int ne =
+        contract_g32_xw<HFX_FP32_PACK>(ci, sv, Ls, bra, ket, S, S + (HFX_FP32_PACK / 2) * sv.group, lane);
     t.prim += ne;
     t.skip += npq - ne;
     if (!ne) continue;
     ++t.quart;
-    if (f32) {
-      ++t.q32;
-      t.p32 += ne;
-    }
+    ++t.q32;
+    t.p32 += ne;
     double deg = 1.0;
     if (sa == sb) deg *= 0.5;
     if (sc == sd) deg *= 0.5;
     if (bra_s == ket_s) deg *= 0.5;
     const int A = __ldg(Ls.sh.bf_off + sa), B = __ldg(Ls.sh.bf_off + sb);
     const int C = __ldg(Ls.sh.bf_off + sc), D = __ldg(Ls.sh.bf_off + sd);
-    // an FP32 quartet leaves its final block in FP64 too (see contract_g32)
+    // the contracted block is in FP64 (see contract_g32_xw)
     digest(ci, S + ci.out_base, 1, A, B, C, D, deg, Ls.P, Ls.K, Ls.ld, lane, 32);
     __syncwarp();
   }
 }
 
-// Periodic quartets [q0, q1) of the launch (FP64), one warp per quartet.
-__device__ __forceinline__ void g32_range_per(const EriClassInfo& ci, const SchedVariant& sv, const EriLaunch& Ls,
-                                              long long q0, long long q1, double* S, double* CF, int lane, Tally& t) {
-  if (q0 >= q1) return;
-  int r = find_row(Ls.qoff, Ls.row_begin, Ls.row_end, q0);
-  for (long long q = q0; q < q1; ++q) {
-    while (__ldg(Ls.qoff + r + 1) <= q) ++r;
-    const int bra_s = Ls.bra_bin_start + (r - Ls.row_begin);
-    const int ket_s = Ls.ket_bin_start + (int)(q - __ldg(Ls.qoff + r));
-    const int bra = __ldg(Ls.sorted + bra_s), ket = __ldg(Ls.sorted + ket_s);
-    PerQuartet pq;
-    if (!per_quartet(Ls, bra, ket, pq)) continue;
-    const int npq = __ldg(Ls.pa.prim_n + bra) * __ldg(Ls.pa.prim_n + ket);
-    const int ne = contract_g32<true>(ci, sv, Ls, bra, ket, S, CF, lane);
-    t.prim += ne;
-    t.skip += npq - ne;
-    if (!ne) continue;
-    ++t.quart;
-    digest_per(ci, S + ci.out_base, 1, pq, Ls.KG, Ls.per.nbf, lane, 32);
-    __syncwarp();
-  }
-}
-
-// The quartet ranges a warp works on.  Static schedules: one range (group_range).
-// Dynamic: chunks claimed from the launch's device counter.  Batched (L.n_sys > 0): chunks
-// of the systems' concatenated quartet lists; a chunk is split at system boundaries
-// (L.seg[s] = first index of system s) and each part runs with that system's record.
-template <bool BATCH, int GS, class F>
-__device__ __forceinline__ void for_each_range(const EriLaunch& L, long long wid, long long nw, int lane, unsigned gm,
-                                               F&& f) {
-  if (!BATCH && L.schedule != 2) {
-    long long q0, q1;
-    group_range(L, wid, nw, q0, q1);
-    f(L, 0, q0, q1);
-    return;
-  }
-  const long long total = L.q_count;
-  while (true) {
-    unsigned long long c = 0;
-    if (lane == 0) c = atomicAdd(L.work, (unsigned long long)L.chunk);
-    c = __shfl_sync(gm, c, 0, GS);
-    long long c0 = (long long)c;
-    if (c0 >= total) break;
-    const long long c1 = min(c0 + L.chunk, total);
-    if constexpr (!BATCH) {
-      f(L, 0, L.q_begin + c0, L.q_begin + c1);
-    } else {
-      while (c0 < c1) {
-        int lo = 0, hi = L.n_sys - 1;  // last s with seg[s] <= c0
-        while (lo < hi) {
-          const int mid = (lo + hi + 1) >> 1;
-          if (__ldg(L.seg + mid) <= c0) lo = mid; else hi = mid - 1;
-        }
-        const long long e = min(c1, __ldg(L.seg + lo + 1));
-        const EriLaunch& Ls = L.batch[lo];
-        f(Ls, lo, Ls.q_begin + (c0 - __ldg(L.seg + lo)), Ls.q_begin + (e - __ldg(L.seg + lo)));
-        c0 = e;
-      }
-    }
-  }
-}
-
-__device__ __forceinline__ void flush_tally(const EriLaunch& L, const Tally& t) {
-  if (!L.counters) return;
-  atomicAdd(L.counters + 0, t.prim);
-  atomicAdd(L.counters + 1, t.quart);
-  atomicAdd(L.counters + 2, t.skip);
-  atomicAdd(L.counters + 3, t.q32);
-  atomicAdd(L.counters + 4, t.p32);
-}
-
-template <int MODE, int PREC, bool BATCH, bool PER = false>
+template <int PREC, bool BATCH>
 __global__ void __launch_bounds__(64, PREC == PREC_MIXED32 ? HFX_G1F_MINB : (BATCH ? HFX_G1B_MINB : HFX_G1_MINB))
     eri_g1_kernel(const EriLaunch L) {
   extern __shared__ double smem[];
@@ -853,59 +533,34 @@ __global__ void __launch_bounds__(64, PREC == PREC_MIXED32 ? HFX_G1F_MINB : (BAT
   const long long ng = (long long)gridDim.x * blockDim.x;
   unsigned long long t0 = 0;
   if (L.busy && threadIdx.x == 0) t0 = globaltimer_ns();
-  if (MODE == 0) {
-    using R = typename std::conditional<PREC == PREC_MIXED32, float, double>::type;
-    const int lane = threadIdx.x & 31;
-    Tally t;
-    G1Queue Q{reinterpret_cast<int4*>(smem + (size_t)L.ci.scratch * blockDim.x) + (threadIdx.x >> 5) * 64, 0};
-    for_each_range<BATCH, 32>(L, gid >> 5, ng >> 5, lane, 0xffffffffu,
-                              [&](const EriLaunch& Ls, int sys, long long q0, long long q1) {
-                                g1_range<BATCH, PREC, R, PER>(L, L.ci, Ls, sys, q0, q1, Sd, st, lane, Q, t);
-                              });
-    g1_drain<BATCH, R, PER>(L, L.ci, Q, lane, Sd, st, t, true);
-    flush_tally(L, t);
-  } else {
-    for (long long t = gid; t < L.diag_n; t += ng) {
-      const int p = __ldg(L.diag_list + t);
-      double mx = 0.0;
-      if (contract_g1<double>(L.ci, L, p, p, Sd, st)) mx = diag_max(L.ci, Sd + L.ci.out_base * st, st);
-      L.diag_Q[p] = sqrt(mx);
-    }
-  }
+  using R = typename std::conditional<PREC == PREC_MIXED32, float, double>::type;
+  const int lane = threadIdx.x & 31;
+  Tally t;
+  G1Queue Q{reinterpret_cast<int4*>(smem + (size_t)L.ci.scratch * blockDim.x) + (threadIdx.x >> 5) * 64, 0};
+  for_each_range<BATCH, 32>(L, gid >> 5, ng >> 5, lane, 0xffffffffu,
+                            [&](const EriLaunch& Ls, int sys, long long q0, long long q1) {
+                              g1_range<BATCH, PREC, R>(L, L.ci, Ls, sys, q0, q1, Sd, st, lane, Q, t);
+                            });
+  g1_drain<BATCH, R>(L, L.ci, Q, lane, Sd, st, t, true);
+  flush_tally(L, t);
   record_busy(L, t0);
 }
 
-template <int MODE, int PREC, bool BATCH, bool PER = false>
-__global__ void __launch_bounds__(64, BATCH ? HFX_G32B_MINB : (PREC == PREC_MIXED32 ? HFX_G32F_MINB : HFX_G32_MINB))
-    eri_g32_kernel(const EriLaunch L) {
+// FP32 pass of a mixed-precision class
+template <bool BATCH>
+__global__ void __launch_bounds__(64, HFX_G32F_MINB) eri_g32_kernel(const EriLaunch L) {
   extern __shared__ __align__(16) double smem[];
   const int lane = threadIdx.x & 31, grp = threadIdx.x >> 5;
   const int gpb = blockDim.x >> 5;
-  double* S = smem + grp * g32_stride(L.sv, PREC);
-  double* CF = S + L.sv.group;
-  const long long gid = (long long)blockIdx.x * gpb + grp;
-  const long long ng = (long long)gridDim.x * gpb;
+  double* S = smem + grp * g32_stride(L.sv);
   unsigned long long t0 = 0;
   if (L.busy && threadIdx.x == 0) t0 = globaltimer_ns();
-  if (MODE == 0) {
-    Tally t;
-    for_each_range<BATCH, 32>(L, gid, ng, lane, 0xffffffffu,
-                              [&](const EriLaunch& Ls, int, long long q0, long long q1) {
-                                if constexpr (PER)
-                                  g32_range_per(L.ci, L.sv, Ls, q0, q1, S, CF, lane, t);
-                                else
-                                  g32_range<PREC>(L.ci, L.sv, Ls, q0, q1, S, CF, lane, t);
-                              });
-    if (lane == 0) flush_tally(L, t);
-  } else {
-    for (long long t = gid; t < L.diag_n; t += ng) {
-      const int p = __ldg(L.diag_list + t);
-      double mx = 0.0;
-      if (contract_g32<false>(L.ci, L.sv, L, p, p, S, CF, lane)) mx = diag_max(L.ci, S + L.ci.out_base, 1);
-      if (lane == 0) L.diag_Q[p] = sqrt(mx);
-      __syncwarp();
-    }
-  }
+  Tally t;
+  for_each_range<BATCH, 32>(L, (long long)blockIdx.x * gpb + grp, (long long)gridDim.x * gpb, lane, 0xffffffffu,
+                            [&](const EriLaunch& Ls, int, long long q0, long long q1) {
+                              g32_range(L.ci, L.sv, Ls, q0, q1, S, lane, t);
+                            });
+  if (lane == 0) flush_tally(L, t);
   record_busy(L, t0);
 }
 
@@ -914,16 +569,12 @@ __global__ void __launch_bounds__(64, BATCH ? HFX_G32B_MINB : (PREC == PREC_MIXE
 // ---------------------------------------------------------------------------
 static const int kBlock = 64;
 
-int eri_group_size(int cls) {
-  // thread-per-quartet for classes whose scratch fits comfortably; warp otherwise
-  return kClassInfo[cls].scratch <= HFX_G1_MAX_SCRATCH ? 1 : 32;
-}
+// Whole warps in every class.  The thread kernel was the default of the nine lowest classes
+// before the Hermite engine, which measured faster in all of them (64-atom diamond, (ss|ss)
+// 17.0 -> 11.2 ms, (pp|ps) 219 -> 129 ms, (dd|ss) 44 -> 26 ms); it runs where a caller asks for it.
+// Groups of 8 or 16 lanes were slower than either in every class.
+int eri_group_size() { return 32; }
 
-// Groups of 8 or 16 lanes (several quartets per warp) were measured on the 64-atom diamond:
-// 1.1x to 10x slower than whole warps in every warp-group class and slower than one thread
-// per quartet in the others, because each group needs its own scratch and coefficient
-// sets, so shared memory caps the resident warps.  The kernel keeps the group size as a
-// template parameter; only 32 is built.
 bool eri_group_size_valid(int gs) { return gs == 1 || gs == 32; }
 
 // Streams of the warp kernel per class (primitive quartets run at a time).  Defaults from a
@@ -958,31 +609,35 @@ int eri_streams(int cls, int streams) {
   return i < 0 ? 0 : kSchedInfo[cls][i].k;
 }
 
-// The kernel instance for a class launch.  gs: lanes per quartet (1 = a thread, 32 = a warp);
-// mode 1 = Schwarz diagonal; prec: precision pass; batch = quartets of several systems.
-template <int PREC>
-static const void* kernel_ptr_p(int gs, bool batch) {
-  if (gs == 1) return batch ? (const void*)eri_g1_kernel<0, PREC, true> : (const void*)eri_g1_kernel<0, PREC, false>;
-  return batch ? (const void*)eri_g32_kernel<0, PREC, true> : (const void*)eri_g32_kernel<0, PREC, false>;
+// The kernel instance for a class launch: FP64 quartets on whole warps run on the Hermite engine
+// (md_*), the FP32 pass on the packed warp kernel, gs = 1 on the thread kernel.
+static bool uses_md(int gs, int prec) { return gs != 1 && prec != PREC_MIXED32; }
+
+static int md_kind(int mode, int prec, bool batch) {
+  return mode == 1 ? MD_DIAG : prec == PREC_PERIODIC ? MD_PER : batch ? MD_BATCH : MD_PLAIN;
 }
 
-static const void* kernel_ptr(int mode, int gs, int prec, bool batch) {
-  if (mode == 1) return gs == 1 ? (const void*)eri_g1_kernel<1, 0, false> : (const void*)eri_g32_kernel<1, 0, false>;
-  if (prec == PREC_PERIODIC)
-    return gs == 1 ? (const void*)eri_g1_kernel<0, 0, false, true> : (const void*)eri_g32_kernel<0, 0, false, true>;
-  if (prec == PREC_MIXED64) return kernel_ptr_p<PREC_MIXED64>(gs, batch);
-  if (prec == PREC_MIXED32) return kernel_ptr_p<PREC_MIXED32>(gs, batch);
-  return kernel_ptr_p<PREC_FP64>(gs, batch);
+template <int PREC>
+static const void* g1_ptr(bool batch) {
+  return batch ? (const void*)eri_g1_kernel<PREC, true> : (const void*)eri_g1_kernel<PREC, false>;
+}
+
+static const void* kernel_ptr(int gs, int prec, bool batch) {
+  if (gs != 1) return batch ? (const void*)eri_g32_kernel<true> : (const void*)eri_g32_kernel<false>;
+  if (prec == PREC_MIXED64) return g1_ptr<PREC_MIXED64>(batch);
+  if (prec == PREC_MIXED32) return g1_ptr<PREC_MIXED32>(batch);
+  return g1_ptr<PREC_FP64>(batch);
 }
 
 static int effective_gs(int gs) { return gs == 1 ? 1 : 32; }
 
 size_t eri_smem_bytes(int cls, int gs, int streams, int prec) {
+  if (uses_md(gs, prec)) return md_smem_bytes(cls);
   // one quartet per thread: interleaved scratch, then a 64-entry quartet queue per warp
   if (gs == 1) return sizeof(double) * (size_t)kClassInfo[cls].scratch * kBlock + sizeof(int4) * 64 * (kBlock / 32);
   const int i = variant_index(cls, streams);
   if (i < 0) return (size_t)1 << 30;
-  return sizeof(double) * (size_t)g32_stride(kSchedInfo[cls][i], prec) * (kBlock / 32);
+  return sizeof(double) * (size_t)g32_stride(kSchedInfo[cls][i]) * (kBlock / 32);
 }
 
 int eri_block_size() { return kBlock; }
@@ -993,26 +648,26 @@ cudaError_t eri_prepare() {
   for (int c = 0; c < HFX_N_CLASSES; ++c) {
     mx = std::max(mx, eri_smem_bytes(c, 1, 0));
     for (int i = 0; i < 3; ++i)
-      if (kSchedInfo[c][i].k) mx = std::max(mx, eri_smem_bytes(c, 32, kSchedInfo[c][i].k));
+      if (kSchedInfo[c][i].k) mx = std::max(mx, eri_smem_bytes(c, 32, kSchedInfo[c][i].k, PREC_MIXED32));
   }
   if (mx > 227 * 1024) mx = 227 * 1024;
-  for (int gs : {1, 32}) {
-    cudaError_t e = cudaFuncSetAttribute(kernel_ptr(1, gs, 0, false), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)mx);
-    if (e != cudaSuccess) return e;
-    for (int prec = 0; prec < 4; ++prec)
-      for (int batch = 0; batch < (prec == PREC_PERIODIC ? 1 : 2); ++batch) {
-        e = cudaFuncSetAttribute(kernel_ptr(0, gs, prec, batch), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mx);
-        if (e != cudaSuccess) return e;
-      }
+  cudaError_t e = md_prepare();
+  if (e != cudaSuccess) return e;
+  auto allow = [&](const void* k) {
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mx);
+  };
+  for (bool batch : {false, true}) {
+    allow(kernel_ptr(32, PREC_MIXED32, batch));
+    for (int prec : {PREC_FP64, PREC_MIXED64, PREC_MIXED32}) allow(kernel_ptr(1, prec, batch));
   }
-  return cudaSuccess;
+  return e;
 }
 
 int eri_blocks_per_sm(int cls, int mode, int gs, int prec, bool batch, int streams) {
-  int n = 0;
   const int g = effective_gs(gs);
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel_ptr(mode, g, prec, batch), kBlock,
+  if (uses_md(g, prec)) return md_blocks_per_sm(cls, md_kind(mode, prec, batch));
+  int n = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel_ptr(g, prec, batch), kBlock,
                                                     eri_smem_bytes(cls, g, streams, prec)) != cudaSuccess)
     return 1;
   return n > 0 ? n : 1;
@@ -1020,16 +675,25 @@ int eri_blocks_per_sm(int cls, int mode, int gs, int prec, bool batch, int strea
 
 int eri_groups_per_block(int gs) { return kBlock / effective_gs(gs); }
 
+// Quartets per claim of the dynamic schedule.  A thread-kernel warp takes 256.  A whole warp takes
+// at most 32 (it tests a claim's quartets with a lane each) and at least 1: a 32nd of an even
+// share of the list, so that the last claims of a launch, while the other warps are done, stay a
+// few per cent of it also for the smallest systems, where a claim of 8 left most warps without one.
+int eri_chunk(int gs, long long n_quartets, long long n_groups) {
+  if (gs == 1) return 256;
+  return (int)std::max(1LL, std::min(32LL, n_quartets / (32 * std::max(1LL, n_groups))));
+}
+
 cudaError_t eri_launch(const EriLaunch& L0, int cls, int mode, int grid, cudaStream_t stream, int gs, int prec,
                        bool batch, int streams) {
   const int g = effective_gs(gs);
+  if (uses_md(g, prec)) return md_launch(L0, cls, md_kind(mode, prec, batch), prec, grid, stream);
   const size_t smem = eri_smem_bytes(cls, g, streams, prec);
   if (smem > 227 * 1024) return cudaErrorInvalidValue;
-  const void* k = kernel_ptr(mode, g, prec, batch);
   EriLaunch L = L0;
   if (g == 32) L.sv = kSchedInfo[cls][variant_index(cls, streams)];
   void* args[] = {(void*)&L};
-  return cudaLaunchKernel(k, dim3(grid), dim3(kBlock), args, smem, stream);
+  return cudaLaunchKernel(kernel_ptr(g, prec, batch), dim3(grid), dim3(kBlock), args, smem, stream);
 }
 
 }  // namespace hfx

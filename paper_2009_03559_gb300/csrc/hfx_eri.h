@@ -9,7 +9,7 @@ struct EriLaunch;
 
 // Group sizes (lanes per quartet): 1 (a thread) or 32 (a warp).  Precision passes `prec`:
 // 0 every quartet in FP64; 1 and 2 the FP64 and FP32 shares of a mixed-precision class.
-int eri_group_size(int cls);  // default for a class: 1 or 32
+int eri_group_size();  // the default: 32
 bool eri_group_size_valid(int gs);
 size_t eri_smem_bytes(int cls, int gs, int streams = 0, int prec = 0);
 int eri_block_size();
@@ -20,6 +20,19 @@ int eri_blocks_per_sm(int cls, int mode, int gs, int prec, bool batch, int strea
 int eri_streams(int cls, int streams);
 bool eri_streams_valid(int cls, int streams);
 int eri_groups_per_block(int gs);
+// quartets per claim of the dynamic schedule, for a list of n_quartets and n_groups groups
+int eri_chunk(int gs, long long n_quartets, long long n_groups);
+
+// The Hermite engine (FP64 quartets on whole warps, hfx_md.cuh) and its pair data.
+// Kinds of launch: one system, a batch of systems, a lattice sum, the Schwarz diagonal.
+enum { MD_PLAIN = 0, MD_BATCH = 1, MD_PER = 2, MD_DIAG = 3 };
+size_t md_smem_bytes(int cls);
+cudaError_t md_prepare();
+int md_blocks_per_sm(int cls, int kind);
+cudaError_t md_launch(const EriLaunch& L, int cls, int kind, int prec, int grid, cudaStream_t stream);
+cudaError_t launch_md_size(int n, const int* pcls, const int* cap, long long* size, cudaStream_t s);
+cudaError_t launch_md_fill(int n, const int* pcls, const double* AB, const int* pp_off, const int* pp_n,
+                           const PrimPair* pp, const long long* md_off, double* md, cudaStream_t s);
 
 }  // namespace hfx
 

@@ -27,6 +27,23 @@ struct EriClassInfo {
 
 extern const EriClassInfo* class_info_host();
 
+// Hermite engine (generated tables, see gen_md_tables.py): the steps of a class ...
+struct MdClassInfo {
+  int Lt;
+  int kc, n_kc, bc, n_bc;              // contraction tables (first entry, entries)
+  int n_row, nab, ncd;                 // rows of Y, function pairs of bra and ket
+  int bra_coef0, bra_coef, bra_set;    // bra pair type: first coefficient, coefficients, sets
+  int ket_coef, ket_set;
+  int z1_round, z1_n, z1_dst, z2_round, z2_n, z2_dst;  // transformation passes
+};
+// ... and the sets and coefficients of a pair type (set: power of 1/2p | of u_b << 4 | of u_a << 8)
+struct MdPairInfo {
+  int coef0, n_coef, n_set;
+  int set[14];
+};
+extern const MdClassInfo* md_class_host();
+extern const MdPairInfo* md_pair_host();
+
 // ---------------------------------------------------------------------------
 // Boys function tables, one per order L = 0..kMaxLt, rows at x_g = g h (h = 1/32,
 // g = 0..kBoysRows-1).  Row g of table L holds the coefficients of the Taylor expansions
@@ -56,6 +73,7 @@ struct __align__(16) PrimPair {
   double PA[3];        // P - A (A = centre of the pair's first shell)
   double C;            // prefactor (see above)
   double inv2p3;       // 3/(2p)
+  double ua, ub;       // a/p and b/p, a and b the exponents of the pair's two shells
   // FP32 copies for the FP32 recurrences
   float pf, inv2pf, PAf[3], Pf[3];
 };
@@ -68,6 +86,8 @@ struct PairArrays {
   const int* prim_n;        // number of surviving primitive pairs
   const double* AB;         // 3 per pair: A - B
   const PrimPair* prim;     // primitive-pair records
+  const long long* md_off;  // first double of the pair's Hermite data in md: the coefficients T of its
+  const double* md;         // type, then the factors W of every surviving primitive pair
 };
 
 struct ShellArrays {
@@ -197,7 +217,9 @@ struct EriLaunch {
   int chunk;                  // schedule 2: quartets per claim
   const double* boys;         // kMaxLt + 1 tables of kBoysTableLen doubles
   double omega, omega2;
-  SchedVariant sv;             // warp kernel: the schedule variant of this class
+  SchedVariant sv;             // packed FP32 warp kernel: the schedule variant of this class
+  MdClassInfo mc;              // FP64 warp kernel: the steps of this class
+  int prec;                    // precision pass (PREC_*)
   const double* P;
   double* K;
   int ld;

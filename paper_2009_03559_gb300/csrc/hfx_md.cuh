@@ -1,0 +1,545 @@
+// Hermite engine: the FP64 warp kernel (one warp evaluates and digests a stream of quartets).
+//
+// What bounds it: the FP64 pipe, one warp instruction per 64 cycles and SM quarter whatever the
+// number of active lanes, so the algorithm with the fewest FP64 warp instructions wins and a
+// handful of resident warps hides everything else (an FMA chain on one warp per quarter already
+// runs at the full rate).  The Hermite form (tables: gen_md_tables.py) contracts over the
+// primitives before it transforms, which leaves (dp|dp) 320 + 225 lane operations per primitive
+// quartet where the Obara-Saika schedule had 2053, and keeps the recursion on the lanes' own
+// registers: no interpreted op, no idle lane.
+//
+// A warp runs a stream of primitive quartets that crosses quartet borders, 32 at a time:
+//   set-up and Hermite recursion, a lane per primitive quartet (results to shared memory);
+//   per run of lanes of one (quartet, bra primitive pair): ket contraction, a lane per H value;
+//   at the end of a bra primitive pair: bra contraction; at the end of a quartet: the two
+//   transformation passes and the digest.
+#pragma once
+#include <type_traits>
+#include "eri_quartets.cuh"
+#include "hfx_eri.h"
+
+namespace hfx {
+
+#define HFX_N_CLASSES 21
+#define HFX_TABLE_QUAL __device__ __align__(16) const
+#include "md_tables.inc"
+#undef HFX_TABLE_QUAL
+
+// n S for a small integer n: doubling and quadrupling are exponent increments (integer pipe).
+// S = 0 or subnormal becomes at most 4 x 2^-1022: nothing next to any integral.
+template <int N>
+__device__ __forceinline__ double times(double x) {
+  if constexpr (N == 1) return x;
+  if constexpr (N == 2) return scale2(x, 1);
+  if constexpr (N == 4) return scale2(x, 2);
+  return x * N;
+}
+
+// compile-time loop: f(integral constant I), ..., f(integral constant N - 1)
+template <int I, int N, class F>
+__device__ __forceinline__ void unrolled(F&& f) {
+  if constexpr (I < N) {
+    f(std::integral_constant<int, I>());
+    unrolled<I + 1, N>(f);
+  }
+}
+
+__host__ __device__ constexpr int n_herm(int n) { return (n + 1) * (n + 2) * (n + 3) / 6; }
+// position of Hermite index (x, y, z) in the list of all by order (x descending, then y)
+__host__ __device__ constexpr int herm_index(int x, int y, int z) {
+  const int n = x + y + z;
+  return n * (n + 1) * (n + 2) / 6 + (n - x) * (n - x + 1) / 2 + (n - x - y);
+}
+
+// S_r, |r| <= L, from the base values B[m] = (2 rho)^m G_m:  rows in m, first along z, from each
+// of them along y, from each of those along x; only the last two rows of a chain stay live.
+template <int L>
+__device__ __forceinline__ void hermite(const double (&B)[L + 1], double X, double Y, double Z, double* out) {
+  double zr[L + 1], zp[L + 1];
+#pragma unroll
+  for (int m = 0; m <= L; ++m) zr[m] = B[m];
+  unrolled<0, L + 1>([&](auto cv) {
+    constexpr int V = decltype(cv)::value;
+    double yr[L + 1 - V], yp[L + 1 - V];
+#pragma unroll
+    for (int m = 0; m <= L - V; ++m) yr[m] = zr[m];
+    unrolled<0, L + 1 - V>([&](auto cu) {
+      constexpr int U = decltype(cu)::value;
+      constexpr int N = L - V - U;
+      double xr[N + 1], xp[N + 1];
+#pragma unroll
+      for (int m = 0; m <= N; ++m) xr[m] = yr[m];
+      unrolled<0, N + 1>([&](auto ct) {
+        constexpr int T = decltype(ct)::value;
+        out[herm_index(T, U, V)] = xr[0];
+#pragma unroll
+        for (int m = 0; m < N - T; ++m) {
+          double v;
+          if constexpr (T == 0)
+            v = X * xr[m + 1];
+          else
+            v = fma(X, xr[m + 1], -times<T>(xp[m + 1]));
+          xp[m] = xr[m];
+          xr[m] = v;
+        }
+        if constexpr (N - T > 0) xp[N - T] = xr[N - T];
+      });
+#pragma unroll
+      for (int m = 0; m < N; ++m) {
+        double v;
+        if constexpr (U == 0)
+          v = Y * yr[m + 1];
+        else
+          v = fma(Y, yr[m + 1], -times<U>(yp[m + 1]));
+        yp[m] = yr[m];
+        yr[m] = v;
+      }
+      if constexpr (N > 0) yp[N] = yr[N];
+    });
+#pragma unroll
+    for (int m = 0; m < L - V; ++m) {
+      double v;
+      if constexpr (V == 0)
+        v = Z * zr[m + 1];
+      else
+        v = fma(Z, zr[m + 1], -times<V>(zp[m + 1]));
+      zp[m] = zr[m];
+      zr[m] = v;
+    }
+    if constexpr (L - V > 0) zp[L - V] = zr[L - V];
+  });
+}
+
+// Set-up of one primitive quartet: B[m] = (2 rho)^m G_m, the base values of the Hermite
+// recursion, with G_m = pref (F_m(T) - kappa^{m+1/2} F_m(kappa T)) (see prim_core, whose downward
+// recursion this is, multiplied through by (2 rho)^m):
+//   B_{m-1} = (R^2 B_m + a_m - c_m e^{-kappa T}) / (2m-1),
+//   a_m = pref (2 rho)^{m-1} e^{-T},  c_m = pref (2 rho)^{m-1} kappa^{m-1/2}.
+// False if the quartet is negligible (kappa T beyond the tables: G_m < e^{-60}).
+template <int L>
+__device__ __forceinline__ bool md_setup(const PrimPair& b, const PrimPair& k, const double* qc, double omega,
+                                         double omega2, const double* __restrict__ tabs, double (&B)[L + 1],
+                                         double* PQ) {
+  const double p = b.p, q = k.p;
+  const double y = rsqrt_nr(p + q);  // 1/sqrt(p+q)
+  const double rho = (p * y) * (q * y);
+  PQ[0] = b.P[0] - qc[0];
+  PQ[1] = b.P[1] - qc[1];
+  PQ[2] = b.P[2] - qc[2];
+  const double R2 = fma(PQ[0], PQ[0], fma(PQ[1], PQ[1], PQ[2] * PQ[2]));
+  const double T = rho * R2;
+  const double pref = (b.C * k.C) * y;
+  const double* tabL = tabs + L * kBoysTableLen;
+  double kap = 0.0, sk = 0.0, kT = 0.0;
+  if (omega2 > 0.0) {
+    sk = omega * rsqrt_nr(omega2 + rho);  // sqrt(kappa)
+    kap = sk * sk;
+    kT = kap * T;
+    if (ge_hi(kT, kBoysXmaxHi)) return false;
+  }
+  double F1, e1 = 0.0;
+  if (!ge_hi(T, kBoysXmaxHi))
+    boys_top(T, tabL, F1, e1);
+  else
+    F1 = boys_asym(L, T);
+  const double r2 = scale2(rho, 1);
+  double pL = pref;  // pref (2 rho)^L
+  if constexpr (L > 0) {
+    double w = r2;
+    pL = (L & 1) ? pref * r2 : pref;
+#pragma unroll
+    for (int i = 1; (L >> i) > 0; ++i) {
+      w = w * w;
+      if ((L >> i) & 1) pL *= w;
+    }
+  }
+  double a[L + 1], g = pL * F1;
+  a[0] = pref * e1;
+#pragma unroll
+  for (int m = 1; m < L; ++m) a[m] = a[m - 1] * r2;
+  if (omega2 > 0.0) {
+    double F2, e2;
+    boys_top(kT, tabL, F2, e2);
+    const double kr = kap * r2;
+    double c[L + 1];
+    c[0] = pref * sk;
+#pragma unroll
+    for (int m = 1; m <= L; ++m) c[m] = c[m - 1] * kr;
+    g = fma(-c[L], F2, g);
+#pragma unroll
+    for (int m = 0; m < L; ++m) a[m] = fma(-c[m], e2, a[m]);
+  }
+  B[L] = g;
+#pragma unroll
+  for (int m = L; m >= 1; --m) {
+    g = fma(R2, g, a[m - 1]);
+    if (m > 1) g *= 1.0 / (2 * m - 1);
+    B[m - 1] = g;
+  }
+  return true;
+}
+
+// Shared memory of one warp, in doubles (offsets; every region starts on an even double).
+struct MdLayout {
+  int rs, ws;                 // strides of a primitive quartet's Hermite integrals and ket factors
+  int R, W, H, A, Tb, Tk, Q;  // H also holds Y, A also the final block
+  int size;
+};
+constexpr int kMdQueue = 64;  // quartets waiting in a warp's queue
+
+inline MdLayout md_layout(const MdClassInfo& c, const MdPairInfo& b, const MdPairInfo& k) {
+  MdLayout l{};
+  auto even = [](int n) { return (n + 1) & ~1; };
+  l.rs = n_herm(c.Lt) | 1;  // odd: the lanes' columns start in different banks
+  l.ws = k.n_set | 1;
+  l.R = 0;
+  l.W = l.R + 32 * l.rs;
+  l.H = l.W + 32 * l.ws;
+  l.A = l.H + even(std::max(c.n_kc, c.n_row * c.ncd));
+  l.Tb = l.A + even(std::max(c.n_bc, c.nab * c.ncd));
+  l.Tk = l.Tb + even(b.n_coef);
+  l.Q = l.Tk + even(k.n_coef);
+  l.size = l.Q + 2 * kMdQueue;
+  return l;
+}
+
+// A sparse pass out[dst] = sum of T[c] in[i] (generated: rounds of 32 outputs of like length).
+__device__ __forceinline__ void md_gather(int round0, int n_round, int dst0, const double* T, const double* in,
+                                          double* out, int lane) {
+  for (int r = 0; r < n_round; ++r) {
+    const uint32_t rd = __ldg(kMdZRound + round0 + r);
+    const uint32_t* w = kMdZ + (rd & 0xFFFFFFu) + lane;
+    const int n = rd >> 24;
+    double v = 0.0;
+    for (int t = 0; t < n; ++t) {
+      const uint32_t e = __ldg(w + 32 * t);
+      v = fma(T[e & 0xFFFFu], in[e >> 16], v);
+    }
+    const uint32_t d = __ldg(kMdZDst + dst0 + 32 * r + lane);
+    if (d != 0xFFFFu) out[d] = v;
+  }
+}
+
+// Digest of the final block into the half matrix A, a lane per output element of the four
+// blocks; every lane runs the same instructions with its own strides, so the outputs of the
+// four blocks share a round (the longest sum counts).
+__device__ __forceinline__ void md_digest(const EriClassInfo& ci, const double* v, int A, int B, int C, int D,
+                                          double deg, const double* __restrict__ P, double* K, int ld, int lane) {
+  const int na = ci.dims[0], nb = ci.dims[1], nc = ci.dims[2], nd = ci.dims[3];
+  const int sb = nc * nd, sa = nb * sb;
+  const int nAC = na * nc, nAD = na * nd, nBC = nb * nc, nout = nAC + nAD + nBC + nb * nd;
+  for (int o = lane; o < nout; o += 32) {
+    int t = o;
+    bool isA = true, isC = true;  // row function of a (else b), column function of c (else d)
+    if (t >= nAC + nAD) {
+      t -= nAC + nAD;
+      isA = false;
+      if (t >= nBC) {
+        t -= nBC;
+        isC = false;
+      }
+    } else if (t >= nAC) {
+      t -= nAC;
+      isC = false;
+    }
+    const int ny = isC ? nc : nd, x = t / ny, y = t - x * ny;
+    const int su = isA ? sb : sa, nu = isA ? nb : na, sw = isC ? 1 : nd, nw = isC ? nd : nc;
+    const double* vp = v + x * (isA ? sa : sb) + y * (isC ? nd : 1);
+    const double* pp = P + (size_t)(isA ? B : A) * ld + (isC ? D : C);
+    double acc = 0.0;
+    int w = 0;
+    const int n = nu * nw;
+    for (int i = 0; i < n; ++i) {
+      acc = fma(vp[w * sw], __ldg(pp + w), acc);
+      if (++w == nw) {
+        w = 0;
+        vp += su;
+        pp += ld;
+      }
+    }
+    atomicAdd(K + (size_t)((isA ? A : B) + x) * ld + (isC ? C : D) + y, deg * acc);
+  }
+}
+
+
+#ifndef HFX_MD_MINB_LO
+#define HFX_MD_MINB_LO 8
+#endif
+#ifndef HFX_MD_MINB_HI
+#define HFX_MD_MINB_HI 4
+#endif
+constexpr int kMdBlock = 64;
+
+template <int LT, int KIND>
+__global__ void __launch_bounds__(kMdBlock, LT <= 4 ? HFX_MD_MINB_LO : HFX_MD_MINB_HI)
+    eri_md_kernel(const __grid_constant__ EriLaunch L, const __grid_constant__ MdLayout ly) {
+  extern __shared__ __align__(16) double smem[];
+  const int lane = threadIdx.x & 31, grp = threadIdx.x >> 5;
+  double* S = smem + grp * ly.size;
+  double* const Rb = S + ly.R;
+  double* const Wb = S + ly.W;
+  double* const H = S + ly.H;
+  double* const A = S + ly.A;
+  int4* const Q = reinterpret_cast<int4*>(S + ly.Q);  // system, bra position, ket position, nb | nk << 16
+  const unsigned lt_mask = (1u << lane) - 1u;
+  const MdClassInfo mc = L.mc;
+  unsigned long long t0 = 0;
+  if (L.busy && threadIdx.x == 0) t0 = globaltimer_ns();
+
+  int head = 0, head_off = 0, tail = 0, waiting = 0;  // queue: entries [head, tail), primitive quartets left
+  bool h_valid = false, a_valid = false;              // the head quartet's H and A hold partial sums
+  int n_eval = 0;                                     // its primitive quartets evaluated so far
+  int tb_sys = -1, tb_bra = -1;                       // whose transformation is in Tb
+  Tally tally;
+
+  auto rec = [&](int sys) -> const EriLaunch& {
+    if constexpr (KIND == MD_BATCH)
+      return L.batch[sys];
+    else
+      return L;
+  };
+  auto pair_id = [&](const EriLaunch& Ls, int pos) -> int {
+    if constexpr (KIND == MD_DIAG)
+      return pos;
+    else
+      return __ldg(Ls.sorted + pos);
+  };
+
+  // H[s, r] (+)= sum over the primitive quartets in slots [p0, p1) of W_s S_r
+  auto ket_contract = [&](int p0, int p1) {
+    auto rounds = [&](int g, auto nc) {
+      constexpr int N = decltype(nc)::value;
+      int ri[N], si[N];
+      double v[N];
+#pragma unroll
+      for (int u = 0; u < N; ++u) {
+        const int e = __ldg(kMdKc + mc.kc + g + 32 * u + lane);  // padded to whole rounds
+        ri[u] = e & 0xFF;
+        si[u] = e >> 8;
+        v[u] = 0.0;
+      }
+      const double* R = Rb + p0 * ly.rs;
+      const double* W = Wb + p0 * ly.ws;
+      for (int p = p0; p < p1; ++p, R += ly.rs, W += ly.ws) {
+#pragma unroll
+        for (int u = 0; u < N; ++u) v[u] = fma(W[si[u]], R[ri[u]], v[u]);
+      }
+#pragma unroll
+      for (int u = 0; u < N; ++u) {
+        const int o = g + 32 * u + lane;
+        if (o < mc.n_kc) H[o] = h_valid ? H[o] + v[u] : v[u];
+      }
+    };
+    int g = 0;
+    for (; g + 96 < mc.n_kc; g += 128) rounds(g, std::integral_constant<int, 4>());
+    const int left = (mc.n_kc - g + 31) >> 5;
+    if (left == 3)
+      rounds(g, std::integral_constant<int, 3>());
+    else if (left == 2)
+      rounds(g, std::integral_constant<int, 2>());
+    else if (left == 1)
+      rounds(g, std::integral_constant<int, 1>());
+    __syncwarp();
+  };
+
+  // A[s', s, r] (+)= W_s' H[s, r] for the bra primitive pair with factors w
+  auto bra_contract = [&](const double* w) {
+    for (int o = lane; o < mc.n_bc; o += 32) {
+      const int e = __ldg(kMdBc + mc.bc + o);
+      const double x = __ldg(w + (e >> 12)), h = H[e & 0xFFF];
+      A[o] = a_valid ? fma(x, h, A[o]) : x * h;
+    }
+    __syncwarp();
+  };
+
+  auto finish = [&](int4 e) {
+    const EriLaunch& Ls = rec(e.x);
+    const int nb = e.w & 0xFFFF, nk = e.w >> 16;
+    tally.prim += n_eval;
+    tally.skip += nb * nk - n_eval;
+    double* Tb = S + ly.Tb;
+    double* Tk = S + ly.Tk;
+    const int bra = pair_id(Ls, e.y), ket = pair_id(Ls, e.z);
+    if (a_valid) {
+      ++tally.quart;
+      const double* mk = Ls.pa.md + __ldg(Ls.pa.md_off + ket);
+      for (int i = lane; i < mc.ket_coef; i += 32) Tk[i] = __ldg(mk + i);
+      if (tb_bra != bra || tb_sys != e.x) {
+        // the bra side carries (-1)^{|p|}: the sign of every second coefficient degree
+        const double* mb = Ls.pa.md + __ldg(Ls.pa.md_off + bra);
+        for (int i = lane; i < mc.bra_coef; i += 32) {
+          const double x = __ldg(mb + i);
+          Tb[i] = __hiloint2double(__double2hiint(x) ^ (__ldg(kMdCoefSign + mc.bra_coef0 + i) << 31),
+                                   __double2loint(x));
+        }
+        tb_bra = bra;
+        tb_sys = e.x;
+      }
+      __syncwarp();
+      md_gather(mc.z1_round, mc.z1_n, mc.z1_dst, Tk, A, H, lane);  // Y takes H's place
+      __syncwarp();
+      md_gather(mc.z2_round, mc.z2_n, mc.z2_dst, Tb, H, A, lane);  // the final block takes A's
+      __syncwarp();
+    }
+    if constexpr (KIND == MD_DIAG) {
+      double mx = 0.0;
+      if (a_valid) {
+        for (int f = lane; f < mc.ncd; f += 32) mx = fmax(mx, fabs(A[f * mc.ncd + f]));
+        for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+      }
+      if (lane == 0) Ls.diag_Q[bra] = sqrt(mx);
+    } else if (a_valid) {
+      if constexpr (KIND == MD_PER) {
+        PerQuartet pq;
+        if (per_quartet(Ls, bra, ket, pq)) digest_per(L.ci, A, 1, pq, Ls.KG, Ls.per.nbf, lane, 32);
+      } else {
+        const int sa = __ldg(Ls.pa.sa + bra), sb = __ldg(Ls.pa.sb + bra);
+        const int sc = __ldg(Ls.pa.sa + ket), sd = __ldg(Ls.pa.sb + ket);
+        double deg = 1.0;
+        if (sa == sb) deg *= 0.5;
+        if (sc == sd) deg *= 0.5;
+        if (e.y == e.z) deg *= 0.5;
+        md_digest(L.ci, A, __ldg(Ls.sh.bf_off + sa), __ldg(Ls.sh.bf_off + sb), __ldg(Ls.sh.bf_off + sc),
+                  __ldg(Ls.sh.bf_off + sd), deg, Ls.P, Ls.K, Ls.ld, lane);
+      }
+    }
+    __syncwarp();
+    a_valid = h_valid = false;
+    n_eval = 0;
+  };
+
+  // the next n (<= 32, <= waiting) primitive quartets of the stream
+  auto batch = [&](int n) {
+    int e = head, off = head_off + lane, ib = 0, ik = 0, nb = 1, nk = 1;
+    bool ok = false;
+    double B[LT + 1], PQ[3];
+    const double* wk = nullptr;
+    if (lane < n) {
+      int4 q = Q[e & (kMdQueue - 1)];
+      int npq = (q.w & 0xFFFF) * (q.w >> 16);
+      while (off >= npq) {
+        off -= npq;
+        q = Q[++e & (kMdQueue - 1)];
+        npq = (q.w & 0xFFFF) * (q.w >> 16);
+      }
+      nb = q.w & 0xFFFF;
+      nk = q.w >> 16;
+      ib = off / nk;
+      ik = off - ib * nk;
+      const EriLaunch& Ls = rec(q.x);
+      const int bra = pair_id(Ls, q.y), ket = pair_id(Ls, q.z);
+      const PrimPair& pb = Ls.pa.prim[__ldg(Ls.pa.prim_off + bra) + ib];
+      const PrimPair& pk = Ls.pa.prim[__ldg(Ls.pa.prim_off + ket) + ik];
+      double qc[3] = {pk.P[0], pk.P[1], pk.P[2]};
+      if constexpr (KIND == MD_PER) {  // the ket pair's image in cell G
+        qc[0] += L.shift[0];
+        qc[1] += L.shift[1];
+        qc[2] += L.shift[2];
+      }
+      wk = Ls.pa.md + __ldg(Ls.pa.md_off + ket) + mc.ket_coef + ik * mc.ket_set;
+      ok = md_setup<LT>(pb, pk, qc, Ls.omega, Ls.omega2, Ls.boys, B, PQ);
+    }
+    const unsigned okm = __ballot_sync(0xffffffffu, ok);
+    if (ok) {
+      const int pos = __popc(okm & lt_mask);
+      double* w = Wb + pos * ly.ws;
+      for (int s = 0; s < mc.ket_set; ++s) w[s] = __ldg(wk + s);
+      hermite<LT>(B, PQ[0], PQ[1], PQ[2], Rb + pos * ly.rs);
+    }
+    __syncwarp();
+    // runs of lanes of one (quartet, bra primitive pair)
+    const int e_up = __shfl_up_sync(0xffffffffu, e, 1), ib_up = __shfl_up_sync(0xffffffffu, ib, 1);
+    unsigned lead = __ballot_sync(0xffffffffu, lane < n && (lane == 0 || e != e_up || ib != ib_up));
+    const unsigned last_k = __ballot_sync(0xffffffffu, ik == nk - 1);
+    const unsigned last_q = __ballot_sync(0xffffffffu, ik == nk - 1 && ib == nb - 1);
+    while (lead) {
+      const int l0 = __ffs(lead) - 1;
+      lead &= lead - 1;
+      const int l1 = lead ? __ffs(lead) - 1 : n;
+      const int p0 = __popc(okm & ((1u << l0) - 1u)), p1 = __popc(okm & (0xffffffffu >> (32 - l1)));
+      if (p1 > p0) {
+        ket_contract(p0, p1);
+        h_valid = true;
+        n_eval += p1 - p0;
+      }
+      if ((last_k >> (l1 - 1)) & 1) {
+        const int4 q = Q[__shfl_sync(0xffffffffu, e, l0) & (kMdQueue - 1)];
+        if (h_valid) {
+          const EriLaunch& Ls = rec(q.x);
+          const int bra = pair_id(Ls, q.y);
+          bra_contract(Ls.pa.md + __ldg(Ls.pa.md_off + bra) + mc.bra_coef +
+                       __shfl_sync(0xffffffffu, ib, l0) * mc.bra_set);
+          a_valid = true;
+          h_valid = false;
+        }
+        if ((last_q >> (l1 - 1)) & 1) finish(q);
+      }
+    }
+    // the stream's new head: after lane n - 1
+    const int e_last = __shfl_sync(0xffffffffu, e, n - 1), off_last = __shfl_sync(0xffffffffu, off, n - 1);
+    const bool done = (last_q >> (n - 1)) & 1;
+    head = done ? e_last + 1 : e_last;
+    head_off = done ? 0 : off_last + 1;
+    waiting -= n;
+    __syncwarp();
+  };
+
+  // a candidate quartet per lane: queue those that pass
+  auto push = [&](bool keep, int sys, int bra_s, int ket_s, int nb, int nk) {
+    keep = keep && nb > 0 && nk > 0;
+    const unsigned m = __ballot_sync(0xffffffffu, keep);
+    if (keep) Q[(tail + __popc(m & lt_mask)) & (kMdQueue - 1)] = make_int4(sys, bra_s, ket_s, nb | (nk << 16));
+    tail += __popc(m);
+    waiting += __reduce_add_sync(0xffffffffu, keep ? nb * nk : 0);
+    __syncwarp();
+    while (waiting >= 32) batch(32);
+  };
+
+  if constexpr (KIND == MD_DIAG) {
+    const long long gw = ((long long)gridDim.x * blockDim.x) >> 5;
+    for (long long t = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; t < L.diag_n; t += gw) {
+      const int p = __ldg(L.diag_list + t), np = __ldg(L.pa.prim_n + p);
+      if (np == 0 && lane == 0) L.diag_Q[p] = 0.0;
+      push(lane == 0, 0, p, p, np, np);
+    }
+  } else {
+    const long long wid = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    for_each_range<KIND == MD_BATCH, 32>(
+        L, wid, ((long long)gridDim.x * blockDim.x) >> 5, lane, 0xffffffffu,
+        [&](const EriLaunch& Ls, int sys, long long q0, long long q1) {
+          if (q0 >= q1) return;
+          int r = find_row(Ls.qoff, Ls.row_begin, Ls.row_end, q0);
+          for (long long base = q0; base < q1; base += 32) {
+            const long long q = base + lane;
+            bool keep = false;
+            int bra_s = 0, ket_s = 0, nb = 0, nk = 0;
+            if (q < q1) {
+              while (__ldg(Ls.qoff + r + 1) <= q) ++r;
+              bra_s = Ls.bra_bin_start + (r - Ls.row_begin);
+              ket_s = Ls.ket_bin_start + (int)(q - __ldg(Ls.qoff + r));
+              const int bra = __ldg(Ls.sorted + bra_s), ket = __ldg(Ls.sorted + ket_s);
+              if constexpr (KIND == MD_PER) {
+                PerQuartet pq;
+                keep = per_quartet(Ls, bra, ket, pq);  // a density block exists for its cell offset
+              } else {
+                const double pm = pmax4(Ls, __ldg(Ls.pa.sa + bra), __ldg(Ls.pa.sb + bra), __ldg(Ls.pa.sa + ket),
+                                        __ldg(Ls.pa.sb + ket));
+                keep = !(Ls.skip_zero && pm == 0.0) &&
+                       !(Ls.dens_tau > 0.0 && __ldg(Ls.Qs + bra_s) * __ldg(Ls.Qs + ket_s) * pm < Ls.dens_tau) &&
+                       dist_keeps(Ls, bra_s, ket_s) && !(L.prec == PREC_MIXED64 && fp32_eligible(Ls, bra_s, ket_s, pm));
+              }
+              if (keep) {
+                nb = __ldg(Ls.pa.prim_n + bra);
+                nk = __ldg(Ls.pa.prim_n + ket);
+              }
+            }
+            push(keep, sys, bra_s, ket_s, nb, nk);
+          }
+        });
+  }
+  if (waiting > 0) batch(waiting);
+  if (KIND != MD_DIAG && lane == 0) flush_tally(L, tally);
+  record_busy(L, t0);
+}
+
+}  // namespace hfx

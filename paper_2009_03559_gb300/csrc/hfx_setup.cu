@@ -187,6 +187,8 @@ __global__ void k_prim_fill(int n_cand, const int* __restrict__ sa, const int* _
       }
       r.C = C;
       r.inv2p3 = 1.5 / p;
+      r.ua = ea / p;
+      r.ub = eb / p;
       r.pf = (float)p;
       r.inv2pf = (float)r.inv2p;
       for (int i = 0; i < 3; ++i) {
