@@ -174,13 +174,12 @@ struct Tally {
   unsigned long long prim = 0, quart = 0, skip = 0, q32 = 0, p32 = 0;
 };
 
-// The quartet ranges a warp works on.  Static schedules: one range (group_range).
+// The quartet ranges a warp (or a team of warps) works on.  Static schedules: one range (group_range).
 // Dynamic: chunks claimed from the launch's device counter.  Batched (L.n_sys > 0): chunks
 // of the systems' concatenated quartet lists; a chunk is split at system boundaries
 // (L.seg[s] = first index of system s) and each part runs with that system's record.
-template <bool BATCH, int GS, class F>
-__device__ __forceinline__ void for_each_range(const EriLaunch& L, long long wid, long long nw, int lane, unsigned gm,
-                                               F&& f) {
+template <bool BATCH, class C, class F>
+__device__ __forceinline__ void for_each_range(const EriLaunch& L, long long wid, long long nw, C&& claim, F&& f) {
   if (!BATCH && L.schedule != 2) {
     long long q0, q1;
     group_range(L, wid, nw, q0, q1);
@@ -189,10 +188,7 @@ __device__ __forceinline__ void for_each_range(const EriLaunch& L, long long wid
   }
   const long long total = L.q_count;
   while (true) {
-    unsigned long long c = 0;
-    if (lane == 0) c = atomicAdd(L.work, (unsigned long long)L.chunk);
-    c = __shfl_sync(gm, c, 0, GS);
-    long long c0 = (long long)c;
+    long long c0 = claim();
     if (c0 >= total) break;
     const long long c1 = min(c0 + L.chunk, total);
     if constexpr (!BATCH) {
@@ -211,6 +207,13 @@ __device__ __forceinline__ void for_each_range(const EriLaunch& L, long long wid
       }
     }
   }
+}
+
+// a warp's claim of the next L.chunk quartets
+__device__ __forceinline__ long long warp_claim(const EriLaunch& L, int lane) {
+  unsigned long long c = 0;
+  if (lane == 0) c = atomicAdd(L.work, (unsigned long long)L.chunk);
+  return (long long)__shfl_sync(0xffffffffu, c, 0);
 }
 
 __device__ __forceinline__ void flush_tally(const EriLaunch& L, const Tally& t) {

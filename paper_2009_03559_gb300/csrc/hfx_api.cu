@@ -225,7 +225,7 @@ EriLaunch hfx::base_launch(hfx_ctx* ctx) {
 
 static int grid_for(hfx_ctx* ctx, int cls, int mode, long long work_items, int gs, int prec = 0,
                     bool batch = false, int streams = 0) {
-  const int groups_per_block = eri_groups_per_block(gs);
+  const int groups_per_block = eri_groups_per_block(cls, gs, mode == 1 ? 0 : prec);
   long long need = (work_items + groups_per_block - 1) / groups_per_block;
   long long cap = (long long)eri_blocks_per_sm(cls, mode, gs, prec, batch, streams) * ctx->n_sm;
   long long g = std::min(need, cap);
@@ -634,7 +634,7 @@ extern "C" int hfx_build_K_periodic(hfx_ctx* ctx, int n_R, const int* R_cells, c
       L.q_count = ctx->cls_q[cp];
       const int gs = eri_group_size();
       const int grid = grid_for(ctx, cp, 0, L.q_count, gs, 3);
-      L.chunk = eri_chunk(gs, L.q_count, (long long)grid * eri_groups_per_block(gs));
+      L.chunk = eri_chunk(gs, L.q_count, (long long)grid * eri_groups_per_block(cp, gs, 3));
       // forward: (p | q + G L) for bra class hi >= ket class lo; reverse (hi > lo): the
       // quartets (p | q + G L) with class(p) = lo < class(q) = hi, evaluated as (q | p - G L)
       for (int rev = 0; rev < (hi > lo ? 2 : 1); ++rev) {
@@ -750,7 +750,7 @@ static int build_K_impl(hfx_ctx* ctx, const double* P, double* K, int ld, int pa
       // FP32 set-up), unless the caller fixed the class's group size
       const int gsp = (prec == 2 && !ctx->gs_override[cp]) ? 32 : gs;
       const int grid = grid_for(ctx, cp, 0, items, gsp, prec, false, streams);
-      L.chunk = eri_chunk(gsp, L.q_count, (long long)grid * eri_groups_per_block(gsp));
+      L.chunk = eri_chunk(gsp, L.q_count, (long long)grid * eri_groups_per_block(cp, gsp, prec));
       L.work = ctx->d_work + cp + 21 * pass;
       CK(eri_launch(L, cp, 0, grid, s, gsp, prec, false, streams));
     }

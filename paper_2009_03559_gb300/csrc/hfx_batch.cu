@@ -181,7 +181,7 @@ int bw_gs(const BatchWork& w, int cp, int prec) { return prec == 2 ? 32 : w.gs[c
 
 int bw_grid(const BatchWork& w, int cp, long long items, int prec) {
   const int gs = bw_gs(w, cp, prec);
-  const long long groups_per_block = eri_groups_per_block(gs);
+  const long long groups_per_block = eri_groups_per_block(cp, gs, prec);
   const long long need = (items + groups_per_block - 1) / groups_per_block;
   const long long cap = (long long)eri_blocks_per_sm(cp, 0, gs, prec, true, w.streams[cp]) * w.n_sm;
   return (int)std::max(1LL, std::min(need, cap));
@@ -191,7 +191,7 @@ int bw_grid(const BatchWork& w, int cp, long long items, int prec) {
 int bw_chunk(const BatchWork& w, int cp, int prec) {
   const int gs = bw_gs(w, cp, prec);
   if (gs == w.gs[cp] && w.chunk[cp]) return w.chunk[cp];
-  return eri_chunk(gs, w.total[cp], (long long)bw_grid(w, cp, w.total[cp], prec) * eri_groups_per_block(gs));
+  return eri_chunk(gs, w.total[cp], (long long)bw_grid(w, cp, w.total[cp], prec) * eri_groups_per_block(cp, gs, prec));
 }
 
 EriLaunch bw_class_launch(const BatchWork& w, int cp, int pass = 0) {
@@ -530,8 +530,9 @@ extern "C" int hfx_batch_tune(hfx_batch* b, const double* const* P, double* cons
     // is not timed on a window that leaves most of the GPU idle
     long long fill = 0;
     for (const Cand& cd : cands) {
-      const long long groups = (long long)eri_blocks_per_sm(cp, 0, cd.gs, bw_prec(w, cp, 0), true, cd.streams) *
-                               w.n_sm * (eri_block_size() / 32);
+      const int pr = bw_prec(w, cp, 0);
+      const long long groups = (long long)eri_blocks_per_sm(cp, 0, cd.gs, pr, true, cd.streams) * w.n_sm *
+                               eri_groups_per_block(cp, cd.gs, pr);
       fill = std::max(fill, 2 * groups * cd.chunk);
     }
     long long win = std::min(total, std::max(16384LL, fill));

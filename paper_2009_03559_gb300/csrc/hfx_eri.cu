@@ -537,7 +537,7 @@ __global__ void __launch_bounds__(64, PREC == PREC_MIXED32 ? HFX_G1F_MINB : (BAT
   const int lane = threadIdx.x & 31;
   Tally t;
   G1Queue Q{reinterpret_cast<int4*>(smem + (size_t)L.ci.scratch * blockDim.x) + (threadIdx.x >> 5) * 64, 0};
-  for_each_range<BATCH, 32>(L, gid >> 5, ng >> 5, lane, 0xffffffffu,
+  for_each_range<BATCH>(L, gid >> 5, ng >> 5, [&]() { return warp_claim(L, lane); },
                             [&](const EriLaunch& Ls, int sys, long long q0, long long q1) {
                               g1_range<BATCH, PREC, R>(L, L.ci, Ls, sys, q0, q1, Sd, st, lane, Q, t);
                             });
@@ -556,7 +556,7 @@ __global__ void __launch_bounds__(64, HFX_G32F_MINB) eri_g32_kernel(const EriLau
   unsigned long long t0 = 0;
   if (L.busy && threadIdx.x == 0) t0 = globaltimer_ns();
   Tally t;
-  for_each_range<BATCH, 32>(L, (long long)blockIdx.x * gpb + grp, (long long)gridDim.x * gpb, lane, 0xffffffffu,
+  for_each_range<BATCH>(L, (long long)blockIdx.x * gpb + grp, (long long)gridDim.x * gpb, [&]() { return warp_claim(L, lane); },
                             [&](const EriLaunch& Ls, int, long long q0, long long q1) {
                               g32_range(L.ci, L.sv, Ls, q0, q1, S, lane, t);
                             });
@@ -640,7 +640,6 @@ size_t eri_smem_bytes(int cls, int gs, int streams, int prec) {
   return sizeof(double) * (size_t)g32_stride(kSchedInfo[cls][i]) * (kBlock / 32);
 }
 
-int eri_block_size() { return kBlock; }
 
 cudaError_t eri_prepare() {
   // allow the largest dynamic shared memory any class needs, for every instance
@@ -673,7 +672,10 @@ int eri_blocks_per_sm(int cls, int mode, int gs, int prec, bool batch, int strea
   return n > 0 ? n : 1;
 }
 
-int eri_groups_per_block(int gs) { return kBlock / effective_gs(gs); }
+int eri_groups_per_block(int cls, int gs, int prec) {
+  if (uses_md(effective_gs(gs), prec)) return md_teams_per_block(cls);
+  return kBlock / effective_gs(gs);
+}
 
 // Quartets per claim of the dynamic schedule.  A thread-kernel warp takes 256.  A whole warp takes
 // at most 32 (it tests a claim's quartets with a lane each) and at least 1: a 32nd of an even

@@ -12,14 +12,14 @@ struct EriLaunch;
 int eri_group_size();  // the default: 32
 bool eri_group_size_valid(int gs);
 size_t eri_smem_bytes(int cls, int gs, int streams = 0, int prec = 0);
-int eri_block_size();
 cudaError_t eri_prepare();
 int eri_blocks_per_sm(int cls, int mode, int gs, int prec, bool batch, int streams = 0);
 // Streams of the warp kernel (primitive quartets run at a time): 0 = the class default;
 // the value a launch with `streams` uses; whether a class has that variant.
 int eri_streams(int cls, int streams);
 bool eri_streams_valid(int cls, int streams);
-int eri_groups_per_block(int gs);
+// independent workers (threads, warps or teams of warps) of a block
+int eri_groups_per_block(int cls, int gs, int prec);
 // quartets per claim of the dynamic schedule, for a list of n_quartets and n_groups groups
 int eri_chunk(int gs, long long n_quartets, long long n_groups);
 
@@ -29,6 +29,7 @@ enum { MD_PLAIN = 0, MD_BATCH = 1, MD_PER = 2, MD_DIAG = 3 };
 size_t md_smem_bytes(int cls);
 cudaError_t md_prepare();
 int md_blocks_per_sm(int cls, int kind);
+int md_teams_per_block(int cls);
 cudaError_t md_launch(const EriLaunch& L, int cls, int kind, int prec, int grid, cudaStream_t stream);
 cudaError_t launch_md_size(int n, const int* pcls, const int* cap, long long* size, cudaStream_t s);
 cudaError_t launch_md_fill(int n, const int* pcls, const double* AB, const int* pp_off, const int* pp_n,

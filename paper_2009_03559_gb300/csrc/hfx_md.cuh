@@ -51,62 +51,95 @@ __host__ __device__ constexpr int herm_index(int x, int y, int z) {
   return n * (n + 1) * (n + 2) / 6 + (n - x) * (n - x + 1) / 2 + (n - x - y);
 }
 
+// Share of the x chains (U, V) of the Hermite recursion that warp W of an NW-warp team runs: a
+// contiguous part of the chains in V-major order with about 1 / NW of the operations.
+template <int L, int NW>
+__host__ __device__ constexpr int chain_owner(int u, int v) {
+  int total = 0, before = 0;
+  for (int vv = 0; vv <= L; ++vv)
+    for (int uu = 0; uu <= L - vv; ++uu) {
+      const int n = L - uu - vv, cost = n * (n + 1) / 2 + n + 1;
+      if (vv < v || (vv == v && uu < u)) before += cost;
+      if (vv == v && uu == u) before += cost / 2;
+      total += cost;
+    }
+  return before * NW / total;
+}
+// the largest u of plane v (with v < 0: the largest v) that has a chain of warp W; -1: none
+template <int L, int NW, int W>
+__host__ __device__ constexpr int chain_last(int v) {
+  int last = -1;
+  for (int vv = 0; vv <= L; ++vv)
+    for (int uu = 0; uu <= L - vv; ++uu)
+      if (chain_owner<L, NW>(uu, vv) == W && (v < 0 || vv == v)) last = v < 0 ? vv : uu;
+  return last;
+}
+
 // S_r, |r| <= L, from the base values B[m] = (2 rho)^m G_m:  rows in m, first along z, from each
 // of them along y, from each of those along x; only the last two rows of a chain stay live.
-template <int L>
+// Warp W of NW writes its share.
+template <int L, int NW, int W>
 __device__ __forceinline__ void hermite(const double (&B)[L + 1], double X, double Y, double Z, double* out) {
+  constexpr int kLastV = chain_last<L, NW, W>(-1);
   double zr[L + 1], zp[L + 1];
 #pragma unroll
   for (int m = 0; m <= L; ++m) zr[m] = B[m];
-  unrolled<0, L + 1>([&](auto cv) {
+  unrolled<0, kLastV + 1>([&](auto cv) {
     constexpr int V = decltype(cv)::value;
+    constexpr int kLastU = chain_last<L, NW, W>(V);
     double yr[L + 1 - V], yp[L + 1 - V];
 #pragma unroll
     for (int m = 0; m <= L - V; ++m) yr[m] = zr[m];
-    unrolled<0, L + 1 - V>([&](auto cu) {
+    unrolled<0, kLastU + 1>([&](auto cu) {
       constexpr int U = decltype(cu)::value;
       constexpr int N = L - V - U;
-      double xr[N + 1], xp[N + 1];
+      if constexpr (chain_owner<L, NW>(U, V) == W) {
+        double xr[N + 1], xp[N + 1];
 #pragma unroll
-      for (int m = 0; m <= N; ++m) xr[m] = yr[m];
-      unrolled<0, N + 1>([&](auto ct) {
-        constexpr int T = decltype(ct)::value;
-        out[herm_index(T, U, V)] = xr[0];
+        for (int m = 0; m <= N; ++m) xr[m] = yr[m];
+        unrolled<0, N + 1>([&](auto ct) {
+          constexpr int T = decltype(ct)::value;
+          out[herm_index(T, U, V)] = xr[0];
 #pragma unroll
-        for (int m = 0; m < N - T; ++m) {
-          double v;
-          if constexpr (T == 0)
-            v = X * xr[m + 1];
-          else
-            v = fma(X, xr[m + 1], -times<T>(xp[m + 1]));
-          xp[m] = xr[m];
-          xr[m] = v;
-        }
-        if constexpr (N - T > 0) xp[N - T] = xr[N - T];
-      });
-#pragma unroll
-      for (int m = 0; m < N; ++m) {
-        double v;
-        if constexpr (U == 0)
-          v = Y * yr[m + 1];
-        else
-          v = fma(Y, yr[m + 1], -times<U>(yp[m + 1]));
-        yp[m] = yr[m];
-        yr[m] = v;
+          for (int m = 0; m < N - T; ++m) {
+            double v;
+            if constexpr (T == 0)
+              v = X * xr[m + 1];
+            else
+              v = fma(X, xr[m + 1], -times<T>(xp[m + 1]));
+            xp[m] = xr[m];
+            xr[m] = v;
+          }
+          if constexpr (N - T > 0) xp[N - T] = xr[N - T];
+        });
       }
-      if constexpr (N > 0) yp[N] = yr[N];
-    });
+      if constexpr (U < kLastU) {
 #pragma unroll
-    for (int m = 0; m < L - V; ++m) {
-      double v;
-      if constexpr (V == 0)
-        v = Z * zr[m + 1];
-      else
-        v = fma(Z, zr[m + 1], -times<V>(zp[m + 1]));
-      zp[m] = zr[m];
-      zr[m] = v;
+        for (int m = 0; m < N; ++m) {
+          double v;
+          if constexpr (U == 0)
+            v = Y * yr[m + 1];
+          else
+            v = fma(Y, yr[m + 1], -times<U>(yp[m + 1]));
+          yp[m] = yr[m];
+          yr[m] = v;
+        }
+        if constexpr (N > 0) yp[N] = yr[N];
+      }
+    });
+    if constexpr (V < kLastV) {
+#pragma unroll
+      for (int m = 0; m < L - V; ++m) {
+        double v;
+        if constexpr (V == 0)
+          v = Z * zr[m + 1];
+        else
+          v = fma(Z, zr[m + 1], -times<V>(zp[m + 1]));
+        zp[m] = zr[m];
+        zr[m] = v;
+      }
+      if constexpr (L - V > 0) zp[L - V] = zr[L - V];
     }
-    if constexpr (L - V > 0) zp[L - V] = zr[L - V];
   });
 }
 
@@ -179,17 +212,28 @@ __device__ __forceinline__ bool md_setup(const PrimPair& b, const PrimPair& k, c
   return true;
 }
 
-// Shared memory of one warp, in doubles (offsets; every region starts on an even double).
+// Warps that work on one stream together (a team): they share its Hermite integrals and
+// contraction buffers, each with an even share of every step's rounds.  The buffers of a lone warp
+// leave 6, 4 and 2 resident warps per SM at L = 6, 7, 8 (FP64 pipe 73, 49 and 26 % busy); teams
+// bring that to 10, 12 and 8.  Up to L = 5 a lone warp's buffers leave 8 to 16 and the pipe 86 to
+// 90 % busy, and a team's barriers would only cost.
+__host__ __device__ constexpr int md_team(int Lt) { return Lt <= 5 ? 1 : (Lt == 6 ? 2 : 4); }
+__host__ __device__ constexpr int md_block(int Lt) { return Lt <= 5 ? 64 : 32 * md_team(Lt); }
+
+// Shared memory of one team, in doubles (offsets; every region starts on an even double).
 struct MdLayout {
   int rs, ws;                 // strides of a primitive quartet's Hermite integrals and ket factors
   int R, W, H, A, Tb, Tk, Q;  // H also holds Y, A also the final block
+  int X;                      // teams: set-up results of every warp's primitive quartets
   int size;
 };
-constexpr int kMdQueue = 64;  // quartets waiting in a warp's queue
+// quartets waiting in a team's queue: fewer than 32 primitive quartets per warp, and 32 more
+__host__ __device__ constexpr int md_queue(int Lt) { return md_team(Lt) == 1 ? 64 : (md_team(Lt) == 2 ? 128 : 256); }
 
 inline MdLayout md_layout(const MdClassInfo& c, const MdPairInfo& b, const MdPairInfo& k) {
   MdLayout l{};
   auto even = [](int n) { return (n + 1) & ~1; };
+  const int nw = md_team(c.Lt);
   l.rs = n_herm(c.Lt) | 1;  // odd: the lanes' columns start in different banks
   l.ws = k.n_set | 1;
   l.R = 0;
@@ -199,20 +243,24 @@ inline MdLayout md_layout(const MdClassInfo& c, const MdPairInfo& b, const MdPai
   l.Tb = l.A + even(std::max(c.n_bc, c.nab * c.ncd));
   l.Tk = l.Tb + even(b.n_coef);
   l.Q = l.Tk + even(k.n_coef);
-  l.size = l.Q + 2 * kMdQueue;
+  l.X = l.Q + 2 * md_queue(c.Lt);
+  // per warp (L + 1) base values and PQ of 32 lanes; the warps' masks and the claim
+  l.size = l.X + (nw > 1 ? nw * (c.Lt + 4) * 32 + 4 : 0);
   return l;
 }
 
-// A sparse pass out[dst] = sum of T[c] in[i] (generated: rounds of 32 outputs of like length).
+// A sparse pass out[dst] = sum of T[c] in[i] (generated: rounds of 32 outputs of like length),
+// rounds w, w + nw, ...
 __device__ __forceinline__ void md_gather(int round0, int n_round, int dst0, const double* T, const double* in,
-                                          double* out, int lane) {
-  for (int r = 0; r < n_round; ++r) {
+                                          double* out, int lane, int w, int nw) {
+  for (int r = w; r < n_round; r += nw) {
     const uint32_t rd = __ldg(kMdZRound + round0 + r);
-    const uint32_t* w = kMdZ + (rd & 0xFFFFFFu) + lane;
+    const uint32_t* word = kMdZ + (rd & 0xFFFFFFu) + lane;
     const int n = rd >> 24;
     double v = 0.0;
+#pragma unroll 4
     for (int t = 0; t < n; ++t) {
-      const uint32_t e = __ldg(w + 32 * t);
+      const uint32_t e = __ldg(word + 32 * t);
       v = fma(T[e & 0xFFFFu], in[e >> 16], v);
     }
     const uint32_t d = __ldg(kMdZDst + dst0 + 32 * r + lane);
@@ -224,11 +272,12 @@ __device__ __forceinline__ void md_gather(int round0, int n_round, int dst0, con
 // blocks; every lane runs the same instructions with its own strides, so the outputs of the
 // four blocks share a round (the longest sum counts).
 __device__ __forceinline__ void md_digest(const EriClassInfo& ci, const double* v, int A, int B, int C, int D,
-                                          double deg, const double* __restrict__ P, double* K, int ld, int lane) {
+                                          double deg, const double* __restrict__ P, double* K, int ld, int o0,
+                                          int ostep) {
   const int na = ci.dims[0], nb = ci.dims[1], nc = ci.dims[2], nd = ci.dims[3];
   const int sb = nc * nd, sa = nb * sb;
   const int nAC = na * nc, nAD = na * nd, nBC = nb * nc, nout = nAC + nAD + nBC + nb * nd;
-  for (int o = lane; o < nout; o += 32) {
+  for (int o = o0; o < nout; o += ostep) {
     int t = o;
     bool isA = true, isC = true;  // row function of a (else b), column function of c (else d)
     if (t >= nAC + nAD) {
@@ -249,6 +298,7 @@ __device__ __forceinline__ void md_digest(const EriClassInfo& ci, const double* 
     double acc = 0.0;
     int w = 0;
     const int n = nu * nw;
+#pragma unroll 4
     for (int i = 0; i < n; ++i) {
       acc = fma(vp[w * sw], __ldg(pp + w), acc);
       if (++w == nw) {
@@ -261,26 +311,25 @@ __device__ __forceinline__ void md_digest(const EriClassInfo& ci, const double* 
   }
 }
 
-
-#ifndef HFX_MD_MINB_LO
-#define HFX_MD_MINB_LO 8
-#endif
-#ifndef HFX_MD_MINB_HI
-#define HFX_MD_MINB_HI 4
-#endif
-constexpr int kMdBlock = 64;
+// resident blocks per SM that the registers must allow: what shared memory allows
+__host__ __device__ constexpr int md_minb(int Lt) { return Lt <= 4 ? 8 : (Lt <= 6 ? 5 : (Lt == 7 ? 3 : 2)); }
 
 template <int LT, int KIND>
-__global__ void __launch_bounds__(kMdBlock, LT <= 4 ? HFX_MD_MINB_LO : HFX_MD_MINB_HI)
+__global__ void __launch_bounds__(md_block(LT), md_minb(LT))
     eri_md_kernel(const __grid_constant__ EriLaunch L, const __grid_constant__ MdLayout ly) {
   extern __shared__ __align__(16) double smem[];
-  const int lane = threadIdx.x & 31, grp = threadIdx.x >> 5;
-  double* S = smem + grp * ly.size;
+  constexpr int NW = md_team(LT), kQ = md_queue(LT), kTeams = md_block(LT) / (32 * NW);
+  const int lane = threadIdx.x & 31;
+  const int wt = NW == 1 ? 0 : (int)(threadIdx.x >> 5);             // warp of the team
+  const int team = NW == 1 ? (int)(threadIdx.x >> 5) : 0;           // team of the block
+  double* S = smem + team * ly.size;
   double* const Rb = S + ly.R;
   double* const Wb = S + ly.W;
   double* const H = S + ly.H;
   double* const A = S + ly.A;
   int4* const Q = reinterpret_cast<int4*>(S + ly.Q);  // system, bra position, ket position, nb | nk << 16
+  double* const X = S + ly.X;
+  unsigned* const Xok = reinterpret_cast<unsigned*>(X + NW * (LT + 4) * 32);  // masks, then the claim
   const unsigned lt_mask = (1u << lane) - 1u;
   const MdClassInfo mc = L.mc;
   unsigned long long t0 = 0;
@@ -292,6 +341,12 @@ __global__ void __launch_bounds__(kMdBlock, LT <= 4 ? HFX_MD_MINB_LO : HFX_MD_MI
   int tb_sys = -1, tb_bra = -1;                       // whose transformation is in Tb
   Tally tally;
 
+  auto sync = [&]() {
+    if constexpr (NW == 1)
+      __syncwarp();
+    else
+      __syncthreads();
+  };
   auto rec = [&](int sys) -> const EriLaunch& {
     if constexpr (KIND == MD_BATCH)
       return L.batch[sys];
@@ -313,7 +368,7 @@ __global__ void __launch_bounds__(kMdBlock, LT <= 4 ? HFX_MD_MINB_LO : HFX_MD_MI
       double v[N];
 #pragma unroll
       for (int u = 0; u < N; ++u) {
-        const int e = __ldg(kMdKc + mc.kc + g + 32 * u + lane);  // padded to whole rounds
+        const int e = __ldg(kMdKc + mc.kc + 32 * (g + NW * u) + lane);  // padded to whole rounds
         ri[u] = e & 0xFF;
         si[u] = e >> 8;
         v[u] = 0.0;
@@ -326,30 +381,43 @@ __global__ void __launch_bounds__(kMdBlock, LT <= 4 ? HFX_MD_MINB_LO : HFX_MD_MI
       }
 #pragma unroll
       for (int u = 0; u < N; ++u) {
-        const int o = g + 32 * u + lane;
+        const int o = 32 * (g + NW * u) + lane;
         if (o < mc.n_kc) H[o] = h_valid ? H[o] + v[u] : v[u];
       }
     };
-    int g = 0;
-    for (; g + 96 < mc.n_kc; g += 128) rounds(g, std::integral_constant<int, 4>());
-    const int left = (mc.n_kc - g + 31) >> 5;
-    if (left == 3)
+    const int n = (mc.n_kc + 31) >> 5;
+    int g = wt;  // this warp's rounds: wt, wt + NW, ...
+    for (; g + 3 * NW < n; g += 4 * NW) rounds(g, std::integral_constant<int, 4>());
+    if (g + 2 * NW < n)
       rounds(g, std::integral_constant<int, 3>());
-    else if (left == 2)
+    else if (g + NW < n)
       rounds(g, std::integral_constant<int, 2>());
-    else if (left == 1)
+    else if (g < n)
       rounds(g, std::integral_constant<int, 1>());
-    __syncwarp();
+    sync();
   };
 
   // A[s', s, r] (+)= W_s' H[s, r] for the bra primitive pair with factors w
   auto bra_contract = [&](const double* w) {
-    for (int o = lane; o < mc.n_bc; o += 32) {
-      const int e = __ldg(kMdBc + mc.bc + o);
-      const double x = __ldg(w + (e >> 12)), h = H[e & 0xFFF];
-      A[o] = a_valid ? fma(x, h, A[o]) : x * h;
-    }
-    __syncwarp();
+    auto rounds = [&](int o, auto nc) {
+      constexpr int N = decltype(nc)::value;
+      double x[N], h[N], a[N];
+#pragma unroll
+      for (int u = 0; u < N; ++u) {
+        const int e = __ldg(kMdBc + mc.bc + o + 32 * NW * u);  // padded to whole rounds
+        x[u] = __ldg(w + (e >> 12));
+        h[u] = H[e & 0xFFF];
+        a[u] = a_valid && o + 32 * NW * u < mc.n_bc ? A[o + 32 * NW * u] : 0.0;
+      }
+#pragma unroll
+      for (int u = 0; u < N; ++u)
+        if (o + 32 * NW * u < mc.n_bc) A[o + 32 * NW * u] = fma(x[u], h[u], a[u]);
+    };
+    const int n = (mc.n_bc + 31) >> 5;
+    int g = wt;
+    for (; g + 3 * NW < n; g += 4 * NW) rounds(32 * g + lane, std::integral_constant<int, 4>());
+    for (; g < n; g += NW) rounds(32 * g + lane, std::integral_constant<int, 1>());
+    sync();
   };
 
   auto finish = [&](int4 e) {
@@ -363,11 +431,11 @@ __global__ void __launch_bounds__(kMdBlock, LT <= 4 ? HFX_MD_MINB_LO : HFX_MD_MI
     if (a_valid) {
       ++tally.quart;
       const double* mk = Ls.pa.md + __ldg(Ls.pa.md_off + ket);
-      for (int i = lane; i < mc.ket_coef; i += 32) Tk[i] = __ldg(mk + i);
+      for (int i = 32 * wt + lane; i < mc.ket_coef; i += 32 * NW) Tk[i] = __ldg(mk + i);
       if (tb_bra != bra || tb_sys != e.x) {
         // the bra side carries (-1)^{|p|}: the sign of every second coefficient degree
         const double* mb = Ls.pa.md + __ldg(Ls.pa.md_off + bra);
-        for (int i = lane; i < mc.bra_coef; i += 32) {
+        for (int i = 32 * wt + lane; i < mc.bra_coef; i += 32 * NW) {
           const double x = __ldg(mb + i);
           Tb[i] = __hiloint2double(__double2hiint(x) ^ (__ldg(kMdCoefSign + mc.bra_coef0 + i) << 31),
                                    __double2loint(x));
@@ -375,11 +443,11 @@ __global__ void __launch_bounds__(kMdBlock, LT <= 4 ? HFX_MD_MINB_LO : HFX_MD_MI
         tb_bra = bra;
         tb_sys = e.x;
       }
-      __syncwarp();
-      md_gather(mc.z1_round, mc.z1_n, mc.z1_dst, Tk, A, H, lane);  // Y takes H's place
-      __syncwarp();
-      md_gather(mc.z2_round, mc.z2_n, mc.z2_dst, Tb, H, A, lane);  // the final block takes A's
-      __syncwarp();
+      sync();
+      md_gather(mc.z1_round, mc.z1_n, mc.z1_dst, Tk, A, H, lane, wt, NW);  // Y takes H's place
+      sync();
+      md_gather(mc.z2_round, mc.z2_n, mc.z2_dst, Tb, H, A, lane, wt, NW);  // the final block takes A's
+      sync();
     }
     if constexpr (KIND == MD_DIAG) {
       double mx = 0.0;
@@ -387,11 +455,12 @@ __global__ void __launch_bounds__(kMdBlock, LT <= 4 ? HFX_MD_MINB_LO : HFX_MD_MI
         for (int f = lane; f < mc.ncd; f += 32) mx = fmax(mx, fabs(A[f * mc.ncd + f]));
         for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
       }
-      if (lane == 0) Ls.diag_Q[bra] = sqrt(mx);
+      if (lane == 0 && wt == 0) Ls.diag_Q[bra] = sqrt(mx);
     } else if (a_valid) {
       if constexpr (KIND == MD_PER) {
         PerQuartet pq;
-        if (per_quartet(Ls, bra, ket, pq)) digest_per(L.ci, A, 1, pq, Ls.KG, Ls.per.nbf, lane, 32);
+        if (per_quartet(Ls, bra, ket, pq))
+          digest_per(L.ci, A, 1, pq, Ls.KG, Ls.per.nbf, 32 * wt + lane, 32 * NW);
       } else {
         const int sa = __ldg(Ls.pa.sa + bra), sb = __ldg(Ls.pa.sb + bra);
         const int sc = __ldg(Ls.pa.sa + ket), sd = __ldg(Ls.pa.sb + ket);
@@ -400,112 +469,179 @@ __global__ void __launch_bounds__(kMdBlock, LT <= 4 ? HFX_MD_MINB_LO : HFX_MD_MI
         if (sc == sd) deg *= 0.5;
         if (e.y == e.z) deg *= 0.5;
         md_digest(L.ci, A, __ldg(Ls.sh.bf_off + sa), __ldg(Ls.sh.bf_off + sb), __ldg(Ls.sh.bf_off + sc),
-                  __ldg(Ls.sh.bf_off + sd), deg, Ls.P, Ls.K, Ls.ld, lane);
+                  __ldg(Ls.sh.bf_off + sd), deg, Ls.P, Ls.K, Ls.ld, 32 * wt + lane, 32 * NW);
       }
     }
-    __syncwarp();
+    sync();
     a_valid = h_valid = false;
     n_eval = 0;
   };
 
-  // the next n (<= 32, <= waiting) primitive quartets of the stream
+  // primitive quartet number pos of the stream: its queue entry, the quartet, the primitive pairs
+  struct Prim {
+    int e, off, nb, nk, ib, ik;
+    int4 q;
+  };
+  auto locate = [&](int pos) {
+    Prim s;
+    s.e = head;
+    s.off = head_off + pos;
+    s.q = Q[s.e & (kQ - 1)];
+    int npq = (s.q.w & 0xFFFF) * (s.q.w >> 16);
+    while (s.off >= npq) {
+      s.off -= npq;
+      s.q = Q[++s.e & (kQ - 1)];
+      npq = (s.q.w & 0xFFFF) * (s.q.w >> 16);
+    }
+    s.nb = s.q.w & 0xFFFF;
+    s.nk = s.q.w >> 16;
+    s.ib = s.off / s.nk;
+    s.ik = s.off - s.ib * s.nk;
+    return s;
+  };
+
+  // the next n (<= 32 NW, <= waiting) primitive quartets of the stream
   auto batch = [&](int n) {
-    int e = head, off = head_off + lane, ib = 0, ik = 0, nb = 1, nk = 1;
+    Prim s{};
+    s.nb = s.nk = 1;
     bool ok = false;
     double B[LT + 1], PQ[3];
-    const double* wk = nullptr;
-    if (lane < n) {
-      int4 q = Q[e & (kMdQueue - 1)];
-      int npq = (q.w & 0xFFFF) * (q.w >> 16);
-      while (off >= npq) {
-        off -= npq;
-        q = Q[++e & (kMdQueue - 1)];
-        npq = (q.w & 0xFFFF) * (q.w >> 16);
-      }
-      nb = q.w & 0xFFFF;
-      nk = q.w >> 16;
-      ib = off / nk;
-      ik = off - ib * nk;
-      const EriLaunch& Ls = rec(q.x);
-      const int bra = pair_id(Ls, q.y), ket = pair_id(Ls, q.z);
-      const PrimPair& pb = Ls.pa.prim[__ldg(Ls.pa.prim_off + bra) + ib];
-      const PrimPair& pk = Ls.pa.prim[__ldg(Ls.pa.prim_off + ket) + ik];
+    if (32 * wt + lane < n) {  // set-up: warp w of the team the w-th 32
+      s = locate(32 * wt + lane);
+      const EriLaunch& Ls = rec(s.q.x);
+      const int bra = pair_id(Ls, s.q.y), ket = pair_id(Ls, s.q.z);
+      const PrimPair& pb = Ls.pa.prim[__ldg(Ls.pa.prim_off + bra) + s.ib];
+      const PrimPair& pk = Ls.pa.prim[__ldg(Ls.pa.prim_off + ket) + s.ik];
       double qc[3] = {pk.P[0], pk.P[1], pk.P[2]};
       if constexpr (KIND == MD_PER) {  // the ket pair's image in cell G
         qc[0] += L.shift[0];
         qc[1] += L.shift[1];
         qc[2] += L.shift[2];
       }
-      wk = Ls.pa.md + __ldg(Ls.pa.md_off + ket) + mc.ket_coef + ik * mc.ket_set;
       ok = md_setup<LT>(pb, pk, qc, Ls.omega, Ls.omega2, Ls.boys, B, PQ);
     }
-    const unsigned okm = __ballot_sync(0xffffffffu, ok);
-    if (ok) {
-      const int pos = __popc(okm & lt_mask);
-      double* w = Wb + pos * ly.ws;
-      for (int s = 0; s < mc.ket_set; ++s) w[s] = __ldg(wk + s);
-      hermite<LT>(B, PQ[0], PQ[1], PQ[2], Rb + pos * ly.rs);
+    unsigned okm = __ballot_sync(0xffffffffu, ok);
+    if constexpr (NW > 1) {
+      double* x = X + wt * (LT + 4) * 32 + lane;
+#pragma unroll
+      for (int m = 0; m <= LT; ++m) x[32 * m] = B[m];
+#pragma unroll
+      for (int i = 0; i < 3; ++i) x[32 * (LT + 1 + i)] = PQ[i];
+      if (lane == 0) Xok[wt] = okm;
+      sync();
     }
-    __syncwarp();
-    // runs of lanes of one (quartet, bra primitive pair)
-    const int e_up = __shfl_up_sync(0xffffffffu, e, 1), ib_up = __shfl_up_sync(0xffffffffu, ib, 1);
-    unsigned lead = __ballot_sync(0xffffffffu, lane < n && (lane == 0 || e != e_up || ib != ib_up));
-    const unsigned last_k = __ballot_sync(0xffffffffu, ik == nk - 1);
-    const unsigned last_q = __ballot_sync(0xffffffffu, ik == nk - 1 && ib == nb - 1);
-    while (lead) {
-      const int l0 = __ffs(lead) - 1;
-      lead &= lead - 1;
-      const int l1 = lead ? __ffs(lead) - 1 : n;
-      const int p0 = __popc(okm & ((1u << l0) - 1u)), p1 = __popc(okm & (0xffffffffu >> (32 - l1)));
-      if (p1 > p0) {
-        ket_contract(p0, p1);
-        h_valid = true;
-        n_eval += p1 - p0;
+    for (int sub = 0; sub < NW && 32 * sub < n; ++sub) {
+      const int ns = min(32, n - 32 * sub);
+      if constexpr (NW > 1) {
+        okm = Xok[sub];
+        ok = (okm >> lane) & 1;
+        s.nb = s.nk = 1;
+        s.ib = s.ik = 0;
+        if (lane < ns) s = locate(32 * sub + lane);
+        const double* x = X + sub * (LT + 4) * 32 + lane;
+#pragma unroll
+        for (int m = 0; m <= LT; ++m) B[m] = x[32 * m];
+#pragma unroll
+        for (int i = 0; i < 3; ++i) PQ[i] = x[32 * (LT + 1 + i)];
       }
-      if ((last_k >> (l1 - 1)) & 1) {
-        const int4 q = Q[__shfl_sync(0xffffffffu, e, l0) & (kMdQueue - 1)];
-        if (h_valid) {
-          const EriLaunch& Ls = rec(q.x);
-          const int bra = pair_id(Ls, q.y);
-          bra_contract(Ls.pa.md + __ldg(Ls.pa.md_off + bra) + mc.bra_coef +
-                       __shfl_sync(0xffffffffu, ib, l0) * mc.bra_set);
-          a_valid = true;
-          h_valid = false;
+      if (ok) {
+        const EriLaunch& Ls = rec(s.q.x);
+        const int ket = pair_id(Ls, s.q.z);
+        const double* wk = Ls.pa.md + __ldg(Ls.pa.md_off + ket) + mc.ket_coef + s.ik * mc.ket_set;
+        const int pos = __popc(okm & lt_mask);
+        double* w = Wb + pos * ly.ws;
+        for (int i = wt; i < mc.ket_set; i += NW) w[i] = __ldg(wk + i);
+        double* R = Rb + pos * ly.rs;
+        if constexpr (NW == 1) hermite<LT, 1, 0>(B, PQ[0], PQ[1], PQ[2], R);
+        if constexpr (NW == 2) {
+          if (wt == 0)
+            hermite<LT, 2, 0>(B, PQ[0], PQ[1], PQ[2], R);
+          else
+            hermite<LT, 2, 1>(B, PQ[0], PQ[1], PQ[2], R);
         }
-        if ((last_q >> (l1 - 1)) & 1) finish(q);
+        if constexpr (NW == 4) {
+          if (wt == 0)
+            hermite<LT, 4, 0>(B, PQ[0], PQ[1], PQ[2], R);
+          else if (wt == 1)
+            hermite<LT, 4, 1>(B, PQ[0], PQ[1], PQ[2], R);
+          else if (wt == 2)
+            hermite<LT, 4, 2>(B, PQ[0], PQ[1], PQ[2], R);
+          else
+            hermite<LT, 4, 3>(B, PQ[0], PQ[1], PQ[2], R);
+        }
+      }
+      sync();
+      // runs of lanes of one (quartet, bra primitive pair)
+      const int e_up = __shfl_up_sync(0xffffffffu, s.e, 1), ib_up = __shfl_up_sync(0xffffffffu, s.ib, 1);
+      unsigned lead = __ballot_sync(0xffffffffu, lane < ns && (lane == 0 || s.e != e_up || s.ib != ib_up));
+      const unsigned last_k = __ballot_sync(0xffffffffu, s.ik == s.nk - 1);
+      const unsigned last_q = __ballot_sync(0xffffffffu, s.ik == s.nk - 1 && s.ib == s.nb - 1);
+      while (lead) {
+        const int l0 = __ffs(lead) - 1;
+        lead &= lead - 1;
+        const int l1 = lead ? __ffs(lead) - 1 : ns;
+        const int p0 = __popc(okm & ((1u << l0) - 1u)), p1 = __popc(okm & (0xffffffffu >> (32 - l1)));
+        if (p1 > p0) {
+          ket_contract(p0, p1);
+          h_valid = true;
+          n_eval += p1 - p0;
+        }
+        if ((last_k >> (l1 - 1)) & 1) {
+          const int4 q = Q[__shfl_sync(0xffffffffu, s.e, l0) & (kQ - 1)];
+          if (h_valid) {
+            const EriLaunch& Ls = rec(q.x);
+            const int bra = pair_id(Ls, q.y);
+            bra_contract(Ls.pa.md + __ldg(Ls.pa.md_off + bra) + mc.bra_coef +
+                         __shfl_sync(0xffffffffu, s.ib, l0) * mc.bra_set);
+            a_valid = true;
+            h_valid = false;
+          }
+          if ((last_q >> (l1 - 1)) & 1) finish(q);
+        }
+      }
+      if (32 * (sub + 1) >= n) {  // the stream's new head: after the last lane
+        const int l = ns - 1;
+        const int e_last = __shfl_sync(0xffffffffu, s.e, l), off_last = __shfl_sync(0xffffffffu, s.off, l);
+        const bool done = (last_q >> l) & 1;
+        head = done ? e_last + 1 : e_last;
+        head_off = done ? 0 : off_last + 1;
       }
     }
-    // the stream's new head: after lane n - 1
-    const int e_last = __shfl_sync(0xffffffffu, e, n - 1), off_last = __shfl_sync(0xffffffffu, off, n - 1);
-    const bool done = (last_q >> (n - 1)) & 1;
-    head = done ? e_last + 1 : e_last;
-    head_off = done ? 0 : off_last + 1;
     waiting -= n;
-    __syncwarp();
+    sync();
   };
 
-  // a candidate quartet per lane: queue those that pass
+  // a candidate quartet per lane (the same in every warp of a team): queue those that pass
   auto push = [&](bool keep, int sys, int bra_s, int ket_s, int nb, int nk) {
     keep = keep && nb > 0 && nk > 0;
     const unsigned m = __ballot_sync(0xffffffffu, keep);
-    if (keep) Q[(tail + __popc(m & lt_mask)) & (kMdQueue - 1)] = make_int4(sys, bra_s, ket_s, nb | (nk << 16));
+    if (keep && wt == 0) Q[(tail + __popc(m & lt_mask)) & (kQ - 1)] = make_int4(sys, bra_s, ket_s, nb | (nk << 16));
     tail += __popc(m);
     waiting += __reduce_add_sync(0xffffffffu, keep ? nb * nk : 0);
-    __syncwarp();
-    while (waiting >= 32) batch(32);
+    sync();
+    while (waiting >= 32 * NW) batch(32 * NW);
   };
 
   if constexpr (KIND == MD_DIAG) {
-    const long long gw = ((long long)gridDim.x * blockDim.x) >> 5;
-    for (long long t = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; t < L.diag_n; t += gw) {
+    for (int t = blockIdx.x * kTeams + team; t < L.diag_n; t += gridDim.x * kTeams) {
       const int p = __ldg(L.diag_list + t), np = __ldg(L.pa.prim_n + p);
-      if (np == 0 && lane == 0) L.diag_Q[p] = 0.0;
+      if (np == 0 && lane == 0 && wt == 0) L.diag_Q[p] = 0.0;
       push(lane == 0, 0, p, p, np, np);
     }
   } else {
-    const long long wid = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    for_each_range<KIND == MD_BATCH, 32>(
-        L, wid, ((long long)gridDim.x * blockDim.x) >> 5, lane, 0xffffffffu,
+    auto claim = [&]() -> long long {
+      unsigned long long c = 0;
+      if (lane == 0 && wt == 0) c = atomicAdd(L.work, (unsigned long long)L.chunk);
+      if constexpr (NW == 1) return (long long)__shfl_sync(0xffffffffu, c, 0);
+      volatile unsigned long long* xc = reinterpret_cast<unsigned long long*>(X + NW * (LT + 4) * 32 + 2);
+      if (threadIdx.x == 0) *xc = c;
+      __syncthreads();
+      c = *xc;
+      __syncthreads();
+      return (long long)c;
+    };
+    for_each_range<KIND == MD_BATCH>(
+        L, blockIdx.x * kTeams + team, (long long)gridDim.x * kTeams, claim,
         [&](const EriLaunch& Ls, int sys, long long q0, long long q1) {
           if (q0 >= q1) return;
           int r = find_row(Ls.qoff, Ls.row_begin, Ls.row_end, q0);
@@ -538,7 +674,7 @@ __global__ void __launch_bounds__(kMdBlock, LT <= 4 ? HFX_MD_MINB_LO : HFX_MD_MI
         });
   }
   if (waiting > 0) batch(waiting);
-  if (KIND != MD_DIAG && lane == 0) flush_tally(L, tally);
+  if (KIND != MD_DIAG && lane == 0 && wt == 0) flush_tally(L, tally);
   record_busy(L, t0);
 }
 

@@ -38,7 +38,12 @@ static MdLayout layout_of(int cls) {
   return md_layout(kMdClass[cls], kMdPair[hi], kMdPair[cls - hi * (hi + 1) / 2]);
 }
 
-size_t md_smem_bytes(int cls) { return sizeof(double) * (size_t)layout_of(cls).size * (kMdBlock / 32); }
+int md_teams_per_block(int cls) {
+  const int l = kMdClass[cls].Lt;
+  return md_block(l) / (32 * md_team(l));
+}
+
+size_t md_smem_bytes(int cls) { return sizeof(double) * (size_t)layout_of(cls).size * md_teams_per_block(cls); }
 
 cudaError_t md_prepare() {
   int mx[kMaxLt + 1] = {};
@@ -55,8 +60,8 @@ cudaError_t md_prepare() {
 
 int md_blocks_per_sm(int cls, int kind) {
   int n = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, md_kernel(kMdClass[cls].Lt, kind), kMdBlock,
-                                                    md_smem_bytes(cls)) != cudaSuccess)
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, md_kernel(kMdClass[cls].Lt, kind),
+                                                    md_block(kMdClass[cls].Lt), md_smem_bytes(cls)) != cudaSuccess)
     return 1;
   return n > 0 ? n : 1;
 }
@@ -67,7 +72,7 @@ cudaError_t md_launch(const EriLaunch& L0, int cls, int kind, int prec, int grid
   L.prec = prec;
   MdLayout ly = layout_of(cls);
   void* args[] = {(void*)&L, (void*)&ly};
-  return cudaLaunchKernel(md_kernel(L.mc.Lt, kind), dim3(grid), dim3(kMdBlock), args, md_smem_bytes(cls), stream);
+  return cudaLaunchKernel(md_kernel(L.mc.Lt, kind), dim3(grid), dim3(md_block(L.mc.Lt)), args, md_smem_bytes(cls), stream);
 }
 
 // ---------------------------------------------------------------------------
