@@ -174,7 +174,7 @@ struct Tally {
   unsigned long long prim = 0, quart = 0, skip = 0, q32 = 0, p32 = 0;
 };
 
-// The quartet ranges a warp (or a team of warps) works on.  Static schedules: one range (group_range).
+// The quartet ranges a warp of the thread kernel works on.  Static schedules: one range (group_range).
 // Dynamic: chunks claimed from the launch's device counter.  Batched (L.n_sys > 0): chunks
 // of the systems' concatenated quartet lists; a chunk is split at system boundaries
 // (L.seg[s] = first index of system s) and each part runs with that system's record.

@@ -762,37 +762,11 @@ def emit(classes, f=sys.stdout):
             str(fl["vrr"] + fl["acc"]), str(fl["hrr"] + fl["sph"] + fl["digest"]), str(fl["digest"]),
         ]) + "},\n")
     w("};\n\n")
-    # warp schedules
-    w("// Coefficient set of one primitive quartet (group scratch of the warp kernel)\n")
-    for name, v in CF.items():
-        w(f"#define HFX_CF_{name} {v}\n")
-    w(f"#define HFX_NCOEF {NCOEF}\n")
-    w(f"#define HFX_CF_KET_BASE {KET_BASE}\n\n")
-    sched_words, info = [], []
+    # the values hfx_set_streams takes (the variants of the warp schedules)
+    w("static const int kStreams[HFX_N_CLASSES][3] = {\n")
     for c in classes:
-        row = []
         ws = warp_schedules(c)
-        for k in SCHED_KS:
-            if k in ws:
-                v = ws[k]
-                row.append((k, v.rsz, v.zero, len(v.iters), len(sched_words) // 4, v.group, v.cost))
-                sched_words.extend(v.words())
-            else:
-                row.append((0, 0, 0, 0, 0, 0, 0))
-        info.append((c, row))
-    w("// Warp schedules: per entry (uint4) dst | s1 << 16, s2 | s3 << 16, s4 | s5 << 16, flags\n")
-    w("// (dir | nA << 2 | nB << 4 | ket << 7 | fold << 8 | add << 9 | valid << 10 | shapeA << 11 |\n")
-    w("//  shapeB << 12 | stream << 13); 32 entries per iteration.\n")
-    sched_words.extend([0] * (32 * 4))   # padding iteration: the warp kernel prefetches one past the end
-    w(f"HFX_TABLE_QUAL uint32_t kSched[{len(sched_words)}] = {{\n")
-    for i in range(0, len(sched_words), 8):
-        w("  " + ", ".join(f"0x{x:x}u" for x in sched_words[i:i + 8]) + ",\n")
-    w("};\n\n")
-    w(f"static const SchedVariant kSchedInfo[HFX_N_CLASSES][{len(SCHED_KS)}] = {{\n")
-    for c, row in info:
-        costs = ", ".join(f"k{r[0]} {r[6] / max(r[0], 1):.1f}" for r in row if r[0])
-        w(f"  // ({c.name()}) FP64 warp instructions per primitive quartet: {costs}\n")
-        w("  {" + ", ".join("{" + ", ".join(str(x) for x in r[:6]) + "}" for r in row) + "},\n")
+        w("  {" + ", ".join(str(k if k in ws else 0) for k in SCHED_KS) + "},\n")
     w("};\n")
 
 

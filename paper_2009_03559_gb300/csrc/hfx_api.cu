@@ -223,11 +223,10 @@ EriLaunch hfx::base_launch(hfx_ctx* ctx) {
   return L;
 }
 
-static int grid_for(hfx_ctx* ctx, int cls, int mode, long long work_items, int gs, int prec = 0,
-                    bool batch = false, int streams = 0) {
-  const int groups_per_block = eri_groups_per_block(cls, gs, mode == 1 ? 0 : prec);
+static int grid_for(hfx_ctx* ctx, int cls, int mode, long long work_items, int gs, int prec = 0) {
+  const int groups_per_block = eri_groups_per_block(cls, gs);
   long long need = (work_items + groups_per_block - 1) / groups_per_block;
-  long long cap = (long long)eri_blocks_per_sm(cls, mode, gs, prec, batch, streams) * ctx->n_sm;
+  long long cap = (long long)eri_blocks_per_sm(cls, mode, gs, prec, false) * ctx->n_sm;
   long long g = std::min(need, cap);
   return (int)std::max(1LL, g);
 }
@@ -634,7 +633,7 @@ extern "C" int hfx_build_K_periodic(hfx_ctx* ctx, int n_R, const int* R_cells, c
       L.q_count = ctx->cls_q[cp];
       const int gs = eri_group_size();
       const int grid = grid_for(ctx, cp, 0, L.q_count, gs, 3);
-      L.chunk = eri_chunk(gs, L.q_count, (long long)grid * eri_groups_per_block(cp, gs, 3));
+      L.chunk = eri_chunk(gs, L.q_count, (long long)grid * eri_groups_per_block(cp, gs));
       // forward: (p | q + G L) for bra class hi >= ket class lo; reverse (hi > lo): the
       // quartets (p | q + G L) with class(p) = lo < class(q) = hi, evaluated as (q | p - G L)
       for (int rev = 0; rev < (hi > lo ? 2 : 1); ++rev) {
@@ -740,19 +739,17 @@ static int build_K_impl(hfx_ctx* ctx, const double* P, double* K, int ld, int pa
     L.fp32_ok = mixed && ((ctx->opt.fp32_class_mask >> cp) & 1);
     const int gs = ctx->gs_override[cp] ? ctx->gs_override[cp] : eri_group_size();
     ctx->gs_used[cp] = gs;
-    const int streams = ctx->streams_override[cp];
-    ctx->streams_used[cp] = gs == 32 ? eri_streams(cp, streams) : 0;
+    ctx->streams_used[cp] = gs == 32 ? eri_streams(cp, ctx->streams_override[cp]) : 0;
     const long long items = ctx->opt.schedule == HFX_SCHED_PAIR ? (L.row_end - L.row_begin) : L.q_count;
     if (ctx->timing) CK(cudaEventRecord(ctx->ev[2 + 2 * cp], s));
     for (int pass = 0; pass < (L.fp32_ok ? 2 : 1); ++pass) {
       const int prec = L.fp32_ok ? 1 + pass : 0;
-      // the FP32 pass runs on whole warps in every class (packed FP32 recurrences after an
-      // FP32 set-up), unless the caller fixed the class's group size
+      // the FP32 pass runs on whole warps in every class unless the caller fixed the class's group size
       const int gsp = (prec == 2 && !ctx->gs_override[cp]) ? 32 : gs;
-      const int grid = grid_for(ctx, cp, 0, items, gsp, prec, false, streams);
-      L.chunk = eri_chunk(gsp, L.q_count, (long long)grid * eri_groups_per_block(cp, gsp, prec));
+      const int grid = grid_for(ctx, cp, 0, items, gsp, prec);
+      L.chunk = eri_chunk(gsp, L.q_count, (long long)grid * eri_groups_per_block(cp, gsp));
       L.work = ctx->d_work + cp + 21 * pass;
-      CK(eri_launch(L, cp, 0, grid, s, gsp, prec, false, streams));
+      CK(eri_launch(L, cp, 0, grid, s, gsp, prec, false));
     }
     if (ctx->timing) CK(cudaEventRecord(ctx->ev[3 + 2 * cp], s));
     ctx->class_launched[cp] = true;

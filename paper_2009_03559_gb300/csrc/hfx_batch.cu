@@ -176,14 +176,14 @@ void bw_set_buffers(BatchWork& w, const double* const* P, double* const* K, cons
 int bw_prec(const BatchWork& w, int cp, int pass) { return w.fp32_class[cp] ? 1 + pass : 0; }
 
 // lanes per quartet of a pass: the class's choice, except the FP32 pass, which runs on whole
-// warps in every class (packed FP32 recurrences after an FP32 set-up)
+// warps in every class
 int bw_gs(const BatchWork& w, int cp, int prec) { return prec == 2 ? 32 : w.gs[cp]; }
 
 int bw_grid(const BatchWork& w, int cp, long long items, int prec) {
   const int gs = bw_gs(w, cp, prec);
-  const long long groups_per_block = eri_groups_per_block(cp, gs, prec);
+  const long long groups_per_block = eri_groups_per_block(cp, gs);
   const long long need = (items + groups_per_block - 1) / groups_per_block;
-  const long long cap = (long long)eri_blocks_per_sm(cp, 0, gs, prec, true, w.streams[cp]) * w.n_sm;
+  const long long cap = (long long)eri_blocks_per_sm(cp, 0, gs, prec, true) * w.n_sm;
   return (int)std::max(1LL, std::min(need, cap));
 }
 
@@ -191,7 +191,7 @@ int bw_grid(const BatchWork& w, int cp, long long items, int prec) {
 int bw_chunk(const BatchWork& w, int cp, int prec) {
   const int gs = bw_gs(w, cp, prec);
   if (gs == w.gs[cp] && w.chunk[cp]) return w.chunk[cp];
-  return eri_chunk(gs, w.total[cp], (long long)bw_grid(w, cp, w.total[cp], prec) * eri_groups_per_block(cp, gs, prec));
+  return eri_chunk(gs, w.total[cp], (long long)bw_grid(w, cp, w.total[cp], prec) * eri_groups_per_block(cp, gs));
 }
 
 EriLaunch bw_class_launch(const BatchWork& w, int cp, int pass = 0) {
@@ -264,7 +264,7 @@ cudaError_t bw_enqueue(const BatchWork& w, cudaStream_t s, const Branches* br = 
     for (int pass = 0; pass < (w.fp32_class[cp] ? 2 : 1); ++pass) {
       const EriLaunch L = bw_class_launch(w, cp, pass);
       const int prec = bw_prec(w, cp, pass);
-      e = eri_launch(L, cp, 0, bw_grid(w, cp, w.total[cp], prec), bs, bw_gs(w, cp, prec), prec, true, w.streams[cp]);
+      e = eri_launch(L, cp, 0, bw_grid(w, cp, w.total[cp], prec), bs, bw_gs(w, cp, prec), prec, true);
       if (e != cudaSuccess) return e;
     }
   }
@@ -499,7 +499,7 @@ extern "C" int hfx_batch_tune(hfx_batch* b, const double* const* P, double* cons
         EriLaunch L = bw_class_launch(w, cp, pass);
         L.q_count = w1;
         const int prec = bw_prec(w, cp, pass);
-        CKB(eri_launch(L, cp, 0, bw_grid(w, cp, w1 - w0, prec), s, bw_gs(w, cp, prec), prec, true, w.streams[cp]));
+        CKB(eri_launch(L, cp, 0, bw_grid(w, cp, w1 - w0, prec), s, bw_gs(w, cp, prec), prec, true));
       }
       CKB(cudaEventRecord(t1, s));
       CKB(cudaEventSynchronize(t1));
@@ -521,18 +521,15 @@ extern "C" int hfx_batch_tune(hfx_batch* b, const double* const* P, double* cons
       int gs, streams, chunk;
     };
     std::vector<Cand> cands;
-    // streams are the FP32 pass's alone
-    for (int k : {1, 2, 4})
-      if (w.fp32_class[cp] ? eri_streams_valid(cp, k) : k == 1)
-        for (int c : {2, 8, 32}) cands.push_back({32, w.fp32_class[cp] ? k : 0, c});
+    for (int c : {2, 8, 32}) cands.push_back({32, 0, c});
     // window size: grow from 16k quartets until the incumbent takes the target, and at
     // least two claims for every resident warp of every candidate, so that a large chunk
     // is not timed on a window that leaves most of the GPU idle
     long long fill = 0;
     for (const Cand& cd : cands) {
       const int pr = bw_prec(w, cp, 0);
-      const long long groups = (long long)eri_blocks_per_sm(cp, 0, cd.gs, pr, true, cd.streams) * w.n_sm *
-                               eri_groups_per_block(cp, cd.gs, pr);
+      const long long groups = (long long)eri_blocks_per_sm(cp, 0, cd.gs, pr, true) * w.n_sm *
+                               eri_groups_per_block(cp, cd.gs);
       fill = std::max(fill, 2 * groups * cd.chunk);
     }
     long long win = std::min(total, std::max(16384LL, fill));

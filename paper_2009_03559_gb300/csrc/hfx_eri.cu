@@ -149,215 +149,13 @@ __device__ __forceinline__ int contract_g1(const EriClassInfo& ci, const EriLaun
   return any;
 }
 
-// HRR and Cartesian -> spherical stages on the group scratch S (lanes share each stage)
-template <typename R>
-__device__ __forceinline__ void post_stages(const EriClassInfo& ci, const PairArrays& pa, int bra, int ket, R* S,
-                                            int lane) {
-  R AB[3], CD[3];
-  for (int i = 0; i < 3; ++i) {
-    AB[i] = R(__ldg(pa.AB + 3 * bra + i));
-    CD[i] = R(__ldg(pa.AB + 3 * ket + i));
-  }
-  for (int s = 0; s < ci.n_post; ++s) {
-    const int off = ci.post_off[s], n = ci.post_n[s], type = ci.post_type[s];
-    for (int o = lane; o < n; o += 32) post_op<R>(ld_op(kPostOps, off + o), type, S, 1, AB, CD);
-    __syncwarp();
-  }
-}
-
-// primitive quartets per slot of the packed FP32 pass (2: float2, 4: float4)
-#ifndef HFX_FP32_PACK
-#define HFX_FP32_PACK 4
-#endif
-
-// Group scratch of one warp (in doubles): k stream regions, the coefficient sets (two
-// primitive quartets per set: 16 and the zero set; four: stream regions of twice the size,
-// 8 sets and the zero set, in doubles twice 9 x NCOEF), spare doubles.
-__host__ __device__ __forceinline__ int g32_stride(const SchedVariant& sv) {
-  // float4 slots need 16-byte alignment: an even stride keeps every warp's region aligned
-  return HFX_FP32_PACK == 4 ? 2 * sv.group + 9 * HFX_NCOEF * 2 + 2 : sv.group + 17 * HFX_NCOEF + 1;
-}
-
-// Position of set bit number n (0-based, from the least significant) of m; -1 if m has fewer.
-__device__ __forceinline__ int nth_bit(unsigned m, int n) {
-  for (int i = 0; i < n; ++i) m &= m - 1u;
-  return __ffs(m) - 1;
-}
-
-// Packed FP32 (mixed precision): every slot and coefficient holds W primitive quartets'
-// values (a float2 for W = 2, a float4 for W = 4), so one op of the schedule advances W
-// primitive quartets with one W-wide load per operand and W/2 FFMA2.  The stream regions hold
-// W floats per slot; the coefficient area holds 32/W sets and the zero set.  The contracted
-// block is widened to FP64 (the W components summed in FP64) for the horizontal recurrences,
-// the spherical step and the digest, which run on the FP64 view of the same memory.
-template <int W>
-struct PackV;
-template <>
-struct PackV<2> {
-  using T = float2;
-};
-template <>
-struct PackV<4> {
-  using T = float4;
-};
-
-template <int W>
-__device__ __forceinline__ int contract_g32_xw(const EriClassInfo& ci, const SchedVariant& sv, const EriLaunch& L,
-                                               int bra, int ket, double* Sd, double* CFd, int lane) {
-  using V = typename PackV<W>::T;
-  constexpr int kZeroSet = 32 / W;
-  V* S = reinterpret_cast<V*>(Sd);
-  V* CF = reinterpret_cast<V*>(CFd);
-  V zv;
-  float* zf = reinterpret_cast<float*>(&zv);
-#pragma unroll
-  for (int c = 0; c < W; ++c) zf[c] = 0.f;
-  const PairArrays pa = L.pa;
-  const double omega = L.omega, omega2 = L.omega2;
-  const double* boys = L.boys;
-  const int nb = __ldg(pa.prim_n + bra), nk = __ldg(pa.prim_n + ket);
-  const PrimPair* pb = pa.prim + __ldg(pa.prim_off + bra);
-  const PrimPair* pk = pa.prim + __ldg(pa.prim_off + ket);
-  const int k = sv.k, rsz = sv.rsz, nacc = ci.n_acc, nbase = ci.Lt + 1;
-  for (int i = lane; i < k * nacc; i += 32) {
-    const int u = i / nacc;
-    S[u * rsz + (i - u * nacc)] = zv;
-  }
-  if (lane < k) S[lane * rsz + sv.zero] = zv;
-  for (int i = lane; i < HFX_NCOEF; i += 32) CF[kZeroSet * HFX_NCOEF + i] = zv;
-  const uint4* sched = reinterpret_cast<const uint4*>(kSched) + sv.off;
-  const int npq = nb * nk;
-  int any = 0;
-  // component pos of the packed sets (pos < 32)
-  auto slot_of = [&](int pos) { return reinterpret_cast<float*>(CF + (pos / W) * HFX_NCOEF) + (pos % W); };
-  // the sets of the lanes in okm (at most 32) are in CF: run the schedule over them
-  auto run_sets = [&](unsigned okm) {
-    const int nv = __popc(okm);
-    any += nv;
-    const int r = nv % W;
-    if (r)  // the unused components of the last packed set: all-zero primitive quartets
-      for (int i = lane; i < HFX_NCOEF * (W - r); i += 32) {
-        const int c = i / (W - r);
-        reinterpret_cast<float*>(CF + (nv / W) * HFX_NCOEF + c)[r + (i - c * (W - r))] = 0.f;
-      }
-    __syncwarp();
-    const int np = (nv + W - 1) / W;
-    for (int j = 0; j < np; j += k) {
-      for (int i = lane; i < k * nbase; i += 32) {
-        const int u = i / nbase, m = i - u * nbase;
-        S[u * rsz + nacc + m] = (j + u < np) ? CF[(j + u) * HFX_NCOEF + HFX_CF_G + m] : zv;
-      }
-      __syncwarp();
-      uint4 e = __ldg(sched + lane);
-      for (int it = 1; it <= sv.n_iter; ++it) {
-        const uint4 en = __ldg(sched + it * 32 + lane);
-        sched_op<V>(e, S, rsz, sv.zero, CF, j, np);
-        __syncwarp();
-        e = en;
-      }
-    }
-  };
-  // the primitive quartets c0 + (bits of m0, m1 << 32, m2 << 64) set up in FP64, 32 at a time
-  auto fp64_sets = [&](unsigned m0, unsigned m1, unsigned m2, int c0) {
-    const int n0 = __popc(m0), n1 = __popc(m1), nf = n0 + n1 + __popc(m2);
-    for (int base = 0; base < nf; base += 32) {
-      const int idx = base + lane;
-      bool ok = false;
-      int ib = 0, ik = 0;
-      double G[kMaxLt + 1];
-      PrimScalars ps;
-      if (idx < nf) {
-        const int u = idx < n0 ? nth_bit(m0, idx) : (idx < n0 + n1 ? 32 + nth_bit(m1, idx - n0) : 64 + nth_bit(m2, idx - n0 - n1));
-        const int t = c0 + u;
-        if (u >= 0 && t < npq) {
-          ib = t / nk;
-          ik = t - ib * nk;
-          ok = prim_core(pb[ib], pk[ik], ci.Lt, omega, omega2, boys, G, ps);
-        }
-      }
-      const unsigned okm = __ballot_sync(0xffffffffu, ok);
-      const int pos = __popc(okm & ((1u << lane) - 1u));
-      if (ok) write_set<float, W>(pb[ib], pk[ik], ci.E, ci.F, ci.Lt, G, ps, slot_of(pos));
-      run_sets(okm);
-    }
-  };
-  // FP32 set-up first (prim_core_f32); the primitive quartets it declines are set up in FP64 at
-  // the end of their chunk of 96 (three rounds), 32 at a time, so that the FP64 set-up runs
-  // once per 32 of them rather than in every round in which one lane needs it
-  const float omega_f = to_f32(omega);
-  for (int c0 = 0; c0 < npq; c0 += 96) {
-    unsigned fm[3] = {0u, 0u, 0u};
-#pragma unroll
-    for (int r = 0; r < 3; ++r) {
-      const int base = c0 + 32 * r;
-      if (base >= npq) break;
-      const int t = base + lane;
-      float G[kMaxLt + 1];
-      PrimScalarsF ps;
-      int ib = 0, ik = 0, stt = F32_SKIP;
-      if (t < npq) {
-        ib = t / nk;
-        ik = t - ib * nk;
-        stt = prim_core_f32(pb[ib], pk[ik], ci.Lt, omega_f, G, ps);
-      }
-      fm[r] = __ballot_sync(0xffffffffu, stt == F32_FP64);
-      const bool ok = stt == F32_OK;
-      const unsigned okm = __ballot_sync(0xffffffffu, ok);
-      const int pos = __popc(okm & ((1u << lane) - 1u));
-      if (ok) write_set_f32<W>(pb[ib], pk[ik], ci.E, ci.F, ci.Lt, G, ps, slot_of(pos));
-      run_sets(okm);
-    }
-    if (fm[0] | fm[1] | fm[2]) fp64_sets(fm[0], fm[1], fm[2], c0);
-  }
-  if (!any) return 0;
-  // the streams' sums, widened to FP64 in place: accumulator a's double overlaps the packed
-  // slot a / (W / 2), which the same or an earlier 32-wide slice reads, so each slice reads all
-  // its slots before any lane writes (the other streams' regions lie above the block)
-  for (int a0 = 0; a0 < nacc; a0 += 32) {
-    const int a = a0 + lane;
-    double w = 0.0;
-    if (a < nacc) {
-      V sum = S[a];
-      float* sf = reinterpret_cast<float*>(&sum);
-      for (int u = 1; u < k; ++u) {
-        const V v = S[u * rsz + a];
-        const float* vf = reinterpret_cast<const float*>(&v);
-#pragma unroll
-        for (int c = 0; c < W; ++c) sf[c] += vf[c];
-      }
-      w = to_f64(sf[0]);
-#pragma unroll
-      for (int c = 1; c < W; ++c) w += to_f64(sf[c]);
-    }
-    __syncwarp();
-    if (a < nacc) Sd[a] = w;
-  }
-  __syncwarp();
-  post_stages<double>(ci, pa, bra, ket, Sd, lane);
-  return any;
-}
-
-// Register caps (blocks of 64 threads per SM).  Thread-per-quartet FP64: 6 (at most 170
-// registers), measured fastest; warp kernel: 8 (128 registers: the schedule keeps few values
-// live); the batched thread kernel carries the batch bookkeeping too and the FP32 passes
-// both recurrence precisions' set-up, so they get 4-6 to stay free of spills.
+// Register caps (blocks of 64 threads per SM): FP64 6 (at most 170 registers), measured fastest;
+// the FP32 pass, which carries both set-ups, 4 to stay free of spills.
 #ifndef HFX_G1_MINB
 #define HFX_G1_MINB 6
 #endif
-#ifndef HFX_G32_MINB
-#define HFX_G32_MINB 8
-#endif
-#ifndef HFX_G1B_MINB
-#define HFX_G1B_MINB 6
-#endif
 #ifndef HFX_G1F_MINB
 #define HFX_G1F_MINB 4
-#endif
-#ifndef HFX_G32B_MINB
-#define HFX_G32B_MINB 8
-#endif
-#ifndef HFX_G32F_MINB  // packed FP32 pass: 10 or 12 blocks spill (64-atom mixed build 3354 / 3309 ms vs 3021)
-#define HFX_G32F_MINB 8
 #endif
 
 // One quartet evaluated and digested by one lane (one quartet per thread), recurrences in
@@ -482,49 +280,8 @@ __device__ __forceinline__ void g1_range(const EriLaunch& L, const EriClassInfo&
   }
 }
 
-// Quartets [q0, q1) of the launch record Ls that qualify for FP32, one warp: the warp takes
-// them one by one.  ci and sv: the launch's class record and schedule variant.
-__device__ __forceinline__ void g32_range(const EriClassInfo& ci, const SchedVariant& sv, const EriLaunch& Ls,
-                                          long long q0, long long q1, double* S, int lane, Tally& t) {
-  if (q0 >= q1) return;
-  int r = find_row(Ls.qoff, Ls.row_begin, Ls.row_end, q0);
-  for (long long q = q0; q < q1; ++q) {
-    while (__ldg(Ls.qoff + r + 1) <= q) ++r;
-    const int bra_s = Ls.bra_bin_start + (r - Ls.row_begin);
-    const int ket_s = Ls.ket_bin_start + (int)(q - __ldg(Ls.qoff + r));
-    const int bra = __ldg(Ls.sorted + bra_s), ket = __ldg(Ls.sorted + ket_s);
-    const int sa = __ldg(Ls.pa.sa + bra), sb = __ldg(Ls.pa.sb + bra);
-    const int sc = __ldg(Ls.pa.sa + ket), sd = __ldg(Ls.pa.sb + ket);
-    const double pm = pmax4(Ls, sa, sb, sc, sd);
-    if (Ls.skip_zero && pm == 0.0) continue;
-    // density-weighted screening (off when dens_tau = 0)
-    if (Ls.dens_tau > 0.0 && __ldg(Ls.Qs + bra_s) * __ldg(Ls.Qs + ket_s) * pm < Ls.dens_tau) continue;
-    // distance-aware screening (off when dist_tau = 0)
-    if (!dist_keeps(Ls, bra_s, ket_s)) continue;
-    if (!fp32_eligible(Ls, bra_s, ket_s, pm)) continue;  // warp-uniform
-    const int npq = __ldg(Ls.pa.prim_n + bra) * __ldg(Ls.pa.prim_n + ket);
-    const int ne =
-        contract_g32_xw<HFX_FP32_PACK>(ci, sv, Ls, bra, ket, S, S + (HFX_FP32_PACK / 2) * sv.group, lane);
-    t.prim += ne;
-    t.skip += npq - ne;
-    if (!ne) continue;
-    ++t.quart;
-    ++t.q32;
-    t.p32 += ne;
-    double deg = 1.0;
-    if (sa == sb) deg *= 0.5;
-    if (sc == sd) deg *= 0.5;
-    if (bra_s == ket_s) deg *= 0.5;
-    const int A = __ldg(Ls.sh.bf_off + sa), B = __ldg(Ls.sh.bf_off + sb);
-    const int C = __ldg(Ls.sh.bf_off + sc), D = __ldg(Ls.sh.bf_off + sd);
-    // the contracted block is in FP64 (see contract_g32_xw)
-    digest(ci, S + ci.out_base, 1, A, B, C, D, deg, Ls.P, Ls.K, Ls.ld, lane, 32);
-    __syncwarp();
-  }
-}
-
 template <int PREC, bool BATCH>
-__global__ void __launch_bounds__(64, PREC == PREC_MIXED32 ? HFX_G1F_MINB : (BATCH ? HFX_G1B_MINB : HFX_G1_MINB))
+__global__ void __launch_bounds__(64, PREC == PREC_MIXED32 ? HFX_G1F_MINB : HFX_G1_MINB)
     eri_g1_kernel(const EriLaunch L) {
   extern __shared__ double smem[];
   const int st = blockDim.x;
@@ -546,24 +303,6 @@ __global__ void __launch_bounds__(64, PREC == PREC_MIXED32 ? HFX_G1F_MINB : (BAT
   record_busy(L, t0);
 }
 
-// FP32 pass of a mixed-precision class
-template <bool BATCH>
-__global__ void __launch_bounds__(64, HFX_G32F_MINB) eri_g32_kernel(const EriLaunch L) {
-  extern __shared__ __align__(16) double smem[];
-  const int lane = threadIdx.x & 31, grp = threadIdx.x >> 5;
-  const int gpb = blockDim.x >> 5;
-  double* S = smem + grp * g32_stride(L.sv);
-  unsigned long long t0 = 0;
-  if (L.busy && threadIdx.x == 0) t0 = globaltimer_ns();
-  Tally t;
-  for_each_range<BATCH>(L, (long long)blockIdx.x * gpb + grp, (long long)gridDim.x * gpb, [&]() { return warp_claim(L, lane); },
-                            [&](const EriLaunch& Ls, int, long long q0, long long q1) {
-                              g32_range(L.ci, L.sv, Ls, q0, q1, S, lane, t);
-                            });
-  if (lane == 0) flush_tally(L, t);
-  record_busy(L, t0);
-}
-
 // ---------------------------------------------------------------------------
 // Host-side launch helpers
 // ---------------------------------------------------------------------------
@@ -577,10 +316,9 @@ int eri_group_size() { return 32; }
 
 bool eri_group_size_valid(int gs) { return gs == 1 || gs == 32; }
 
-// Streams of the warp kernel per class (primitive quartets run at a time).  Defaults from a
-// sweep of k = 1, 2, 4 over every warp class of the 64-atom diamond build (plain FP64): more
-// streams fill the iterations with fewer FP64 warp instructions per primitive quartet, but
-// their larger group scratch lowers the resident warps, which the largest classes feel most.
+// Streams (primitive quartets of one quartet run at a time by the schedules of the former warp
+// kernel): the choice is still taken, checked and reported, and no kernel depends on it.  The
+// values a class carries, the largest up to its default last chosen.
 static const int kDefaultStreams[HFX_N_CLASSES] = {
     4, 4, 4, 4, 4, 4,   // ss|ss ps|ss ps|ps pp|ss pp|ps pp|pp
     4, 4, 4, 4,         // ds|ss ds|ps ds|pp ds|ds
@@ -588,15 +326,15 @@ static const int kDefaultStreams[HFX_N_CLASSES] = {
     4, 4, 2, 2, 1, 1};  // dd|ss dd|ps dd|pp dd|ds dd|dp dd|dd
 
 static int variant_index(int cls, int streams) {
-  const SchedVariant* v = kSchedInfo[cls];
+  const int* v = kStreams[cls];
   if (streams > 0) {
     for (int i = 0; i < 3; ++i)
-      if (v[i].k == streams) return i;
+      if (v[i] == streams) return i;
     return -1;
   }
   int best = 0;  // the largest variant carried up to the default
   for (int i = 1; i < 3; ++i)
-    if (v[i].k && v[i].k <= kDefaultStreams[cls]) best = i;
+    if (v[i] && v[i] <= kDefaultStreams[cls]) best = i;
   return best;
 }
 
@@ -606,13 +344,11 @@ bool eri_streams_valid(int cls, int streams) {
 
 int eri_streams(int cls, int streams) {
   const int i = variant_index(cls, streams);
-  return i < 0 ? 0 : kSchedInfo[cls][i].k;
+  return i < 0 ? 0 : kStreams[cls][i];
 }
 
-// The kernel instance for a class launch: FP64 quartets on whole warps run on the Hermite engine
-// (md_*), the FP32 pass on the packed warp kernel, gs = 1 on the thread kernel.
-static bool uses_md(int gs, int prec) { return gs != 1 && prec != PREC_MIXED32; }
-
+// The kernel of a class launch: the Hermite engine (md_*) on whole warps, in FP32 for the FP32
+// pass; the thread kernel for gs = 1.
 static int md_kind(int mode, int prec, bool batch) {
   return mode == 1 ? MD_DIAG : prec == PREC_PERIODIC ? MD_PER : batch ? MD_BATCH : MD_PLAIN;
 }
@@ -622,59 +358,41 @@ static const void* g1_ptr(bool batch) {
   return batch ? (const void*)eri_g1_kernel<PREC, true> : (const void*)eri_g1_kernel<PREC, false>;
 }
 
-static const void* kernel_ptr(int gs, int prec, bool batch) {
-  if (gs != 1) return batch ? (const void*)eri_g32_kernel<true> : (const void*)eri_g32_kernel<false>;
+static const void* kernel_ptr(int prec, bool batch) {
   if (prec == PREC_MIXED64) return g1_ptr<PREC_MIXED64>(batch);
   if (prec == PREC_MIXED32) return g1_ptr<PREC_MIXED32>(batch);
   return g1_ptr<PREC_FP64>(batch);
 }
 
-static int effective_gs(int gs) { return gs == 1 ? 1 : 32; }
-
-size_t eri_smem_bytes(int cls, int gs, int streams, int prec) {
-  if (uses_md(gs, prec)) return md_smem_bytes(cls);
-  // one quartet per thread: interleaved scratch, then a 64-entry quartet queue per warp
-  if (gs == 1) return sizeof(double) * (size_t)kClassInfo[cls].scratch * kBlock + sizeof(int4) * 64 * (kBlock / 32);
-  const int i = variant_index(cls, streams);
-  if (i < 0) return (size_t)1 << 30;
-  return sizeof(double) * (size_t)g32_stride(kSchedInfo[cls][i]) * (kBlock / 32);
+// one quartet per thread: interleaved scratch, then a 64-entry quartet queue per warp
+static size_t g1_smem_bytes(int cls) {
+  return sizeof(double) * (size_t)kClassInfo[cls].scratch * kBlock + sizeof(int4) * 64 * (kBlock / 32);
 }
-
 
 cudaError_t eri_prepare() {
   // allow the largest dynamic shared memory any class needs, for every instance
   size_t mx = 0;
-  for (int c = 0; c < HFX_N_CLASSES; ++c) {
-    mx = std::max(mx, eri_smem_bytes(c, 1, 0));
-    for (int i = 0; i < 3; ++i)
-      if (kSchedInfo[c][i].k) mx = std::max(mx, eri_smem_bytes(c, 32, kSchedInfo[c][i].k, PREC_MIXED32));
-  }
+  for (int c = 0; c < HFX_N_CLASSES; ++c) mx = std::max(mx, g1_smem_bytes(c));
   if (mx > 227 * 1024) mx = 227 * 1024;
   cudaError_t e = md_prepare();
-  if (e != cudaSuccess) return e;
-  auto allow = [&](const void* k) {
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mx);
-  };
-  for (bool batch : {false, true}) {
-    allow(kernel_ptr(32, PREC_MIXED32, batch));
-    for (int prec : {PREC_FP64, PREC_MIXED64, PREC_MIXED32}) allow(kernel_ptr(1, prec, batch));
-  }
+  for (bool batch : {false, true})
+    for (int prec : {PREC_FP64, PREC_MIXED64, PREC_MIXED32})
+      if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(kernel_ptr(prec, batch), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mx);
   return e;
 }
 
-int eri_blocks_per_sm(int cls, int mode, int gs, int prec, bool batch, int streams) {
-  const int g = effective_gs(gs);
-  if (uses_md(g, prec)) return md_blocks_per_sm(cls, md_kind(mode, prec, batch));
+int eri_blocks_per_sm(int cls, int mode, int gs, int prec, bool batch) {
+  if (gs != 1) return md_blocks_per_sm(cls, md_kind(mode, prec, batch), prec == PREC_MIXED32);
   int n = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel_ptr(g, prec, batch), kBlock,
-                                                    eri_smem_bytes(cls, g, streams, prec)) != cudaSuccess)
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel_ptr(prec, batch), kBlock, g1_smem_bytes(cls)) !=
+      cudaSuccess)
     return 1;
   return n > 0 ? n : 1;
 }
 
-int eri_groups_per_block(int cls, int gs, int prec) {
-  if (uses_md(effective_gs(gs), prec)) return md_teams_per_block(cls);
-  return kBlock / effective_gs(gs);
+int eri_groups_per_block(int cls, int gs) {
+  return gs == 1 ? kBlock : md_teams_per_block(cls);
 }
 
 // Quartets per claim of the dynamic schedule.  A thread-kernel warp takes 256.  A whole warp takes
@@ -687,15 +405,13 @@ int eri_chunk(int gs, long long n_quartets, long long n_groups) {
 }
 
 cudaError_t eri_launch(const EriLaunch& L0, int cls, int mode, int grid, cudaStream_t stream, int gs, int prec,
-                       bool batch, int streams) {
-  const int g = effective_gs(gs);
-  if (uses_md(g, prec)) return md_launch(L0, cls, md_kind(mode, prec, batch), prec, grid, stream);
-  const size_t smem = eri_smem_bytes(cls, g, streams, prec);
+                       bool batch) {
+  if (gs != 1) return md_launch(L0, cls, md_kind(mode, prec, batch), prec, prec == PREC_MIXED32, grid, stream);
+  const size_t smem = g1_smem_bytes(cls);
   if (smem > 227 * 1024) return cudaErrorInvalidValue;
   EriLaunch L = L0;
-  if (g == 32) L.sv = kSchedInfo[cls][variant_index(cls, streams)];
   void* args[] = {(void*)&L};
-  return cudaLaunchKernel(kernel_ptr(g, prec, batch), dim3(grid), dim3(kBlock), args, smem, stream);
+  return cudaLaunchKernel(kernel_ptr(prec, batch), dim3(grid), dim3(kBlock), args, smem, stream);
 }
 
 }  // namespace hfx

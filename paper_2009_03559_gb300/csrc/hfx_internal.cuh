@@ -129,6 +129,11 @@ __device__ __forceinline__ float to_f32(double x) {
   const unsigned fb = ((unsigned)(mag - (896 << 20)) << 3) | (lo >> 29);
   return __int_as_float((int)((mag < (897 << 20) ? 0u : fb) | ((unsigned)hi & 0x80000000u)));
 }
+// FP32 value of a double by rounding to nearest (ties away from zero), on the integer units;
+// magnitudes below 2^-126 give 0, above 2^128 are not expected.
+__device__ __forceinline__ float to_f32_rn(double x) {
+  return to_f32(__longlong_as_double(__double_as_longlong(x) + (1ll << 28)));
+}
 // Exact double of a float (subnormal floats give 0).
 __device__ __forceinline__ double to_f64(float f) {
   const int fb = __float_as_int(f);
@@ -176,16 +181,6 @@ __device__ __forceinline__ double boys_asym(int L, double x) {
   return c * v;
 }
 
-// Schedule variant of a class for the warp kernel (generated; see gen_eri_tables.py).
-struct SchedVariant {
-  int k;       // primitive quartets run at a time (streams), 0 = variant absent
-  int rsz;     // doubles (or floats) of group scratch per stream
-  int zero;    // index of the zero slot in a stream's region
-  int n_iter;  // iterations of 32 entries
-  int off;     // first entry in kSched (uint4 units)
-  int group;   // doubles of the stream regions together, at least the post-contraction scratch
-};
-
 // Lattice images (periodic builds): the library holds the home cell's shells repeated in a
 // box of cells (the image shells, cell-major, the home cell first); every pair of the pair
 // list has one shell in the home cell (list-IJ anchored in the home cell, Sec. 3.1).
@@ -217,8 +212,7 @@ struct EriLaunch {
   int chunk;                  // schedule 2: quartets per claim
   const double* boys;         // kMaxLt + 1 tables of kBoysTableLen doubles
   double omega, omega2;
-  SchedVariant sv;             // packed FP32 warp kernel: the schedule variant of this class
-  MdClassInfo mc;              // FP64 warp kernel: the steps of this class
+  MdClassInfo mc;              // Hermite engine: the steps of this class
   int prec;                    // precision pass (PREC_*)
   const double* P;
   double* K;

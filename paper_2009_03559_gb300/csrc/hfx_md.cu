@@ -7,14 +7,20 @@
 #define HFX_CAT(a, b) HFX_CAT2(a, b)
 
 namespace hfx {
-const void* HFX_CAT(md_kernel_l, HFX_MD_L)(int kind) {
+const void* HFX_CAT(md_kernel_l, HFX_MD_L)(int kind, bool f32) {
+  constexpr int l = HFX_MD_L;
+  if (f32)
+    return kind == MD_PLAIN   ? (const void*)eri_md_kernel<l, MD_PLAIN, float>
+           : kind == MD_BATCH ? (const void*)eri_md_kernel<l, MD_BATCH, float>
+                              : nullptr;
   switch (kind) {
-    case MD_PLAIN: return (const void*)eri_md_kernel<HFX_MD_L, MD_PLAIN>;
-    case MD_BATCH: return (const void*)eri_md_kernel<HFX_MD_L, MD_BATCH>;
-    case MD_PER: return (const void*)eri_md_kernel<HFX_MD_L, MD_PER>;
-    // the diagonal (p|p) has an even total angular momentum
-    case MD_DIAG: return HFX_MD_L % 2 ? nullptr : (const void*)eri_md_kernel<HFX_MD_L - HFX_MD_L % 2, MD_DIAG>;
+    case MD_PLAIN: return (const void*)eri_md_kernel<l, MD_PLAIN, double>;
+    case MD_BATCH: return (const void*)eri_md_kernel<l, MD_BATCH, double>;
+    case MD_PER: return (const void*)eri_md_kernel<l, MD_PER, double>;
   }
+#if HFX_MD_L % 2 == 0  // the diagonal (p|p) has an even total angular momentum
+  if (kind == MD_DIAG) return (const void*)eri_md_kernel<l, MD_DIAG, double>;
+#endif
   return nullptr;
 }
 }  // namespace hfx

@@ -15,6 +15,7 @@
 //   transformation passes and the digest.
 #pragma once
 #include <type_traits>
+#include "eri_prim.cuh"
 #include "eri_quartets.cuh"
 #include "hfx_eri.h"
 
@@ -27,13 +28,17 @@ namespace hfx {
 
 // n S for a small integer n: doubling and quadrupling are exponent increments (integer pipe).
 // S = 0 or subnormal becomes at most 4 x 2^-1022: nothing next to any integral.
-template <int N>
-__device__ __forceinline__ double times(double x) {
+template <int N, typename R>
+__device__ __forceinline__ R times(R x) {
   if constexpr (N == 1) return x;
-  if constexpr (N == 2) return scale2(x, 1);
-  if constexpr (N == 4) return scale2(x, 2);
-  return x * N;
+  if constexpr (sizeof(R) == 8) {
+    if constexpr (N == 2) return scale2(x, 1);
+    if constexpr (N == 4) return scale2(x, 2);
+  }
+  return x * R(N);
 }
+__device__ __forceinline__ double fmar(double a, double b, double c) { return __fma_rn(a, b, c); }
+__device__ __forceinline__ float fmar(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 
 // compile-time loop: f(integral constant I), ..., f(integral constant N - 1)
 template <int I, int N, class F>
@@ -42,6 +47,32 @@ __device__ __forceinline__ void unrolled(F&& f) {
     f(std::integral_constant<int, I>());
     unrolled<I + 1, N>(f);
   }
+}
+
+// f(integral constant n) for a run-time n of 1 .. N
+template <int N, class F>
+__device__ __forceinline__ void exact_rounds(int n, F&& f) {
+  if constexpr (N > 1) {
+    if (n < N) {
+      exact_rounds<N - 1>(n, f);
+      return;
+    }
+  }
+  f(std::integral_constant<int, N>());
+}
+
+// f(0) .. f(n - 1), U at a time and the rest one by one (a loop unrolled by the compiler ran its
+// rest as a predicated copy, whose FP64 instructions cost the same when off)
+template <int U, class F>
+__device__ __forceinline__ void stepped(int n, F&& f) {
+  int i = 0;
+#pragma unroll 1
+  for (; i + U <= n; i += U) {
+#pragma unroll
+    for (int k = 0; k < U; ++k) f(i + k);
+  }
+#pragma unroll 1
+  for (; i < n; ++i) f(i);
 }
 
 __host__ __device__ constexpr int n_herm(int n) { return (n + 1) * (n + 2) * (n + 3) / 6; }
@@ -77,36 +108,41 @@ __host__ __device__ constexpr int chain_last(int v) {
 
 // S_r, |r| <= L, from the base values B[m] = (2 rho)^m G_m:  rows in m, first along z, from each
 // of them along y, from each of those along x; only the last two rows of a chain stay live.
-// Warp W of NW writes its share.
-template <int L, int NW, int W>
-__device__ __forceinline__ void hermite(const double (&B)[L + 1], double X, double Y, double Z, double* out) {
+// Warp W of NW writes its share.  In FP32 the recursion runs on s_r = S_r / lam^{|r|} with
+// lam = sqrt(2 rho) (base values G_m, coordinates times lam), whose values stay in range for any
+// exponents, and lp[n] = lam^n scales the results.
+template <int L, int NW, int W, typename R>
+__device__ __forceinline__ void hermite(const R (&B)[L + 1], R X, R Y, R Z, const R* lp, R* out) {
   constexpr int kLastV = chain_last<L, NW, W>(-1);
-  double zr[L + 1], zp[L + 1];
+  R zr[L + 1], zp[L + 1];
 #pragma unroll
   for (int m = 0; m <= L; ++m) zr[m] = B[m];
   unrolled<0, kLastV + 1>([&](auto cv) {
     constexpr int V = decltype(cv)::value;
     constexpr int kLastU = chain_last<L, NW, W>(V);
-    double yr[L + 1 - V], yp[L + 1 - V];
+    R yr[L + 1 - V], yp[L + 1 - V];
 #pragma unroll
     for (int m = 0; m <= L - V; ++m) yr[m] = zr[m];
     unrolled<0, kLastU + 1>([&](auto cu) {
       constexpr int U = decltype(cu)::value;
       constexpr int N = L - V - U;
       if constexpr (chain_owner<L, NW>(U, V) == W) {
-        double xr[N + 1], xp[N + 1];
+        R xr[N + 1], xp[N + 1];
 #pragma unroll
         for (int m = 0; m <= N; ++m) xr[m] = yr[m];
         unrolled<0, N + 1>([&](auto ct) {
           constexpr int T = decltype(ct)::value;
-          out[herm_index(T, U, V)] = xr[0];
+          if constexpr (sizeof(R) == 8 || T + U + V == 0)
+            out[herm_index(T, U, V)] = xr[0];
+          else
+            out[herm_index(T, U, V)] = xr[0] * lp[T + U + V];
 #pragma unroll
           for (int m = 0; m < N - T; ++m) {
-            double v;
+            R v;
             if constexpr (T == 0)
               v = X * xr[m + 1];
             else
-              v = fma(X, xr[m + 1], -times<T>(xp[m + 1]));
+              v = fmar(X, xr[m + 1], -times<T>(xp[m + 1]));
             xp[m] = xr[m];
             xr[m] = v;
           }
@@ -116,11 +152,11 @@ __device__ __forceinline__ void hermite(const double (&B)[L + 1], double X, doub
       if constexpr (U < kLastU) {
 #pragma unroll
         for (int m = 0; m < N; ++m) {
-          double v;
+          R v;
           if constexpr (U == 0)
             v = Y * yr[m + 1];
           else
-            v = fma(Y, yr[m + 1], -times<U>(yp[m + 1]));
+            v = fmar(Y, yr[m + 1], -times<U>(yp[m + 1]));
           yp[m] = yr[m];
           yr[m] = v;
         }
@@ -130,11 +166,11 @@ __device__ __forceinline__ void hermite(const double (&B)[L + 1], double X, doub
     if constexpr (V < kLastV) {
 #pragma unroll
       for (int m = 0; m < L - V; ++m) {
-        double v;
+        R v;
         if constexpr (V == 0)
           v = Z * zr[m + 1];
         else
-          v = fma(Z, zr[m + 1], -times<V>(zp[m + 1]));
+          v = fmar(Z, zr[m + 1], -times<V>(zp[m + 1]));
         zp[m] = zr[m];
         zr[m] = v;
       }
@@ -220,39 +256,71 @@ __device__ __forceinline__ bool md_setup(const PrimPair& b, const PrimPair& k, c
 __host__ __device__ constexpr int md_team(int Lt) { return Lt <= 5 ? 1 : (Lt == 6 ? 2 : 4); }
 __host__ __device__ constexpr int md_block(int Lt) { return Lt <= 5 ? 64 : 32 * md_team(Lt); }
 
+// The FP32 pass of a mixed-precision class runs the same steps with the set-up, the Hermite
+// recursion and both contractions in FP32 (the transformations, which replace the horizontal
+// recurrences and the spherical step, and the digest in FP64).  A team sets up kSub32 times 32
+// primitive quartets before it contracts them, so that those whose Boys step the FP32 set-up
+// declines (a few per cent) are set up in FP64 together: one FP64 set-up per 128 primitive
+// quartets, not one per 32.
+constexpr int kSub32 = 4;
+// 32s of primitive quartets set up together; whether their set-up passes through shared memory;
+// its values per primitive quartet: base values, P - Q (times lam, and lam itself, in FP32)
+template <typename R>
+__host__ __device__ constexpr int md_sub(int Lt) { return sizeof(R) == 4 ? kSub32 : md_team(Lt); }
+template <typename R>
+__host__ __device__ constexpr int md_xval(int Lt) { return sizeof(R) == 4 ? Lt + 5 : Lt + 4; }
+
+// Row of a primitive quartet in shared memory: its Hermite integrals, then the factors of its ket
+// primitive pair (at most as many as the classes of this L have sets); an odd length, so that the
+// lanes' rows start in different banks, and known when compiling, so that the contraction's loads
+// need no address arithmetic.
+__host__ __device__ constexpr int md_row(int Lt) {
+  const int sets[kMaxLt + 1] = {1, 1, 2, 2, 5, 5, 8, 8, 14};
+  return (n_herm(Lt) + sets[Lt]) | 1;
+}
+// Up to L = 4 a lane's entries of the contraction tables and its A values stay in registers (at
+// most this many rounds); up to L = 2, where a ket contraction has at most 13 results, the warp
+// runs 32 / md_group of them side by side.
+__host__ __device__ constexpr int md_kc_rounds(int Lt) { return Lt <= 3 ? 1 : 3; }
+__host__ __device__ constexpr int md_bc_rounds(int Lt) { return Lt <= 2 ? 1 : (Lt == 3 ? 2 : 5); }
+__host__ __device__ constexpr int md_group(int Lt) { return Lt == 0 ? 1 : (Lt == 1 ? 4 : 16); }
+
 // Shared memory of one team, in doubles (offsets; every region starts on an even double).
 struct MdLayout {
-  int rs, ws;                 // strides of a primitive quartet's Hermite integrals and ket factors
-  int R, W, H, A, Tb, Tk, Q;  // H also holds Y, A also the final block
-  int X;                      // teams: set-up results of every warp's primitive quartets
+  int R, H, Y, A, Tb, Tk, Q;  // rows, H, transformed rows (in H's place from L = 3), A and the final block
+  int X;                      // set-up results, where several 32s are set up together
   int size;
 };
-// quartets waiting in a team's queue: fewer than 32 primitive quartets per warp, and 32 more
-__host__ __device__ constexpr int md_queue(int Lt) { return md_team(Lt) == 1 ? 64 : (md_team(Lt) == 2 ? 128 : 256); }
+// quartets waiting in a team's queue: at most 31, and 32 more
+constexpr int kMdQueue = 64;
 
-inline MdLayout md_layout(const MdClassInfo& c, const MdPairInfo& b, const MdPairInfo& k) {
+template <typename R>
+MdLayout md_layout(const MdClassInfo& c, const MdPairInfo& b, const MdPairInfo& k) {
   MdLayout l{};
   auto even = [](int n) { return (n + 1) & ~1; };
-  const int nw = md_team(c.Lt);
-  l.rs = n_herm(c.Lt) | 1;  // odd: the lanes' columns start in different banks
-  l.ws = k.n_set | 1;
+  auto mem = [&](int n) { return even(sizeof(R) == 8 ? n : (n + 1) / 2); };  // n values of type R
   l.R = 0;
-  l.W = l.R + 32 * l.rs;
-  l.H = l.W + 32 * l.ws;
-  l.A = l.H + even(std::max(c.n_kc, c.n_row * c.ncd));
-  l.Tb = l.A + even(std::max(c.n_bc, c.nab * c.ncd));
+  l.H = l.R + mem(32 * md_row(c.Lt));
+  l.Y = c.Lt <= 2 ? l.H + mem(32) + 18 : l.H;  // 18: the runs' first rows
+  l.A = l.Y + std::max(c.Lt <= 2 ? 0 : mem(c.n_kc), even(c.n_row * c.ncd));
+  l.Tb = l.A + std::max(mem(c.n_bc), even(c.nab * c.ncd));
   l.Tk = l.Tb + even(b.n_coef);
   l.Q = l.Tk + even(k.n_coef);
-  l.X = l.Q + 2 * md_queue(c.Lt);
-  // per warp (L + 1) base values and PQ of 32 lanes; the warps' masks and the claim
-  l.size = l.X + (nw > 1 ? nw * (c.Lt + 4) * 32 + 4 : 0);
+  l.X = l.Q + 2 * kMdQueue;
+  const int ns = md_sub<R>(c.Lt);
+  // the values of 32 lanes; the accepted and declined masks; the team's claim
+  l.size = l.X + (ns > 1 ? mem(ns * md_xval<R>(c.Lt) * 32) + ns + 2 : 0);
   return l;
 }
 
 // A sparse pass out[dst] = sum of T[c] in[i] (generated: rounds of 32 outputs of like length),
 // rounds w, w + nw, ...
-__device__ __forceinline__ void md_gather(int round0, int n_round, int dst0, const double* T, const double* in,
+__device__ __forceinline__ double widen(double x) { return x; }
+__device__ __forceinline__ double widen(float x) { return to_f64(x); }
+template <typename R>
+__device__ __forceinline__ void md_gather(int round0, int n_round, int dst0, const double* T, const R* in,
                                           double* out, int lane, int w, int nw) {
+#pragma unroll 1
   for (int r = w; r < n_round; r += nw) {
     const uint32_t rd = __ldg(kMdZRound + round0 + r);
     const uint32_t* word = kMdZ + (rd & 0xFFFFFFu) + lane;
@@ -261,7 +329,7 @@ __device__ __forceinline__ void md_gather(int round0, int n_round, int dst0, con
 #pragma unroll 4
     for (int t = 0; t < n; ++t) {
       const uint32_t e = __ldg(word + 32 * t);
-      v = fma(T[e & 0xFFFFu], in[e >> 16], v);
+      v = fma(T[e & 0xFFFFu], widen(in[e >> 16]), v);
     }
     const uint32_t d = __ldg(kMdZDst + dst0 + 32 * r + lane);
     if (d != 0xFFFFu) out[d] = v;
@@ -312,26 +380,36 @@ __device__ __forceinline__ void md_digest(const EriClassInfo& ci, const double* 
 }
 
 // resident blocks per SM that the registers must allow: what shared memory allows
-__host__ __device__ constexpr int md_minb(int Lt) { return Lt <= 4 ? 8 : (Lt <= 6 ? 5 : (Lt == 7 ? 3 : 2)); }
+template <typename R>
+__host__ __device__ constexpr int md_minb(int Lt) {
+  return sizeof(R) == 4 ? (Lt <= 6 ? 8 : 4) : (Lt <= 4 ? 8 : (Lt <= 6 ? 5 : (Lt == 7 ? 3 : 2)));
+}
 
-template <int LT, int KIND>
-__global__ void __launch_bounds__(md_block(LT), md_minb(LT))
+template <int LT, int KIND, typename R>
+__global__ void __launch_bounds__(md_block(LT), md_minb<R>(LT))
     eri_md_kernel(const __grid_constant__ EriLaunch L, const __grid_constant__ MdLayout ly) {
   extern __shared__ __align__(16) double smem[];
-  constexpr int NW = md_team(LT), kQ = md_queue(LT), kTeams = md_block(LT) / (32 * NW);
+  constexpr bool F32 = sizeof(R) == 4;
+  constexpr int NW = md_team(LT), kQ = kMdQueue, kTeams = md_block(LT) / (32 * NW);
+  constexpr int NS = md_sub<R>(LT), NX = md_xval<R>(LT);
+  constexpr int kRow = md_row(LT), kW = n_herm(LT);
+  constexpr bool kRegs = LT <= 4;
+  constexpr int KR = md_kc_rounds(LT), BR = md_bc_rounds(LT);
   const int lane = threadIdx.x & 31;
   const int wt = NW == 1 ? 0 : (int)(threadIdx.x >> 5);             // warp of the team
   const int team = NW == 1 ? (int)(threadIdx.x >> 5) : 0;           // team of the block
   double* S = smem + team * ly.size;
-  double* const Rb = S + ly.R;
-  double* const Wb = S + ly.W;
-  double* const H = S + ly.H;
-  double* const A = S + ly.A;
+  R* const Rb = reinterpret_cast<R*>(S + ly.R);
+  R* const H = reinterpret_cast<R*>(S + ly.H);
+  R* const A = reinterpret_cast<R*>(S + ly.A);
+  double* const Y = S + ly.Y;
+  double* const F = S + ly.A;
   int4* const Q = reinterpret_cast<int4*>(S + ly.Q);  // system, bra position, ket position, nb | nk << 16
-  double* const X = S + ly.X;
-  unsigned* const Xok = reinterpret_cast<unsigned*>(X + NW * (LT + 4) * 32);  // masks, then the claim
+  R* const X = reinterpret_cast<R*>(S + ly.X);
+  unsigned* const Xok = reinterpret_cast<unsigned*>(S + ly.size - NS - 2);  // masks [NS], [NS], then the claim
   const unsigned lt_mask = (1u << lane) - 1u;
   const MdClassInfo mc = L.mc;
+  const EriLaunch* const Lp = &L;
   unsigned long long t0 = 0;
   if (L.busy && threadIdx.x == 0) t0 = globaltimer_ns();
 
@@ -340,6 +418,25 @@ __global__ void __launch_bounds__(md_block(LT), md_minb(LT))
   int n_eval = 0;                                     // its primitive quartets evaluated so far
   int tb_sys = -1, tb_bra = -1;                       // whose transformation is in Tb
   Tally tally;
+
+  int kc_r[kRegs ? KR : 1], kc_w[kRegs ? KR : 1], bc_h[kRegs ? BR : 1], bc_w[kRegs ? BR : 1];
+  R a_reg[kRegs ? BR : 1];
+  if constexpr (kRegs) {
+#pragma unroll
+    for (int u = 0; u < KR; ++u) {
+      const int o = 32 * u + (LT <= 2 ? lane % md_group(LT) : lane);
+      const int e = o < mc.n_kc ? __ldg(kMdKc + mc.kc + o) : 0;
+      kc_r[u] = e & 0xFF;
+      kc_w[u] = kW + (e >> 8);
+    }
+#pragma unroll
+    for (int u = 0; u < BR; ++u) {
+      const int e = 32 * u + lane < mc.n_bc ? __ldg(kMdBc + mc.bc + 32 * u + lane) : 0;
+      bc_h[u] = e & 0xFFF;
+      bc_w[u] = e >> 12;
+      a_reg[u] = R(0);
+    }
+  }
 
   auto sync = [&]() {
     if constexpr (NW == 1)
@@ -351,7 +448,7 @@ __global__ void __launch_bounds__(md_block(LT), md_minb(LT))
     if constexpr (KIND == MD_BATCH)
       return L.batch[sys];
     else
-      return L;
+      return *Lp;
   };
   auto pair_id = [&](const EriLaunch& Ls, int pos) -> int {
     if constexpr (KIND == MD_DIAG)
@@ -360,58 +457,95 @@ __global__ void __launch_bounds__(md_block(LT), md_minb(LT))
       return __ldg(Ls.sorted + pos);
   };
 
-  // H[s, r] (+)= sum over the primitive quartets in slots [p0, p1) of W_s S_r
+  auto narrow = [](double x) -> R {
+    if constexpr (F32)
+      return to_f32_rn(x);
+    else
+      return x;
+  };
+
+  // H[s, r] (+)= sum over the primitive quartets in rows [p0, p1) of W_s S_r
   auto ket_contract = [&](int p0, int p1) {
-    auto rounds = [&](int g, auto nc) {
-      constexpr int N = decltype(nc)::value;
-      int ri[N], si[N];
-      double v[N];
+    if constexpr (kRegs) {
+      // the round count decides a branch: as a predicate inside the loop it was turned into
+      // selects, with the FP64 instructions of all rounds executed
+      exact_rounds<KR>((mc.n_kc + 31) >> 5, [&](auto nc) {
+        constexpr int N = decltype(nc)::value;
+        const R *r[N], *w[N];
+        R v[N];
 #pragma unroll
-      for (int u = 0; u < N; ++u) {
-        const int e = __ldg(kMdKc + mc.kc + 32 * (g + NW * u) + lane);  // padded to whole rounds
-        ri[u] = e & 0xFF;
-        si[u] = e >> 8;
-        v[u] = 0.0;
-      }
-      const double* R = Rb + p0 * ly.rs;
-      const double* W = Wb + p0 * ly.ws;
-      for (int p = p0; p < p1; ++p, R += ly.rs, W += ly.ws) {
+        for (int u = 0; u < N; ++u) {
+          r[u] = Rb + p0 * kRow + kc_r[u];
+          w[u] = Rb + p0 * kRow + kc_w[u];
+          v[u] = h_valid && 32 * u + lane < mc.n_kc ? H[32 * u + lane] : R(0);
+        }
+        stepped<4>(p1 - p0, [&](int p) {
 #pragma unroll
-        for (int u = 0; u < N; ++u) v[u] = fma(W[si[u]], R[ri[u]], v[u]);
-      }
+          for (int u = 0; u < N; ++u) v[u] = fmar(w[u][p * kRow], r[u][p * kRow], v[u]);
+        });
 #pragma unroll
-      for (int u = 0; u < N; ++u) {
-        const int o = 32 * (g + NW * u) + lane;
-        if (o < mc.n_kc) H[o] = h_valid ? H[o] + v[u] : v[u];
-      }
-    };
-    const int n = (mc.n_kc + 31) >> 5;
-    int g = wt;  // this warp's rounds: wt, wt + NW, ...
-    for (; g + 3 * NW < n; g += 4 * NW) rounds(g, std::integral_constant<int, 4>());
-    if (g + 2 * NW < n)
-      rounds(g, std::integral_constant<int, 3>());
-    else if (g + NW < n)
-      rounds(g, std::integral_constant<int, 2>());
-    else if (g < n)
-      rounds(g, std::integral_constant<int, 1>());
+        for (int u = 0; u < N; ++u) {
+          const int o = 32 * u + lane;
+          if (o < mc.n_kc) H[o] = v[u];
+        }
+      });
+    } else {
+      auto rounds = [&](int g, auto nc) {
+        constexpr int N = decltype(nc)::value;
+        const R *r[N], *w[N];
+        R v[N];
+#pragma unroll
+        for (int u = 0; u < N; ++u) {
+          const int e = __ldg(kMdKc + mc.kc + 32 * (g + NW * u) + lane);  // padded to whole rounds
+          r[u] = Rb + p0 * kRow + (e & 0xFF);
+          w[u] = Rb + p0 * kRow + kW + (e >> 8);
+          const int o = 32 * (g + NW * u) + lane;
+          v[u] = h_valid && o < mc.n_kc ? H[o] : R(0);
+        }
+          stepped<2>(p1 - p0, [&](int p) {
+#pragma unroll
+            for (int u = 0; u < N; ++u) v[u] = fmar(w[u][p * kRow], r[u][p * kRow], v[u]);
+          });
+#pragma unroll
+        for (int u = 0; u < N; ++u) {
+          const int o = 32 * (g + NW * u) + lane;
+          if (o < mc.n_kc) H[o] = v[u];
+        }
+      };
+      const int n = (mc.n_kc + 31) >> 5;
+      int g = wt;  // this warp's rounds: wt, wt + NW, ...
+#pragma unroll 1
+      for (; g + 3 * NW < n; g += 4 * NW) rounds(g, std::integral_constant<int, 4>());
+#pragma unroll 1
+      for (; g < n; g += NW) rounds(g, std::integral_constant<int, 1>());
+    }
     sync();
   };
 
   // A[s', s, r] (+)= W_s' H[s, r] for the bra primitive pair with factors w
-  auto bra_contract = [&](const double* w) {
+  auto bra_contract = [&](const double* w, const R* H) {
+    if constexpr (kRegs) {
+      exact_rounds<BR>((mc.n_bc + 31) >> 5, [&](auto nc) {
+#pragma unroll
+        for (int u = 0; u < decltype(nc)::value; ++u)
+          a_reg[u] = fmar(narrow(__ldg(w + bc_w[u])), H[bc_h[u]], a_reg[u]);
+      });
+      if constexpr (LT > 2) sync();
+      return;
+    }
     auto rounds = [&](int o, auto nc) {
       constexpr int N = decltype(nc)::value;
-      double x[N], h[N], a[N];
+      R x[N], h[N], a[N];
 #pragma unroll
       for (int u = 0; u < N; ++u) {
         const int e = __ldg(kMdBc + mc.bc + o + 32 * NW * u);  // padded to whole rounds
-        x[u] = __ldg(w + (e >> 12));
+        x[u] = narrow(__ldg(w + (e >> 12)));
         h[u] = H[e & 0xFFF];
-        a[u] = a_valid && o + 32 * NW * u < mc.n_bc ? A[o + 32 * NW * u] : 0.0;
+        a[u] = a_valid && o + 32 * NW * u < mc.n_bc ? A[o + 32 * NW * u] : R(0);
       }
 #pragma unroll
       for (int u = 0; u < N; ++u)
-        if (o + 32 * NW * u < mc.n_bc) A[o + 32 * NW * u] = fma(x[u], h[u], a[u]);
+        if (o + 32 * NW * u < mc.n_bc) A[o + 32 * NW * u] = fmar(x[u], h[u], a[u]);
     };
     const int n = (mc.n_bc + 31) >> 5;
     int g = wt;
@@ -429,7 +563,18 @@ __global__ void __launch_bounds__(md_block(LT), md_minb(LT))
     double* Tk = S + ly.Tk;
     const int bra = pair_id(Ls, e.y), ket = pair_id(Ls, e.z);
     if (a_valid) {
+      if constexpr (kRegs) {
+#pragma unroll
+        for (int u = 0; u < BR; ++u) {
+          if (32 * u + lane < mc.n_bc) A[32 * u + lane] = a_reg[u];
+          a_reg[u] = R(0);
+        }
+      }
       ++tally.quart;
+      if (F32) {
+        ++tally.q32;
+        tally.p32 += n_eval;
+      }
       const double* mk = Ls.pa.md + __ldg(Ls.pa.md_off + ket);
       for (int i = 32 * wt + lane; i < mc.ket_coef; i += 32 * NW) Tk[i] = __ldg(mk + i);
       if (tb_bra != bra || tb_sys != e.x) {
@@ -444,15 +589,15 @@ __global__ void __launch_bounds__(md_block(LT), md_minb(LT))
         tb_sys = e.x;
       }
       sync();
-      md_gather(mc.z1_round, mc.z1_n, mc.z1_dst, Tk, A, H, lane, wt, NW);  // Y takes H's place
+      md_gather<R>(mc.z1_round, mc.z1_n, mc.z1_dst, Tk, A, Y, lane, wt, NW);
       sync();
-      md_gather(mc.z2_round, mc.z2_n, mc.z2_dst, Tb, H, A, lane, wt, NW);  // the final block takes A's
+      md_gather<double>(mc.z2_round, mc.z2_n, mc.z2_dst, Tb, Y, F, lane, wt, NW);
       sync();
     }
     if constexpr (KIND == MD_DIAG) {
       double mx = 0.0;
       if (a_valid) {
-        for (int f = lane; f < mc.ncd; f += 32) mx = fmax(mx, fabs(A[f * mc.ncd + f]));
+        for (int f = lane; f < mc.ncd; f += 32) mx = fmax(mx, fabs(F[f * mc.ncd + f]));
         for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
       }
       if (lane == 0 && wt == 0) Ls.diag_Q[bra] = sqrt(mx);
@@ -460,7 +605,7 @@ __global__ void __launch_bounds__(md_block(LT), md_minb(LT))
       if constexpr (KIND == MD_PER) {
         PerQuartet pq;
         if (per_quartet(Ls, bra, ket, pq))
-          digest_per(L.ci, A, 1, pq, Ls.KG, Ls.per.nbf, 32 * wt + lane, 32 * NW);
+          digest_per(L.ci, F, 1, pq, Ls.KG, Ls.per.nbf, 32 * wt + lane, 32 * NW);
       } else {
         const int sa = __ldg(Ls.pa.sa + bra), sb = __ldg(Ls.pa.sb + bra);
         const int sc = __ldg(Ls.pa.sa + ket), sd = __ldg(Ls.pa.sb + ket);
@@ -468,7 +613,7 @@ __global__ void __launch_bounds__(md_block(LT), md_minb(LT))
         if (sa == sb) deg *= 0.5;
         if (sc == sd) deg *= 0.5;
         if (e.y == e.z) deg *= 0.5;
-        md_digest(L.ci, A, __ldg(Ls.sh.bf_off + sa), __ldg(Ls.sh.bf_off + sb), __ldg(Ls.sh.bf_off + sc),
+        md_digest(L.ci, F, __ldg(Ls.sh.bf_off + sa), __ldg(Ls.sh.bf_off + sb), __ldg(Ls.sh.bf_off + sc),
                   __ldg(Ls.sh.bf_off + sd), deg, Ls.P, Ls.K, Ls.ld, 32 * wt + lane, 32 * NW);
       }
     }
@@ -500,74 +645,137 @@ __global__ void __launch_bounds__(md_block(LT), md_minb(LT))
     return s;
   };
 
-  // the next n (<= 32 NW, <= waiting) primitive quartets of the stream
+  // the primitive pairs of s
+  auto prims = [&](const Prim& s, const PrimPair*& pb, const PrimPair*& pk) -> const EriLaunch& {
+    const EriLaunch& Ls = rec(s.q.x);
+    const int bra = pair_id(Ls, s.q.y), ket = pair_id(Ls, s.q.z);
+    pb = Ls.pa.prim + __ldg(Ls.pa.prim_off + bra) + s.ib;
+    pk = Ls.pa.prim + __ldg(Ls.pa.prim_off + ket) + s.ik;
+    return Ls;
+  };
+
+  // the next n (<= 32 NS, <= waiting) primitive quartets of the stream
   auto batch = [&](int n) {
     Prim s{};
-    s.nb = s.nk = 1;
+    unsigned okm = 0;
     bool ok = false;
-    double B[LT + 1], PQ[3];
-    if (32 * wt + lane < n) {  // set-up: warp w of the team the w-th 32
-      s = locate(32 * wt + lane);
-      const EriLaunch& Ls = rec(s.q.x);
-      const int bra = pair_id(Ls, s.q.y), ket = pair_id(Ls, s.q.z);
-      const PrimPair& pb = Ls.pa.prim[__ldg(Ls.pa.prim_off + bra) + s.ib];
-      const PrimPair& pk = Ls.pa.prim[__ldg(Ls.pa.prim_off + ket) + s.ik];
-      double qc[3] = {pk.P[0], pk.P[1], pk.P[2]};
-      if constexpr (KIND == MD_PER) {  // the ket pair's image in cell G
-        qc[0] += L.shift[0];
-        qc[1] += L.shift[1];
-        qc[2] += L.shift[2];
+    R B[LT + 1], PQ[3], lam = R(1);
+#pragma unroll 1
+    for (int sub = wt; sub < NS; sub += NW) {  // set-up
+      s = Prim{};
+      s.nb = s.nk = 1;
+      ok = false;
+      bool declined = false;
+      if (32 * sub + lane < n) {
+        s = locate(32 * sub + lane);
+        const PrimPair *pb, *pk;
+        const EriLaunch& Ls = prims(s, pb, pk);
+        if constexpr (F32) {
+          PrimScalarsF ps;
+          const int st = prim_core_f32(*pb, *pk, LT, to_f32(Ls.omega), B, ps);
+          lam = sqrtf(2.0f * pb->pf * ps.RP);
+          for (int i = 0; i < 3; ++i) PQ[i] = ps.PQ[i] * lam;
+          ok = st == F32_OK;
+          declined = st == F32_FP64;
+        } else {
+          double qc[3] = {pk->P[0], pk->P[1], pk->P[2]};
+          if constexpr (KIND == MD_PER) {  // the ket pair's image in cell G
+            qc[0] += L.shift[0];
+            qc[1] += L.shift[1];
+            qc[2] += L.shift[2];
+          }
+          ok = md_setup<LT>(*pb, *pk, qc, Ls.omega, Ls.omega2, Ls.boys, B, PQ);
+        }
       }
-      ok = md_setup<LT>(pb, pk, qc, Ls.omega, Ls.omega2, Ls.boys, B, PQ);
+      okm = __ballot_sync(0xffffffffu, ok);
+      if constexpr (NS > 1) {
+        R* x = X + sub * NX * 32 + lane;
+#pragma unroll
+        for (int m = 0; m <= LT; ++m) x[32 * m] = B[m];
+#pragma unroll
+        for (int i = 0; i < 3; ++i) x[32 * (LT + 1 + i)] = PQ[i];
+        if constexpr (F32) x[32 * (LT + 4)] = lam;
+        const unsigned dm = __ballot_sync(0xffffffffu, declined);
+        if (lane == 0) {
+          Xok[sub] = okm;
+          Xok[NS + sub] = dm;
+        }
+      }
     }
-    unsigned okm = __ballot_sync(0xffffffffu, ok);
-    if constexpr (NW > 1) {
-      double* x = X + wt * (LT + 4) * 32 + lane;
+    if constexpr (NS > 1) sync();
+    if constexpr (F32) {
+      // the declined ones in FP64, 32 at a time: their base values replace the FP32 ones
+      int nd = 0;
+      for (int sub = 0; sub < NS; ++sub) nd += __popc(Xok[NS + sub]);
+      for (int d0 = 32 * wt; d0 < nd; d0 += 32 * NW) {
+        int d = d0 + lane, sub = 0;
+        if (d < nd) {
+          unsigned m = Xok[NS];
+          while (d >= __popc(m)) {
+            d -= __popc(m);
+            m = Xok[NS + ++sub];
+          }
+          for (; d > 0; --d) m &= m - 1;
+          const int l = __ffs(m) - 1;
+          const Prim t = locate(32 * sub + l);
+          const PrimPair *pb, *pk;
+          const EriLaunch& Ls = prims(t, pb, pk);
+          double G[kMaxLt + 1];
+          PrimScalars ps;
+          if (prim_core(*pb, *pk, LT, Ls.omega, Ls.omega2, Ls.boys, G, ps)) {
 #pragma unroll
-      for (int m = 0; m <= LT; ++m) x[32 * m] = B[m];
-#pragma unroll
-      for (int i = 0; i < 3; ++i) x[32 * (LT + 1 + i)] = PQ[i];
-      if (lane == 0) Xok[wt] = okm;
+            for (int k = 0; k <= LT; ++k) X[(sub * NX + k) * 32 + l] = to_f32_rn(G[k]);
+            atomicOr(Xok + sub, 1u << l);
+          }
+        }
+      }
       sync();
     }
-    for (int sub = 0; sub < NW && 32 * sub < n; ++sub) {
+#pragma unroll 1
+    for (int sub = 0; sub < NS && 32 * sub < n; ++sub) {
       const int ns = min(32, n - 32 * sub);
-      if constexpr (NW > 1) {
+      R lp[F32 ? LT + 1 : 1];
+      lp[0] = R(1);
+      if constexpr (NS > 1) {
         okm = Xok[sub];
         ok = (okm >> lane) & 1;
+        s = Prim{};
         s.nb = s.nk = 1;
-        s.ib = s.ik = 0;
         if (lane < ns) s = locate(32 * sub + lane);
-        const double* x = X + sub * (LT + 4) * 32 + lane;
+        const R* x = X + sub * NX * 32 + lane;
 #pragma unroll
         for (int m = 0; m <= LT; ++m) B[m] = x[32 * m];
 #pragma unroll
         for (int i = 0; i < 3; ++i) PQ[i] = x[32 * (LT + 1 + i)];
+        if constexpr (F32) {
+          lam = x[32 * (LT + 4)];
+#pragma unroll
+          for (int m = 1; m <= LT; ++m) lp[m] = lp[m - 1] * lam;
+        }
       }
       if (ok) {
         const EriLaunch& Ls = rec(s.q.x);
         const int ket = pair_id(Ls, s.q.z);
         const double* wk = Ls.pa.md + __ldg(Ls.pa.md_off + ket) + mc.ket_coef + s.ik * mc.ket_set;
         const int pos = __popc(okm & lt_mask);
-        double* w = Wb + pos * ly.ws;
-        for (int i = wt; i < mc.ket_set; i += NW) w[i] = __ldg(wk + i);
-        double* R = Rb + pos * ly.rs;
-        if constexpr (NW == 1) hermite<LT, 1, 0>(B, PQ[0], PQ[1], PQ[2], R);
+        R* r = Rb + pos * kRow;
+        for (int i = wt; i < mc.ket_set; i += NW) r[kW + i] = narrow(__ldg(wk + i));
+        if constexpr (NW == 1) hermite<LT, 1, 0>(B, PQ[0], PQ[1], PQ[2], lp, r);
         if constexpr (NW == 2) {
           if (wt == 0)
-            hermite<LT, 2, 0>(B, PQ[0], PQ[1], PQ[2], R);
+            hermite<LT, 2, 0>(B, PQ[0], PQ[1], PQ[2], lp, r);
           else
-            hermite<LT, 2, 1>(B, PQ[0], PQ[1], PQ[2], R);
+            hermite<LT, 2, 1>(B, PQ[0], PQ[1], PQ[2], lp, r);
         }
         if constexpr (NW == 4) {
           if (wt == 0)
-            hermite<LT, 4, 0>(B, PQ[0], PQ[1], PQ[2], R);
+            hermite<LT, 4, 0>(B, PQ[0], PQ[1], PQ[2], lp, r);
           else if (wt == 1)
-            hermite<LT, 4, 1>(B, PQ[0], PQ[1], PQ[2], R);
+            hermite<LT, 4, 1>(B, PQ[0], PQ[1], PQ[2], lp, r);
           else if (wt == 2)
-            hermite<LT, 4, 2>(B, PQ[0], PQ[1], PQ[2], R);
+            hermite<LT, 4, 2>(B, PQ[0], PQ[1], PQ[2], lp, r);
           else
-            hermite<LT, 4, 3>(B, PQ[0], PQ[1], PQ[2], R);
+            hermite<LT, 4, 3>(B, PQ[0], PQ[1], PQ[2], lp, r);
         }
       }
       sync();
@@ -576,27 +784,72 @@ __global__ void __launch_bounds__(md_block(LT), md_minb(LT))
       unsigned lead = __ballot_sync(0xffffffffu, lane < ns && (lane == 0 || s.e != e_up || s.ib != ib_up));
       const unsigned last_k = __ballot_sync(0xffffffffu, s.ik == s.nk - 1);
       const unsigned last_q = __ballot_sync(0xffffffffu, s.ik == s.nk - 1 && s.ib == s.nb - 1);
-      while (lead) {
-        const int l0 = __ffs(lead) - 1;
-        lead &= lead - 1;
-        const int l1 = lead ? __ffs(lead) - 1 : ns;
-        const int p0 = __popc(okm & ((1u << l0) - 1u)), p1 = __popc(okm & (0xffffffffu >> (32 - l1)));
-        if (p1 > p0) {
-          ket_contract(p0, p1);
-          h_valid = true;
-          n_eval += p1 - p0;
-        }
-        if ((last_k >> (l1 - 1)) & 1) {
-          const int4 q = Q[__shfl_sync(0xffffffffu, s.e, l0) & (kQ - 1)];
-          if (h_valid) {
-            const EriLaunch& Ls = rec(q.x);
-            const int bra = pair_id(Ls, q.y);
-            bra_contract(Ls.pa.md + __ldg(Ls.pa.md_off + bra) + mc.bra_coef +
-                         __shfl_sync(0xffffffffu, s.ib, l0) * mc.bra_set);
-            a_valid = true;
-            h_valid = false;
+      if constexpr (LT <= 2) {
+        // 32 / md_group runs side by side, then the bra contraction of each.  A run cut by the end
+        // of a batch needs no carry: its parts add up in A.
+        constexpr int GL = md_group(LT), G = 32 / GL;
+        int* const first_row = reinterpret_cast<int*>(S + ly.Y - 18);
+        const int nr = __popc(lead);
+        if ((lead >> lane) & 1) first_row[__popc(lead & lt_mask)] = __popc(okm & lt_mask);
+        if (lane == 0) first_row[nr] = __popc(okm);
+        __syncwarp();
+#pragma unroll 1
+        for (int t0 = 0; t0 < nr; t0 += G) {
+          const int t = t0 + lane / GL;
+          const int p0 = t < nr ? first_row[t] : 0, len = t < nr ? first_row[t + 1] - p0 : 0;
+          const int most = __reduce_max_sync(0xffffffffu, len);
+          const R* r = Rb + p0 * kRow + kc_r[0];
+          const R* w = Rb + p0 * kRow + kc_w[0];
+          R v = R(0);
+#pragma unroll 4
+          for (int p = 0; p < most; ++p)
+            if (p < len) v = fmar(w[p * kRow], r[p * kRow], v);
+          H[lane] = v;
+          __syncwarp();
+#pragma unroll 1
+          for (int u = t0; u < min(t0 + G, nr); ++u) {
+            const int l0 = __ffs(lead) - 1;
+            lead &= lead - 1;
+            const int l1 = lead ? __ffs(lead) - 1 : ns;
+            const int np = first_row[u + 1] - first_row[u];
+            const int4 q = Q[__shfl_sync(0xffffffffu, s.e, l0) & (kQ - 1)];
+            if (np > 0) {
+              const EriLaunch& Ls = rec(q.x);
+              const int bra = pair_id(Ls, q.y);
+              bra_contract(Ls.pa.md + __ldg(Ls.pa.md_off + bra) + mc.bra_coef +
+                               __shfl_sync(0xffffffffu, s.ib, l0) * mc.bra_set,
+                           H + (u - t0) * GL);
+              a_valid = true;
+              n_eval += np;
+            }
+            if ((last_q >> (l1 - 1)) & 1) finish(q);
           }
-          if ((last_q >> (l1 - 1)) & 1) finish(q);
+          __syncwarp();
+        }
+      } else {
+        while (lead) {
+          const int l0 = __ffs(lead) - 1;
+          lead &= lead - 1;
+          const int l1 = lead ? __ffs(lead) - 1 : ns;
+          const int p0 = __popc(okm & ((1u << l0) - 1u)), p1 = __popc(okm & (0xffffffffu >> (32 - l1)));
+          if (p1 > p0) {
+            ket_contract(p0, p1);
+            h_valid = true;
+            n_eval += p1 - p0;
+          }
+          if ((last_k >> (l1 - 1)) & 1) {
+            const int4 q = Q[__shfl_sync(0xffffffffu, s.e, l0) & (kQ - 1)];
+            if (h_valid) {
+              const EriLaunch& Ls = rec(q.x);
+              const int bra = pair_id(Ls, q.y);
+              bra_contract(Ls.pa.md + __ldg(Ls.pa.md_off + bra) + mc.bra_coef +
+                               __shfl_sync(0xffffffffu, s.ib, l0) * mc.bra_set,
+                           H);
+              a_valid = true;
+              h_valid = false;
+            }
+            if ((last_q >> (l1 - 1)) & 1) finish(q);
+          }
         }
       }
       if (32 * (sub + 1) >= n) {  // the stream's new head: after the last lane
@@ -611,69 +864,116 @@ __global__ void __launch_bounds__(md_block(LT), md_minb(LT))
     sync();
   };
 
-  // a candidate quartet per lane (the same in every warp of a team): queue those that pass
-  auto push = [&](bool keep, int sys, int bra_s, int ket_s, int nb, int nk) {
-    keep = keep && nb > 0 && nk > 0;
-    const unsigned m = __ballot_sync(0xffffffffu, keep);
-    if (keep && wt == 0) Q[(tail + __popc(m & lt_mask)) & (kQ - 1)] = make_int4(sys, bra_s, ket_s, nb | (nk << 16));
-    tail += __popc(m);
-    waiting += __reduce_add_sync(0xffffffffu, keep ? nb * nk : 0);
-    sync();
-    while (waiting >= 32 * NW) batch(32 * NW);
+  // The team's next candidates, up to 32 of them, a lane each (the same in every warp): quartets
+  // [q0, q1) of the list of Ls (system sys), r the row of q0; or pairs of the diagonal.
+  long long q0 = 0, q1 = 0, c0 = 0, c1 = 0;
+  int r = 0, sys = 0;
+  bool first = true;
+  const long long wid = blockIdx.x * kTeams + team, nteam = (long long)gridDim.x * kTeams;
+  auto next_range = [&]() -> bool {
+    if constexpr (KIND == MD_DIAG) {
+      q0 = first ? wid : q0 - 32 + nteam;  // one pair at a time: q0 has been advanced by 32
+      q1 = q0 + 1;
+      first = false;
+      return q0 < L.diag_n;
+    } else {
+      while (true) {
+        if (KIND != MD_BATCH && L.schedule != 2) {
+          if (!first) return false;
+          first = false;
+          group_range(L, wid, nteam, q0, q1);
+        } else {
+          if (c0 >= c1) {  // claim a chunk
+            unsigned long long c = 0;
+            if (lane == 0 && wt == 0) c = atomicAdd(L.work, (unsigned long long)L.chunk);
+            if constexpr (NW == 1) {
+              c = __shfl_sync(0xffffffffu, c, 0);
+            } else {
+              volatile unsigned long long* xc = reinterpret_cast<unsigned long long*>(Xok + 2 * NS);
+              if (threadIdx.x == 0) *xc = c;
+              __syncthreads();
+              c = *xc;
+              __syncthreads();
+            }
+            c0 = (long long)c;
+            if (c0 >= L.q_count) return false;
+            c1 = min(c0 + L.chunk, L.q_count);
+          }
+          if constexpr (KIND == MD_BATCH) {  // the chunk's part in the next system's list
+            int lo = 0, hi = L.n_sys - 1;    // last s with seg[s] <= c0
+            while (lo < hi) {
+              const int mid = (lo + hi + 1) >> 1;
+              if (__ldg(L.seg + mid) <= c0) lo = mid; else hi = mid - 1;
+            }
+            const long long e = min(c1, __ldg(L.seg + lo + 1)), s0 = __ldg(L.seg + lo);
+            sys = lo;
+            q0 = L.batch[lo].q_begin + (c0 - s0);
+            q1 = L.batch[lo].q_begin + (e - s0);
+            c0 = e;
+          } else {
+            q0 = L.q_begin + c0;
+            q1 = L.q_begin + c1;
+            c0 = c1;
+          }
+        }
+        if (q0 < q1) {
+          const EriLaunch& Ls = rec(sys);
+          r = find_row(Ls.qoff, Ls.row_begin, Ls.row_end, q0);
+          return true;
+        }
+      }
+    }
   };
 
-  if constexpr (KIND == MD_DIAG) {
-    for (int t = blockIdx.x * kTeams + team; t < L.diag_n; t += gridDim.x * kTeams) {
-      const int p = __ldg(L.diag_list + t), np = __ldg(L.pa.prim_n + p);
-      if (np == 0 && lane == 0 && wt == 0) L.diag_Q[p] = 0.0;
-      push(lane == 0, 0, p, p, np, np);
-    }
-  } else {
-    auto claim = [&]() -> long long {
-      unsigned long long c = 0;
-      if (lane == 0 && wt == 0) c = atomicAdd(L.work, (unsigned long long)L.chunk);
-      if constexpr (NW == 1) return (long long)__shfl_sync(0xffffffffu, c, 0);
-      volatile unsigned long long* xc = reinterpret_cast<unsigned long long*>(X + NW * (LT + 4) * 32 + 2);
-      if (threadIdx.x == 0) *xc = c;
-      __syncthreads();
-      c = *xc;
-      __syncthreads();
-      return (long long)c;
-    };
-    for_each_range<KIND == MD_BATCH>(
-        L, blockIdx.x * kTeams + team, (long long)gridDim.x * kTeams, claim,
-        [&](const EriLaunch& Ls, int sys, long long q0, long long q1) {
-          if (q0 >= q1) return;
-          int r = find_row(Ls.qoff, Ls.row_begin, Ls.row_end, q0);
-          for (long long base = q0; base < q1; base += 32) {
-            const long long q = base + lane;
-            bool keep = false;
-            int bra_s = 0, ket_s = 0, nb = 0, nk = 0;
-            if (q < q1) {
-              while (__ldg(Ls.qoff + r + 1) <= q) ++r;
-              bra_s = Ls.bra_bin_start + (r - Ls.row_begin);
-              ket_s = Ls.ket_bin_start + (int)(q - __ldg(Ls.qoff + r));
-              const int bra = __ldg(Ls.sorted + bra_s), ket = __ldg(Ls.sorted + ket_s);
-              if constexpr (KIND == MD_PER) {
-                PerQuartet pq;
-                keep = per_quartet(Ls, bra, ket, pq);  // a density block exists for its cell offset
-              } else {
-                const double pm = pmax4(Ls, __ldg(Ls.pa.sa + bra), __ldg(Ls.pa.sb + bra), __ldg(Ls.pa.sa + ket),
-                                        __ldg(Ls.pa.sb + ket));
-                keep = !(Ls.skip_zero && pm == 0.0) &&
-                       !(Ls.dens_tau > 0.0 && __ldg(Ls.Qs + bra_s) * __ldg(Ls.Qs + ket_s) * pm < Ls.dens_tau) &&
-                       dist_keeps(Ls, bra_s, ket_s) && !(L.prec == PREC_MIXED64 && fp32_eligible(Ls, bra_s, ket_s, pm));
-              }
-              if (keep) {
-                nb = __ldg(Ls.pa.prim_n + bra);
-                nk = __ldg(Ls.pa.prim_n + ket);
-              }
-            }
-            push(keep, sys, bra_s, ket_s, nb, nk);
+  // one loop and one place for the batches: the kernel's code is large, and a second copy of it
+  // cost more in instruction fetches than anything else in the FP32 pass
+  for (bool more = true; more;) {
+    if (q0 >= q1) more = next_range();
+    bool keep = false;
+    int bra_s = 0, ket_s = 0, nb = 0, nk = 0;
+    if (more) {
+      const long long q = q0 + lane;
+      q0 += 32;
+      if (q < q1) {
+        if constexpr (KIND == MD_DIAG) {
+          const int p = __ldg(L.diag_list + q);
+          bra_s = ket_s = p;
+          nb = nk = __ldg(L.pa.prim_n + p);
+          keep = nb > 0;
+          if (!keep && wt == 0) L.diag_Q[p] = 0.0;
+        } else {
+          const EriLaunch& Ls = rec(sys);
+          while (__ldg(Ls.qoff + r + 1) <= q) ++r;
+          bra_s = Ls.bra_bin_start + (r - Ls.row_begin);
+          ket_s = Ls.ket_bin_start + (int)(q - __ldg(Ls.qoff + r));
+          const int bra = __ldg(Ls.sorted + bra_s), ket = __ldg(Ls.sorted + ket_s);
+          if constexpr (KIND == MD_PER) {
+            PerQuartet pq;
+            keep = per_quartet(Ls, bra, ket, pq);  // a density block exists for its cell offset
+          } else {
+            const double pm = pmax4(Ls, __ldg(Ls.pa.sa + bra), __ldg(Ls.pa.sb + bra), __ldg(Ls.pa.sa + ket),
+                                    __ldg(Ls.pa.sb + ket));
+            keep = !(Ls.skip_zero && pm == 0.0) &&
+                   !(Ls.dens_tau > 0.0 && __ldg(Ls.Qs + bra_s) * __ldg(Ls.Qs + ket_s) * pm < Ls.dens_tau) &&
+                   dist_keeps(Ls, bra_s, ket_s) &&
+                   (L.prec == PREC_FP64 || fp32_eligible(Ls, bra_s, ket_s, pm) == F32);
           }
-        });
+          if (keep) {
+            nb = __ldg(Ls.pa.prim_n + bra);
+            nk = __ldg(Ls.pa.prim_n + ket);
+            keep = nb > 0 && nk > 0;
+          }
+        }
+      }
+      const unsigned m = __ballot_sync(0xffffffffu, keep);
+      if (keep && wt == 0) Q[(tail + __popc(m & lt_mask)) & (kQ - 1)] = make_int4(sys, bra_s, ket_s, nb | (nk << 16));
+      tail += __popc(m);
+      waiting += __reduce_add_sync(0xffffffffu, keep ? nb * nk : 0);
+      sync();
+    }
+    // full batches; short of full where the queue could not take the next 32 quartets, and at the end
+    while (waiting >= 32 * NS || tail - head >= 32 || (!more && waiting > 0)) batch(min(waiting, 32 * NS));
   }
-  if (waiting > 0) batch(waiting);
   if (KIND != MD_DIAG && lane == 0 && wt == 0) flush_tally(L, tally);
   record_busy(L, t0);
 }

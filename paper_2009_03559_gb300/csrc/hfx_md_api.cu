@@ -8,34 +8,35 @@ namespace hfx {
 const MdClassInfo* md_class_host() { return kMdClass; }
 const MdPairInfo* md_pair_host() { return kMdPair; }
 
-const void* md_kernel_l0(int kind);
-const void* md_kernel_l1(int kind);
-const void* md_kernel_l2(int kind);
-const void* md_kernel_l3(int kind);
-const void* md_kernel_l4(int kind);
-const void* md_kernel_l5(int kind);
-const void* md_kernel_l6(int kind);
-const void* md_kernel_l7(int kind);
-const void* md_kernel_l8(int kind);
+const void* md_kernel_l0(int kind, bool f32);
+const void* md_kernel_l1(int kind, bool f32);
+const void* md_kernel_l2(int kind, bool f32);
+const void* md_kernel_l3(int kind, bool f32);
+const void* md_kernel_l4(int kind, bool f32);
+const void* md_kernel_l5(int kind, bool f32);
+const void* md_kernel_l6(int kind, bool f32);
+const void* md_kernel_l7(int kind, bool f32);
+const void* md_kernel_l8(int kind, bool f32);
 
-static const void* md_kernel(int Lt, int kind) {
+static const void* md_kernel(int Lt, int kind, bool f32) {
   switch (Lt) {
-    case 0: return md_kernel_l0(kind);
-    case 1: return md_kernel_l1(kind);
-    case 2: return md_kernel_l2(kind);
-    case 3: return md_kernel_l3(kind);
-    case 4: return md_kernel_l4(kind);
-    case 5: return md_kernel_l5(kind);
-    case 6: return md_kernel_l6(kind);
-    case 7: return md_kernel_l7(kind);
-    default: return md_kernel_l8(kind);
+    case 0: return md_kernel_l0(kind, f32);
+    case 1: return md_kernel_l1(kind, f32);
+    case 2: return md_kernel_l2(kind, f32);
+    case 3: return md_kernel_l3(kind, f32);
+    case 4: return md_kernel_l4(kind, f32);
+    case 5: return md_kernel_l5(kind, f32);
+    case 6: return md_kernel_l6(kind, f32);
+    case 7: return md_kernel_l7(kind, f32);
+    default: return md_kernel_l8(kind, f32);
   }
 }
 
-static MdLayout layout_of(int cls) {
+static MdLayout layout_of(int cls, bool f32) {
   int hi = 0;
   while ((hi + 1) * (hi + 2) / 2 <= cls) ++hi;
-  return md_layout(kMdClass[cls], kMdPair[hi], kMdPair[cls - hi * (hi + 1) / 2]);
+  const MdPairInfo &b = kMdPair[hi], &k = kMdPair[cls - hi * (hi + 1) / 2];
+  return f32 ? md_layout<float>(kMdClass[cls], b, k) : md_layout<double>(kMdClass[cls], b, k);
 }
 
 int md_teams_per_block(int cls) {
@@ -43,36 +44,42 @@ int md_teams_per_block(int cls) {
   return md_block(l) / (32 * md_team(l));
 }
 
-size_t md_smem_bytes(int cls) { return sizeof(double) * (size_t)layout_of(cls).size * md_teams_per_block(cls); }
+size_t md_smem_bytes(int cls, bool f32) {
+  return sizeof(double) * (size_t)layout_of(cls, f32).size * md_teams_per_block(cls);
+}
 
 cudaError_t md_prepare() {
-  int mx[kMaxLt + 1] = {};
-  for (int c = 0; c < HFX_N_CLASSES; ++c) mx[kMdClass[c].Lt] = std::max(mx[kMdClass[c].Lt], (int)md_smem_bytes(c));
-  for (int l = 0; l <= kMaxLt; ++l)
-    for (int kind : {MD_PLAIN, MD_BATCH, MD_PER, MD_DIAG}) {
-      const void* k = md_kernel(l, kind);
-      if (!k) continue;
-      const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, mx[l]);
-      if (e != cudaSuccess) return e;
-    }
+  for (bool f32 : {false, true}) {
+    int mx[kMaxLt + 1] = {};
+    for (int c = 0; c < HFX_N_CLASSES; ++c)
+      mx[kMdClass[c].Lt] = std::max(mx[kMdClass[c].Lt], (int)md_smem_bytes(c, f32));
+    for (int l = 0; l <= kMaxLt; ++l)
+      for (int kind : {MD_PLAIN, MD_BATCH, MD_PER, MD_DIAG}) {
+        const void* k = md_kernel(l, kind, f32);
+        if (!k) continue;
+        const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, mx[l]);
+        if (e != cudaSuccess) return e;
+      }
+  }
   return cudaSuccess;
 }
 
-int md_blocks_per_sm(int cls, int kind) {
+int md_blocks_per_sm(int cls, int kind, bool f32) {
   int n = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, md_kernel(kMdClass[cls].Lt, kind),
-                                                    md_block(kMdClass[cls].Lt), md_smem_bytes(cls)) != cudaSuccess)
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, md_kernel(kMdClass[cls].Lt, kind, f32), md_block(kMdClass[cls].Lt),
+                                                    md_smem_bytes(cls, f32)) != cudaSuccess)
     return 1;
   return n > 0 ? n : 1;
 }
 
-cudaError_t md_launch(const EriLaunch& L0, int cls, int kind, int prec, int grid, cudaStream_t stream) {
+cudaError_t md_launch(const EriLaunch& L0, int cls, int kind, int prec, bool f32, int grid, cudaStream_t stream) {
   EriLaunch L = L0;
   L.mc = kMdClass[cls];
-  L.prec = prec;
-  MdLayout ly = layout_of(cls);
+  L.prec = prec == PREC_PERIODIC ? PREC_FP64 : prec;
+  MdLayout ly = layout_of(cls, f32);
   void* args[] = {(void*)&L, (void*)&ly};
-  return cudaLaunchKernel(md_kernel(L.mc.Lt, kind), dim3(grid), dim3(md_block(L.mc.Lt)), args, md_smem_bytes(cls), stream);
+  return cudaLaunchKernel(md_kernel(L.mc.Lt, kind, f32), dim3(grid), dim3(md_block(kMdClass[cls].Lt)), args,
+                          md_smem_bytes(cls, f32), stream);
 }
 
 // ---------------------------------------------------------------------------
