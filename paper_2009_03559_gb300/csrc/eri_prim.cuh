@@ -33,11 +33,8 @@ __device__ __forceinline__ bool prim_core(const PrimPair& b, const PrimPair& k, 
   const double T = rho * fma(ps.PQ[0], ps.PQ[0], fma(ps.PQ[1], ps.PQ[1], ps.PQ[2] * ps.PQ[2]));
   const double pref = (b.C * k.C) * y;
   const double* tabL = tabs + Lt * kBoysTableLen;
-  double F1, e1 = 0.0;
-  if (!ge_hi(T, kBoysXmaxHi))
-    boys_top(T, tabL, F1, e1);
-  else
-    F1 = boys_asym(Lt, T);
+  double F1, e1;
+  boys_any(Lt, T, tabL, F1, e1);
   const double T2 = T + T;
   if (omega2 > 0.0) {
     const double sk = omega * rsqrt_nr(omega2 + rho);   // sqrt(kappa)

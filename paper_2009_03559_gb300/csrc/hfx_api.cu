@@ -186,14 +186,13 @@ static int init_basis_impl(hfx_ctx** out, int n_atoms, const double* xyz, int n_
 }
 
 // Flops (add/mul 1, fma 2) of one primitive-quartet set-up as written in prim_core and
-// write_set, with the table branch of both Boys evaluations (each: the offset from the
-// grid point and two seven-term Horner chains, 25 flops; the asymptotic branch taken for
-// T >= 60 costs 7 + 2 Lt and is not counted separately).
+// prim_setup, with both Boys evaluations (each: the offset from the grid point and two
+// Horner chains of three FP64 steps, 13 flops; their FP32 steps are not counted).
 static double setup_flops(int E, int F, int Lt, bool erfc) {
   // s, rsqrt(s), 1/s, rho/p, rho/q, rho, PQ, r2, T, pref, Boys(T), 2T
-  double f = 1 + 5 + 1 + 2 + 1 + 3 + 5 + 1 + 2 + 25 + 1;
+  double f = 1 + 5 + 1 + 2 + 1 + 3 + 5 + 1 + 2 + 13 + 1;
   if (erfc)
-    f += 7 + 1 + 1 + 25 + 1 + Lt + 1 + 3 + 5.0 * Lt;  // sqrt(kappa), kappa, kT, Boys(kT), c_m, G recursion
+    f += 7 + 1 + 1 + 13 + 1 + Lt + 1 + 3 + 5.0 * Lt;  // sqrt(kappa), kappa, kT, Boys(kT), c_m, G recursion
   else
     f += 1 + 1 + 3.0 * Lt;
   if (E > 0) f += 3;   // W - P
@@ -201,7 +200,7 @@ static double setup_flops(int E, int F, int Lt, bool erfc) {
   return f;
 }
 // a primitive quartet dropped at kappa T >= table end costs the set-up up to that test
-static double skip_flops() { return 47 + 7 + 1 + 1; }
+static double skip_flops() { return 35 + 7 + 1 + 1; }
 
 EriLaunch hfx::base_launch(hfx_ctx* ctx) {
   EriLaunch L;

@@ -45,22 +45,26 @@ extern const MdClassInfo* md_class_host();
 extern const MdPairInfo* md_pair_host();
 
 // ---------------------------------------------------------------------------
-// Boys function tables, one per order L = 0..kMaxLt, rows at x_g = g h (h = 1/32,
-// g = 0..kBoysRows-1).  Row g of table L holds the coefficients of the Taylor expansions
-// about x_g in powers of d = x - x_g:
-//   [0] x_g,  [1 + k] (-1)^k F_{L+k}(x_g) / k!,  [8 + k] (-1)^k exp(-x_g) / k!  (k = 0..6),
-//   [15] 0,
-// with F_m(x) = int_0^1 u^{2m} exp(-x u^2) du.  Seven terms with |d| <= h/2 leave a
-// relative error below 5e-17.
+// Boys function tables, one per order L = 0..kMaxLt, with F_m(x) = int_0^1 u^{2m} exp(-x u^2) du.
+// A row holds the Taylor coefficients about its grid point x_g in powers of d = x - x_g:
+//   doubles [0] x_g, [1..3] f_0, f_1, f_2, [4] e_0 = exp(-x_g), [5] e_0 / 2, then floats
+//   [12..14] f_3, f_4, f_5;  f_k = (-1)^k F_{L+k}(x_g) / k!,  exp(-x) = e_0 - e_0 d + e_0/2 d^2 - ...
+// Rows 0..kBoysRows-1: x_g = g / 256 up to 60.  |d| <= 1/512, so the terms from the third on are
+// below 1.3e-9 of the value and their FP32 rounding below 8e-17: they cost no FP64 instruction
+// (with the former spacing of 1/32 both chains had six).  The rows after them hold the asymptote
+// (2L-1)!!/2^{L+1} sqrt(pi) t^{-L-1/2} for t = 1 + g / 1024 in [1, 4], e_0 = 0: T >= 60 is looked
+// up as t = T / 4^k and the value scaled by 2^{-k(2L+1)}, exponent arithmetic on the integer pipe
+// (the neglected part of F_L is below exp(-60) relative).
 // ---------------------------------------------------------------------------
-constexpr int kBoysRowLen = 16;
-constexpr float kBoysInvStepF = 32.0f;
-constexpr double kBoysStep = 1.0 / 32.0;
+constexpr int kBoysRowLen = 8;
+constexpr int kBoysPerUnit = 256;
 constexpr double kBoysXmax = 60.0;
 constexpr int kBoysXmaxHi = 0x404E0000;   // high word of 60.0 (low word 0)
-constexpr int kBoysRows = 60 * 32 + 2;
+constexpr int kBoysRows = 60 * kBoysPerUnit + 2;
+constexpr int kBoysTailPerUnit = 1024;
+constexpr int kBoysTailRows = 3 * kBoysTailPerUnit + 1;
 constexpr int kMaxLt = 8;
-constexpr int kBoysTableLen = kBoysRows * kBoysRowLen;   // doubles per order
+constexpr int kBoysTableLen = (kBoysRows + kBoysTailRows) * kBoysRowLen;   // doubles per order
 
 // ---------------------------------------------------------------------------
 // Primitive-pair record (one per surviving primitive pair of a shell pair).
@@ -152,33 +156,37 @@ __device__ __forceinline__ double rsqrt_nr(double x) {
   return fma(hy, r, y);
 }
 
-// F_L(x) and exp(-x) for 0 <= x < kBoysXmax from the table of order L (13 FP64
-// instructions: the offset from the grid point and two Horner chains).
-__device__ __forceinline__ void boys_top(double x, const double* __restrict__ tabL, double& F, double& e) {
-  const int g = __float2int_rn(approx_f32(x) * kBoysInvStepF);
+// F_L(x) and exp(-x) from row g of the table of order L: 7 FP64 instructions.
+__device__ __forceinline__ void boys_row(double x, const double* __restrict__ tabL, int g, double& F, double& e) {
   const double2* row = reinterpret_cast<const double2*>(tabL + g * kBoysRowLen);
-  const double2 r0 = __ldg(row), r1 = __ldg(row + 1), r2 = __ldg(row + 2), r3 = __ldg(row + 3);
-  const double2 r4 = __ldg(row + 4), r5 = __ldg(row + 5), r6 = __ldg(row + 6), r7 = __ldg(row + 7);
+  const double2 r0 = __ldg(row), r1 = __ldg(row + 1), r2 = __ldg(row + 2);
+  const float4 r3 = __ldg(reinterpret_cast<const float4*>(row + 3));
   const double d = x - r0.x;
-  F = fma(fma(fma(fma(fma(fma(r3.y, d, r3.x), d, r2.y), d, r2.x), d, r1.y), d, r1.x), d, r0.y);
-  e = fma(fma(fma(fma(fma(fma(r7.x, d, r6.y), d, r6.x), d, r5.y), d, r5.x), d, r4.y), d, r4.x);
+  const float df = to_f32(d), ef = to_f32(r2.x);
+  const double f3 = to_f64(fmaf(df, fmaf(df, r3.z, r3.y), r3.x));
+  const double e3 = to_f64(ef * fmaf(df, fmaf(df, -1.0f / 120, 1.0f / 24), -1.0f / 6));
+  F = fma(fma(fma(f3, d, r1.y), d, r1.x), d, r0.y);
+  e = fma(fma(fma(e3, d, r2.y), d, -r2.x), d, r2.x);
 }
 
-// F_L(x) for x >= kBoysXmax: (2L-1)!!/2^{L+1} sqrt(pi) x^{-L-1/2} (the neglected terms are
-// below exp(-60) relative); exp(-x) is taken as 0.
-__device__ __forceinline__ double boys_asym(int L, double x) {
-  const double y = rsqrt_nr(x);
-  const double y2 = y * y;
-  double v = y;
-  double c = 0.886226925452758014;  // sqrt(pi)/2
-#pragma unroll
-  for (int m = 0; m < kMaxLt; ++m) {
-    if (m < L) {
-      v *= y2;
-      c *= (m + 0.5);
-    }
+// the same for 0 <= x < kBoysXmax
+__device__ __forceinline__ void boys_top(double x, const double* __restrict__ tabL, double& F, double& e) {
+  boys_row(x, tabL, __float2int_rn(approx_f32(x) * (float)kBoysPerUnit), F, e);
+}
+
+// F_L(x) and exp(-x) (0 from kBoysXmax on) for any x >= 0, by one sequence of instructions
+__device__ __forceinline__ void boys_any(int L, double x, const double* __restrict__ tabL, double& F, double& e) {
+  const bool tail = ge_hi(x, kBoysXmaxHi);
+  const int k = tail ? ((__double2hiint(x) >> 20) - 1023) >> 1 : 0;
+  const double t = scale2(x, -2 * k);
+  const float f = approx_f32(t);
+  const int g = tail ? kBoysRows + __float2int_rn((f - 1.0f) * (float)kBoysTailPerUnit)
+                     : __float2int_rn(f * (float)kBoysPerUnit);
+  boys_row(t, tabL, g, F, e);
+  if (tail) {
+    const int hi = __double2hiint(F), up = k * (2 * L + 1);
+    F = (hi >> 20) > up ? scale2(F, -up) : 0.0;
   }
-  return c * v;
 }
 
 // Lattice images (periodic builds): the library holds the home cell's shells repeated in a

@@ -206,11 +206,8 @@ __device__ __forceinline__ bool md_setup(const PrimPair& b, const PrimPair& k, c
     kT = kap * T;
     if (ge_hi(kT, kBoysXmaxHi)) return false;
   }
-  double F1, e1 = 0.0;
-  if (!ge_hi(T, kBoysXmaxHi))
-    boys_top(T, tabL, F1, e1);
-  else
-    F1 = boys_asym(L, T);
+  double F1, e1;
+  boys_any(L, T, tabL, F1, e1);
   const double r2 = scale2(rho, 1);
   double pL = pref;  // pref (2 rho)^L
   if constexpr (L > 0) {

@@ -34,14 +34,38 @@ __global__ void k_normalize(int n_shells, const int* __restrict__ l, const int* 
 }
 
 // ---------------------------------------------------------------------------
-// Boys tables: at x_g = g h, F_15(x_g) from its series exp(-x) sum_k (2x)^k / ((31)(33)...(31+2k)),
+// Boys tables: at x_g, F_15(x_g) from its series exp(-x) sum_k (2x)^k / ((31)(33)...(31+2k)),
 // lower orders by the downward recursion F_{m-1} = (2x F_m + e^{-x}) / (2m-1); then for every
-// order L = 0..kMaxLt the row of Taylor coefficients [x_g, (-1)^k F_{L+k}/k!, (-1)^k e^{-x_g}/k!].
+// order L = 0..kMaxLt its row; the rows of the tail from the asymptote (layout: kBoysRowLen).
 // ---------------------------------------------------------------------------
+__device__ __forceinline__ void put_boys_row(double* row, double x, const double* f, double e) {
+  row[0] = x;
+  for (int k = 0; k < 3; ++k) row[1 + k] = f[k];
+  row[4] = e;
+  row[5] = 0.5 * e;
+  float* r = reinterpret_cast<float*>(row + 6);
+  for (int k = 0; k < 3; ++k) r[k] = (float)f[3 + k];
+  r[3] = 0.f;
+}
+
 __global__ void k_boys_table(double* __restrict__ tab) {
   const int g = blockIdx.x * blockDim.x + threadIdx.x;
-  if (g >= kBoysRows) return;
-  const double x = g * kBoysStep;
+  if (g >= kBoysRows + kBoysTailRows) return;
+  double f[6];
+  if (g >= kBoysRows) {
+    const double t = 1.0 + (double)(g - kBoysRows) / kBoysTailPerUnit;
+    double c = 0.886226925452758014;  // (2L-1)!!/2^{L+1} sqrt(pi)
+    for (int L = 0; L <= kMaxLt; ++L) {
+      const double a = L + 0.5;
+      f[0] = c / sqrt(t);
+      for (int m = 0; m < L; ++m) f[0] /= t;
+      for (int k = 1; k < 6; ++k) f[k] = -f[k - 1] * (a + k - 1) / (k * t);
+      put_boys_row(tab + (size_t)L * kBoysTableLen + (size_t)g * kBoysRowLen, t, f, 0.0);
+      c *= a;
+    }
+    return;
+  }
+  const double x = (double)g / kBoysPerUnit;
   const int M = 15;
   double term = 1.0 / (2 * M + 1), sum = term;
   for (int k = 1; k < 4000; ++k) {
@@ -53,16 +77,10 @@ __global__ void k_boys_table(double* __restrict__ tab) {
   double Fm[M + 1];
   Fm[M] = e * sum;
   for (int m = M; m >= 1; --m) Fm[m - 1] = (2.0 * x * Fm[m] + e) / (2 * m - 1);
-  const double inv_fact[7] = {1.0, 1.0, 1.0 / 2, 1.0 / 6, 1.0 / 24, 1.0 / 120, 1.0 / 720};
+  const double inv_fact[6] = {1.0, -1.0, 1.0 / 2, -1.0 / 6, 1.0 / 24, -1.0 / 120};
   for (int L = 0; L <= kMaxLt; ++L) {
-    double* row = tab + (size_t)L * kBoysTableLen + (size_t)g * kBoysRowLen;
-    row[0] = x;
-    for (int k = 0; k < 7; ++k) {
-      const double sg = (k & 1) ? -inv_fact[k] : inv_fact[k];
-      row[1 + k] = sg * Fm[L + k];
-      row[8 + k] = sg * e;
-    }
-    row[15] = 0.0;
+    for (int k = 0; k < 6; ++k) f[k] = inv_fact[k] * Fm[L + k];
+    put_boys_row(tab + (size_t)L * kBoysTableLen + (size_t)g * kBoysRowLen, x, f, e);
   }
 }
 
@@ -592,7 +610,7 @@ cudaError_t launch_pmax_blocks(int n_R, int ns, int nbf, const int* bf_off, cons
 }
 
 cudaError_t launch_boys_table(double* tab, cudaStream_t s) {
-  k_boys_table<<<nblk(kBoysRows, 128), 128, 0, s>>>(tab);
+  k_boys_table<<<nblk(kBoysRows + kBoysTailRows, 128), 128, 0, s>>>(tab);
   return cudaGetLastError();
 }
 

@@ -1,0 +1,56 @@
+"""The Hermite engine where it can go wrong: arguments of the Boys tables at their seams, and
+streams of quartets with very few and very many primitive quartets (queue, runs cut by batch
+ends, teams of warps), against the oracle."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2009_03559_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def hfx_mod():
+    from paper_2009_03559_gb300 import hfx
+    return hfx
+
+
+def check(hfx_mod, s, P, tol, **kw):
+    Ko, eo = oracle.Screen(oracle.Basis(s)).build_K(P, "sym")
+    h = hfx_mod.HFX(s, **kw).build_pairs()
+    h.set_timing(True)
+    K = h.build_K(torch.from_numpy(P).cuda()).cpu().numpy()
+    assert np.abs(K - Ko).max() <= tol * np.abs(Ko).max(), np.abs(K - Ko).max()
+    assert abs(h.energy() - eo) <= tol * np.abs(Ko).max() * s.n_bf
+    return h
+
+
+# exponents 1 on both atoms: rho = 1 for the quartets of two same-atom pairs, T = R^2.  60 is where
+# the rows of the asymptote begin, powers of 4 where their scaling by 4^k changes, 1/512 off a grid
+# point the largest distance from one.  Tolerance: 16 doubles' rounding in each of some 30 steps.
+@pytest.mark.parametrize("T", [1e-6, 1.0 / 512, 17.0 + 1.0 / 512, 59.998, 60.0, 60.002, 63.999, 64.001, 255.99, 256.01,
+                               4095.9, 4096.1, 1e6])
+@pytest.mark.parametrize("omega", [0.0, 0.11])
+def test_boys_seams(hfx_mod, T, omega):
+    ls = [0, 1, 2]
+    xyz = np.array([[0.0, 0.0, 0.0], [0.6, 0.48, 0.64]]) * np.sqrt(T)
+    s = inputs.System("pair", xyz, np.repeat([0, 1], 3).astype(np.int32), np.array(ls * 2, np.int32),
+                      np.ones(6, np.int32), np.ones(6), np.ones(6), omega=omega, tau=0.0)
+    rng = np.random.default_rng(11)
+    P = rng.standard_normal((s.n_bf, s.n_bf))
+    check(hfx_mod, s, P + P.T, 16 * 30 * 1.2e-16)
+
+
+@pytest.mark.parametrize("nprim,atoms", [(1, 5), (2, 3), (8, 1), (8, 2)])
+@pytest.mark.parametrize("mixed", [False, True])
+def test_streams_of_few_and_many_primitives(hfx_mod, nprim, atoms, mixed):
+    s = inputs.diamond_system(atoms, seed=40 + nprim, nprim=nprim, tau=1e-12, alpha_range=(0.2, 4.0))
+    P = inputs.density_matrix(s)
+    kw = dict(precision=hfx_mod.HFX_MIXED, fp32_class_mask=hfx_mod.ALL_CLASS_MASK, fp32_tau=1e-3) if mixed else {}
+    h = check(hfx_mod, s, P, 1e-6 if mixed else 1e-12, **kw)
+    st = h.stats()
+    assert sum(st["quartets_evaluated_class"]) > 0
+    if mixed and atoms > 1:  # (the quartets of one atom are all large: its mixed build is the FP64 pass)
+        assert sum(st["quartets_fp32_class"]) > 0
