@@ -82,9 +82,10 @@ __device__ __forceinline__ CoefRgT<float> coef_f32(const CoefRg& c, int E, int F
 
 // Set-up into registers (one quartet per thread).
 __device__ __forceinline__ bool prim_setup(const PrimPair& b, const PrimPair& k, int E, int F, int Lt, double omega,
-                                           double omega2, const double* __restrict__ tabs, CoefRg& c, double* Gm) {
+                                           double omega2, const double* __restrict__ tabs, CoefRg& c, double* Gm,
+                                           const Fp64& op) {
   PrimScalars ps;
-  if (!prim_core(b, k, Lt, omega, omega2, tabs, Gm, ps)) return false;
+  if (!prim_core(b, k, Lt, omega, omega2, tabs, Gm, ps, op)) return false;
   if (E > 0) {
     c.PA[0] = b.PA[0]; c.PA[1] = b.PA[1]; c.PA[2] = b.PA[2];
     c.WP[0] = -ps.RP * ps.PQ[0]; c.WP[1] = -ps.RP * ps.PQ[1]; c.WP[2] = -ps.RP * ps.PQ[2];   // W - P
@@ -103,9 +104,9 @@ __device__ __forceinline__ bool prim_setup(const PrimPair& b, const PrimPair& k,
 
 // Register coefficients from the FP32 set-up (one quartet per thread).
 __device__ __forceinline__ int prim_setup_f32(const PrimPair& b, const PrimPair& k, int E, int F, int Lt,
-                                              float omega_f, CoefRgT<float>& c, float* G) {
+                                              float omega_f, CoefRgT<float>& c, float* G, const Fp64& op) {
   PrimScalarsF ps;
-  const int st = prim_core_f32(b, k, Lt, omega_f, G, ps);
+  const int st = prim_core_f32(b, k, Lt, omega_f, G, ps, op);
   if (st != F32_OK) return st;
   if (E > 0) {
     c.PA[0] = b.PAf[0]; c.PA[1] = b.PAf[1]; c.PA[2] = b.PAf[2];

@@ -18,42 +18,43 @@ struct PrimScalars {
 //   G_{m-1} = (2T G_m + pref e^{-T} - pref kappa^{m-1/2} e^{-kappa T}) / (2m-1).
 // Returns false if the quartet is negligible (kappa T beyond the tables: G_m < e^{-60}).
 __device__ __forceinline__ bool prim_core(const PrimPair& b, const PrimPair& k, int Lt, double omega, double omega2,
-                                          const double* __restrict__ tabs, double* G, PrimScalars& ps) {
+                                          const double* __restrict__ tabs, double* G, PrimScalars& ps,
+                                          const Fp64& op) {
   const double p = b.p, q = k.p;
-  const double s = p + q;
-  const double y = rsqrt_nr(s);   // 1/sqrt(p+q)
-  const double inv_s = y * y;
+  const double s = op.add(p, q);
+  const double y = rsqrt_nr(s, op);   // 1/sqrt(p+q)
+  const double inv_s = op.mul(y, y);
   ps.inv_s = inv_s;
-  ps.RP = q * inv_s;              // rho / p
-  ps.RQ = p * inv_s;              // rho / q
-  const double rho = p * ps.RP;
-  ps.PQ[0] = b.P[0] - k.P[0];
-  ps.PQ[1] = b.P[1] - k.P[1];
-  ps.PQ[2] = b.P[2] - k.P[2];
-  const double T = rho * fma(ps.PQ[0], ps.PQ[0], fma(ps.PQ[1], ps.PQ[1], ps.PQ[2] * ps.PQ[2]));
-  const double pref = (b.C * k.C) * y;
+  ps.RP = op.mul(q, inv_s);       // rho / p
+  ps.RQ = op.mul(p, inv_s);       // rho / q
+  const double rho = op.mul(p, ps.RP);
+  ps.PQ[0] = op.sub(b.P[0], k.P[0]);
+  ps.PQ[1] = op.sub(b.P[1], k.P[1]);
+  ps.PQ[2] = op.sub(b.P[2], k.P[2]);
+  const double T = op.mul(rho, fma(ps.PQ[0], ps.PQ[0], fma(ps.PQ[1], ps.PQ[1], op.mul(ps.PQ[2], ps.PQ[2]))));
+  const double pref = op.mul(op.mul(b.C, k.C), y);
   const double* tabL = tabs + Lt * kBoysTableLen;
   double F1, e1;
-  boys_any(Lt, T, tabL, F1, e1);
-  const double T2 = T + T;
+  boys_any(Lt, T, tabL, F1, e1, op);
+  const double T2 = op.add(T, T);
   if (omega2 > 0.0) {
-    const double sk = omega * rsqrt_nr(omega2 + rho);   // sqrt(kappa)
-    const double kap = sk * sk;
-    const double kT = kap * T;
+    const double sk = op.mul(omega, rsqrt_nr(op.add(rho, omega2), op));   // sqrt(kappa)
+    const double kap = op.mul(sk, sk);
+    const double kT = op.mul(kap, T);
     if (ge_hi(kT, kBoysXmaxHi)) return false;
     double F2, e2;
-    boys_top(kT, tabL, F2, e2);
+    boys_top(kT, tabL, F2, e2, op);
     // c[m] = pref kappa^{m-1/2}, m = 1..Lt+1
     double c[kMaxLt + 2];
-    c[1] = pref * sk;
+    c[1] = op.mul(pref, sk);
 #pragma unroll
     for (int m = 1; m <= kMaxLt; ++m)
-      if (m <= Lt) c[m + 1] = c[m] * kap;
-    const double pe1 = pref * e1;
+      if (m <= Lt) c[m + 1] = op.mul(c[m], kap);
+    const double pe1 = op.mul(pref, e1);
     double g = 0.0;
 #pragma unroll
     for (int m = 0; m <= kMaxLt; ++m)
-      if (m == Lt) g = fma(-c[m + 1], F2, pref * F1);
+      if (m == Lt) g = fma(-c[m + 1], F2, op.mul(pref, F1));
     G[Lt] = g;
 #pragma unroll
     for (int m = kMaxLt; m >= 1; --m) {
@@ -63,8 +64,8 @@ __device__ __forceinline__ bool prim_core(const PrimPair& b, const PrimPair& k, 
       }
     }
   } else {
-    const double pe1 = pref * e1;
-    double g = pref * F1;
+    const double pe1 = op.mul(pref, e1);
+    double g = op.mul(pref, F1);
     G[Lt] = g;
 #pragma unroll
     for (int m = kMaxLt; m >= 1; --m) {
@@ -98,7 +99,7 @@ struct PrimScalarsF {
 enum { F32_SKIP = 0, F32_OK = 1, F32_FP64 = 2 };
 
 __device__ __forceinline__ int prim_core_f32(const PrimPair& b, const PrimPair& k, int Lt, float omega_f, float* G,
-                                             PrimScalarsF& ps) {
+                                             PrimScalarsF& ps, const Fp64& op) {
   const float p = b.pf, q = k.pf;
   const float y = rsqrtf(p + q);  // 1/sqrt(p+q)
   const float inv_s = y * y;
@@ -106,9 +107,9 @@ __device__ __forceinline__ int prim_core_f32(const PrimPair& b, const PrimPair& 
   ps.RP = q * inv_s;
   ps.RQ = p * inv_s;
   const float rho = p * ps.RP;
-  ps.PQ[0] = to_f32(b.P[0] - k.P[0]);
-  ps.PQ[1] = to_f32(b.P[1] - k.P[1]);
-  ps.PQ[2] = to_f32(b.P[2] - k.P[2]);
+  ps.PQ[0] = to_f32(op.sub(b.P[0], k.P[0]));
+  ps.PQ[1] = to_f32(op.sub(b.P[1], k.P[1]));
+  ps.PQ[2] = to_f32(op.sub(b.P[2], k.P[2]));
   const float T = rho * fmaf(ps.PQ[0], ps.PQ[0], fmaf(ps.PQ[1], ps.PQ[1], ps.PQ[2] * ps.PQ[2]));
   const float sk = omega_f * rsqrtf(fmaf(omega_f, omega_f, rho));  // sqrt(kappa)
   const float kap = sk * sk;

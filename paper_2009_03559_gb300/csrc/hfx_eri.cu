@@ -30,6 +30,8 @@ __device__ __forceinline__ int contract_g1(const EriClassInfo& ci, const EriLaun
   const PairArrays pa = L.pa;
   const double omega = L.omega, omega2 = L.omega2;
   const double* boys = L.boys;
+  Fp64 op;
+  op.init();
   R* V = S + ci.work_base * sts;
   const int nb = __ldg(pa.prim_n + bra), nk = __ldg(pa.prim_n + ket);
   const PrimPair* pb = pa.prim + __ldg(pa.prim_off + bra);
@@ -61,7 +63,7 @@ __device__ __forceinline__ int contract_g1(const EriClassInfo& ci, const EriLaun
       const int ib = t / nk, ik = t - ib * nk;
       CoefRg c;
       double Gm[kMaxLt + 1];
-      if (!prim_setup(pb[ib], pk[ik], ci.E, ci.F, ci.Lt, omega, omega2, boys, c, Gm)) return false;
+      if (!prim_setup(pb[ib], pk[ik], ci.E, ci.F, ci.Lt, omega, omega2, boys, c, Gm, op)) return false;
       cf = coef_f32(c, ci.E, ci.F);
       for (int m = 0; m <= ci.Lt; ++m) Gf[m] = to_f32(Gm[m]);
       return true;
@@ -77,7 +79,7 @@ __device__ __forceinline__ int contract_g1(const EriClassInfo& ci, const EriLaun
         const int ib = t / nk, ik = t - ib * nk;
         CoefRgT<float> cf;
         float Gf[kMaxLt + 1];
-        const int stt = prim_setup_f32(pb[ib], pk[ik], ci.E, ci.F, ci.Lt, omega_f, cf, Gf);
+        const int stt = prim_setup_f32(pb[ib], pk[ik], ci.E, ci.F, ci.Lt, omega_f, cf, Gf, op);
         if (stt == F32_SKIP) continue;
         if (stt == F32_FP64) {
           const int u = t - c0;
@@ -128,7 +130,7 @@ __device__ __forceinline__ int contract_g1(const EriClassInfo& ci, const EriLaun
       const int ib = t / nk, ik = t - ib * nk;
       CoefRg c;
       double Gm[kMaxLt + 1];
-      if (!prim_setup(pb[ib], pk[ik], ci.E, ci.F, ci.Lt, omega, omega2, boys, c, Gm)) continue;
+      if (!prim_setup(pb[ib], pk[ik], ci.E, ci.F, ci.Lt, omega, omega2, boys, c, Gm, op)) continue;
       ++any;
       vrr(c, Gm);
     }

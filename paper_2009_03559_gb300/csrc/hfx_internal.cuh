@@ -146,22 +146,52 @@ __device__ __forceinline__ double to_f64(float f) {
   return __hiloint2double(((mag >> 3) + (896 << 20)) | (fb & (int)0x80000000), mag << 29);
 }
 
+// ---------------------------------------------------------------------------
+// FP64 instructions with three vector-register operands.  A DFMA of three registers takes 16
+// cycles of an SM; DADD, DMUL and a DFMA with a constant, immediate or zero-register operand take
+// 19 (measured: chains of each form on 8 warps, 16.00 and 19.00 cycles per warp instruction).  So
+// sums and products are written as a DFMA with 1 or -0 from a register that the compiler cannot
+// see through; both are exact, so the results are those of the plain operations.
+// ---------------------------------------------------------------------------
+constexpr int kFp64Recip = 8;
+static __device__ double kFp64Operands[kFp64Recip + kMaxLt + 1] = {
+    1.0, -0.0, 3.0, 5.0, 7.0, 0.0, 0.0, 0.0,              // one, -0, multipliers
+    -1.0, 1.0, 1.0 / 3, 1.0 / 5, 1.0 / 7, 1.0 / 9, 1.0 / 11, 1.0 / 13, 1.0 / 15};  // [kFp64Recip + m] 1 / (2m - 1)
+// operand i, loaded where this stands (not hoisted: registers are scarce) ...
+__device__ __forceinline__ double fp64_operand(int i) {
+  double v;
+  asm volatile("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(kFp64Operands + i));
+  return v;
+}
+// ... and the two of all sums and products, held by a kernel from its start
+struct Fp64 {
+  double one, nzero;
+  __device__ __forceinline__ void init() {
+    one = fp64_operand(0);
+    nzero = fp64_operand(1);
+  }
+  __device__ __forceinline__ double mul(double a, double b) const { return __fma_rn(a, b, nzero); }
+  __device__ __forceinline__ double add(double a, double b) const { return __fma_rn(a, one, b); }
+  __device__ __forceinline__ double sub(double a, double b) const { return __fma_rn(-b, one, a); }
+};
+
 // 1/sqrt(x) for x > 0 in FP32 range: FP32 hardware seed (relative error below 2^-22),
 // one Newton-Raphson step (the error squares: below 1e-13 relative).  3 FP64 instructions.
-__device__ __forceinline__ double rsqrt_nr(double x) {
+__device__ __forceinline__ double rsqrt_nr(double x, const Fp64& op) {
   const float yf = rsqrtf(approx_f32(x));
   const double y = widen_f32(yf);
   const double hy = widen_f32(yf, -1);            // y / 2
-  const double r = fma(-x * y, y, 1.0);           // 1 - x y^2
+  const double r = fma(-op.mul(x, y), y, op.one); // 1 - x y^2
   return fma(hy, r, y);
 }
 
 // F_L(x) and exp(-x) from row g of the table of order L: 7 FP64 instructions.
-__device__ __forceinline__ void boys_row(double x, const double* __restrict__ tabL, int g, double& F, double& e) {
+__device__ __forceinline__ void boys_row(double x, const double* __restrict__ tabL, int g, double& F, double& e,
+                                         const Fp64& op) {
   const double2* row = reinterpret_cast<const double2*>(tabL + g * kBoysRowLen);
   const double2 r0 = __ldg(row), r1 = __ldg(row + 1), r2 = __ldg(row + 2);
   const float4 r3 = __ldg(reinterpret_cast<const float4*>(row + 3));
-  const double d = x - r0.x;
+  const double d = op.sub(x, r0.x);
   const float df = to_f32(d), ef = to_f32(r2.x);
   const double f3 = to_f64(fmaf(df, fmaf(df, r3.z, r3.y), r3.x));
   const double e3 = to_f64(ef * fmaf(df, fmaf(df, -1.0f / 120, 1.0f / 24), -1.0f / 6));
@@ -170,19 +200,21 @@ __device__ __forceinline__ void boys_row(double x, const double* __restrict__ ta
 }
 
 // the same for 0 <= x < kBoysXmax
-__device__ __forceinline__ void boys_top(double x, const double* __restrict__ tabL, double& F, double& e) {
-  boys_row(x, tabL, __float2int_rn(approx_f32(x) * (float)kBoysPerUnit), F, e);
+__device__ __forceinline__ void boys_top(double x, const double* __restrict__ tabL, double& F, double& e,
+                                         const Fp64& op) {
+  boys_row(x, tabL, __float2int_rn(approx_f32(x) * (float)kBoysPerUnit), F, e, op);
 }
 
 // F_L(x) and exp(-x) (0 from kBoysXmax on) for any x >= 0, by one sequence of instructions
-__device__ __forceinline__ void boys_any(int L, double x, const double* __restrict__ tabL, double& F, double& e) {
+__device__ __forceinline__ void boys_any(int L, double x, const double* __restrict__ tabL, double& F, double& e,
+                                         const Fp64& op) {
   const bool tail = ge_hi(x, kBoysXmaxHi);
   const int k = tail ? ((__double2hiint(x) >> 20) - 1023) >> 1 : 0;
   const double t = scale2(x, -2 * k);
   const float f = approx_f32(t);
   const int g = tail ? kBoysRows + __float2int_rn((f - 1.0f) * (float)kBoysTailPerUnit)
                      : __float2int_rn(f * (float)kBoysPerUnit);
-  boys_row(t, tabL, g, F, e);
+  boys_row(t, tabL, g, F, e, op);
   if (tail) {
     const int hi = __double2hiint(F), up = k * (2 * L + 1);
     F = (hi >> 20) > up ? scale2(F, -up) : 0.0;

@@ -28,15 +28,23 @@ namespace hfx {
 
 // n S for a small integer n: doubling and quadrupling are exponent increments (integer pipe).
 // S = 0 or subnormal becomes at most 4 x 2^-1022: nothing next to any integral.
-template <int N, typename R>
-__device__ __forceinline__ R times(R x) {
+template <int N>
+__device__ __forceinline__ double times(double x, const Fp64& op) {
   if constexpr (N == 1) return x;
-  if constexpr (sizeof(R) == 8) {
-    if constexpr (N == 2) return scale2(x, 1);
-    if constexpr (N == 4) return scale2(x, 2);
-  }
-  return x * R(N);
+  if constexpr (N == 2) return scale2(x, 1);
+  if constexpr (N == 3) return op.mul(x, fp64_operand(2));
+  if constexpr (N == 4) return scale2(x, 2);
+  if constexpr (N == 5) return op.mul(x, fp64_operand(3));
+  if constexpr (N == 6) return scale2(op.mul(x, fp64_operand(2)), 1);
+  if constexpr (N == 7) return op.mul(x, fp64_operand(4));
+  return x;  // not reached: a chain of order L <= 8 raises with N <= 7
 }
+template <int N>
+__device__ __forceinline__ float times(float x, const Fp64&) {
+  return x * float(N);
+}
+__device__ __forceinline__ float mulr(float a, float b, const Fp64&) { return a * b; }
+__device__ __forceinline__ double mulr(double a, double b, const Fp64& op) { return op.mul(a, b); }
 __device__ __forceinline__ double fmar(double a, double b, double c) { return __fma_rn(a, b, c); }
 __device__ __forceinline__ float fmar(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 
@@ -112,7 +120,8 @@ __host__ __device__ constexpr int chain_last(int v) {
 // lam = sqrt(2 rho) (base values G_m, coordinates times lam), whose values stay in range for any
 // exponents, and lp[n] = lam^n scales the results.
 template <int L, int NW, int W, typename R>
-__device__ __forceinline__ void hermite(const R (&B)[L + 1], R X, R Y, R Z, const R* lp, R* out) {
+__device__ __forceinline__ void hermite(const R (&B)[L + 1], R X, R Y, R Z, const R* lp, R* out,
+                                        const Fp64& op) {
   constexpr int kLastV = chain_last<L, NW, W>(-1);
   R zr[L + 1], zp[L + 1];
 #pragma unroll
@@ -140,9 +149,9 @@ __device__ __forceinline__ void hermite(const R (&B)[L + 1], R X, R Y, R Z, cons
           for (int m = 0; m < N - T; ++m) {
             R v;
             if constexpr (T == 0)
-              v = X * xr[m + 1];
+              v = mulr(X, xr[m + 1], op);
             else
-              v = fmar(X, xr[m + 1], -times<T>(xp[m + 1]));
+              v = fmar(X, xr[m + 1], -times<T>(xp[m + 1], op));
             xp[m] = xr[m];
             xr[m] = v;
           }
@@ -154,9 +163,9 @@ __device__ __forceinline__ void hermite(const R (&B)[L + 1], R X, R Y, R Z, cons
         for (int m = 0; m < N; ++m) {
           R v;
           if constexpr (U == 0)
-            v = Y * yr[m + 1];
+            v = mulr(Y, yr[m + 1], op);
           else
-            v = fmar(Y, yr[m + 1], -times<U>(yp[m + 1]));
+            v = fmar(Y, yr[m + 1], -times<U>(yp[m + 1], op));
           yp[m] = yr[m];
           yr[m] = v;
         }
@@ -168,9 +177,9 @@ __device__ __forceinline__ void hermite(const R (&B)[L + 1], R X, R Y, R Z, cons
       for (int m = 0; m < L - V; ++m) {
         R v;
         if constexpr (V == 0)
-          v = Z * zr[m + 1];
+          v = mulr(Z, zr[m + 1], op);
         else
-          v = fmar(Z, zr[m + 1], -times<V>(zp[m + 1]));
+          v = fmar(Z, zr[m + 1], -times<V>(zp[m + 1], op));
         zp[m] = zr[m];
         zr[m] = v;
       }
@@ -188,49 +197,49 @@ __device__ __forceinline__ void hermite(const R (&B)[L + 1], R X, R Y, R Z, cons
 template <int L>
 __device__ __forceinline__ bool md_setup(const PrimPair& b, const PrimPair& k, const double* qc, double omega,
                                          double omega2, const double* __restrict__ tabs, double (&B)[L + 1],
-                                         double* PQ) {
+                                         double* PQ, const Fp64& op) {
   const double p = b.p, q = k.p;
-  const double y = rsqrt_nr(p + q);  // 1/sqrt(p+q)
-  const double rho = (p * y) * (q * y);
-  PQ[0] = b.P[0] - qc[0];
-  PQ[1] = b.P[1] - qc[1];
-  PQ[2] = b.P[2] - qc[2];
-  const double R2 = fma(PQ[0], PQ[0], fma(PQ[1], PQ[1], PQ[2] * PQ[2]));
-  const double T = rho * R2;
-  const double pref = (b.C * k.C) * y;
+  const double y = rsqrt_nr(op.add(p, q), op);  // 1/sqrt(p+q)
+  const double rho = op.mul(op.mul(p, y), op.mul(q, y));
+  PQ[0] = op.sub(b.P[0], qc[0]);
+  PQ[1] = op.sub(b.P[1], qc[1]);
+  PQ[2] = op.sub(b.P[2], qc[2]);
+  const double R2 = fma(PQ[0], PQ[0], fma(PQ[1], PQ[1], op.mul(PQ[2], PQ[2])));
+  const double T = op.mul(rho, R2);
+  const double pref = op.mul(op.mul(b.C, k.C), y);
   const double* tabL = tabs + L * kBoysTableLen;
   double kap = 0.0, sk = 0.0, kT = 0.0;
   if (omega2 > 0.0) {
-    sk = omega * rsqrt_nr(omega2 + rho);  // sqrt(kappa)
-    kap = sk * sk;
-    kT = kap * T;
+    sk = op.mul(omega, rsqrt_nr(op.add(rho, omega2), op));  // sqrt(kappa)
+    kap = op.mul(sk, sk);
+    kT = op.mul(kap, T);
     if (ge_hi(kT, kBoysXmaxHi)) return false;
   }
   double F1, e1;
-  boys_any(L, T, tabL, F1, e1);
+  boys_any(L, T, tabL, F1, e1, op);
   const double r2 = scale2(rho, 1);
   double pL = pref;  // pref (2 rho)^L
   if constexpr (L > 0) {
     double w = r2;
-    pL = (L & 1) ? pref * r2 : pref;
+    pL = (L & 1) ? op.mul(pref, r2) : pref;
 #pragma unroll
     for (int i = 1; (L >> i) > 0; ++i) {
-      w = w * w;
-      if ((L >> i) & 1) pL *= w;
+      w = op.mul(w, w);
+      if ((L >> i) & 1) pL = op.mul(pL, w);
     }
   }
-  double a[L + 1], g = pL * F1;
-  a[0] = pref * e1;
+  double a[L + 1], g = op.mul(pL, F1);
+  a[0] = op.mul(pref, e1);
 #pragma unroll
-  for (int m = 1; m < L; ++m) a[m] = a[m - 1] * r2;
+  for (int m = 1; m < L; ++m) a[m] = op.mul(a[m - 1], r2);
   if (omega2 > 0.0) {
     double F2, e2;
-    boys_top(kT, tabL, F2, e2);
-    const double kr = kap * r2;
+    boys_top(kT, tabL, F2, e2, op);
+    const double kr = op.mul(kap, r2);
     double c[L + 1];
-    c[0] = pref * sk;
+    c[0] = op.mul(pref, sk);
 #pragma unroll
-    for (int m = 1; m <= L; ++m) c[m] = c[m - 1] * kr;
+    for (int m = 1; m <= L; ++m) c[m] = op.mul(c[m - 1], kr);
     g = fma(-c[L], F2, g);
 #pragma unroll
     for (int m = 0; m < L; ++m) a[m] = fma(-c[m], e2, a[m]);
@@ -239,7 +248,7 @@ __device__ __forceinline__ bool md_setup(const PrimPair& b, const PrimPair& k, c
 #pragma unroll
   for (int m = L; m >= 1; --m) {
     g = fma(R2, g, a[m - 1]);
-    if (m > 1) g *= 1.0 / (2 * m - 1);
+    if (m > 1) g = op.mul(g, fp64_operand(kFp64Recip + m));
     B[m - 1] = g;
   }
   return true;
@@ -338,7 +347,7 @@ __device__ __forceinline__ void md_gather(int round0, int n_round, int dst0, con
 // four blocks share a round (the longest sum counts).
 __device__ __forceinline__ void md_digest(const EriClassInfo& ci, const double* v, int A, int B, int C, int D,
                                           double deg, const double* __restrict__ P, double* K, int ld, int o0,
-                                          int ostep) {
+                                          int ostep, const Fp64& op) {
   const int na = ci.dims[0], nb = ci.dims[1], nc = ci.dims[2], nd = ci.dims[3];
   const int sb = nc * nd, sa = nb * sb;
   const int nAC = na * nc, nAD = na * nd, nBC = nb * nc, nout = nAC + nAD + nBC + nb * nd;
@@ -372,7 +381,7 @@ __device__ __forceinline__ void md_digest(const EriClassInfo& ci, const double* 
         pp += ld;
       }
     }
-    atomicAdd(K + (size_t)((isA ? A : B) + x) * ld + (isC ? C : D) + y, deg * acc);
+    atomicAdd(K + (size_t)((isA ? A : B) + x) * ld + (isC ? C : D) + y, op.mul(deg, acc));
   }
 }
 
@@ -415,6 +424,9 @@ __global__ void __launch_bounds__(md_block(LT), md_minb<R>(LT))
   int n_eval = 0;                                     // its primitive quartets evaluated so far
   int tb_sys = -1, tb_bra = -1;                       // whose transformation is in Tb
   Tally tally;
+  Fp64 op;
+  op.init();
+  const double omega = op.mul(L.omega, op.one), omega2 = op.mul(L.omega2, op.one);
 
   int kc_r[kRegs ? KR : 1], kc_w[kRegs ? KR : 1], bc_h[kRegs ? BR : 1], bc_w[kRegs ? BR : 1];
   R a_reg[kRegs ? BR : 1];
@@ -611,7 +623,7 @@ __global__ void __launch_bounds__(md_block(LT), md_minb<R>(LT))
         if (sc == sd) deg *= 0.5;
         if (e.y == e.z) deg *= 0.5;
         md_digest(L.ci, F, __ldg(Ls.sh.bf_off + sa), __ldg(Ls.sh.bf_off + sb), __ldg(Ls.sh.bf_off + sc),
-                  __ldg(Ls.sh.bf_off + sd), deg, Ls.P, Ls.K, Ls.ld, 32 * wt + lane, 32 * NW);
+                  __ldg(Ls.sh.bf_off + sd), deg, Ls.P, Ls.K, Ls.ld, 32 * wt + lane, 32 * NW, op);
       }
     }
     sync();
@@ -669,7 +681,7 @@ __global__ void __launch_bounds__(md_block(LT), md_minb<R>(LT))
         const EriLaunch& Ls = prims(s, pb, pk);
         if constexpr (F32) {
           PrimScalarsF ps;
-          const int st = prim_core_f32(*pb, *pk, LT, to_f32(Ls.omega), B, ps);
+          const int st = prim_core_f32(*pb, *pk, LT, to_f32(Ls.omega), B, ps, op);
           lam = sqrtf(2.0f * pb->pf * ps.RP);
           for (int i = 0; i < 3; ++i) PQ[i] = ps.PQ[i] * lam;
           ok = st == F32_OK;
@@ -677,11 +689,13 @@ __global__ void __launch_bounds__(md_block(LT), md_minb<R>(LT))
         } else {
           double qc[3] = {pk->P[0], pk->P[1], pk->P[2]};
           if constexpr (KIND == MD_PER) {  // the ket pair's image in cell G
-            qc[0] += L.shift[0];
-            qc[1] += L.shift[1];
-            qc[2] += L.shift[2];
+            qc[0] = op.add(qc[0], L.shift[0]);
+            qc[1] = op.add(qc[1], L.shift[1]);
+            qc[2] = op.add(qc[2], L.shift[2]);
           }
-          ok = md_setup<LT>(*pb, *pk, qc, Ls.omega, Ls.omega2, Ls.boys, B, PQ);
+          // (a kernel parameter is a constant operand: one product makes it a register's)
+          const double om = KIND == MD_BATCH ? Ls.omega : omega, om2 = KIND == MD_BATCH ? Ls.omega2 : omega2;
+          ok = md_setup<LT>(*pb, *pk, qc, om, om2, Ls.boys, B, PQ, op);
         }
       }
       okm = __ballot_sync(0xffffffffu, ok);
@@ -719,7 +733,7 @@ __global__ void __launch_bounds__(md_block(LT), md_minb<R>(LT))
           const EriLaunch& Ls = prims(t, pb, pk);
           double G[kMaxLt + 1];
           PrimScalars ps;
-          if (prim_core(*pb, *pk, LT, Ls.omega, Ls.omega2, Ls.boys, G, ps)) {
+          if (prim_core(*pb, *pk, LT, Ls.omega, Ls.omega2, Ls.boys, G, ps, op)) {
 #pragma unroll
             for (int k = 0; k <= LT; ++k) X[(sub * NX + k) * 32 + l] = to_f32_rn(G[k]);
             atomicOr(Xok + sub, 1u << l);
@@ -757,22 +771,22 @@ __global__ void __launch_bounds__(md_block(LT), md_minb<R>(LT))
         const int pos = __popc(okm & lt_mask);
         R* r = Rb + pos * kRow;
         for (int i = wt; i < mc.ket_set; i += NW) r[kW + i] = narrow(__ldg(wk + i));
-        if constexpr (NW == 1) hermite<LT, 1, 0>(B, PQ[0], PQ[1], PQ[2], lp, r);
+        if constexpr (NW == 1) hermite<LT, 1, 0>(B, PQ[0], PQ[1], PQ[2], lp, r, op);
         if constexpr (NW == 2) {
           if (wt == 0)
-            hermite<LT, 2, 0>(B, PQ[0], PQ[1], PQ[2], lp, r);
+            hermite<LT, 2, 0>(B, PQ[0], PQ[1], PQ[2], lp, r, op);
           else
-            hermite<LT, 2, 1>(B, PQ[0], PQ[1], PQ[2], lp, r);
+            hermite<LT, 2, 1>(B, PQ[0], PQ[1], PQ[2], lp, r, op);
         }
         if constexpr (NW == 4) {
           if (wt == 0)
-            hermite<LT, 4, 0>(B, PQ[0], PQ[1], PQ[2], lp, r);
+            hermite<LT, 4, 0>(B, PQ[0], PQ[1], PQ[2], lp, r, op);
           else if (wt == 1)
-            hermite<LT, 4, 1>(B, PQ[0], PQ[1], PQ[2], lp, r);
+            hermite<LT, 4, 1>(B, PQ[0], PQ[1], PQ[2], lp, r, op);
           else if (wt == 2)
-            hermite<LT, 4, 2>(B, PQ[0], PQ[1], PQ[2], lp, r);
+            hermite<LT, 4, 2>(B, PQ[0], PQ[1], PQ[2], lp, r, op);
           else
-            hermite<LT, 4, 3>(B, PQ[0], PQ[1], PQ[2], lp, r);
+            hermite<LT, 4, 3>(B, PQ[0], PQ[1], PQ[2], lp, r, op);
         }
       }
       sync();
