@@ -8,8 +8,8 @@
 // Layout: one warp runs one restart; its lanes share the radial grid r_i = i h (lane j owns the
 // points i = j + 1 + 32 t), so every sum over the grid is a per-lane partial sum followed by one
 // warp reduction.  Everything is FP64.  Per warp, shared memory holds the targets y_i, the
-// reduction scratch, a dense system for the local search and the genetic search's two
-// populations.  The genetic step and the local search are separate kernels (each gets its own
+// reduction scratch, a dense system for the local search, the genetic search's two
+// populations and, where it fits, the Gaussians on the grid.  The genetic step and the local search are separate kernels (each gets its own
 // register budget); a third picks the best restart per function.
 //
 // Gaussians on the grid: for an exponent a and beta = a h^2, exp(-beta i^2) moves along one lane's
@@ -46,12 +46,15 @@
 #include <string>
 
 #include "hfx.h"
+#include "hfx_internal.cuh"
 
 namespace hfx {
 void set_global_error(const std::string& msg);
 }
 
 namespace {
+
+using hfx::Fp64;
 
 constexpr int kMaxM = 6;
 constexpr int kMaxUnknowns = 2 * kMaxM;
@@ -96,8 +99,15 @@ __host__ __device__ constexpr int n_tri(int m) { return m * (m + 1) / 2; }
 // reduction scratch rows: A0, A1, A2 (three triangles), two gradients, one spare
 __host__ __device__ constexpr int n_red(int m) { return 3 * n_tri(m) + 2 * m + 1; }
 
-__host__ __device__ inline int warp_smem_doubles(int M, int npad, int P) {
-  return npad + n_red(M) * 33 + kMatDoubles + 10 * P * M + 2 * P;
+enum Which { kGenetic, kLocal, kProject };
+
+// Shared memory of one warp: targets, reduction rows, then per kernel the dense system (local
+// search), the populations (genetic step) and, with `store`, the Gaussians on the grid, kept by
+// the pass of the normal equations for the pass of the residual.
+__host__ __device__ inline int warp_smem_doubles(Which w, int M, int npad, int P, bool store) {
+  const int rows = w == kLocal ? n_red(M) : n_tri(M) + M;
+  return npad + rows * 33 + (w == kLocal ? kMatDoubles : 0) + (w == kGenetic ? 10 * P * M + 2 * P : 0) +
+         (store ? M * npad : 0);
 }
 
 // pop: genes u_m = ln alpha_m; al: alpha_m; fac: per Gaussian exp(-beta), exp(-64 beta) and
@@ -107,28 +117,36 @@ struct WarpMem {
   double* y;
   double* red;
   double* mat;
+  double* gauss;  // M x npad
   double* pop[2];
   double* al[2];
   double* fac[2];
   double* fit[2];
 };
 
-__device__ __forceinline__ WarpMem warp_mem(int M, int npad, int P) {
+template <Which W, int M, bool STORE>
+__device__ __forceinline__ WarpMem warp_mem(int npad, int P) {
   extern __shared__ double smem[];
   const int w = threadIdx.x >> 5;
-  double* base = smem + (size_t)w * warp_smem_doubles(M, npad, P);
-  WarpMem m;
-  m.y = base;
+  WarpMem m{};
+  m.y = smem + (size_t)w * warp_smem_doubles(W, M, npad, P, STORE);
   m.red = m.y + npad;
-  m.mat = m.red + n_red(M) * 33;
-  m.pop[0] = m.mat + kMatDoubles;
-  m.pop[1] = m.pop[0] + P * M;
-  m.al[0] = m.pop[1] + P * M;
-  m.al[1] = m.al[0] + P * M;
-  m.fac[0] = m.al[1] + P * M;
-  m.fac[1] = m.fac[0] + 3 * P * M;
-  m.fit[0] = m.fac[1] + 3 * P * M;
-  m.fit[1] = m.fit[0] + P;
+  double* next = m.red + (W == kLocal ? n_red(M) : n_tri(M) + M) * 33;
+  if constexpr (W == kLocal) m.mat = next;
+  if constexpr (STORE) {
+    m.gauss = next;
+    next += M * npad;
+  }
+  if constexpr (W == kGenetic) {
+    m.pop[0] = next;
+    m.pop[1] = m.pop[0] + P * M;
+    m.al[0] = m.pop[1] + P * M;
+    m.al[1] = m.al[0] + P * M;
+    m.fac[0] = m.al[1] + P * M;
+    m.fac[1] = m.fac[0] + 3 * P * M;
+    m.fit[0] = m.fac[1] + 3 * P * M;
+    m.fit[1] = m.fit[0] + P;
+  }
   return m;
 }
 
@@ -168,45 +186,46 @@ __device__ __forceinline__ double uniform01(unsigned long long seed, unsigned lo
 // ---------------------------------------------------------------------------
 // totals left in red[k * 33 + 32]
 template <int NV>
-__device__ __forceinline__ void warp_sum_smem(const double (&v)[NV], double* red, int lane) {
+__device__ __forceinline__ void warp_sum_smem(const double (&v)[NV], double* red, int lane, const Fp64& op) {
 #pragma unroll
   for (int k = 0; k < NV; ++k) red[k * 33 + lane] = v[k];
   __syncwarp();
-  for (int k = lane; k < NV; k += 32) {
-    const double* row = red + k * 33;
-    double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
+  // four lanes a row, each the sum of every fourth value in order, then (s0 + s1) + (s2 + s3): the
+  // order of one lane with four sums, in a quarter of the instructions
+  for (int k0 = 0; k0 < NV; k0 += 8) {
+    const int k = k0 + (lane >> 2), c = lane & 3;
+    const double* row = red + min(k, NV - 1) * 33 + c;
+    double s = 0.0;
 #pragma unroll
-    for (int j = 0; j < 32; j += 4) {
-      s0 += row[j];
-      s1 += row[j + 1];
-      s2 += row[j + 2];
-      s3 += row[j + 3];
-    }
-    red[k * 33 + 32] = (s0 + s1) + (s2 + s3);
+    for (int j = 0; j < 32; j += 4) s = op.add(s, row[j]);
+    s = op.add(s, __shfl_xor_sync(0xffffffffu, s, 1));
+    s = op.add(s, __shfl_xor_sync(0xffffffffu, s, 2));
+    __syncwarp();
+    if (c == 0 && k < NV) red[k * 33 + 32] = s;
   }
   __syncwarp();
 }
 
 template <int NV>
-__device__ __forceinline__ void warp_sum(double (&v)[NV], double* red, int lane) {
-  warp_sum_smem<NV>(v, red, lane);
+__device__ __forceinline__ void warp_sum(double (&v)[NV], double* red, int lane, const Fp64& op) {
+  warp_sum_smem<NV>(v, red, lane, op);
 #pragma unroll
   for (int k = 0; k < NV; ++k) v[k] = red[k * 33 + 32];
   __syncwarp();
 }
 
-__device__ __forceinline__ double warp_sum1(double v) {
+__device__ __forceinline__ double warp_sum1(double v, const Fp64& op) {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  for (int o = 16; o > 0; o >>= 1) v = op.add(v, __shfl_xor_sync(0xffffffffu, v, o));
   return __shfl_sync(0xffffffffu, v, 0);  // lane 0's order for everyone
 }
 
 // inclusive product of v over lanes 0..lane
-__device__ __forceinline__ double scan_mul(double v, int lane) {
+__device__ __forceinline__ double scan_mul(double v, int lane, const Fp64& op) {
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
     const double t = __shfl_up_sync(0xffffffffu, v, o);
-    if (lane >= o) v *= t;
+    if (lane >= o) v = op.mul(v, t);
   }
   return v;
 }
@@ -231,21 +250,21 @@ struct LaneGauss {
   // per Gaussian, by product scans over the lanes: with a = exp(-beta), lane j's first point
   // i0 = j + 1 has exp(-beta i0^2) = prod_{k <= j} a^{2k+1} and exp(-beta (64 i0 + 1024)) =
   // exp(-1024 beta) exp(-64 beta)^{j+1}; the step factor is exp(-1024 beta)^2
-  __device__ __forceinline__ void init_scan(const double* f, int lane) {
+  __device__ __forceinline__ void init_scan(const double* f, int lane, const Fp64& op) {
 #pragma unroll
     for (int m = 0; m < M; ++m) {
       const double a = f[3 * m], q = f[3 * m + 1], s = f[3 * m + 2];
-      const double r = a * scan_mul(lane == 0 ? 1.0 : a * a, lane);  // a^{2 lane + 1}
-      e[m] = scan_mul(r, lane);
-      c[m] = s * scan_mul(q, lane);
-      d[m] = s * s;
+      const double r = op.mul(a, scan_mul(lane == 0 ? 1.0 : op.mul(a, a), lane, op));  // a^{2 lane + 1}
+      e[m] = scan_mul(r, lane, op);
+      c[m] = op.mul(s, scan_mul(q, lane, op));
+      d[m] = op.mul(s, s);
     }
   }
-  __device__ __forceinline__ void step() {
+  __device__ __forceinline__ void step(const Fp64& op) {
 #pragma unroll
     for (int m = 0; m < M; ++m) {
-      e[m] *= c[m];
-      c[m] *= d[m];
+      e[m] = op.mul(e[m], c[m]);
+      c[m] = op.mul(c[m], d[m]);
     }
   }
 };
@@ -253,7 +272,7 @@ struct LaneGauss {
 // err(alpha, D) over the warp's grid, given the lane's Gaussian state at its first point
 template <int M>
 __device__ __forceinline__ double residual(LaneGauss<M> g, const double (&D)[M], const NaoArgs& A, const double* y,
-                                           int lane) {
+                                           int lane, const Fp64& op) {
   double s = 0.0;
   const int T = A.npad >> 5;
   for (int t = 0; t < T; ++t) {
@@ -262,17 +281,32 @@ __device__ __forceinline__ double residual(LaneGauss<M> g, const double (&D)[M],
     double f = 0.0;
 #pragma unroll
     for (int m = 0; m < M; ++m) f = fma(D[m], valid ? g.e[m] : 0.0, f);
-    const double res = f - y[i0];
+    const double res = op.sub(f, y[i0]);
     s = fma(res, res, s);
-    g.step();
+    g.step(op);
   }
-  return warp_sum1(s);
+  return warp_sum1(s, op);
+}
+
+// the same from the Gaussians kept on the grid
+template <int M>
+__device__ __forceinline__ double residual_kept(const double* gauss, const double (&D)[M], const NaoArgs& A,
+                                                const double* y, int lane, const Fp64& op) {
+  double s = 0.0;
+  for (int i0 = lane; i0 < A.npad; i0 += 32) {
+    double f = op.mul(D[0], gauss[i0]);
+#pragma unroll
+    for (int m = 1; m < M; ++m) f = fma(D[m], gauss[m * A.npad + i0], f);
+    const double res = op.sub(f, y[i0]);
+    s = fma(res, res, s);
+  }
+  return warp_sum1(s, op);
 }
 
 // Cholesky solve of a small SPD system held in registers (every lane the same), packed lower
 // triangle a[i (i + 1) / 2 + j]; false on a pivot that is not positive.
 template <int N>
-__device__ __forceinline__ bool chol_solve_reg(double (&a)[n_tri(N)], double (&b)[N]) {
+__device__ __forceinline__ bool chol_solve_reg(double (&a)[n_tri(N)], double (&b)[N], const Fp64& op) {
   double rd[N];
 #pragma unroll
   for (int j = 0; j < N; ++j) {
@@ -286,7 +320,7 @@ __device__ __forceinline__ bool chol_solve_reg(double (&a)[n_tri(N)], double (&b
       double t = a[n_tri(i) + j];
 #pragma unroll
       for (int k = 0; k < j; ++k) t = fma(-a[n_tri(i) + k], a[n_tri(j) + k], t);
-      a[n_tri(i) + j] = t * rd[j];
+      a[n_tri(i) + j] = op.mul(t, rd[j]);
     }
   }
 #pragma unroll
@@ -294,26 +328,28 @@ __device__ __forceinline__ bool chol_solve_reg(double (&a)[n_tri(N)], double (&b
     double t = b[i];
 #pragma unroll
     for (int k = 0; k < i; ++k) t = fma(-a[n_tri(i) + k], b[k], t);
-    b[i] = t * rd[i];
+    b[i] = op.mul(t, rd[i]);
   }
 #pragma unroll
   for (int i = N - 1; i >= 0; --i) {
     double t = b[i];
 #pragma unroll
     for (int k = i + 1; k < N; ++k) t = fma(-a[n_tri(k) + i], b[k], t);
-    b[i] = t * rd[i];
+    b[i] = op.mul(t, rd[i]);
   }
   return true;
 }
 
 // Variable projection: D minimising err for fixed alpha (ridged normal equations), and err there.
-template <int M>
+// STORE: the residual reads the Gaussians that the first pass left in shared memory instead of
+// running their recurrence again (2 M of its 3 M + 2 FP64 instructions per point).
+template <int M, bool STORE>
 __device__ __forceinline__ double project(const double (&alpha)[M], double (&D)[M], const NaoArgs& A,
-                                          const WarpMem& wm, int lane, const double* fac = nullptr) {
+                                          const WarpMem& wm, int lane, const Fp64& op, const double* fac = nullptr) {
   constexpr int NA = n_tri(M);
   LaneGauss<M> g0;
   if (fac)
-    g0.init_scan(fac, lane);
+    g0.init_scan(fac, lane, op);
   else
     g0.init(alpha, A.h * A.h, lane);
   LaneGauss<M> g = g0;
@@ -327,16 +363,19 @@ __device__ __forceinline__ double project(const double (&alpha)[M], double (&D)[
     const double yv = wm.y[i0];
     double ev[M];
 #pragma unroll
-    for (int m = 0; m < M; ++m) ev[m] = valid ? g.e[m] : 0.0;
+    for (int m = 0; m < M; ++m) {
+      ev[m] = valid ? g.e[m] : 0.0;
+      if constexpr (STORE) wm.gauss[m * A.npad + i0] = ev[m];
+    }
 #pragma unroll
     for (int i = 0; i < M; ++i) {
 #pragma unroll
       for (int j = 0; j <= i; ++j) acc[n_tri(i) + j] = fma(ev[i], ev[j], acc[n_tri(i) + j]);
       acc[NA + i] = fma(yv, ev[i], acc[NA + i]);
     }
-    g.step();
+    g.step(op);
   }
-  warp_sum(acc, wm.red, lane);
+  warp_sum(acc, wm.red, lane, op);
   double a[NA];
 #pragma unroll
   for (int i = 0; i < M; ++i) {
@@ -345,11 +384,14 @@ __device__ __forceinline__ double project(const double (&alpha)[M], double (&D)[
     a[n_tri(i) + i] += kRidge * acc[n_tri(i) + i];
     D[i] = acc[NA + i];
   }
-  if (!chol_solve_reg<M>(a, D)) {
+  if (!chol_solve_reg<M>(a, D, op)) {
 #pragma unroll
     for (int m = 0; m < M; ++m) D[m] = 0.0;
   }
-  return residual<M>(g0, D, A, wm.y, lane);
+  if constexpr (STORE)
+    return residual_kept<M>(wm.gauss, D, A, wm.y, lane, op);
+  else
+    return residual<M>(g0, D, A, wm.y, lane, op);
 }
 
 // ---------------------------------------------------------------------------
@@ -385,13 +427,13 @@ __device__ __forceinline__ double reflect_box(double c, double lo, double hi) {
   return fmin(fmax(c, lo), hi);
 }
 
-template <int M>
+template <int M, bool STORE>
 __device__ __forceinline__ double eval_individual(const double* al, const double* fac, const NaoArgs& A,
-                                                  const WarpMem& wm, int lane) {
+                                                  const WarpMem& wm, int lane, const Fp64& op) {
   double alpha[M], D[M];
 #pragma unroll
   for (int m = 0; m < M; ++m) alpha[m] = al[m];
-  return project<M>(alpha, D, A, wm, lane, fac);
+  return project<M, STORE>(alpha, D, A, wm, lane, op, fac);
 }
 
 // alpha = exp(u) and the grid-recurrence factors of one individual, into shared memory
@@ -410,7 +452,7 @@ __device__ __forceinline__ void store_individual(const double (&u)[M], double h2
   }
 }
 
-template <int M>
+template <int M, bool STORE>
 __global__ void __launch_bounds__(kWarps * 32) nao_genetic_kernel(NaoArgs A) {
   const int lane = threadIdx.x & 31;
   const long long q = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -418,7 +460,9 @@ __global__ void __launch_bounds__(kWarps * 32) nao_genetic_kernel(NaoArgs A) {
   const int f = (int)(q / A.N);
   const int P = A.P, G = A.G;
   constexpr int S = 4 + 2 * M;
-  const WarpMem wm = warp_mem(M, A.npad, P);
+  const WarpMem wm = warp_mem<kGenetic, M, STORE>(A.npad, P);
+  Fp64 op;
+  op.init();
   load_targets(A, f, wm.y, lane);
   auto ctr = [&](int g, int j, int k) -> unsigned long long {
     return (((unsigned long long)q * (unsigned long long)(G + 1) + (unsigned long long)g) * (unsigned long long)P +
@@ -436,7 +480,7 @@ __global__ void __launch_bounds__(kWarps * 32) nao_genetic_kernel(NaoArgs A) {
   }
   __syncwarp();
   for (int j = 0; j < P; ++j) {
-    const double fj = eval_individual<M>(wm.al[0] + j * M, wm.fac[0] + 3 * j * M, A, wm, lane);
+    const double fj = eval_individual<M, STORE>(wm.al[0] + j * M, wm.fac[0] + 3 * j * M, A, wm, lane, op);
     if (lane == 0) wm.fit[0][j] = fj;
   }
   __syncwarp();
@@ -484,7 +528,7 @@ __global__ void __launch_bounds__(kWarps * 32) nao_genetic_kernel(NaoArgs A) {
     }
     __syncwarp();
     for (int j = 1; j < P; ++j) {
-      const double fj = eval_individual<M>(nal + j * M, nfac + 3 * j * M, A, wm, lane);
+      const double fj = eval_individual<M, STORE>(nal + j * M, nfac + 3 * j * M, A, wm, lane, op);
       if (lane == 0) nfit[j] = fj;
     }
     __syncwarp();
@@ -494,7 +538,7 @@ __global__ void __launch_bounds__(kWarps * 32) nao_genetic_kernel(NaoArgs A) {
   double alpha[M], D[M];
 #pragma unroll
   for (int m = 0; m < M; ++m) alpha[m] = wm.al[cur][e * M + m];
-  const double fe = project<M>(alpha, D, A, wm, lane, wm.fac[cur] + 3 * e * M);
+  const double fe = project<M, STORE>(alpha, D, A, wm, lane, op, wm.fac[cur] + 3 * e * M);
   if (lane == 0) {
 #pragma unroll
     for (int m = 0; m < M; ++m) {
@@ -554,7 +598,9 @@ __global__ void __launch_bounds__(kWarps * 32) nao_local_kernel(NaoArgs A) {
   constexpr int NA = n_tri(M);
   constexpr int NU = 2 * M;
   constexpr int NS = 3 * NA + 2 * M;  // sums of one Jacobian pass
-  const WarpMem wm = warp_mem(M, A.npad, A.P);
+  const WarpMem wm = warp_mem<kLocal, M, false>(A.npad, A.P);
+  Fp64 op;
+  op.init();
   load_targets(A, f, wm.y, lane);
   const double h2 = A.h * A.h;
   double xa[M], xd[M];
@@ -565,7 +611,7 @@ __global__ void __launch_bounds__(kWarps * 32) nao_local_kernel(NaoArgs A) {
   }
   LaneGauss<M> g;
   g.init(xa, h2, lane);
-  double E = residual<M>(g, xd, A, wm.y, lane);
+  double E = residual<M>(g, xd, A, wm.y, lane, op);
   double lam = kLambda0;
   bool needJ = true;
   int it = 0, jpass = 0;
@@ -614,9 +660,9 @@ __global__ void __launch_bounds__(kWarps * 32) nao_local_kernel(NaoArgs A) {
           acc[3 * NA + i] += qv;
           acc[3 * NA + M + i] = fma(r2, qv, acc[3 * NA + M + i]);
         }
-        gg.step();
+        gg.step(op);
       }
-      warp_sum_smem<NS>(acc, wm.red, lane);
+      warp_sum_smem<NS>(acc, wm.red, lane, op);
       // g = J^T res: d/d alpha_m = -D_m sum r^2 e_m res, d/d D_m = sum e_m res
       double dmax = 0.0;
 #pragma unroll
@@ -673,7 +719,7 @@ __global__ void __launch_bounds__(kWarps * 32) nao_local_kernel(NaoArgs A) {
     __syncwarp();
     LaneGauss<M> gt;
     gt.init(xta, h2, lane);
-    const double Et = residual<M>(gt, xtd, A, wm.y, lane);
+    const double Et = residual<M>(gt, xtd, A, wm.y, lane, op);
     if (Et < E * kTieFactor) {
       const bool conv = (E - Et) <= kConv * E;
 #pragma unroll
@@ -742,7 +788,7 @@ __global__ void nao_best_kernel(int n_fun, int N, int M, const double* r_alpha, 
 }
 
 // Variable projection for given exponent sets (one warp per set).
-template <int M>
+template <int M, bool STORE>
 __global__ void __launch_bounds__(kWarps * 32) nao_project_kernel(NaoArgs A) {
   const int lane = threadIdx.x & 31;
   const long long s = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -756,12 +802,14 @@ __global__ void __launch_bounds__(kWarps * 32) nao_project_kernel(NaoArgs A) {
     }
     return;
   }
-  const WarpMem wm = warp_mem(M, A.npad, A.P);
+  const WarpMem wm = warp_mem<kProject, M, STORE>(A.npad, A.P);
+  Fp64 op;
+  op.init();
   load_targets(A, f, wm.y, lane);
   double alpha[M], D[M];
 #pragma unroll
   for (int m = 0; m < M; ++m) alpha[m] = __ldg(A.set_alpha + s * M + m);
-  const double e = project<M>(alpha, D, A, wm, lane);
+  const double e = project<M, STORE>(alpha, D, A, wm, lane, op);
   if (lane == 0) {
 #pragma unroll
     for (int m = 0; m < M; ++m) A.set_D[s * M + m] = D[m];
@@ -772,35 +820,50 @@ __global__ void __launch_bounds__(kWarps * 32) nao_project_kernel(NaoArgs A) {
 // ---------------------------------------------------------------------------
 // Host side
 // ---------------------------------------------------------------------------
-enum Which { kGenetic, kLocal, kProject };
-
 template <int M>
-const void* kernel_of(Which w) {
+const void* kernel_of(Which w, bool store) {
   switch (w) {
-    case kGenetic: return (const void*)nao_genetic_kernel<M>;
+    case kGenetic: return store ? (const void*)nao_genetic_kernel<M, true> : (const void*)nao_genetic_kernel<M, false>;
     case kLocal: return (const void*)nao_local_kernel<M>;
-    default: return (const void*)nao_project_kernel<M>;
+    default: return store ? (const void*)nao_project_kernel<M, true> : (const void*)nao_project_kernel<M, false>;
   }
 }
 
-const void* kernel_for(int M, Which w) {
+const void* kernel_for(int M, Which w, bool store) {
   switch (M) {
-    case 1: return kernel_of<1>(w);
-    case 2: return kernel_of<2>(w);
-    case 3: return kernel_of<3>(w);
-    case 4: return kernel_of<4>(w);
-    case 5: return kernel_of<5>(w);
-    default: return kernel_of<6>(w);
+    case 1: return kernel_of<1>(w, store);
+    case 2: return kernel_of<2>(w, store);
+    case 3: return kernel_of<3>(w, store);
+    case 4: return kernel_of<4>(w, store);
+    case 5: return kernel_of<5>(w, store);
+    default: return kernel_of<6>(w, store);
   }
+}
+
+// restarts per block: up to kWarps, as many as the shared memory of a block holds
+int warps_per_block(size_t per_warp) {
+  return (int)std::max<size_t>(1, std::min<size_t>(kWarps, kMaxBlockSmem / per_warp));
+}
+
+// warps an SM holds by shared memory (228 KB, 1 KB of it per block reserved)
+int resident_warps(size_t per_warp) {
+  const int w = warps_per_block(per_warp);
+  return (int)(228 * 1024 / (w * per_warp + 1024)) * w;
 }
 
 int launch(Which w, int M, const NaoArgs& a, long long n_warps, cudaStream_t s) {
   if (n_warps <= 0) return HFX_OK;
-  // up to kWarps restarts per block, as many as the shared memory of a block holds
-  const size_t per_warp = (size_t)warp_smem_doubles(M, a.npad, a.P) * sizeof(double);
-  const int warps = (int)std::max<size_t>(1, std::min<size_t>(kWarps, kMaxBlockSmem / per_warp));
+  // the Gaussians are kept on the grid where that leaves 8 warps per SM or costs none: two warps
+  // per SM quarter keep the FP64 pipe busy, fewer do not
+  auto bytes = [&](bool store) {
+    return (size_t)warp_smem_doubles(w, M, a.npad, a.P, store) * sizeof(double);
+  };
+  const bool store = w != kLocal && bytes(true) <= kMaxBlockSmem &&
+                     (resident_warps(bytes(true)) >= 8 || resident_warps(bytes(true)) == resident_warps(bytes(false)));
+  const size_t per_warp = bytes(store);
+  const int warps = warps_per_block(per_warp);
   const size_t smem = warps * per_warp;
-  const void* k = kernel_for(M, w);
+  const void* k = kernel_for(M, w, store);
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) {
     hfx::set_global_error(std::string("nao: shared memory request refused: ") + cudaGetErrorString(e));
