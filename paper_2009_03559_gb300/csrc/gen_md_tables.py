@@ -145,6 +145,36 @@ class Gather:
             self.dst += [outs[lanes[l]][0] if l < len(lanes) else 0xFFFF for l in range(32)]
 
 
+class Digest:
+    """The sums of the four blocks A_ac, A_ad, A_bc, A_bd over the final block (a, b, c, d), as lane
+    tasks: (row of b instead of a, column of d instead of c, row, column, first u, first w, terms), u
+    and w the two summed indices, w running fastest.  A sum is cut into tasks of at most `chunk`
+    terms (each adds its part to the matrix), the tasks dealt to lanes by length: the chunk that
+    costs the fewest instructions, a round counting its longest task and two more."""
+
+    def __init__(self, dims):
+        na, nb, nc, nd = dims
+        best = None
+        for chunk in range(1, 26):
+            tasks = []
+            for isb in (0, 1):
+                for isd in (0, 1):
+                    nw = nc if isd else nd
+                    n = (na if isb else nb) * nw
+                    parts = -(-n // chunk)
+                    cuts = [n * i // parts for i in range(parts + 1)]
+                    for x in range(nb if isb else na):
+                        for y in range(nd if isd else nc):
+                            tasks += [(isb, isd, x, y, c0 // nw, c0 % nw, c1 - c0) for c0, c1 in zip(cuts, cuts[1:])]
+            tasks.sort(key=lambda s: -s[6])
+            cost = sum(tasks[r][6] + 2 for r in range(0, len(tasks), 32))
+            if best is None or (cost, len(tasks)) < best[:2]:
+                best = (cost, len(tasks), tasks)
+        self.cost, _, tasks = best
+        tasks = tasks + [(0,) * 7] * (-len(tasks) % 32)
+        self.words = [b | d << 1 | x << 2 | y << 5 | u << 8 | w << 11 | n << 14 for b, d, x, y, u, w, n in tasks]
+
+
 class MdClass:
     def __init__(self, hi, lo):
         self.hi, self.lo = hi, lo
@@ -170,6 +200,9 @@ class MdClass:
         self.z2 = Gather([(ab * self.ncd + f, [(c, b.row[sb, p] * self.ncd + f) for c, sb, p in b.terms(ab)])
                           for ab in range(self.nab) for f in range(self.ncd)])
 
+        self.dims = [2 * l + 1 for l in (*PAIR_CLASSES[hi], *PAIR_CLASSES[lo])]
+        self.digest = Digest(self.dims)
+
     def name(self):
         L = "spd"
         return "(" + "|".join("".join(L[x] for x in PAIR_CLASSES[c]) for c in (self.hi, self.lo)) + ")"
@@ -190,7 +223,7 @@ def classes():
 
 def emit(w):
     cl = classes()
-    kc, bc, zw, zd, zr, rows = [], [], [], [], [], []
+    kc, bc, zw, zd, zr, dg, rows = [], [], [], [], [], [], []
     for c in cl:
         r = dict(kc=len(kc), nkc=len(c.kc), bc=len(bc), nbc=len(c.bc))
         kc += [i | (s << 8) for i, s in c.kc]
@@ -203,6 +236,8 @@ def emit(w):
             zr += [(len(zw) + o) | (n << 24) for o, n in g.rounds]
             zw += g.words
             zd += g.dst
+        r["dig"] = (len(dg), len(c.digest.words) // 32)
+        dg += c.digest.words
         rows.append((c, r))
     assert len(zw) < 1 << 24
     w("// Generated by gen_md_tables.py -- do not edit by hand.\n#pragma once\n\n")
@@ -219,6 +254,8 @@ def emit(w):
     arr("kMdZ", "uint32_t", zw)
     arr("kMdZDst", "uint16_t", zd)
     arr("kMdZRound", "uint32_t", zr)
+    w("// digest: row b | column d << 1 | row << 2 | column << 5 | first u << 8 | first w << 11 | terms << 14\n")
+    arr("kMdDigest", "uint32_t", dg)
     # coefficients per pair type: polynomials over the 35 monomials of AB up to degree 4
     mono = {m: i for i, m in enumerate(m for n in range(5) for m in monos(n))}
     poly, cf, sign, info = [], [], [], []
@@ -241,11 +278,11 @@ def emit(w):
     for c, r in rows:
         z = (sum(n for _, n in c.z1.rounds), sum(n for _, n in c.z2.rounds))
         w(f"  // {c.name()}: Hermite recursion {c.r_ops()} instructions on every primitive quartet's lane, contraction "
-          f"{-(-len(c.kc) // 32)} per primitive quartet, {-(-len(c.bc) // 32)} per bra pair, transformation {z[0]} + {z[1]}\n")
+          f"{-(-len(c.kc) // 32)} per primitive quartet, {-(-len(c.bc) // 32)} per bra pair, transformation {z[0]} + {z[1]}, digest {c.digest.cost}\n")
         b, k = info[c.hi], info[c.lo]
         w(f"  {{{c.Lt}, {r['kc']}, {r['nkc']}, {r['bc']}, {r['nbc']}, {c.n_rows}, {c.nab}, {c.ncd}, "
           f"{b[0]}, {b[1]}, {b[2]}, {k[1]}, {k[2]}, "
-          f"{r['z1'][0]}, {r['z1'][1]}, {r['z1'][2]}, {r['z2'][0]}, {r['z2'][1]}, {r['z2'][2]}}},\n")
+          f"{r['z1'][0]}, {r['z1'][1]}, {r['z1'][2]}, {r['z2'][0]}, {r['z2'][1]}, {r['z2'][2]}, {r['dig'][0]}, {r['dig'][1]}}},\n")
     w("};\n")
 
 
@@ -253,7 +290,7 @@ if __name__ == "__main__":
     if "--summary" in sys.argv:
         for c in classes():
             print(c.name(), "L", c.Lt, "R", c.r_ops(), "kc", len(c.kc), "bc", len(c.bc), "rows", c.n_rows,
-                  "z1", sum(n for _, n in c.z1.rounds), "z2", sum(n for _, n in c.z2.rounds), "coefs",
+                  "z1", sum(n for _, n in c.z1.rounds), "z2", sum(n for _, n in c.z2.rounds), "digest", c.digest.cost, len(c.digest.words) // 32, "coefs",
                   len(PAIRS[c.hi].coefs), len(PAIRS[c.lo].coefs), "Y", c.n_rows * c.ncd)
     else:
         emit(sys.stdout.write)

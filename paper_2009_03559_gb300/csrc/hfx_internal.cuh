@@ -35,6 +35,7 @@ struct MdClassInfo {
   int bra_coef0, bra_coef, bra_set;    // bra pair type: first coefficient, coefficients, sets
   int ket_coef, ket_set;
   int z1_round, z1_n, z1_dst, z2_round, z2_n, z2_dst;  // transformation passes
+  int dig, dig_n;                      // digest (first round, rounds)
 };
 // ... and the sets and coefficients of a pair type (set: power of 1/2p | of u_b << 4 | of u_a << 8)
 struct MdPairInfo {

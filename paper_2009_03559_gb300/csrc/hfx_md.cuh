@@ -267,7 +267,8 @@ __host__ __device__ constexpr int md_block(int Lt) { return Lt <= 5 ? 64 : 32 * 
 // recurrences and the spherical step, and the digest in FP64).  A team sets up kSub32 times 32
 // primitive quartets before it contracts them, so that those whose Boys step the FP32 set-up
 // declines (a few per cent) are set up in FP64 together: one FP64 set-up per 128 primitive
-// quartets, not one per 32.
+// quartets, not one per 32.  (6 and 8 times 32: fewer FP64 set-ups, but their shared memory costs
+// resident warps, 64-atom mixed build 1153 -> 1185 and 1221 ms.)
 constexpr int kSub32 = 4;
 // 32s of primitive quartets set up together; whether their set-up passes through shared memory;
 // its values per primitive quartet: base values, P - Q (times lam, and lam itself, in FP32)
@@ -342,53 +343,46 @@ __device__ __forceinline__ void md_gather(int round0, int n_round, int dst0, con
   }
 }
 
-// Digest of the final block into the half matrix A, a lane per output element of the four
-// blocks; every lane runs the same instructions with its own strides, so the outputs of the
-// four blocks share a round (the longest sum counts).
-__device__ __forceinline__ void md_digest(const EriClassInfo& ci, const double* v, int A, int B, int C, int D,
-                                          double deg, const double* __restrict__ P, double* K, int ld, int o0,
-                                          int ostep, const Fp64& op) {
-  const int na = ci.dims[0], nb = ci.dims[1], nc = ci.dims[2], nd = ci.dims[3];
-  const int sb = nc * nd, sa = nb * sb;
-  const int nAC = na * nc, nAD = na * nd, nBC = nb * nc, nout = nAC + nAD + nBC + nb * nd;
-  for (int o = o0; o < nout; o += ostep) {
-    int t = o;
-    bool isA = true, isC = true;  // row function of a (else b), column function of c (else d)
-    if (t >= nAC + nAD) {
-      t -= nAC + nAD;
-      isA = false;
-      if (t >= nBC) {
-        t -= nBC;
-        isC = false;
-      }
-    } else if (t >= nAC) {
-      t -= nAC;
-      isC = false;
-    }
-    const int ny = isC ? nc : nd, x = t / ny, y = t - x * ny;
-    const int su = isA ? sb : sa, nu = isA ? nb : na, sw = isC ? 1 : nd, nw = isC ? nd : nc;
-    const double* vp = v + x * (isA ? sa : sb) + y * (isC ? nd : 1);
-    const double* pp = P + (size_t)(isA ? B : A) * ld + (isC ? D : C);
-    double acc = 0.0;
-    int w = 0;
-    const int n = nu * nw;
-#pragma unroll 4
+// Digest of the final block into the half matrix A: rounds w, w + nw, ... of 32 generated tasks, a
+// lane per (part of a) sum.  Every lane runs the same instructions with its own strides, so the
+// sums of the four blocks share a round, and long sums (the 25 terms of A_bd in (ds|ds)) are cut so
+// that a round's longest does not set the pace (64 atoms: FP64 build 1819 -> 1795 ms, mixed
+// 1193 -> 1153 ms, whose FP32 pass the digest weighs on most).
+__device__ __forceinline__ void md_digest(const MdClassInfo& mc, const int4& dim, const double* v, int A, int B,
+                                          int C, int D, double deg, const double* __restrict__ P, double* K, int ld,
+                                          int lane, int w0, int nw0, const Fp64& op) {
+  const int sb = dim.z * dim.w, sa = dim.y * sb;
+#pragma unroll 1
+  for (int r = w0; r < mc.dig_n; r += nw0) {
+    const uint32_t e = __ldg(kMdDigest + mc.dig + 32 * r + lane);
+    const bool isB = e & 1, isD = e & 2;
+    const int x = (e >> 2) & 7, y = (e >> 5) & 7, u = (e >> 8) & 7, n = (e >> 14) & 31;
+    int w = (e >> 11) & 7;
+    const int su = isB ? sa : sb, sw = isD ? dim.w : 1, nw = isD ? dim.z : dim.w;
+    const double* vp = v + x * (isB ? sb : sa) + y * (isD ? 1 : dim.w) + u * su + w * sw;
+    const double* pp = P + (size_t)((isB ? A : B) + u) * ld + (isD ? C : D) + w;
+    double acc = op.nzero;
+    // at the end of a row of w: v to the next u's first w, P to the next row's
+    const int vskip = su - nw * sw, pskip = ld - nw;
+#pragma unroll 1
     for (int i = 0; i < n; ++i) {
-      acc = fma(vp[w * sw], __ldg(pp + w), acc);
+      acc = fma(*vp, __ldg(pp), acc);
+      vp += sw;
+      ++pp;
       if (++w == nw) {
         w = 0;
-        vp += su;
-        pp += ld;
+        vp += vskip;
+        pp += pskip;
       }
     }
-    atomicAdd(K + (size_t)((isA ? A : B) + x) * ld + (isC ? C : D) + y, op.mul(deg, acc));
+    if (n) atomicAdd(K + (size_t)((isB ? B : A) + x) * ld + (isD ? D : C) + y, op.mul(deg, acc));
   }
 }
 
 // resident blocks per SM that the registers must allow: what shared memory allows
 template <typename R>
 __host__ __device__ constexpr int md_minb(int Lt) {
-  return sizeof(R) == 4 ? (Lt <= 6 ? 8 : 4) : (Lt <= 4 ? 8 : (Lt <= 6 ? 5 : (Lt == 7 ? 3 : 2)));
+  return sizeof(R) == 4 ? (Lt <= 3 ? 10 : (Lt <= 6 ? 8 : 4)) : (Lt <= 4 ? 8 : (Lt <= 6 ? 5 : (Lt == 7 ? 3 : 2)));
 }
 
 template <int LT, int KIND, typename R>
@@ -416,6 +410,7 @@ __global__ void __launch_bounds__(md_block(LT), md_minb<R>(LT))
   const unsigned lt_mask = (1u << lane) - 1u;
   const MdClassInfo mc = L.mc;
   const EriLaunch* const Lp = &L;
+  const int4 dims = make_int4(L.ci.dims[0], L.ci.dims[1], L.ci.dims[2], L.ci.dims[3]);
   unsigned long long t0 = 0;
   if (L.busy && threadIdx.x == 0) t0 = globaltimer_ns();
 
@@ -622,8 +617,8 @@ __global__ void __launch_bounds__(md_block(LT), md_minb<R>(LT))
         if (sa == sb) deg *= 0.5;
         if (sc == sd) deg *= 0.5;
         if (e.y == e.z) deg *= 0.5;
-        md_digest(L.ci, F, __ldg(Ls.sh.bf_off + sa), __ldg(Ls.sh.bf_off + sb), __ldg(Ls.sh.bf_off + sc),
-                  __ldg(Ls.sh.bf_off + sd), deg, Ls.P, Ls.K, Ls.ld, 32 * wt + lane, 32 * NW, op);
+        md_digest(mc, dims, F, __ldg(Ls.sh.bf_off + sa), __ldg(Ls.sh.bf_off + sb), __ldg(Ls.sh.bf_off + sc),
+                  __ldg(Ls.sh.bf_off + sd), deg, Ls.P, Ls.K, Ls.ld, lane, wt, NW, op);
       }
     }
     sync();

@@ -93,3 +93,31 @@ def test_tables_reproduce_oracle_integrals(ci):
     ref = expected(os_class, [np.array([*e, *f]) for e in bra for f in ket], cen, omega)
     scale = np.abs(ref).max()
     assert np.allclose(got, ref.reshape(-1), rtol=1e-10, atol=1e-12 * scale), (c.name(), np.abs(got - ref.reshape(-1)).max())
+
+
+@pytest.mark.parametrize("ci", range(21), ids=[c.name() for c in MD])
+def test_digest_tasks_make_the_four_blocks(ci):
+    """Every term of every sum once: A_ac += v P_bd, A_ad += v P_bc, A_bc += v P_ad, A_bd += v P_ac."""
+    c = MD[ci]
+    na, nb, nc, nd = c.dims
+    rng = np.random.default_rng(ci)
+    v = rng.standard_normal(c.dims)
+    P = rng.standard_normal((4, 4, 5, 5))  # P[i, j]: block of shells i, j (a, b, c, d = 0 .. 3)
+    got = {}
+    for e in c.digest.words:
+        isb, isd, x, y, u, w, n = e & 1, (e >> 1) & 1, (e >> 2) & 7, (e >> 5) & 7, (e >> 8) & 7, (e >> 11) & 7, e >> 14
+        acc = 0.0
+        for _ in range(n):
+            a, b = (u, x) if isb else (x, u)
+            cc, d = (w, y) if isd else (y, w)
+            acc += v[a, b, cc, d] * P[0 if isb else 1, 2 if isd else 3][u, w]
+            w += 1
+            if w == (nc if isd else nd):
+                u, w = u + 1, 0
+        if n:
+            got[isb, isd, x, y] = got.get((isb, isd, x, y), 0.0) + acc
+    want = {(0, 0): np.einsum("abcd,bd->ac", v, P[1, 3][:nb, :nd]), (0, 1): np.einsum("abcd,bc->ad", v, P[1, 2][:nb, :nc]),
+            (1, 0): np.einsum("abcd,ad->bc", v, P[0, 3][:na, :nd]), (1, 1): np.einsum("abcd,ac->bd", v, P[0, 2][:na, :nc])}
+    assert len(got) == sum(w.size for w in want.values())
+    for (isb, isd, x, y), val in got.items():
+        assert abs(val - want[isb, isd][x, y]) <= 1e-13
