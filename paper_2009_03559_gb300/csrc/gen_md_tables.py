@@ -221,6 +221,11 @@ def classes():
     return [MdClass(hi, lo) for hi in range(6) for lo in range(hi + 1)]
 
 
+# warps that work on one stream together (the kernel's choice and its reasons: hfx_md.cuh)
+def team(Lt):
+    return 1 if Lt <= 5 else (2 if Lt == 6 else 4)
+
+
 def emit(w):
     cl = classes()
     kc, bc, zw, zd, zr, dg, rows = [], [], [], [], [], [], []
@@ -256,6 +261,17 @@ def emit(w):
     arr("kMdZRound", "uint32_t", zr)
     w("// digest: row b | column d << 1 | row << 2 | column << 5 | first u << 8 | first w << 11 | terms << 14\n")
     arr("kMdDigest", "uint32_t", dg)
+    by_l = [[c for c in cl if c.Lt == l] for l in range(9)]
+    rounds = lambda n, l: -(-(-(-n // 32)) // team(l))  # noqa: E731
+    w("// by total angular momentum: warps of a team; the most rounds a warp of it has in a ket and in a\n"
+      "// bra contraction; the most sets of a ket\n")
+    for name, v in (("md_team", [team(l) for l in range(9)]),
+                    ("md_kc_rounds", [max(rounds(len(c.kc), l) for c in by_l[l]) for l in range(9)]),
+                    ("md_bc_rounds", [max(rounds(len(c.bc), l) for c in by_l[l]) for l in range(9)]),
+                    ("md_ket_sets", [max(len(PAIRS[c.lo].sets) for c in by_l[l]) for l in range(9)])):
+        w(f"__host__ __device__ constexpr int {name}(int Lt) {{\n  const int v[9] = {{{', '.join(map(str, v))}}};\n"
+          "  return v[Lt];\n}\n")
+    w("\n")
     # coefficients per pair type: polynomials over the 35 monomials of AB up to degree 4
     mono = {m: i for i, m in enumerate(m for n in range(5) for m in monos(n))}
     poly, cf, sign, info = [], [], [], []

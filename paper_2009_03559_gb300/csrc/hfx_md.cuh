@@ -66,7 +66,7 @@ __device__ __forceinline__ void exact_rounds(int n, F&& f) {
       return;
     }
   }
-  f(std::integral_constant<int, N>());
+  if (n >= N) f(std::integral_constant<int, N>());  // (n may be 0: a team's last warps)
 }
 
 // f(0) .. f(n - 1), U at a time and the rest one by one (a loop unrolled by the compiler ran its
@@ -259,8 +259,10 @@ __device__ __forceinline__ bool md_setup(const PrimPair& b, const PrimPair& k, c
 // leave 6, 4 and 2 resident warps per SM at L = 6, 7, 8 (FP64 pipe 73, 49 and 26 % busy); teams
 // bring that to 10, 12 and 8.  Up to L = 5 a lone warp's buffers leave 8 to 16 and the pipe 86 to
 // 90 % busy, and a team's barriers would only cost.
-__host__ __device__ constexpr int md_team(int Lt) { return Lt <= 5 ? 1 : (Lt == 6 ? 2 : 4); }
-__host__ __device__ constexpr int md_block(int Lt) { return Lt <= 5 ? 64 : 32 * md_team(Lt); }
+// (md_team: 1 up to L = 5, then 2, 4, 4)
+// threads per block: two lone warps up to L = 4, one at L = 5 (whose 23 KB a warp fill the SM better
+// in single pieces: (dp|pp) 199 -> 193 ms at 64 atoms), one team beyond
+__host__ __device__ constexpr int md_block(int Lt) { return Lt <= 4 ? 64 : 32 * md_team(Lt); }
 
 // The FP32 pass of a mixed-precision class runs the same steps with the set-up, the Hermite
 // recursion and both contractions in FP32 (the transformations, which replace the horizontal
@@ -271,25 +273,24 @@ __host__ __device__ constexpr int md_block(int Lt) { return Lt <= 5 ? 64 : 32 * 
 // resident warps, 64-atom mixed build 1153 -> 1185 and 1221 ms.)
 constexpr int kSub32 = 4;
 // 32s of primitive quartets set up together; whether their set-up passes through shared memory;
-// its values per primitive quartet: base values, P - Q (times lam, and lam itself, in FP32)
+// its values per primitive quartet: base values, P - Q (in FP32 times lam, lam, and where it belongs)
 template <typename R>
 __host__ __device__ constexpr int md_sub(int Lt) { return sizeof(R) == 4 ? kSub32 : md_team(Lt); }
 template <typename R>
-__host__ __device__ constexpr int md_xval(int Lt) { return sizeof(R) == 4 ? Lt + 5 : Lt + 4; }
+__host__ __device__ constexpr int md_xval(int Lt) { return sizeof(R) == 4 ? Lt + 6 : Lt + 4; }
 
 // Row of a primitive quartet in shared memory: its Hermite integrals, then the factors of its ket
 // primitive pair (at most as many as the classes of this L have sets); an odd length, so that the
 // lanes' rows start in different banks, and known when compiling, so that the contraction's loads
 // need no address arithmetic.
 __host__ __device__ constexpr int md_row(int Lt) {
-  const int sets[kMaxLt + 1] = {1, 1, 2, 2, 5, 5, 8, 8, 14};
-  return (n_herm(Lt) + sets[Lt]) | 1;
+  return (n_herm(Lt) + md_ket_sets(Lt)) | 1;
 }
-// Up to L = 4 a lane's entries of the contraction tables and its A values stay in registers (at
-// most this many rounds); up to L = 2, where a ket contraction has at most 13 results, the warp
-// runs 32 / md_group of them side by side.
-__host__ __device__ constexpr int md_kc_rounds(int Lt) { return Lt <= 3 ? 1 : 3; }
-__host__ __device__ constexpr int md_bc_rounds(int Lt) { return Lt <= 2 ? 1 : (Lt == 3 ? 2 : 5); }
+// Up to L = 4, in FP32 up to L = 7, a lane's entries of the contraction tables and its A values stay
+// in registers (at most this many rounds of a warp of the team); up to L = 2, where a ket
+// contraction has at most 13 results, the warp runs 32 / md_group of them side by side.
+template <typename R>
+__host__ __device__ constexpr bool md_in_regs(int Lt) { return Lt <= (sizeof(R) == 4 ? 7 : 4); }
 __host__ __device__ constexpr int md_group(int Lt) { return Lt == 0 ? 1 : (Lt == 1 ? 4 : 16); }
 
 // Shared memory of one team, in doubles (offsets; every region starts on an even double).
@@ -313,7 +314,7 @@ MdLayout md_layout(const MdClassInfo& c, const MdPairInfo& b, const MdPairInfo& 
   l.Tb = l.A + std::max(mem(c.n_bc), even(c.nab * c.ncd));
   l.Tk = l.Tb + even(b.n_coef);
   l.Q = l.Tk + even(k.n_coef);
-  l.X = l.Q + 2 * kMdQueue;
+  l.X = l.Q + 4 * kMdQueue;
   const int ns = md_sub<R>(c.Lt);
   // the values of 32 lanes; the accepted and declined masks; the team's claim
   l.size = l.X + (ns > 1 ? mem(ns * md_xval<R>(c.Lt) * 32) + ns + 2 : 0);
@@ -382,7 +383,8 @@ __device__ __forceinline__ void md_digest(const MdClassInfo& mc, const int4& dim
 // resident blocks per SM that the registers must allow: what shared memory allows
 template <typename R>
 __host__ __device__ constexpr int md_minb(int Lt) {
-  return sizeof(R) == 4 ? (Lt <= 3 ? 10 : (Lt <= 6 ? 8 : 4)) : (Lt <= 4 ? 8 : (Lt <= 6 ? 5 : (Lt == 7 ? 3 : 2)));
+  const int f32[kMaxLt + 1] = {10, 10, 10, 10, 8, 12, 7, 4, 4}, f64[kMaxLt + 1] = {8, 8, 8, 8, 8, 10, 5, 3, 2};
+  return sizeof(R) == 4 ? f32[Lt] : f64[Lt];
 }
 
 template <int LT, int KIND, typename R>
@@ -393,7 +395,7 @@ __global__ void __launch_bounds__(md_block(LT), md_minb<R>(LT))
   constexpr int NW = md_team(LT), kQ = kMdQueue, kTeams = md_block(LT) / (32 * NW);
   constexpr int NS = md_sub<R>(LT), NX = md_xval<R>(LT);
   constexpr int kRow = md_row(LT), kW = n_herm(LT);
-  constexpr bool kRegs = LT <= 4;
+  constexpr bool kRegs = md_in_regs<R>(LT);
   constexpr int KR = md_kc_rounds(LT), BR = md_bc_rounds(LT);
   const int lane = threadIdx.x & 31;
   const int wt = NW == 1 ? 0 : (int)(threadIdx.x >> 5);             // warp of the team
@@ -405,6 +407,9 @@ __global__ void __launch_bounds__(md_block(LT), md_minb<R>(LT))
   double* const Y = S + ly.Y;
   double* const F = S + ly.A;
   int4* const Q = reinterpret_cast<int4*>(S + ly.Q);  // system, bra position, ket position, nb | nk << 16
+  // the bra's and the ket's first primitive pair, and where their Hermite data begin (in fours of
+  // doubles): looked up once per quartet, not once per primitive quartet and run
+  uint4* const Qo = reinterpret_cast<uint4*>(Q + kQ);
   R* const X = reinterpret_cast<R*>(S + ly.X);
   unsigned* const Xok = reinterpret_cast<unsigned*>(S + ly.size - NS - 2);  // masks [NS], [NS], then the claim
   const unsigned lt_mask = (1u << lane) - 1u;
@@ -428,14 +433,14 @@ __global__ void __launch_bounds__(md_block(LT), md_minb<R>(LT))
   if constexpr (kRegs) {
 #pragma unroll
     for (int u = 0; u < KR; ++u) {
-      const int o = 32 * u + (LT <= 2 ? lane % md_group(LT) : lane);
+      const int o = 32 * (wt + NW * u) + (LT <= 2 ? lane % md_group(LT) : lane);
       const int e = o < mc.n_kc ? __ldg(kMdKc + mc.kc + o) : 0;
       kc_r[u] = e & 0xFF;
       kc_w[u] = kW + (e >> 8);
     }
 #pragma unroll
     for (int u = 0; u < BR; ++u) {
-      const int e = 32 * u + lane < mc.n_bc ? __ldg(kMdBc + mc.bc + 32 * u + lane) : 0;
+      const int o = 32 * (wt + NW * u) + lane, e = o < mc.n_bc ? __ldg(kMdBc + mc.bc + o) : 0;
       bc_h[u] = e & 0xFFF;
       bc_w[u] = e >> 12;
       a_reg[u] = R(0);
@@ -468,12 +473,15 @@ __global__ void __launch_bounds__(md_block(LT), md_minb<R>(LT))
       return x;
   };
 
+  // this warp's rounds of n results: wt, wt + NW, ...
+  auto team_rounds = [&](int n) { return (((n + 31) >> 5) - wt + NW - 1) / NW; };
+
   // H[s, r] (+)= sum over the primitive quartets in rows [p0, p1) of W_s S_r
   auto ket_contract = [&](int p0, int p1) {
     if constexpr (kRegs) {
       // the round count decides a branch: as a predicate inside the loop it was turned into
       // selects, with the FP64 instructions of all rounds executed
-      exact_rounds<KR>((mc.n_kc + 31) >> 5, [&](auto nc) {
+      exact_rounds<KR>(team_rounds(mc.n_kc), [&](auto nc) {
         constexpr int N = decltype(nc)::value;
         const R *r[N], *w[N];
         R v[N];
@@ -481,7 +489,8 @@ __global__ void __launch_bounds__(md_block(LT), md_minb<R>(LT))
         for (int u = 0; u < N; ++u) {
           r[u] = Rb + p0 * kRow + kc_r[u];
           w[u] = Rb + p0 * kRow + kc_w[u];
-          v[u] = h_valid && 32 * u + lane < mc.n_kc ? H[32 * u + lane] : R(0);
+          const int o = 32 * (wt + NW * u) + lane;
+          v[u] = h_valid && o < mc.n_kc ? H[o] : R(0);
         }
         stepped<4>(p1 - p0, [&](int p) {
 #pragma unroll
@@ -489,7 +498,7 @@ __global__ void __launch_bounds__(md_block(LT), md_minb<R>(LT))
         });
 #pragma unroll
         for (int u = 0; u < N; ++u) {
-          const int o = 32 * u + lane;
+          const int o = 32 * (wt + NW * u) + lane;
           if (o < mc.n_kc) H[o] = v[u];
         }
       });
@@ -529,11 +538,17 @@ __global__ void __launch_bounds__(md_block(LT), md_minb<R>(LT))
   // A[s', s, r] (+)= W_s' H[s, r] for the bra primitive pair with factors w
   auto bra_contract = [&](const double* w, const R* H) {
     if constexpr (kRegs) {
-      exact_rounds<BR>((mc.n_bc + 31) >> 5, [&](auto nc) {
+      const int n = team_rounds(mc.n_bc);
+      if constexpr (F32) {  // spare rounds cost less than copies of the code
 #pragma unroll
-        for (int u = 0; u < decltype(nc)::value; ++u)
-          a_reg[u] = fmar(narrow(__ldg(w + bc_w[u])), H[bc_h[u]], a_reg[u]);
-      });
+        for (int u = 0; u < BR; ++u)
+          if (u < n) a_reg[u] = fmar(narrow(__ldg(w + bc_w[u])), H[bc_h[u]], a_reg[u]);
+      } else {
+        exact_rounds<BR>(n, [&](auto nc) {
+#pragma unroll
+          for (int u = 0; u < decltype(nc)::value; ++u) a_reg[u] = fmar(__ldg(w + bc_w[u]), H[bc_h[u]], a_reg[u]);
+        });
+      }
       if constexpr (LT > 2) sync();
       return;
     }
@@ -558,7 +573,8 @@ __global__ void __launch_bounds__(md_block(LT), md_minb<R>(LT))
     sync();
   };
 
-  auto finish = [&](int4 e) {
+  auto finish = [&](int slot) {
+    const int4 e = Q[slot];
     const EriLaunch& Ls = rec(e.x);
     const int nb = e.w & 0xFFFF, nk = e.w >> 16;
     tally.prim += n_eval;
@@ -566,11 +582,13 @@ __global__ void __launch_bounds__(md_block(LT), md_minb<R>(LT))
     double* Tb = S + ly.Tb;
     double* Tk = S + ly.Tk;
     const int bra = pair_id(Ls, e.y), ket = pair_id(Ls, e.z);
+    const uint4 eo = Qo[slot];
     if (a_valid) {
       if constexpr (kRegs) {
 #pragma unroll
         for (int u = 0; u < BR; ++u) {
-          if (32 * u + lane < mc.n_bc) A[32 * u + lane] = a_reg[u];
+          const int o = 32 * (wt + NW * u) + lane;
+          if (o < mc.n_bc) A[o] = a_reg[u];
           a_reg[u] = R(0);
         }
       }
@@ -579,11 +597,11 @@ __global__ void __launch_bounds__(md_block(LT), md_minb<R>(LT))
         ++tally.q32;
         tally.p32 += n_eval;
       }
-      const double* mk = Ls.pa.md + __ldg(Ls.pa.md_off + ket);
+      const double* mk = Ls.pa.md + 4ull * eo.w;
       for (int i = 32 * wt + lane; i < mc.ket_coef; i += 32 * NW) Tk[i] = __ldg(mk + i);
       if (tb_bra != bra || tb_sys != e.x) {
         // the bra side carries (-1)^{|p|}: the sign of every second coefficient degree
-        const double* mb = Ls.pa.md + __ldg(Ls.pa.md_off + bra);
+        const double* mb = Ls.pa.md + 4ull * eo.z;
         for (int i = 32 * wt + lane; i < mc.bra_coef; i += 32 * NW) {
           const double x = __ldg(mb + i);
           Tb[i] = __hiloint2double(__double2hiint(x) ^ (__ldg(kMdCoefSign + mc.bra_coef0 + i) << 31),
@@ -628,34 +646,38 @@ __global__ void __launch_bounds__(md_block(LT), md_minb<R>(LT))
 
   // primitive quartet number pos of the stream: its queue entry, the quartet, the primitive pairs
   struct Prim {
-    int e, off, nb, nk, ib, ik;
+    int e, nb, nk, ib, ik;
     int4 q;
   };
   auto locate = [&](int pos) {
     Prim s;
     s.e = head;
-    s.off = head_off + pos;
+    int off = head_off + pos;
     s.q = Q[s.e & (kQ - 1)];
     int npq = (s.q.w & 0xFFFF) * (s.q.w >> 16);
-    while (s.off >= npq) {
-      s.off -= npq;
+    while (off >= npq) {
+      off -= npq;
       s.q = Q[++s.e & (kQ - 1)];
       npq = (s.q.w & 0xFFFF) * (s.q.w >> 16);
     }
     s.nb = s.q.w & 0xFFFF;
     s.nk = s.q.w >> 16;
-    s.ib = s.off / s.nk;
-    s.ik = s.off - s.ib * s.nk;
+    s.ib = off / s.nk;
+    s.ik = off - s.ib * s.nk;
     return s;
   };
 
   // the primitive pairs of s
   auto prims = [&](const Prim& s, const PrimPair*& pb, const PrimPair*& pk) -> const EriLaunch& {
     const EriLaunch& Ls = rec(s.q.x);
-    const int bra = pair_id(Ls, s.q.y), ket = pair_id(Ls, s.q.z);
-    pb = Ls.pa.prim + __ldg(Ls.pa.prim_off + bra) + s.ib;
-    pk = Ls.pa.prim + __ldg(Ls.pa.prim_off + ket) + s.ik;
+    const uint4 o = Qo[s.e & (kQ - 1)];
+    pb = Ls.pa.prim + o.x + s.ib;
+    pk = Ls.pa.prim + o.y + s.ik;
     return Ls;
+  };
+  // the factors of the bra primitive pair ib of the quartet in a slot
+  auto bra_factors = [&](int slot, int ib) {
+    return rec(Q[slot].x).pa.md + 4ull * Qo[slot].z + mc.bra_coef + ib * mc.bra_set;
   };
 
   // the next n (<= 32 NS, <= waiting) primitive quartets of the stream
@@ -700,7 +722,11 @@ __global__ void __launch_bounds__(md_block(LT), md_minb<R>(LT))
         for (int m = 0; m <= LT; ++m) x[32 * m] = B[m];
 #pragma unroll
         for (int i = 0; i < 3; ++i) x[32 * (LT + 1 + i)] = PQ[i];
-        if constexpr (F32) x[32 * (LT + 4)] = lam;
+        if constexpr (F32) {
+          x[32 * (LT + 4)] = lam;
+          x[32 * (LT + 5)] = __int_as_float((s.e & (kQ - 1)) | (s.ib << 6) | (s.ik << 12) |
+                                            (s.ik == s.nk - 1 ? 1 << 18 : 0) | (s.ib == s.nb - 1 ? 1 << 19 : 0));
+        }
         const unsigned dm = __ballot_sync(0xffffffffu, declined);
         if (lane == 0) {
           Xok[sub] = okm;
@@ -747,8 +773,17 @@ __global__ void __launch_bounds__(md_block(LT), md_minb<R>(LT))
         ok = (okm >> lane) & 1;
         s = Prim{};
         s.nb = s.nk = 1;
-        if (lane < ns) s = locate(32 * sub + lane);
         const R* x = X + sub * NX * 32 + lane;
+        if constexpr (F32) {
+          const int p = lane < ns ? __float_as_int(x[32 * (LT + 5)]) : 0;
+          s.e = head + (((p & (kQ - 1)) - head) & (kQ - 1));
+          s.ib = (p >> 6) & 63;
+          s.ik = (p >> 12) & 63;
+          s.nk = s.ik + ((p >> 18) & 1 ? 1 : 2);  // only what tells the last ones
+          s.nb = s.ib + ((p >> 19) & 1 ? 1 : 2);
+        } else if (lane < ns) {
+          s = locate(32 * sub + lane);
+        }
 #pragma unroll
         for (int m = 0; m <= LT; ++m) B[m] = x[32 * m];
 #pragma unroll
@@ -760,9 +795,8 @@ __global__ void __launch_bounds__(md_block(LT), md_minb<R>(LT))
         }
       }
       if (ok) {
-        const EriLaunch& Ls = rec(s.q.x);
-        const int ket = pair_id(Ls, s.q.z);
-        const double* wk = Ls.pa.md + __ldg(Ls.pa.md_off + ket) + mc.ket_coef + s.ik * mc.ket_set;
+        const int slot = s.e & (kQ - 1);
+        const double* wk = rec(Q[slot].x).pa.md + 4ull * Qo[slot].w + mc.ket_coef + s.ik * mc.ket_set;
         const int pos = __popc(okm & lt_mask);
         R* r = Rb + pos * kRow;
         for (int i = wt; i < mc.ket_set; i += NW) r[kW + i] = narrow(__ldg(wk + i));
@@ -818,17 +852,13 @@ __global__ void __launch_bounds__(md_block(LT), md_minb<R>(LT))
             lead &= lead - 1;
             const int l1 = lead ? __ffs(lead) - 1 : ns;
             const int np = first_row[u + 1] - first_row[u];
-            const int4 q = Q[__shfl_sync(0xffffffffu, s.e, l0) & (kQ - 1)];
+            const int slot = __shfl_sync(0xffffffffu, s.e, l0) & (kQ - 1), ib = __shfl_sync(0xffffffffu, s.ib, l0);
             if (np > 0) {
-              const EriLaunch& Ls = rec(q.x);
-              const int bra = pair_id(Ls, q.y);
-              bra_contract(Ls.pa.md + __ldg(Ls.pa.md_off + bra) + mc.bra_coef +
-                               __shfl_sync(0xffffffffu, s.ib, l0) * mc.bra_set,
-                           H + (u - t0) * GL);
+              bra_contract(bra_factors(slot, ib), H + (u - t0) * GL);
               a_valid = true;
               n_eval += np;
             }
-            if ((last_q >> (l1 - 1)) & 1) finish(q);
+            if ((last_q >> (l1 - 1)) & 1) finish(slot);
           }
           __syncwarp();
         }
@@ -844,26 +874,23 @@ __global__ void __launch_bounds__(md_block(LT), md_minb<R>(LT))
             n_eval += p1 - p0;
           }
           if ((last_k >> (l1 - 1)) & 1) {
-            const int4 q = Q[__shfl_sync(0xffffffffu, s.e, l0) & (kQ - 1)];
+            const int slot = __shfl_sync(0xffffffffu, s.e, l0) & (kQ - 1), ib = __shfl_sync(0xffffffffu, s.ib, l0);
             if (h_valid) {
-              const EriLaunch& Ls = rec(q.x);
-              const int bra = pair_id(Ls, q.y);
-              bra_contract(Ls.pa.md + __ldg(Ls.pa.md_off + bra) + mc.bra_coef +
-                               __shfl_sync(0xffffffffu, s.ib, l0) * mc.bra_set,
-                           H);
+              bra_contract(bra_factors(slot, ib), H);
               a_valid = true;
               h_valid = false;
             }
-            if ((last_q >> (l1 - 1)) & 1) finish(q);
+            if ((last_q >> (l1 - 1)) & 1) finish(slot);
           }
         }
       }
       if (32 * (sub + 1) >= n) {  // the stream's new head: after the last lane
         const int l = ns - 1;
-        const int e_last = __shfl_sync(0xffffffffu, s.e, l), off_last = __shfl_sync(0xffffffffu, s.off, l);
+        const int e_last = __shfl_sync(0xffffffffu, s.e, l);
+        const int ib_last = __shfl_sync(0xffffffffu, s.ib, l), ik_last = __shfl_sync(0xffffffffu, s.ik, l);
         const bool done = (last_q >> l) & 1;
         head = done ? e_last + 1 : e_last;
-        head_off = done ? 0 : off_last + 1;
+        head_off = done ? 0 : ib_last * (Q[e_last & (kQ - 1)].w >> 16) + ik_last + 1;
       }
     }
     waiting -= n;
@@ -972,7 +999,13 @@ __global__ void __launch_bounds__(md_block(LT), md_minb<R>(LT))
         }
       }
       const unsigned m = __ballot_sync(0xffffffffu, keep);
-      if (keep && wt == 0) Q[(tail + __popc(m & lt_mask)) & (kQ - 1)] = make_int4(sys, bra_s, ket_s, nb | (nk << 16));
+      if (keep && wt == 0) {
+        const EriLaunch& Ls = rec(sys);
+        const int slot = (tail + __popc(m & lt_mask)) & (kQ - 1), bra = pair_id(Ls, bra_s), ket = pair_id(Ls, ket_s);
+        Q[slot] = make_int4(sys, bra_s, ket_s, nb | (nk << 16));
+        Qo[slot] = make_uint4(__ldg(Ls.pa.prim_off + bra), __ldg(Ls.pa.prim_off + ket),
+                              (unsigned)(__ldg(Ls.pa.md_off + bra) >> 2), (unsigned)(__ldg(Ls.pa.md_off + ket) >> 2));
+      }
       tail += __popc(m);
       waiting += __reduce_add_sync(0xffffffffu, keep ? nb * nk : 0);
       sync();

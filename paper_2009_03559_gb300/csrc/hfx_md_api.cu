@@ -101,7 +101,7 @@ __global__ void k_md_size(int n, const int* __restrict__ pcls, const int* __rest
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= n) return;
   const MdPairInfo& t = info.t[pcls[c]];
-  size[c] = t.n_coef + (long long)t.n_set * cap[c];
+  size[c] = (t.n_coef + (long long)t.n_set * cap[c] + 3) & ~3ll;  // the engine counts in fours
 }
 
 // one warp per pair
