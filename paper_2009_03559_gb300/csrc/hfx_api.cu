@@ -329,6 +329,7 @@ extern "C" int hfx_build_pairs(hfx_ctx* ctx) {
   {
     EriLaunch L = base_launch(ctx);
     int start = 0;
+    bool follows = false;
     for (int pc = 0; pc < 6; ++pc) {
       if (cnt[pc] > 0) {
         const int cls = pc * (pc + 1) / 2 + pc;
@@ -337,7 +338,9 @@ extern "C" int hfx_build_pairs(hfx_ctx* ctx) {
         L.diag_n = cnt[pc];
         L.diag_Q = ctx->d_Q;
         const int gs = eri_group_size();
-        CK(eri_launch(L, cls, 1, grid_for(ctx, cls, 1, cnt[pc], gs), s, gs, 0, false));
+        const int grid = grid_for(ctx, cls, 1, cnt[pc], gs);
+        CK(eri_launch(L, cls, 1, grid, s, gs, 0, false, follows));
+        follows = eri_overlap(gs, cnt[pc], (long long)grid * eri_groups_per_block(cls, gs));
       }
       start += cnt[pc];
     }
@@ -618,6 +621,7 @@ extern "C" int hfx_build_K_periodic(hfx_ctx* ctx, int n_R, const int* R_cells, c
       sh[i] = G[0] * ctx->lattice[i] + G[1] * ctx->lattice[3 + i] + G[2] * ctx->lattice[6 + i];
     L.KG = K_G + (size_t)g * nbf * nbf;
     CK(cudaMemsetAsync(ctx->d_work, 0, 64 * sizeof(unsigned long long), s));
+    bool follows = false;
     for (int cp = 0; cp < 21; ++cp) {
       if (ctx->cls_q[cp] == 0) continue;
       int hi = 0;
@@ -642,7 +646,8 @@ extern "C" int hfx_build_K_periodic(hfx_ctx* ctx, int n_R, const int* R_cells, c
           L.shift[i] = rev ? -sh[i] : sh[i];
         }
         L.work = ctx->d_work + cp + 21 * rev;
-        CK(eri_launch(L, cp, 0, grid, s, gs, 3, false));
+        CK(eri_launch(L, cp, 0, grid, s, gs, 3, false, follows));
+        follows = eri_overlap(gs, L.q_count, (long long)grid * eri_groups_per_block(cp, gs));
       }
     }
   }
@@ -714,6 +719,7 @@ static int build_K_impl(hfx_ctx* ctx, const double* P, double* K, int ld, int pa
   L.dist = ctx->d_dist;
   L.Qs = ctx->d_Qs;
   if (ctx->timing) L.busy = ctx->d_busy;
+  bool follows = false;  // this launch may start before the one before it has ended
   for (int cp = 0; cp < 21; ++cp) {
     ctx->class_launched[cp] = false;
     if (ctx->cls_q[cp] == 0) continue;
@@ -740,7 +746,10 @@ static int build_K_impl(hfx_ctx* ctx, const double* P, double* K, int ld, int pa
     ctx->gs_used[cp] = gs;
     ctx->streams_used[cp] = gs == 32 ? eri_streams(cp, ctx->streams_override[cp]) : 0;
     const long long items = ctx->opt.schedule == HFX_SCHED_PAIR ? (L.row_end - L.row_begin) : L.q_count;
-    if (ctx->timing) CK(cudaEventRecord(ctx->ev[2 + 2 * cp], s));
+    if (ctx->timing) {
+      CK(cudaEventRecord(ctx->ev[2 + 2 * cp], s));
+      follows = false;  // class times are those of launches by themselves
+    }
     for (int pass = 0; pass < (L.fp32_ok ? 2 : 1); ++pass) {
       const int prec = L.fp32_ok ? 1 + pass : 0;
       // the FP32 pass runs on whole warps in every class unless the caller fixed the class's group size
@@ -748,7 +757,8 @@ static int build_K_impl(hfx_ctx* ctx, const double* P, double* K, int ld, int pa
       const int grid = grid_for(ctx, cp, 0, items, gsp, prec);
       L.chunk = eri_chunk(gsp, L.q_count, (long long)grid * eri_groups_per_block(cp, gsp));
       L.work = ctx->d_work + cp + 21 * pass;
-      CK(eri_launch(L, cp, 0, grid, s, gsp, prec, false));
+      CK(eri_launch(L, cp, 0, grid, s, gsp, prec, false, follows));
+      follows = !ctx->timing && eri_overlap(gsp, L.q_count, (long long)grid * eri_groups_per_block(cp, gsp));
     }
     if (ctx->timing) CK(cudaEventRecord(ctx->ev[3 + 2 * cp], s));
     ctx->class_launched[cp] = true;

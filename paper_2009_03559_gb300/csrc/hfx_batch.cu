@@ -248,6 +248,7 @@ cudaError_t bw_enqueue(const BatchWork& w, cudaStream_t s, const Branches* br = 
   }
   std::sort(order, order + 21, [&](int a, int b) { return cost[a] > cost[b]; });
   double load[kBranches] = {};
+  bool follows[kBranches] = {};  // the branch's next launch may start before the last has ended
   if (nb > 1) {
     if ((e = cudaEventRecord(br->fork, s)) != cudaSuccess) return e;
     for (int i = 0; i < nb - 1; ++i)
@@ -264,7 +265,10 @@ cudaError_t bw_enqueue(const BatchWork& w, cudaStream_t s, const Branches* br = 
     for (int pass = 0; pass < (w.fp32_class[cp] ? 2 : 1); ++pass) {
       const EriLaunch L = bw_class_launch(w, cp, pass);
       const int prec = bw_prec(w, cp, pass);
-      e = eri_launch(L, cp, 0, bw_grid(w, cp, w.total[cp], prec), bs, bw_gs(w, cp, prec), prec, true);
+      const int gs = bw_gs(w, cp, prec);
+      const int grid = bw_grid(w, cp, w.total[cp], prec);
+      e = eri_launch(L, cp, 0, grid, bs, gs, prec, true, follows[bi]);
+      follows[bi] = eri_overlap(gs, w.total[cp], (long long)grid * eri_groups_per_block(cp, gs));
       if (e != cudaSuccess) return e;
     }
   }

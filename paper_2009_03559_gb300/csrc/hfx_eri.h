@@ -21,6 +21,8 @@ bool eri_streams_valid(int cls, int streams);
 int eri_groups_per_block(int cls, int gs);
 // quartets per claim of the dynamic schedule, for a list of n_quartets and n_groups groups
 int eri_chunk(int gs, long long n_quartets, long long n_groups);
+// whether the next class launch may overlap this one
+bool eri_overlap(int gs, long long n_quartets, long long n_groups);
 
 // The Hermite engine (quartets on whole warps, hfx_md.cuh; f32: the FP32 pass) and its pair data.
 // Kinds of launch: one system, a batch of systems, a lattice sum, the Schwarz diagonal.
@@ -29,7 +31,8 @@ size_t md_smem_bytes(int cls, bool f32);
 cudaError_t md_prepare();
 int md_blocks_per_sm(int cls, int kind, bool f32);
 int md_teams_per_block(int cls);
-cudaError_t md_launch(const EriLaunch& L, int cls, int kind, int prec, bool f32, int grid, cudaStream_t stream);
+cudaError_t md_launch(const EriLaunch& L, int cls, int kind, int prec, bool f32, int grid, cudaStream_t stream,
+                      bool overlap);
 cudaError_t launch_md_size(int n, const int* pcls, const int* cap, long long* size, cudaStream_t s);
 cudaError_t launch_md_fill(int n, const int* pcls, const double* AB, const int* pp_off, const int* pp_n,
                            const PrimPair* pp, const long long* md_off, double* md, cudaStream_t s);
@@ -37,6 +40,8 @@ cudaError_t launch_md_fill(int n, const int* pcls, const double* AB, const int* 
 }  // namespace hfx
 
 namespace hfx {
+// overlap: the launch before it on the stream is another class or pass of the same build, and this
+// one need not wait for it (warps; the thread kernel always waits)
 cudaError_t eri_launch(const EriLaunch& L, int cls, int mode, int grid, cudaStream_t stream, int gs, int prec,
-                       bool batch);
+                       bool batch, bool overlap = false);
 }

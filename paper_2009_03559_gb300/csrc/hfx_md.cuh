@@ -390,6 +390,8 @@ __host__ __device__ constexpr int md_minb(int Lt) {
 template <int LT, int KIND, typename R>
 __global__ void __launch_bounds__(md_block(LT), md_minb<R>(LT))
     eri_md_kernel(const __grid_constant__ EriLaunch L, const __grid_constant__ MdLayout ly) {
+  // the next class's launch may start (see md_launch): nothing it reads comes from this one
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   extern __shared__ __align__(16) double smem[];
   constexpr bool F32 = sizeof(R) == 4;
   constexpr int NW = md_team(LT), kQ = kMdQueue, kTeams = md_block(LT) / (32 * NW);
@@ -1015,6 +1017,8 @@ __global__ void __launch_bounds__(md_block(LT), md_minb<R>(LT))
   }
   if (KIND != MD_DIAG && lane == 0 && wt == 0) flush_tally(L, tally);
   record_busy(L, t0);
+  // a launch completes after the one before it, so that what follows the last waits for all
+  asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 }  // namespace hfx

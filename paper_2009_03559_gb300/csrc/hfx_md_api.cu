@@ -72,14 +72,29 @@ int md_blocks_per_sm(int cls, int kind, bool f32) {
   return n > 0 ? n : 1;
 }
 
-cudaError_t md_launch(const EriLaunch& L0, int cls, int kind, int prec, bool f32, int grid, cudaStream_t stream) {
+// overlap: the launch may start while the one before it on the stream (a class launch of the same
+// build) still runs.  The launches of a build are independent (their K updates are atomic, their
+// work counters apart), so the last quartets of one class, with most SMs idle, run beside the
+// first of the next.  Each kernel lets its successor start at once and itself ends only after its
+// predecessor has (griddepcontrol), so the build's last launch ends after all of them.
+cudaError_t md_launch(const EriLaunch& L0, int cls, int kind, int prec, bool f32, int grid, cudaStream_t stream,
+                      bool overlap) {
   EriLaunch L = L0;
   L.mc = kMdClass[cls];
   L.prec = prec == PREC_PERIODIC ? PREC_FP64 : prec;
   MdLayout ly = layout_of(cls, f32);
   void* args[] = {(void*)&L, (void*)&ly};
-  return cudaLaunchKernel(md_kernel(L.mc.Lt, kind, f32), dim3(grid), dim3(md_block(kMdClass[cls].Lt)), args,
-                          md_smem_bytes(cls, f32), stream);
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = overlap ? 1 : 0;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(md_block(L.mc.Lt));
+  cfg.dynamicSmemBytes = md_smem_bytes(cls, f32);
+  cfg.stream = stream;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelExC(&cfg, md_kernel(L.mc.Lt, kind, f32), args);
 }
 
 // ---------------------------------------------------------------------------
