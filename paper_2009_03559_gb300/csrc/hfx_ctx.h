@@ -84,7 +84,7 @@ struct hfx_ctx {
       *p = nullptr;
       *cap = 0;
     }
-    const int r = alloc(p, n);
+    const int r = alloc(p, n, false, true);
     if (r == HFX_OK) *cap = n;
     return r;
   }
@@ -101,20 +101,45 @@ struct hfx_ctx {
     err = std::string(what) + ": " + cudaGetErrorString(e);
     return e == cudaErrorMemoryAllocation ? HFX_ERR_OOM : HFX_ERR_CUDA;
   }
+  // Tables up to kSlabPiece bytes share slabs of kSlab bytes: a new context and its pair list make
+  // some fifty tables, and a cudaMalloc and cudaFree for each took a fifth of a small system's
+  // first build.  A slab lives as long as its scope; own: an allocation of its own in any case.
+  static constexpr size_t kSlab = 1 << 20, kSlabPiece = 1 << 17;
+  struct Slab {
+    char* p = nullptr;
+    size_t used = 0;
+  };
+  Slab slabs[2];  // of the context, of the pair list
   template <class T>
-  int alloc(T** p, size_t n, bool pair_scope = false) {
+  int alloc(T** p, size_t n, bool pair_scope = false, bool own = false) {
     *p = nullptr;
     if (n == 0) n = 1;
     if (hfx::alloc_fault_due()) return fail(HFX_ERR_OOM, "cudaMalloc: injected allocation failure");
-    cudaError_t e = cudaMalloc((void**)p, n * sizeof(T));
+    const size_t need = (n * sizeof(T) + 255) & ~(size_t)255;
+    const bool piece = !own && need <= kSlabPiece;
+    Slab& s = slabs[pair_scope];
+    if (piece && s.p && s.used + need <= kSlab) {
+      *p = (T*)(s.p + s.used);
+      s.used += need;
+      return HFX_OK;
+    }
+    const size_t size = piece ? kSlab : n * sizeof(T);
+    void* q = nullptr;
+    cudaError_t e = cudaMalloc(&q, size);
     if (e != cudaSuccess) return cuda_fail("cudaMalloc", e);
-    (pair_scope ? pair_allocs : allocs).push_back(*p);
-    (pair_scope ? pair_bytes : bytes) += n * sizeof(T);
+    (pair_scope ? pair_allocs : allocs).push_back(q);
+    (pair_scope ? pair_bytes : bytes) += size;
+    *p = (T*)q;
+    if (piece) {
+      s.p = (char*)q;
+      s.used = need;
+    }
     return HFX_OK;
   }
   void free_pairs() {
     for (void* p : pair_allocs) cudaFree(p);
     pair_allocs.clear();
+    slabs[1] = Slab();
     pair_bytes = 0;
     pairs_ready = false;
   }

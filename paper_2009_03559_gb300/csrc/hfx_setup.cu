@@ -48,28 +48,36 @@ __device__ __forceinline__ void put_boys_row(double* row, double x, const double
   r[3] = 0.f;
 }
 
-__global__ void k_boys_table(double* __restrict__ tab) {
-  const int g = blockIdx.x * blockDim.x + threadIdx.x;
-  if (g >= kBoysRows + kBoysTailRows) return;
+// blocks [0, tail_block): a thread per row below 60; then a thread per order and tail row.  The series
+// multiplies by reciprocals that the block makes once: with a division per term, and all orders of a
+// tail row on one thread, the table took longer than the rest of a small system's set-up.
+constexpr int kBoysBlock = 128, kBoysTerms = 512;
+constexpr int kBoysTailBlock = (kBoysRows + kBoysBlock - 1) / kBoysBlock;
+__global__ void __launch_bounds__(kBoysBlock) k_boys_table(double* __restrict__ tab) {
   double f[6];
-  if (g >= kBoysRows) {
-    const double t = 1.0 + (double)(g - kBoysRows) / kBoysTailPerUnit;
+  if (blockIdx.x >= kBoysTailBlock) {
+    const int i = (blockIdx.x - kBoysTailBlock) * blockDim.x + threadIdx.x, L = i / kBoysTailRows;
+    if (L > kMaxLt) return;
+    const int g = i - L * kBoysTailRows;
+    const double t = 1.0 + (double)g / kBoysTailPerUnit;
     double c = 0.886226925452758014;  // (2L-1)!!/2^{L+1} sqrt(pi)
-    for (int L = 0; L <= kMaxLt; ++L) {
-      const double a = L + 0.5;
-      f[0] = c / sqrt(t);
-      for (int m = 0; m < L; ++m) f[0] /= t;
-      for (int k = 1; k < 6; ++k) f[k] = -f[k - 1] * (a + k - 1) / (k * t);
-      put_boys_row(tab + (size_t)L * kBoysTableLen + (size_t)g * kBoysRowLen, t, f, 0.0);
-      c *= a;
-    }
+    for (int m = 0; m < L; ++m) c *= m + 0.5;
+    f[0] = c / sqrt(t);
+    for (int m = 0; m < L; ++m) f[0] /= t;
+    for (int k = 1; k < 6; ++k) f[k] = -f[k - 1] * (L + k - 0.5) / (k * t);
+    put_boys_row(tab + (size_t)L * kBoysTableLen + (size_t)(kBoysRows + g) * kBoysRowLen, t, f, 0.0);
     return;
   }
-  const double x = (double)g / kBoysPerUnit;
   const int M = 15;
-  double term = 1.0 / (2 * M + 1), sum = term;
-  for (int k = 1; k < 4000; ++k) {
-    term *= 2.0 * x / (2 * M + 2 * k + 1);
+  __shared__ double rcp[kBoysTerms];  // 1 / (2 M + 2 k + 1)
+  for (int k = threadIdx.x; k < kBoysTerms; k += blockDim.x) rcp[k] = 1.0 / (2 * M + 2 * k + 1);
+  __syncthreads();
+  const int g = blockIdx.x * blockDim.x + threadIdx.x;
+  if (g >= kBoysRows) return;
+  const double x = (double)g / kBoysPerUnit;
+  double term = rcp[0], sum = term;
+  for (int k = 1; k < kBoysTerms; ++k) {  // (some 250 terms at x = 60)
+    term *= 2.0 * x * rcp[k];
     sum += term;
     if (term < 1e-18 * sum) break;
   }
@@ -610,7 +618,7 @@ cudaError_t launch_pmax_blocks(int n_R, int ns, int nbf, const int* bf_off, cons
 }
 
 cudaError_t launch_boys_table(double* tab, cudaStream_t s) {
-  k_boys_table<<<nblk(kBoysRows + kBoysTailRows, 128), 128, 0, s>>>(tab);
+  k_boys_table<<<kBoysTailBlock + nblk((kMaxLt + 1) * kBoysTailRows, kBoysBlock), kBoysBlock, 0, s>>>(tab);
   return cudaGetLastError();
 }
 
