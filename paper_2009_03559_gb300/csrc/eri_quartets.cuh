@@ -171,7 +171,7 @@ __device__ __forceinline__ void digest_per(const EriClassInfo& ci, const double*
 
 // Per-thread tallies of one kernel, added to the launch's counters once at the end.
 struct Tally {
-  unsigned long long prim = 0, quart = 0, skip = 0, q32 = 0, p32 = 0;
+  unsigned long long prim = 0, quart = 0, skip = 0, q32 = 0, p32 = 0, run = 0;
 };
 
 // The quartet ranges a warp of the thread kernel works on.  Static schedules: one range (group_range).
@@ -223,6 +223,7 @@ __device__ __forceinline__ void flush_tally(const EriLaunch& L, const Tally& t) 
   atomicAdd(L.counters + 2, t.skip);
   atomicAdd(L.counters + 3, t.q32);
   atomicAdd(L.counters + 4, t.p32);
+  atomicAdd(L.counters + 5, t.run);
 }
 
 }  // namespace hfx

@@ -207,6 +207,20 @@ class MdClass:
         L = "spd"
         return "(" + "|".join("".join(L[x] for x in PAIR_CLASSES[c]) for c in (self.hi, self.lo)) + ")"
 
+    def flops(self):
+        """Add/mul 1, fma 2: per primitive quartet (Hermite recursion, ket contraction), per run of a
+        bra primitive pair (bra contraction), per quartet (transformations and digest, digest alone)."""
+        r = 0
+        for o in range(1, self.Lt + 1):
+            for t in monos(o):
+                n = t[0] or t[1] or t[2]
+                r += (self.Lt - o + 1) * (1 if n == 1 else (3 if n - 1 in (3, 5, 6, 7) else 2))
+        terms = self.n_rows * sum(len(PAIRS[self.lo].T[f]) for f in range(self.ncd))
+        terms += self.ncd * sum(len(PAIRS[self.hi].T[f]) for f in range(self.nab))
+        na, nb, nc, nd = self.dims
+        dig = 8 * na * nb * nc * nd + (na + nb) * (nc + nd)
+        return r + 2 * len(self.kc), 2 * len(self.bc), 2 * terms + dig, dig
+
     def r_ops(self):
         """FP64 instructions of the Hermite recursion, x last (2 S is an exponent increment)."""
         n = 0
@@ -286,6 +300,11 @@ def emit(w):
     arr("kMdCoefSign", "unsigned char", sign)
     arr("kMdTermMono", "unsigned char", [m for m, _ in poly])
     arr("kMdTermVal", "double", [v for _, v in poly], hexa=False)
+    w("// flops (add/mul 1, fma 2) per primitive quartet, per bra run, per quartet, of it in the digest\n")
+    w("static const int kMdFlops[HFX_N_CLASSES][4] = {\n")
+    for c in cl:
+        w(f"  {{{', '.join(map(str, c.flops()))}}},\n")
+    w("};\n\n")
     w("static const MdPairInfo kMdPair[6] = {\n")
     for (off, n, ns), p in zip(info, PAIRS):
         st = [(k + h) | (i << 4) | (j << 8) for k, i, j, h in p.sets] + [0] * (14 - len(p.sets))

@@ -199,6 +199,11 @@ static double setup_flops(int E, int F, int Lt, bool erfc) {
   if (F > 0) f += 4;   // W - Q, 3/(2(p+q))
   return f;
 }
+// The same for the Hermite engine's md_setup: s, 1/sqrt(s), rho, P - Q, R^2, T, prefactor, Boys(T),
+// pref (2 rho)^L, the a and B chains; with kappa: its root, kappa T, Boys(kappa T), the c chain.
+static double md_setup_flops(int Lt, bool erfc) {
+  return 1 + 5 + 3 + 3 + 5 + 1 + 2 + 13 + 4 + 1 + 4.0 * Lt + (erfc ? 1 + 5 + 3 + 13 + 2 + 2 + 3.0 * Lt : 0.0);
+}
 // a primitive quartet dropped at kappa T >= table end costs the set-up up to that test
 static double skip_flops() { return 35 + 7 + 1 + 1; }
 
@@ -836,18 +841,24 @@ extern "C" int hfx_get_stats(hfx_ctx* ctx, hfx_stats* out) {
       st.prim_quartets_class[cp] = (int64_t)c[0];
       st.quartets_evaluated_class[cp] = (int64_t)c[1];
       st.quartets_fp32_class[cp] = (int64_t)c[3];
-      // FP64: the set-up and the recurrences of FP64 quartets, every digest; FP32: the set-up
-      // and the recurrences of FP32 quartets (the few primitive quartets whose Boys step the
-      // FP32 set-up declines are set up in FP64 but counted here as FP32)
-      const double su = setup_flops(ci.E, ci.F, ci.Lt, ctx->opt.omega > 0.0);
-      const double f64 = (double)(c[0] - c[4]) * (su + ci.flops_prim) +
-                         (double)(c[1] - c[3]) * (ci.flops_quartet - ci.flops_digest) +
-                         (double)c[1] * ci.flops_digest + (double)c[2] * skip_flops();
-      const double f32 = (double)c[4] * (su + ci.flops_prim) + (double)c[3] * (ci.flops_quartet - ci.flops_digest);
+      // FP64: the set-up, recursion and contraction of FP64 primitive quartets, every transformation
+      // (in the thread kernel: of FP64 quartets) and digest; FP32: the set-up and the recursion and
+      // contraction of FP32 primitive quartets (the few whose Boys step the FP32 set-up declines are
+      // set up in FP64 but counted here as FP32)
+      const bool md = ctx->gs_used[cp] != 1;
+      const double su = md ? md_setup_flops(ci.Lt, ctx->opt.omega > 0.0)
+                           : setup_flops(ci.E, ci.F, ci.Lt, ctx->opt.omega > 0.0);
+      const int* mf = md_flops_host()[cp];
+      const double prim = md ? mf[0] : ci.flops_prim, quart = md ? mf[2] : ci.flops_quartet;
+      const double dig = md ? mf[3] : ci.flops_digest, runs = md ? (double)c[5] * mf[1] : 0.0;
+      const double part32 = c[0] ? (double)c[4] / (double)c[0] : 0.0, q64 = md ? (double)c[1] : (double)(c[1] - c[3]);
+      const double f64 = (double)(c[0] - c[4]) * (su + prim) + (1.0 - part32) * runs + q64 * (quart - dig) +
+                         (double)c[1] * dig + (double)c[2] * skip_flops();
+      const double f32 = (double)c[4] * (su + prim) + part32 * runs + ((double)c[1] - q64) * (quart - dig);
       st.flops_class[cp] = f64 + f32;
       fl += f64;
       fl32 += f32;
-      st.flops_recurrence_class[cp] = (double)c[0] * ci.flops_prim + (double)c[1] * ci.flops_quartet;
+      st.flops_recurrence_class[cp] = (double)c[0] * prim + runs + (double)c[1] * quart;
       flr += st.flops_recurrence_class[cp];
       nsp += (double)c[0] * (ctx->opt.omega > 0.0 ? 2.0 : 1.0) + (double)c[2];
     }

@@ -13,8 +13,9 @@ bool alloc_fault_due();
 }  // namespace hfx
 
 // device counters per class: primitive quartets evaluated, quartets evaluated, primitive
-// quartets dropped at the Boys step, quartets in FP32, primitive quartets in FP32
-constexpr int kNCnt = 5;
+// quartets dropped at the Boys step, quartets in FP32, primitive quartets in FP32, runs of a bra
+// primitive pair (Hermite engine)
+constexpr int kNCnt = 6;
 
 struct hfx_ctx {
   cudaStream_t stream = nullptr;

@@ -44,6 +44,8 @@ struct MdPairInfo {
 };
 extern const MdClassInfo* md_class_host();
 extern const MdPairInfo* md_pair_host();
+// per class: flops per primitive quartet, per run of a bra primitive pair, per quartet, in its digest
+extern const int (*md_flops_host())[4];
 
 // ---------------------------------------------------------------------------
 // Boys function tables, one per order L = 0..kMaxLt, with F_m(x) = int_0^1 u^{2m} exp(-x u^2) du.

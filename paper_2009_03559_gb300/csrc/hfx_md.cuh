@@ -267,15 +267,17 @@ __host__ __device__ constexpr int md_block(int Lt) { return Lt <= 4 ? 64 : 32 * 
 // The FP32 pass of a mixed-precision class runs the same steps with the set-up, the Hermite
 // recursion and both contractions in FP32 (the transformations, which replace the horizontal
 // recurrences and the spherical step, and the digest in FP64).  A team sets up kSub32 times 32
-// primitive quartets before it contracts them, so that those whose Boys step the FP32 set-up
-// declines (a few per cent) are set up in FP64 together: one FP64 set-up per 128 primitive
-// quartets, not one per 32.  (6 and 8 times 32: fewer FP64 set-ups, but their shared memory costs
-// resident warps, 64-atom mixed build 1153 -> 1185 and 1221 ms.)
-constexpr int kSub32 = 4;
+// primitive quartets before it contracts them (at least its warps' 32 each), so that those whose
+// Boys step the FP32 set-up declines (a few per cent) are set up in FP64 together and not in every
+// 32.  More of them save FP64 set-ups and cost shared memory, hence resident warps (64-atom mixed
+// build: 2 times 1095 ms, 4 times 1104, 6 times 1185, 8 times 1221).
+constexpr int kSub32 = 2;
 // 32s of primitive quartets set up together; whether their set-up passes through shared memory;
 // its values per primitive quartet: base values, P - Q (in FP32 times lam, lam, and where it belongs)
 template <typename R>
-__host__ __device__ constexpr int md_sub(int Lt) { return sizeof(R) == 4 ? kSub32 : md_team(Lt); }
+__host__ __device__ constexpr int md_sub(int Lt) {
+  return sizeof(R) == 4 && kSub32 > md_team(Lt) ? kSub32 : md_team(Lt);
+}
 template <typename R>
 __host__ __device__ constexpr int md_xval(int Lt) { return sizeof(R) == 4 ? Lt + 6 : Lt + 4; }
 
@@ -317,7 +319,7 @@ MdLayout md_layout(const MdClassInfo& c, const MdPairInfo& b, const MdPairInfo& 
   l.X = l.Q + 4 * kMdQueue;
   const int ns = md_sub<R>(c.Lt);
   // the values of 32 lanes; the accepted and declined masks; the team's claim
-  l.size = l.X + (ns > 1 ? mem(ns * md_xval<R>(c.Lt) * 32) + ns + 2 : 0);
+  l.size = even(l.X + (ns > 1 ? mem(ns * md_xval<R>(c.Lt) * 32) + ns + 2 : 0));  // 16-byte entries in Q
   return l;
 }
 
@@ -539,6 +541,7 @@ __global__ void __launch_bounds__(md_block(LT), md_minb<R>(LT))
 
   // A[s', s, r] (+)= W_s' H[s, r] for the bra primitive pair with factors w
   auto bra_contract = [&](const double* w, const R* H) {
+    ++tally.run;
     if constexpr (kRegs) {
       const int n = team_rounds(mc.n_bc);
       if constexpr (F32) {  // spare rounds cost less than copies of the code

@@ -7,6 +7,7 @@ namespace hfx {
 
 const MdClassInfo* md_class_host() { return kMdClass; }
 const MdPairInfo* md_pair_host() { return kMdPair; }
+const int (*md_flops_host())[4] { return kMdFlops; }
 
 const void* md_kernel_l0(int kind, bool f32);
 const void* md_kernel_l1(int kind, bool f32);
