@@ -74,6 +74,41 @@ extern "C" int hfx_init_basis(hfx_ctx** out, int n_atoms, const double* xyz, int
   return init_basis_impl(out, n_atoms, xyz, n_shells, shell_atom, shell_l, shell_nprim, alpha, coef, opt, stream);
 }
 
+// Quartet classes whose FP32 pass stays in FP32's range.  A Hermite integral of order up to L is at
+// most C_ab C_cd (2 rho)^{L/2} / sqrt(p+q) <= f_ab f_cd with f_ab = C_ab p^{(L-1)/4} (rho <= sqrt(pq)/2)
+// and C_ab ~ w_a w_b / p, w = (8 alpha)^{(2l+3)/4} for a normalised shell; f grows with both exponents
+// (for L < 5 after p^{-z} <= (4ab)^{-z/2}), so the extremes of the shells' exponents bound it.  1e34 and 1e-22
+// leave room for contraction weights, and for integrals far below the largest of their quartet.
+// (d shells up to 7e3 in (dd|dd), p shells up to 1e8 in (pp|pp); beyond, the class runs in FP64.)
+static int fp32_range_mask(int n_shells, const int* l, const int* nprim, const double* alpha) {
+  double lo[3] = {1e300, 1e300, 1e300}, hi[3] = {0.0, 0.0, 0.0};
+  for (int s = 0, k = 0; s < n_shells; ++s)
+    for (int i = 0; i < nprim[s]; ++i, ++k) {
+      lo[l[s]] = std::min(lo[l[s]], alpha[k]);
+      hi[l[s]] = std::max(hi[l[s]], alpha[k]);
+    }
+  const int pl[6][2] = {{0, 0}, {1, 0}, {1, 1}, {2, 0}, {2, 1}, {2, 2}};
+  int mask = 0;
+  for (int b = 0; b < 6; ++b)
+    for (int k = 0; k <= b; ++k) {
+      const int L = pl[b][0] + pl[b][1] + pl[k][0] + pl[k][1];
+      const double z = (L - 5) / 4.0;
+      auto size = [&](const double* a) {  // log10 of the bound, all exponents at a[l]
+        double v = 0.0;
+        for (const int* p : {pl[b], pl[k]}) {
+          const double x = a[p[0]], y = a[p[1]];
+          v += 0.75 + 0.25 * (2 * p[0] + 3) * std::log10(8.0 * x) + 0.25 * (2 * p[1] + 3) * std::log10(8.0 * y) +
+               (z >= 0.0 ? z * std::log10(x + y) : 0.5 * z * (std::log10(4.0 * x) + std::log10(y)));
+        }
+        return v;
+      };
+      bool present = true;
+      for (const int* p : {pl[b], pl[k]}) present = present && hi[p[0]] > 0.0 && hi[p[1]] > 0.0;
+      if (!present || (size(hi) < 34.0 && size(lo) > -22.0)) mask |= 1 << (b * (b + 1) / 2 + k);
+    }
+  return mask;
+}
+
 static int init_basis_impl(hfx_ctx** out, int n_atoms, const double* xyz, int n_shells, const int* shell_atom,
                            const int* shell_l, const int* shell_nprim, const double* alpha, const double* coef,
                            const hfx_options* opt, void* stream, bool periodic) {
@@ -139,6 +174,7 @@ static int init_basis_impl(hfx_ctx** out, int n_atoms, const double* xyz, int n_
   ctx->n_bf = nb;
   ctx->n_prim = np;
   ctx->h_l.assign(shell_l, shell_l + n_shells);
+  ctx->fp32_range = fp32_range_mask(n_shells, shell_l, shell_nprim, alpha);
   cudaDeviceGetAttribute(&ctx->n_sm, cudaDevAttrMultiProcessorCount, dev);
   auto bail = [&](int code) {
     g_init_err = ctx->err;
@@ -746,7 +782,7 @@ static int build_K_impl(hfx_ctx* ctx, const double* P, double* K, int ld, int pa
     // mixed precision: a class allowed FP32 runs two passes over its quartet list, the
     // quartets that stay FP64 then those whose recurrences run in FP32, each with a kernel
     // compiled for its precision alone (registers, hence resident warps, of its own)
-    L.fp32_ok = mixed && ((ctx->opt.fp32_class_mask >> cp) & 1);
+    L.fp32_ok = mixed && ((ctx->fp32_mask() >> cp) & 1);
     const int gs = ctx->gs_override[cp] ? ctx->gs_override[cp] : eri_group_size();
     ctx->gs_used[cp] = gs;
     ctx->streams_used[cp] = gs == 32 ? eri_streams(cp, ctx->streams_override[cp]) : 0;

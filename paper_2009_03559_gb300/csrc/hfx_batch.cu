@@ -100,7 +100,7 @@ void bw_fill(BatchWork& w, hfx_ctx* const* ctxs, int n, double* const* pmax, dou
   w.mixed = false;
   for (int cp = 0; cp < 21; ++cp) {
     w.fp32_class[cp] = false;
-    for (int s = 0; s < n; ++s) w.fp32_class[cp] = w.fp32_class[cp] || (mixed && ((ctxs[s]->opt.fp32_class_mask >> cp) & 1));
+    for (int s = 0; s < n; ++s) w.fp32_class[cp] = w.fp32_class[cp] || (mixed && ((ctxs[s]->fp32_mask() >> cp) & 1));
     w.mixed = w.mixed || w.fp32_class[cp];
   }
   for (int cp = 0; cp < 21; ++cp) {
@@ -131,7 +131,7 @@ void bw_fill(BatchWork& w, hfx_ctx* const* ctxs, int n, double* const* pmax, dou
       L.pmax = w.pmax ? pmax[s] : nullptr;
       L.ns = c->n_shells;
       L.skip_zero = c->opt.skip_zero_p;
-      L.fp32_ok = mixed && ((c->opt.fp32_class_mask >> cp) & 1);
+      L.fp32_ok = mixed && ((c->fp32_mask() >> cp) & 1);
       L.fp32_tau = c->opt.fp32_tau;
       L.pglob = glob ? pglob[s] : nullptr;
       L.dens_tau = c->opt.density_tau;

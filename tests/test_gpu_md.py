@@ -54,3 +54,39 @@ def test_streams_of_few_and_many_primitives(hfx_mod, nprim, atoms, mixed):
     assert sum(st["quartets_evaluated_class"]) > 0
     if mixed and atoms > 1:  # (the quartets of one atom are all large: its mixed build is the FP64 pass)
         assert sum(st["quartets_fp32_class"]) > 0
+
+
+@pytest.mark.parametrize("alpha", [4e8, 3e10, 2e-10])
+def test_mixed_build_at_the_ends_of_the_fp32_range(hfx_mod, alpha):
+    """Powers of 2 rho and the prefactors leave FP32's range for such exponents: classes within it take
+    the FP32 pass, the others the FP64 pass, all finite and right (a tiny density makes every quartet
+    eligible)."""
+    xyz = np.array([[0.0, 0.0, 0.0], [1.0, 0.8, -0.6]])
+    s = inputs.System("pair", xyz, np.repeat([0, 1], 3).astype(np.int32), np.array([0, 1, 2] * 2, np.int32),
+                      np.ones(6, np.int32), np.full(6, alpha) * np.array([1.0, 0.7, 0.9, 0.8, 1.0, 0.6]), np.ones(6),
+                      omega=0.11, tau=0.0)
+    P = 1e-14 * (np.ones((s.n_bf, s.n_bf)) + np.eye(s.n_bf))
+    h = check(hfx_mod, s, P, 1e-6, precision=hfx_mod.HFX_MIXED, fp32_class_mask=hfx_mod.ALL_CLASS_MASK,
+              prim_tau=0.0)  # (the oracle drops no primitive pairs)
+    n32 = h.stats()["quartets_fp32_class"]
+    assert n32[0] > 0 and n32[20] == 0  # (ss|ss) within, (dd|dd) beyond
+
+
+@pytest.mark.parametrize("mixed", [False, True])
+def test_build_inside_a_captured_graph(hfx_mod, mixed):
+    """Overlapping class launches (a small system) as a captured graph, replayed for another density."""
+    s, P0 = inputs.config1(3)
+    h = hfx_mod.HFX(s, stream=torch.cuda.Stream(), precision=hfx_mod.HFX_MIXED if mixed else hfx_mod.HFX_FP64)
+    h.build_pairs()
+    P, K = torch.from_numpy(P0).cuda(), torch.empty(P0.shape, dtype=torch.float64, device="cuda")
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=h.stream):
+        h.build_K(P, K)
+    for seed in (1, 2):
+        P1 = inputs.density_matrix(s, seed=seed, truncate_bohr=10.0)
+        P.copy_(torch.from_numpy(P1))
+        graph.replay()
+        torch.cuda.synchronize()
+        Ko, _ = oracle.Screen(oracle.Basis(s)).build_K(P1, "sym")
+        assert np.abs(K.cpu().numpy() - Ko).max() <= (1e-7 if mixed else 1e-12) * np.abs(Ko).max()
