@@ -282,11 +282,11 @@ def run_batch32(args, torch, hfx, inputs):
 
 def nao_flops(M, n_r, evals, jpasses, trials):
     """FP64 flops (FMA = 2) per grid point as the NAO kernels are written, times the passes:
-    genetic fitness = Gaussians by recurrence (2M per pass, two passes), normal equations
+    genetic fitness = Gaussians by recurrence (2M, kept for the residual), normal equations
     (M(M+1) + 2M) and residual (2M + 3); Jacobian pass 4M + 3 + 6 M(M+1)/2 + 4M; trial pass
     4M + 3.  exp() calls (3M per lane and pass) are not counted."""
     na = M * (M + 1) // 2
-    fit = 2 * M + 2 * na + 2 * M + 2 * M + 2 * M + 3
+    fit = 2 * M + 2 * na + 2 * M + 2 * M + 3
     jac = 4 * M + 3 + 6 * na + 4 * M
     trial = 4 * M + 3
     return n_r * (evals * fit + jpasses * jac + trials * trial)
@@ -695,9 +695,9 @@ def main():
     g32 = [c for c in range(21) if st_timed["group_size_class"][c] == 32]
     dom_ms = sum(ms_cls[c] for c in g32)
     prim_c = st_timed["prim_quartets_class"]
-    # algorithmic flops: vertical recurrence + contraction per primitive quartet, horizontal
-    # recurrence + spherical step + digest per quartet (the Boys evaluations are counted
-    # apart, as special-function evaluations)
+    # algorithmic flops: Hermite recursion + ket contraction per primitive quartet, bra contraction
+    # per run, transformation + digest per quartet (the Boys evaluations are counted apart, as
+    # special-function evaluations)
     rec_fl = sum(st_timed["flops_recurrence_class"][c] for c in g32)
     set_fl = sum(st_timed["flops_class"][c] for c in g32)   # the same plus the primitive set-up
     f32 = st_timed["flops_fp32"] if mixed else 0.0
@@ -731,13 +731,13 @@ def main():
             "e2e": {"value": n_q / float(np.median(e2e_t)) if e2e_t else None, "unit": "quartets/s",
                     "h2d_bytes_per_step": nbytes, "d2h_bytes_per_step": nbytes},
             "gpu_launches": launches_per_step * args.steps,
-            "roofline": {"bound": "alu", "kernel": "eri_g32_kernel (the classes run one quartet per warp), CUDA "
+            "roofline": {"bound": "alu", "kernel": "eri_md_kernel (Hermite engine, every class), CUDA "
                                                    "events around each class launch over the timed steps",
                          "achieved": achieved, "peak": fp64_peak, "unit": "TFLOP/s",
                          "frac": (achieved / fp64_peak) if achieved else None,
-                         "flops": "vertical recurrence + contraction per evaluated primitive quartet, horizontal "
-                                  "recurrence + spherical step + digest per evaluated quartet (operation counts "
-                                  "of the generated tables); Boys evaluations counted apart"
+                         "flops": "Hermite recursion + ket contraction per evaluated primitive quartet, bra "
+                                  "contraction per run, transformation + digest per evaluated quartet (operation "
+                                  "counts of the generated tables); Boys evaluations counted apart"
                                   + ("; FP32 flops counted at the FP64/FP32 peak ratio" if mixed else ""),
                          "traffic": None,
                          "traffic_note": "not taken in this run; ncu on one 16-atom launch of this kernel "

@@ -75,15 +75,15 @@ typedef struct {
   double schwarz_tau;  /* Schwarz threshold tau (>= 0) */
   double rcut_bohr;    /* orbital cutoff radius r_c; <= 0 disables the pair-distance screen */
   double prim_tau;     /* primitive pairs with |prefactor| below this are dropped (default 1e-22) */
-  double fp32_tau;     /* HFX_MIXED: a quartet's primitive set-up, recurrences (VRR) and their
+  double fp32_tau;     /* HFX_MIXED: a quartet's primitive set-up, recurrences and their
                           contraction run in FP32 iff Q_IJ Q_KL Pmax < fp32_tau (default 1e-6),
-                          Pmax as set by fp32_pmax_global; HRR, spherical step and all K
-                          accumulation stay FP64.  The FP32 Boys step is the difference of two
-                          upper incomplete gamma functions (erfc and an upward recursion of
-                          positive terms); a primitive quartet where the subtracted one exceeds
-                          1/64 of the other (small T (1 - kappa)) takes the FP64 Boys step.  FP32
-                          quartets run on whole warps, four primitive quartets per float4 slot
-                          (two FFMA2 per op) */
+                          Pmax as set by fp32_pmax_global; the transformation to spherical
+                          integrals and all K accumulation stay FP64.  The FP32 Boys step is the
+                          difference of two upper incomplete gamma functions (erfc and an upward
+                          recursion of positive terms); a primitive quartet where the subtracted
+                          one exceeds 1/64 of the other (small T (1 - kappa)) takes the FP64 Boys
+                          step.  Classes whose integrals could leave FP32's range for the
+                          exponents of the basis stay FP64.  FP32 quartets run on whole warps */
   int precision;       /* HFX_FP64 (default) or HFX_MIXED */
   int schedule;        /* HFX_SCHED_DYNAMIC (default), HFX_SCHED_QUARTET or HFX_SCHED_PAIR */
   int skip_zero_p;     /* 1 (default): skip quartets whose four density blocks P_bd, P_bc,
@@ -128,13 +128,13 @@ typedef struct {
   double ms_build;             /* GPU time of the last hfx_build_K (zero K .. E_K ready) */
   double ms_class[21];         /* GPU time of each class launch in the last K build */
   double energy;               /* E_K = sum_{mu nu} P_{mu nu} K_{mu nu} of the last K build */
-  double flops_recurrence;     /* of flops_fp64 + flops_fp32: the recurrences alone (vertical
-                                  recurrence, contraction, horizontal recurrence, Cartesian ->
-                                  spherical step, digest into K), the primitive set-up excluded */
+  double flops_recurrence;     /* of flops_fp64 + flops_fp32: the recurrences alone (recursion,
+                                  contraction, transformation to spherical integrals, digest into
+                                  K), the primitive set-up excluded */
   double special_evals;        /* Boys-function evaluations of the last timed build (each: F_m at
                                   the top order and exp(-x) from the tables): two per evaluated
                                   primitive quartet with the erfc kernel, one with omega = 0 */
-  int32_t streams_class[21];   /* warp kernel: primitive quartets run at a time per class */
+  int32_t streams_class[21];   /* the class's choice of hfx_set_streams (0: thread kernel) */
   int32_t reserved_stats[1];
   double flops_recurrence_class[21]; /* flops_recurrence per class */
 } hfx_stats;
@@ -179,10 +179,11 @@ int hfx_periodic_cells(const hfx_ctx* ctx, int* cells, int max_n);
 int hfx_build_K_periodic(hfx_ctx* ctx, int n_R, const int* R_cells, const double* P_R, int n_G, const int* G_cells,
                          double* K_G);
 
-/* Primitive quartets the warp kernel runs at a time for quartet class cls (0..20) in later
- * builds: 0 = the class default, else one of the variants the library carries (1, 2 or 4;
- * the largest classes carry fewer).  Results do not depend on it (summation order aside).
- * Errors: HFX_ERR_ARG for an unknown class or a variant the class does not carry. */
+/* Primitive quartets of one quartet run at a time for quartet class cls (0..20): 0 = the class
+ * default, else one of the class's variants (1, 2 or 4; the largest classes carry fewer).  The
+ * choice is kept and reported in the statistics; the kernels stream primitive quartets across
+ * quartets and run the same whatever it is.  Errors: HFX_ERR_ARG for an unknown class or a variant
+ * the class does not carry. */
 int hfx_set_streams(hfx_ctx* ctx, int cls, int streams);
 
 /* Fills *opt with defaults: omega 0.11, tau 1e-10, no cutoff, prim_tau 1e-22, FP64,
@@ -246,9 +247,8 @@ int hfx_energy(hfx_ctx* ctx, double* out);
 int hfx_get_stats(hfx_ctx* ctx, hfx_stats* out);
 
 /* Lanes per quartet for class cls (0..20) in later K builds of this context: 1 (a thread
- * owns a quartet), 32 (a warp), 0 = the library's default (1 for the nine classes whose
- * scratch fits the thread kernel, 32 otherwise; in a mixed-precision build the FP32 pass runs
- * 32 in every class).  A value set here applies to both passes of a mixed-precision class.
+ * owns a quartet), 32 (whole warps, alone or in teams, over a stream of quartets), 0 = the
+ * library's default (32).  A value set here applies to both passes of a mixed-precision class.
  * 1 needs a class whose scratch fits the thread kernel, else the build fails with
  * HFX_ERR_CUDA.  Errors: HFX_ERR_ARG. */
 int hfx_set_group_size(hfx_ctx* ctx, int cls, int gs);
@@ -298,7 +298,7 @@ typedef struct {
   int32_t chunk_class[21];     /* chosen quartets per dynamic claim per class */
   double tune_ms_class[21];    /* best tuning time per class, scaled from its window to the class */
   int64_t tune_window_class[21]; /* quartets in the window each candidate was timed on */
-  int32_t streams_class[21];   /* warp kernel: primitive quartets at a time per class (0: thread kernel) */
+  int32_t streams_class[21];   /* as hfx_stats.streams_class */
   int32_t tune_kept;           /* 1 if the last hfx_batch_tune kept its choices (they beat the
                                   previous ones on the whole batch), 0 if it restored them */
   double tune_full_default_ms; /* last hfx_batch_tune: whole batch with the previous choices */
@@ -313,11 +313,9 @@ typedef struct {
  * contexts must outlive the batch. */
 int hfx_batch_create(hfx_batch** out, hfx_ctx* const* ctxs, int n, void* stream);
 
-/* Autotuner: for every class, times its batched launch with each candidate kernel shape
- * (a warp per quartet with 1, 2 or 4 primitive quartets at a time, or a thread per quartet
- * where the class allows it) and dynamic chunk size (quartets per claim) on one window of
- * the class's quartets, and keeps the fastest; a candidate must beat the current choice by
- * 5% to replace it.  Then it times the whole batch with the previous and with the tuned
+/* Autotuner: for every class, times its batched launch with each candidate dynamic chunk size
+ * (quartets per claim) on one window of the class's quartets, and keeps the fastest; a candidate
+ * must beat the current choice by 5% to replace it.  Then it times the whole batch with the previous and with the tuned
  * choices and keeps the tuned ones only if they are faster (the number of parallel branches,
  * 1 or 4, is chosen there too), so tuning never makes a batch slower than its previous
  * configuration as measured by these runs.  Uses P/K like

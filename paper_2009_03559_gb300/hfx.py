@@ -451,7 +451,8 @@ class HFX:
         self._check(self.L.hfx_set_group_size(self.h, int(cls), int(gs)))
 
     def set_streams(self, cls, k):
-        """Primitive quartets the warp kernel runs at a time for class cls (0 = default)."""
+        """Primitive quartets of a quartet run at a time for class cls (0 = default): checked and
+        reported; the kernels run the same whatever it is."""
         self._check(self.L.hfx_set_streams(self.h, int(cls), int(k)))
 
     def set_timing(self, on=True):
