@@ -5,19 +5,20 @@
 // under alpha_m >= alpha_min; Algorithm 1: N restarts, each a constrained genetic search for a
 // starting point followed by a constrained local search, the restart with the smallest err kept).
 //
-// Layout: one warp runs one restart; its lanes share the radial grid r_i = i h (lane j owns the
-// points i = j + 1 + 32 t), so every sum over the grid is a per-lane partial sum followed by one
-// warp reduction.  Everything is FP64.  Per warp, shared memory holds the targets y_i, the
-// reduction scratch, a dense system for the local search, the genetic search's two
-// populations and, where it fits, the Gaussians on the grid.  The genetic step and the local search are separate kernels (each gets its own
-// register budget); a third picks the best restart per function.
+// Layout: a warp's lanes share the radial grid r_i = i h (lane j owns the points i = j + 1 + 32 t),
+// so every sum over the grid is a per-lane partial sum followed by one warp reduction.  Everything
+// is FP64.  The genetic step runs one restart per block, its warps sharing each generation's
+// individuals, the local search one restart per warp.  Shared memory holds the targets y_i, the
+// reduction scratch of each warp, a dense system for the local search, the genetic search's two
+// populations and, where it fits, the Gaussians on the grid.  The genetic step and the local
+// search are separate kernels (each gets its own register budget); a third picks the best restart
+// per function.
 //
 // Gaussians on the grid: for an exponent a and beta = a h^2, exp(-beta i^2) moves along one lane's
 // points (i -> i + 32) by the factor exp(-beta (64 i + 1024)), and that factor by exp(-2048 beta):
 // two exp() calls per Gaussian and lane plus the lane-independent one, then two multiplies per
 // point (the local search).  In the genetic step an individual's alpha = exp(u) and the factors
-// exp(-beta), exp(-64 beta), exp(-1024 beta) are made once, by the lane that makes the
-// individual, and kept with its genes; a lane's start values are then products over the lanes
+// exp(-beta), exp(-64 beta), exp(-1024 beta) are made once and kept with its genes; a lane's start values are then products over the lanes
 // below it (warp product scans), so evaluating an individual calls no exp().
 //
 // The paper names the two searches but does not spell them out; the readings (shared with the
@@ -62,7 +63,7 @@ constexpr int kMatLd = kMaxUnknowns + 1;
 constexpr int kMatDoubles = kMaxUnknowns * kMatLd + kMatLd;  // matrix + right-hand side
 constexpr int kMaxNr = 1024;
 constexpr int kMaxPop = 64;
-constexpr int kWarps = 4;  // warps (restarts) per block at most
+constexpr int kWarps = 4;  // warps per block at most
 constexpr size_t kMaxBlockSmem = 227 * 1024;
 
 constexpr double kRidge = 1e-12;
@@ -101,18 +102,20 @@ __host__ __device__ constexpr int n_red(int m) { return 3 * n_tri(m) + 2 * m + 1
 
 enum Which { kGenetic, kLocal, kProject };
 
-// Shared memory of one warp: targets, reduction rows, then per kernel the dense system (local
-// search), the populations (genetic step) and, with `store`, the Gaussians on the grid, kept by
-// the pass of the normal equations for the pass of the residual.
-__host__ __device__ inline int warp_smem_doubles(Which w, int M, int npad, int P, bool store) {
+// Shared memory: of a genetic step's block the targets and the populations; of each warp the
+// targets (else), the reduction rows, the dense system (local search) and, with `store`, the
+// Gaussians on the grid, kept by the pass of the normal equations for the pass of the residual.
+__host__ __device__ inline int block_smem_doubles(Which w, int M, int npad, int P) {
+  return w == kGenetic ? npad + 10 * P * M + 2 * P : 0;
+}
+__host__ __device__ inline int warp_smem_doubles(Which w, int M, int npad, bool store) {
   const int rows = w == kLocal ? n_red(M) : n_tri(M) + M;
-  return npad + rows * 33 + (w == kLocal ? kMatDoubles : 0) + (w == kGenetic ? 10 * P * M + 2 * P : 0) +
-         (store ? M * npad : 0);
+  return (w == kGenetic ? 0 : npad) + rows * 33 + (w == kLocal ? kMatDoubles : 0) + (store ? M * npad : 0);
 }
 
 // pop: genes u_m = ln alpha_m; al: alpha_m; fac: per Gaussian exp(-beta), exp(-64 beta) and
 // exp(-1024 beta), beta = alpha_m h^2, the factors of the grid recurrence (made once per
-// individual by the lane that makes it)
+// individual)
 struct WarpMem {
   double* y;
   double* red;
@@ -129,16 +132,10 @@ __device__ __forceinline__ WarpMem warp_mem(int npad, int P) {
   extern __shared__ double smem[];
   const int w = threadIdx.x >> 5;
   WarpMem m{};
-  m.y = smem + (size_t)w * warp_smem_doubles(W, M, npad, P, STORE);
-  m.red = m.y + npad;
-  double* next = m.red + (W == kLocal ? n_red(M) : n_tri(M) + M) * 33;
-  if constexpr (W == kLocal) m.mat = next;
-  if constexpr (STORE) {
-    m.gauss = next;
-    next += M * npad;
-  }
+  double* next = smem + block_smem_doubles(W, M, npad, P) + (size_t)w * warp_smem_doubles(W, M, npad, STORE);
   if constexpr (W == kGenetic) {
-    m.pop[0] = next;
+    m.y = smem;
+    m.pop[0] = smem + npad;
     m.pop[1] = m.pop[0] + P * M;
     m.al[0] = m.pop[1] + P * M;
     m.al[1] = m.al[0] + P * M;
@@ -146,14 +143,22 @@ __device__ __forceinline__ WarpMem warp_mem(int npad, int P) {
     m.fac[1] = m.fac[0] + 3 * P * M;
     m.fit[0] = m.fac[1] + 3 * P * M;
     m.fit[1] = m.fit[0] + P;
+  } else {
+    m.y = next;
+    next += npad;
   }
+  m.red = next;
+  next += (W == kLocal ? n_red(M) : n_tri(M) + M) * 33;
+  if constexpr (W == kLocal) m.mat = next;
+  if constexpr (STORE) m.gauss = next;
   return m;
 }
 
 // y_i = phi(r_i) / r_i^l on the padded grid (zero beyond n_r)
+template <Which W>
 __device__ __forceinline__ void load_targets(const NaoArgs& A, int f, double* y, int lane) {
   const int l = __ldg(A.l + f);
-  for (int i0 = lane; i0 < A.npad; i0 += 32) {
+  for (int i0 = lane; i0 < A.npad; i0 += W == kGenetic ? blockDim.x : 32) {
     double v = 0.0;
     if (i0 < A.n_r) {
       const double r = A.h * (double)(i0 + 1);
@@ -357,7 +362,7 @@ __device__ __forceinline__ double project(const double (&alpha)[M], double (&D)[
 #pragma unroll
   for (int k = 0; k < NA + M; ++k) acc[k] = 0.0;
   const int T = A.npad >> 5;
-  for (int t = 0; t < T; ++t) {
+  auto point = [&](int t) {
     const int i0 = lane + 32 * t;
     const bool valid = i0 < A.n_r;
     const double yv = wm.y[i0];
@@ -373,8 +378,12 @@ __device__ __forceinline__ double project(const double (&alpha)[M], double (&D)[
       for (int j = 0; j <= i; ++j) acc[n_tri(i) + j] = fma(ev[i], ev[j], acc[n_tri(i) + j]);
       acc[NA + i] = fma(yv, ev[i], acc[NA + i]);
     }
+  };
+  for (int t = 0; t + 1 < T; ++t) {
+    point(t);
     g.step(op);
   }
+  point(T - 1);
   warp_sum(acc, wm.red, lane, op);
   double a[NA];
 #pragma unroll
@@ -395,7 +404,7 @@ __device__ __forceinline__ double project(const double (&alpha)[M], double (&D)[
 }
 
 // ---------------------------------------------------------------------------
-// Genetic step (one warp per restart)
+// Genetic step (one block per restart)
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ bool better(double fa, double fb) { return fa < fb * kTieFactor; }
 
@@ -436,34 +445,40 @@ __device__ __forceinline__ double eval_individual(const double* al, const double
   return project<M, STORE>(alpha, D, A, wm, lane, op, fac);
 }
 
-// alpha = exp(u) and the grid-recurrence factors of one individual, into shared memory
-template <int M>
-__device__ __forceinline__ void store_individual(const double (&u)[M], double h2, double* pop, double* al,
-                                                 double* fac) {
-#pragma unroll
-  for (int m = 0; m < M; ++m) {
-    const double a = exp(u[m]);
+// alpha = exp(u) and the grid-recurrence factors of genes j0 .. j1, a gene per thread
+__device__ __forceinline__ void gene_factors(int j0, int j1, int tid, double h2, const double* pop, double* al,
+                                             double* fac) {
+  for (int j = j0 + tid; j < j1; j += blockDim.x) {
+    const double a = exp(pop[j]);
     const double beta = a * h2;
-    pop[m] = u[m];
-    al[m] = a;
-    fac[3 * m] = exp(-beta);
-    fac[3 * m + 1] = exp(-64.0 * beta);
-    fac[3 * m + 2] = exp(-1024.0 * beta);
+    al[j] = a;
+    fac[3 * j] = exp(-beta);
+    fac[3 * j + 1] = exp(-64.0 * beta);
+    fac[3 * j + 2] = exp(-1024.0 * beta);
   }
 }
 
+// One restart per block.  The individuals of a generation are independent: the block's warps take
+// every W-th of them, one lane of the first warp makes each individual's genes, and a thread per
+// gene its factors.  Which warp is first turns with the block and the generation (a warp sits on
+// one quarter of the SM, and the first has the genes to make and the odd individual to evaluate).
+// Against a restart per warp: 1280 restarts are 8.4 to an SM, which with 8 resident warps took a
+// second pass that was nearly empty, and the shared targets and populations leave room for 12
+// warps per SM instead of 8 (M = 3, 512 points, population 32).  10 functions: 46.5 -> 33.4 ms
+// of FP64 pipe time 28 ms; 20 functions x 512 restarts: 257 -> 250 ms (67 to an SM).
 template <int M, bool STORE>
 __global__ void __launch_bounds__(kWarps * 32) nao_genetic_kernel(NaoArgs A) {
   const int lane = threadIdx.x & 31;
-  const long long q = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (q >= (long long)A.n_fun * A.N) return;  // whole warps leave together
+  const int W = blockDim.x >> 5;
+  const long long q = blockIdx.x;
   const int f = (int)(q / A.N);
   const int P = A.P, G = A.G;
   constexpr int S = 4 + 2 * M;
   const WarpMem wm = warp_mem<kGenetic, M, STORE>(A.npad, P);
   Fp64 op;
   op.init();
-  load_targets(A, f, wm.y, lane);
+  load_targets<kGenetic>(A, f, wm.y, threadIdx.x);
+  auto place = [&](int g) { return (int)((threadIdx.x >> 5) + blockIdx.x + (unsigned)g) % W; };
   auto ctr = [&](int g, int j, int k) -> unsigned long long {
     return (((unsigned long long)q * (unsigned long long)(G + 1) + (unsigned long long)g) * (unsigned long long)P +
             (unsigned long long)j) * (unsigned long long)S + (unsigned long long)k;
@@ -471,19 +486,22 @@ __global__ void __launch_bounds__(kWarps * 32) nao_genetic_kernel(NaoArgs A) {
   const double span = __dsub_rn(A.hi, A.lo);
   const double h2 = A.h * A.h;
   // initial population
-  for (int j = lane; j < P; j += 32) {
+  for (int j = threadIdx.x; j < P; j += blockDim.x) {
     double u[M];
 #pragma unroll
     for (int m = 0; m < M; ++m) u[m] = __dadd_rn(A.lo, __dmul_rn(uniform01(A.seed, ctr(0, j, m)), span));
     sort_genes<M>(u);
-    store_individual<M>(u, h2, wm.pop[0] + j * M, wm.al[0] + j * M, wm.fac[0] + 3 * j * M);
+#pragma unroll
+    for (int m = 0; m < M; ++m) wm.pop[0][j * M + m] = u[m];
   }
-  __syncwarp();
-  for (int j = 0; j < P; ++j) {
+  __syncthreads();
+  gene_factors(0, P * M, threadIdx.x, h2, wm.pop[0], wm.al[0], wm.fac[0]);
+  __syncthreads();
+  for (int j = place(0); j < P; j += W) {
     const double fj = eval_individual<M, STORE>(wm.al[0] + j * M, wm.fac[0] + 3 * j * M, A, wm, lane, op);
     if (lane == 0) wm.fit[0][j] = fj;
   }
-  __syncwarp();
+  __syncthreads();
   int cur = 0;
   for (int g = 1; g <= G; ++g) {
     const double* pop = wm.pop[cur];
@@ -492,8 +510,9 @@ __global__ void __launch_bounds__(kWarps * 32) nao_genetic_kernel(NaoArgs A) {
     double* nal = wm.al[cur ^ 1];
     double* nfac = wm.fac[cur ^ 1];
     double* nfit = wm.fit[cur ^ 1];
-    const int e = best_index(fit, P);
-    for (int j = lane; j < P; j += 32) {
+    const int w = place(g);
+    const int e = w == 0 ? best_index(fit, P) : 0;
+    for (int j = w == 0 ? lane : P; j < P; j += 32) {
       if (j == 0) {
 #pragma unroll
         for (int m = 0; m < M; ++m) {
@@ -524,16 +543,20 @@ __global__ void __launch_bounds__(kWarps * 32) nao_genetic_kernel(NaoArgs A) {
         c[m] = reflect_box(v, A.lo, A.hi);
       }
       sort_genes<M>(c);
-      store_individual<M>(c, h2, npop + j * M, nal + j * M, nfac + 3 * j * M);
+#pragma unroll
+      for (int m = 0; m < M; ++m) npop[j * M + m] = c[m];
     }
-    __syncwarp();
-    for (int j = 1; j < P; ++j) {
+    __syncthreads();
+    gene_factors(M, P * M, 32 * w + lane, h2, npop, nal, nfac);
+    __syncthreads();
+    for (int j = 1 + w; j < P; j += W) {
       const double fj = eval_individual<M, STORE>(nal + j * M, nfac + 3 * j * M, A, wm, lane, op);
       if (lane == 0) nfit[j] = fj;
     }
-    __syncwarp();
+    __syncthreads();
     cur ^= 1;
   }
+  if (place(0) != 0) return;
   const int e = best_index(wm.fit[cur], P);
   double alpha[M], D[M];
 #pragma unroll
@@ -601,7 +624,7 @@ __global__ void __launch_bounds__(kWarps * 32) nao_local_kernel(NaoArgs A) {
   const WarpMem wm = warp_mem<kLocal, M, false>(A.npad, A.P);
   Fp64 op;
   op.init();
-  load_targets(A, f, wm.y, lane);
+  load_targets<kLocal>(A, f, wm.y, lane);
   const double h2 = A.h * A.h;
   double xa[M], xd[M];
 #pragma unroll
@@ -805,7 +828,7 @@ __global__ void __launch_bounds__(kWarps * 32) nao_project_kernel(NaoArgs A) {
   const WarpMem wm = warp_mem<kProject, M, STORE>(A.npad, A.P);
   Fp64 op;
   op.init();
-  load_targets(A, f, wm.y, lane);
+  load_targets<kProject>(A, f, wm.y, lane);
   double alpha[M], D[M];
 #pragma unroll
   for (int m = 0; m < M; ++m) alpha[m] = __ldg(A.set_alpha + s * M + m);
@@ -840,36 +863,34 @@ const void* kernel_for(int M, Which w, bool store) {
   }
 }
 
-// restarts per block: up to kWarps, as many as the shared memory of a block holds
-int warps_per_block(size_t per_warp) {
-  return (int)std::max<size_t>(1, std::min<size_t>(kWarps, kMaxBlockSmem / per_warp));
-}
-
-// warps an SM holds by shared memory (228 KB, 1 KB of it per block reserved)
-int resident_warps(size_t per_warp) {
-  const int w = warps_per_block(per_warp);
-  return (int)(228 * 1024 / (w * per_warp + 1024)) * w;
-}
-
-int launch(Which w, int M, const NaoArgs& a, long long n_warps, cudaStream_t s) {
-  if (n_warps <= 0) return HFX_OK;
+int launch(Which w, int M, const NaoArgs& a, long long n, cudaStream_t s) {
+  if (n <= 0) return HFX_OK;
+  // warps per block: as many as the shared memory of a block holds, up to kWarps; in the genetic
+  // step no more than a generation has new individuals
+  const size_t shared = (size_t)block_smem_doubles(w, M, a.npad, a.P) * sizeof(double);
+  auto per_warp = [&](bool store) { return (size_t)warp_smem_doubles(w, M, a.npad, store) * sizeof(double); };
+  auto warps_per_block = [&](bool store) {
+    const size_t fit = shared < kMaxBlockSmem ? (kMaxBlockSmem - shared) / per_warp(store) : 0;
+    return (int)std::min<size_t>(w == kGenetic ? std::min(kWarps, a.P - 1) : kWarps, fit);
+  };
+  // warps an SM holds by shared memory (228 KB, 1 KB of it per block reserved)
+  auto resident = [&](bool store) {
+    const int nw = warps_per_block(store);
+    return nw ? (int)(228 * 1024 / (shared + nw * per_warp(store) + 1024)) * nw : 0;
+  };
   // the Gaussians are kept on the grid where that leaves 8 warps per SM or costs none: two warps
   // per SM quarter keep the FP64 pipe busy, fewer do not
-  auto bytes = [&](bool store) {
-    return (size_t)warp_smem_doubles(w, M, a.npad, a.P, store) * sizeof(double);
-  };
-  const bool store = w != kLocal && bytes(true) <= kMaxBlockSmem &&
-                     (resident_warps(bytes(true)) >= 8 || resident_warps(bytes(true)) == resident_warps(bytes(false)));
-  const size_t per_warp = bytes(store);
-  const int warps = warps_per_block(per_warp);
-  const size_t smem = warps * per_warp;
+  const bool store = w != kLocal && warps_per_block(true) > 0 &&
+                     (resident(true) >= 8 || resident(true) == resident(false));
+  const int warps = std::max(1, warps_per_block(store));
+  const size_t smem = shared + warps * per_warp(store);
   const void* k = kernel_for(M, w, store);
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) {
     hfx::set_global_error(std::string("nao: shared memory request refused: ") + cudaGetErrorString(e));
     return HFX_ERR_CUDA;
   }
-  const long long blocks = (n_warps + warps - 1) / warps;
+  const long long blocks = w == kGenetic ? n : (n + warps - 1) / warps;
   void* args[] = {(void*)&a};
   e = cudaLaunchKernel(k, dim3((unsigned)blocks), dim3(warps * 32), args, smem, s);
   if (e != cudaSuccess) {

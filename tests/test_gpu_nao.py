@@ -184,3 +184,21 @@ def test_largest_options(fitter):
         assert out["r_ga_err"][it] == pytest.approx(N.err(p["ga_alpha"], p["ga_D"], N.targets(phi[0], 2, h), r),
                                                     rel=1e-8)
     assert out["err"][0] == pytest.approx(ref["best"]["err"], rel=1e-6)
+
+
+@pytest.mark.parametrize("P", [2, 3, 4, 5, 33, 64])
+def test_genetic_step_at_block_shapes(fitter, P):
+    """Populations that give blocks of one, two, three and four warps, a remainder of individuals per
+    warp, more individuals than lanes."""
+    hfx, rs, F = fitter
+    r = N.grid(rs.phi.shape[1], rs.h)
+    o = hfx.nao_options(n_gauss=2, n_restarts=3, population=P, generations=3, seed=5)
+    a, _, e = (x.cpu().numpy() for x in F.genetic(o))
+    agree = 0
+    for f in range(F.n_fun):
+        y = N.targets(rs.phi[f], int(rs.l[f]), rs.h)
+        for it in range(3):
+            q = f * 3 + it
+            a_o, _, e_o = N.genetic(q, y, r, 2, P, 3, 0.1, 1000.0, 5)
+            agree += int(abs(e[q] - e_o) <= 1e-10 * e_o and np.allclose(a[q], a_o, rtol=1e-12))
+    assert agree >= 0.9 * F.n_fun * 3
