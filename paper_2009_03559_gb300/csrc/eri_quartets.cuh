@@ -96,11 +96,11 @@ __device__ __forceinline__ void record_busy(const EriLaunch& L, unsigned long lo
 }
 
 // ---------------------------------------------------------------------------
-// Periodic quartets (Eq. vx with lattice images): the launch for cell G evaluates
+// Periodic quartets (Eq. vx with lattice images): the pass for cell G evaluates
 // (X | Y + shift) for bra pair X and ket pair Y of the home-anchored pair list and adds
 //   K^G_{ab} += sum_{c,d} (a c | b d) P^{R}_{cd},   R = cell(d) - cell(c),
 // where a is the home-cell shell of the pair holding the row function (X for a forward
-// launch, Y for a reverse one), c its partner, b the home-cell shell of the other pair
+// pass, Y for a reverse one), c its partner, b the home-cell shell of the other pair
 // (in cell G) and d its partner.  Every ordered pair of pairs is one quartet (no
 // permutational symmetry is used across cells), so the degeneracy factor is 1.
 // ---------------------------------------------------------------------------
@@ -110,8 +110,10 @@ struct PerQuartet {
   const double* PR;          // density block P^R
 };
 
-__device__ __forceinline__ bool per_quartet(const EriLaunch& L, int bra, int ket, PerQuartet& q) {
+__device__ __forceinline__ bool per_quartet(const EriLaunch& L, int pass, int bra, int ket, PerQuartet& q) {
   const PeriodicInfo& pi = L.per;
+  const PerCell& cell = pi.cells[pass];
+  const bool reverse = __ldg(&cell.reverse);
   const int sax = __ldg(L.pa.sa + bra), sbx = __ldg(L.pa.sb + bra);
   const int say = __ldg(L.pa.sa + ket), sby = __ldg(L.pa.sb + ket);
   const bool hx = __ldg(pi.home_first + bra), hy = __ldg(pi.home_first + ket);
@@ -123,7 +125,7 @@ __device__ __forceinline__ bool per_quartet(const EriLaunch& L, int bra, int ket
   int idx = 0;
   for (int i = 0; i < 3; ++i) {
     const int d = __ldg(cy + i) - __ldg(cx + i);
-    const int R = L.gcell[i] + (L.reverse ? -d : d);
+    const int R = __ldg(&cell.gcell[i]) + (reverse ? -d : d);
     if (R < -pi.rb || R > pi.rb) return false;
     idx = idx * w + (R + pi.rb);
   }
@@ -131,12 +133,12 @@ __device__ __forceinline__ bool per_quartet(const EriLaunch& L, int bra, int ket
   if (blk < 0) return false;
   // an exactly zero density block P^R_{cd} makes the quartet's contribution exactly zero
   {
-    const int c = L.reverse ? oys : oxs, d = L.reverse ? oxs : oys;
+    const int c = reverse ? oys : oxs, d = reverse ? oxs : oys;
     if (__ldg(pi.pmax + ((size_t)blk * pi.nsh + c % pi.nsh) * pi.nsh + d % pi.nsh) == 0.0) return false;
   }
   q.PR = pi.P + (size_t)blk * pi.nbf * pi.nbf;
   const int phx = hx ? 0 : 1, pox = 1 - phx, phy = hy ? 2 : 3, poy = 5 - phy;
-  if (!L.reverse) {
+  if (!reverse) {
     q.pa = phx; q.pc = pox; q.pb = phy; q.pd = poy;
     q.bfa = __ldg(pi.shell_bf + hxs); q.bfc = __ldg(pi.shell_bf + oxs);
     q.bfb = __ldg(pi.shell_bf + hys); q.bfd = __ldg(pi.shell_bf + oys);

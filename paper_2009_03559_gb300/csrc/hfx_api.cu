@@ -646,52 +646,62 @@ extern "C" int hfx_build_K_periodic(hfx_ctx* ctx, int n_R, const int* R_cells, c
   L.per.pmax = d_pmaxR;
   L.per.nsh = ctx->n_home_shells;
   L.schedule = HFX_SCHED_DYNAMIC;
+  // K^{-G} = (K^G)^T (exchanging bra and ket pairs maps the quartets of cell G onto those of
+  // cell -G): a cell whose opposite came earlier in the list is a transpose.
+  // forward passes: (p | q + G L) for bra class hi >= ket class lo; reverse ones (hi > lo): the
+  // quartets (p | q + G L) with class(p) = lo < class(q) = hi, evaluated as (q | p - G L)
+  std::vector<int> mirror(n_G, -1);
+  std::vector<PerCell> cells, back;
   for (int g = 0; g < n_G; ++g) {
     const int* G = G_cells + 3 * g;
-    // K^{-G} = (K^G)^T (exchanging bra and ket pairs maps the quartets of cell G onto those of
-    // cell -G): a cell whose opposite came earlier in the list is a transpose
-    int mirror = -1;
-    for (int j = 0; j < g && mirror < 0; ++j)
-      if (G_cells[3 * j] == -G[0] && G_cells[3 * j + 1] == -G[1] && G_cells[3 * j + 2] == -G[2]) mirror = j;
-    if (mirror >= 0) {
-      CK(launch_transpose(nbf, K_G + (size_t)mirror * nbf * nbf, K_G + (size_t)g * nbf * nbf, s));
-      continue;
+    for (int j = 0; j < g && mirror[g] < 0; ++j)
+      if (G_cells[3 * j] == -G[0] && G_cells[3 * j + 1] == -G[1] && G_cells[3 * j + 2] == -G[2]) mirror[g] = j;
+    if (mirror[g] >= 0) continue;
+    PerCell f{}, r{};
+    f.KG = r.KG = K_G + (size_t)g * nbf * nbf;
+    r.reverse = 1;
+    for (int i = 0; i < 3; ++i) {
+      f.gcell[i] = r.gcell[i] = G[i];
+      f.shift[i] = G[0] * ctx->lattice[i] + G[1] * ctx->lattice[3 + i] + G[2] * ctx->lattice[6 + i];
+      r.shift[i] = -f.shift[i];
     }
-    double sh[3];
-    for (int i = 0; i < 3; ++i)
-      sh[i] = G[0] * ctx->lattice[i] + G[1] * ctx->lattice[3 + i] + G[2] * ctx->lattice[6 + i];
-    L.KG = K_G + (size_t)g * nbf * nbf;
-    CK(cudaMemsetAsync(ctx->d_work, 0, 64 * sizeof(unsigned long long), s));
-    bool follows = false;
-    for (int cp = 0; cp < 21; ++cp) {
-      if (ctx->cls_q[cp] == 0) continue;
-      int hi = 0;
-      while ((hi + 1) * (hi + 2) / 2 <= cp) ++hi;
-      const int lo = cp - hi * (hi + 1) / 2;
-      L.ci = class_info_host()[cp];
-      L.row_begin = ctx->rt.row_base[cp];
-      L.row_end = ctx->rt.row_base[cp + 1];
-      L.bra_bin_start = ctx->rt.bin_start[hi];
-      L.ket_bin_start = ctx->rt.bin_start[lo];
-      L.q_begin = ctx->cls_qbegin[cp];
-      L.q_count = ctx->cls_q[cp];
-      const int gs = eri_group_size();
-      const int grid = grid_for(ctx, cp, 0, L.q_count, gs, 3);
-      L.chunk = eri_chunk(gs, L.q_count, (long long)grid * eri_groups_per_block(cp, gs));
-      // forward: (p | q + G L) for bra class hi >= ket class lo; reverse (hi > lo): the
-      // quartets (p | q + G L) with class(p) = lo < class(q) = hi, evaluated as (q | p - G L)
-      for (int rev = 0; rev < (hi > lo ? 2 : 1); ++rev) {
-        L.reverse = rev;
-        for (int i = 0; i < 3; ++i) {
-          L.gcell[i] = G[i];
-          L.shift[i] = rev ? -sh[i] : sh[i];
-        }
-        L.work = ctx->d_work + cp + 21 * rev;
-        CK(eri_launch(L, cp, 0, grid, s, gs, 3, false, follows));
-        follows = eri_overlap(gs, L.q_count, (long long)grid * eri_groups_per_block(cp, gs));
-      }
-    }
+    cells.push_back(f);
+    back.push_back(r);
   }
+  const int n_fwd = (int)cells.size();
+  cells.insert(cells.end(), back.begin(), back.end());
+  RK(ctx->scratch(&ctx->d_cells, &ctx->cells_cap, cells.size()));
+  CK(cudaMemcpyAsync(ctx->d_cells, cells.data(), sizeof(PerCell) * cells.size(), cudaMemcpyHostToDevice, s));
+  L.per.cells = ctx->d_cells;
+  CK(cudaMemsetAsync(ctx->d_work, 0, 64 * sizeof(unsigned long long), s));
+  bool follows = false;
+  // One launch per class runs the passes of all cells, both ways: a pass by itself is a few quartets
+  // a warp, and the latency of one quartet (25 us for (ss|ss), 140 us for (dd|dd)) was most of a
+  // launch (s, p, d shells, 4 cells: 36 launches a cell, 3.65 -> 1.92 ms a build in all, FP64 pipe
+  // time 1.2 ms).  The classes of the longest quartets go first.
+  for (int cp = 20; cp >= 0; --cp) {
+    if (ctx->cls_q[cp] == 0) continue;
+    int hi = 0;
+    while ((hi + 1) * (hi + 2) / 2 <= cp) ++hi;
+    const int lo = cp - hi * (hi + 1) / 2;
+    L.ci = class_info_host()[cp];
+    L.row_begin = ctx->rt.row_base[cp];
+    L.row_end = ctx->rt.row_base[cp + 1];
+    L.bra_bin_start = ctx->rt.bin_start[hi];
+    L.ket_bin_start = ctx->rt.bin_start[lo];
+    L.q_begin = ctx->cls_qbegin[cp];
+    L.per.n_list = ctx->cls_q[cp];
+    L.q_count = ctx->cls_q[cp] * (hi > lo ? 2 * n_fwd : n_fwd);
+    const int gs = eri_group_size();
+    const int grid = grid_for(ctx, cp, 0, L.q_count, gs, 3);
+    L.chunk = eri_chunk(gs, L.q_count, (long long)grid * eri_groups_per_block(cp, gs));
+    L.work = ctx->d_work + cp;
+    CK(eri_launch(L, cp, 0, grid, s, gs, 3, false, follows));
+    follows = eri_overlap(gs, L.q_count, (long long)grid * eri_groups_per_block(cp, gs));
+  }
+  for (int g = 0; g < n_G; ++g)
+    if (mirror[g] >= 0)
+      CK(launch_transpose(nbf, K_G + (size_t)mirror[g] * nbf * nbf, K_G + (size_t)g * nbf * nbf, s));
   if (ctx->timing) CK(cudaEventRecord(ctx->ev[1], s));
   return HFX_OK;
 }

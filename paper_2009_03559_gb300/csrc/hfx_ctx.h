@@ -69,11 +69,13 @@ struct hfx_ctx {
   int *d_shell_cell = nullptr, *d_shell_bf = nullptr, *d_cell_xyz = nullptr;
   unsigned char* d_home_first = nullptr;  // per candidate pair (pair scope)
   // per periodic build, reused while large enough: cell map of the density blocks, their
-  // block maxima
+  // block maxima, the passes over the quartet lists
   int* d_rmap = nullptr;
   size_t rmap_cap = 0;
   double* d_pmaxR = nullptr;
   size_t pmaxR_cap = 0;
+  hfx::PerCell* d_cells = nullptr;
+  size_t cells_cap = 0;
   // a context-lifetime buffer of at least n elements in *p (capacity *cap), reallocated when short
   template <class T>
   int scratch(T** p, size_t* cap, size_t n) {

@@ -227,6 +227,7 @@ __device__ __forceinline__ void boys_any(int L, double x, const double* __restri
 // Lattice images (periodic builds): the library holds the home cell's shells repeated in a
 // box of cells (the image shells, cell-major, the home cell first); every pair of the pair
 // list has one shell in the home cell (list-IJ anchored in the home cell, Sec. 3.1).
+struct PerCell;
 struct PeriodicInfo {
   const int* shell_cell;            // image shell -> cell index (0 = home cell)
   const int* shell_bf;              // image shell -> first function in the home-cell numbering
@@ -238,6 +239,18 @@ struct PeriodicInfo {
   int nbf;
   const double* pmax;               // max |P^R| per (R, home shell, home shell): n_R x nsh x nsh
   int nsh;                          // shells of the home cell
+  const PerCell* cells;             // the launch's passes over the quartet list of the class
+  long long n_list;                 // quartets of the list
+};
+
+// A pass over the list of a class: quartets (bra | ket + shift) of cell G; reverse = 0: the bra pair
+// carries the row function of K^G, 1: the ket pair does (the pass then evaluates (q | p - G L) for
+// the quartet (p | q + G L) of a lower bra class)
+struct PerCell {
+  double shift[3];
+  double* KG;  // K^G, nbf x nbf
+  int gcell[3];
+  int reverse;
 };
 
 // Arguments of one class launch (passed by value).
@@ -283,14 +296,8 @@ struct EriLaunch {
   int n_sys;
   const long long* seg;
   const EriLaunch* batch;
-  // periodic launch: quartets (bra | ket + shift) of the pair list for the cell G; reverse = 0:
-  // the bra pair carries the row function of K^G, 1: the ket pair does (the launch then
-  // evaluates (q | p - G L) for the quartet (p | q + G L) of a lower bra class)
+  // periodic launch: the list of the class once for each of per.cells (q_count = all of them)
   PeriodicInfo per;
-  double shift[3];
-  int gcell[3];
-  int reverse;
-  double* KG;                 // K^G, nbf x nbf
 };
 
 

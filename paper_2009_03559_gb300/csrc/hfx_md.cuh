@@ -631,8 +631,8 @@ __global__ void __launch_bounds__(md_block(LT), md_minb<R>(LT))
     } else if (a_valid) {
       if constexpr (KIND == MD_PER) {
         PerQuartet pq;
-        if (per_quartet(Ls, bra, ket, pq))
-          digest_per(L.ci, F, 1, pq, Ls.KG, Ls.per.nbf, 32 * wt + lane, 32 * NW);
+        if (per_quartet(Ls, e.x, bra, ket, pq))
+          digest_per(L.ci, F, 1, pq, Ls.per.cells[e.x].KG, Ls.per.nbf, 32 * wt + lane, 32 * NW);
       } else {
         const int sa = __ldg(Ls.pa.sa + bra), sb = __ldg(Ls.pa.sb + bra);
         const int sc = __ldg(Ls.pa.sa + ket), sd = __ldg(Ls.pa.sb + ket);
@@ -711,9 +711,10 @@ __global__ void __launch_bounds__(md_block(LT), md_minb<R>(LT))
         } else {
           double qc[3] = {pk->P[0], pk->P[1], pk->P[2]};
           if constexpr (KIND == MD_PER) {  // the ket pair's image in cell G
-            qc[0] = op.add(qc[0], L.shift[0]);
-            qc[1] = op.add(qc[1], L.shift[1]);
-            qc[2] = op.add(qc[2], L.shift[2]);
+            const double* shift = L.per.cells[s.q.x].shift;
+            qc[0] = op.add(qc[0], __ldg(shift));
+            qc[1] = op.add(qc[1], __ldg(shift + 1));
+            qc[2] = op.add(qc[2], __ldg(shift + 2));
           }
           // (a kernel parameter is a constant operand: one product makes it a register's)
           const double om = KIND == MD_BATCH ? Ls.omega : omega, om2 = KIND == MD_BATCH ? Ls.omega2 : omega2;
@@ -916,7 +917,7 @@ __global__ void __launch_bounds__(md_block(LT), md_minb<R>(LT))
       return q0 < L.diag_n;
     } else {
       while (true) {
-        if (KIND != MD_BATCH && L.schedule != 2) {
+        if (KIND != MD_BATCH && KIND != MD_PER && L.schedule != 2) {
           if (!first) return false;
           first = false;
           group_range(L, wid, nteam, q0, q1);
@@ -947,6 +948,12 @@ __global__ void __launch_bounds__(md_block(LT), md_minb<R>(LT))
             sys = lo;
             q0 = L.batch[lo].q_begin + (c0 - s0);
             q1 = L.batch[lo].q_begin + (e - s0);
+            c0 = e;
+          } else if constexpr (KIND == MD_PER) {  // the chunk's part in the next pass over the list
+            sys = (int)(c0 / L.per.n_list);
+            const long long s0 = sys * L.per.n_list, e = min(c1, s0 + L.per.n_list);
+            q0 = L.q_begin + (c0 - s0);
+            q1 = L.q_begin + (e - s0);
             c0 = e;
           } else {
             q0 = L.q_begin + c0;
@@ -987,7 +994,7 @@ __global__ void __launch_bounds__(md_block(LT), md_minb<R>(LT))
           const int bra = __ldg(Ls.sorted + bra_s), ket = __ldg(Ls.sorted + ket_s);
           if constexpr (KIND == MD_PER) {
             PerQuartet pq;
-            keep = per_quartet(Ls, bra, ket, pq);  // a density block exists for its cell offset
+            keep = per_quartet(Ls, sys, bra, ket, pq);  // a density block exists for its cell offset
           } else {
             const double pm = pmax4(Ls, __ldg(Ls.pa.sa + bra), __ldg(Ls.pa.sb + bra), __ldg(Ls.pa.sa + ket),
                                     __ldg(Ls.pa.sb + ket));

@@ -70,3 +70,18 @@ def test_missing_density_blocks_contribute_nothing(hfx_mod):
     P_R = inputs.periodic_density(ps, r_cells=2, seed=80, truncate_bohr=10.0)
     P_R = {R: v for R, v in P_R.items() if max(abs(x) for x in R) <= 1}
     check(hfx_mod, ps, P_R, [(0, 0, 0), (1, 0, 0)])
+
+
+@pytest.mark.parametrize("G_list", [[(1, 0, 0)], [(0, 0, 0), (0, 1, 0), (0, -1, 0), (1, 1, 0), (-1, -1, 0), (0, 2, 0)]])
+def test_cells_together_or_one_by_one(hfx_mod, G_list):
+    """A class launch runs every listed cell's pass over its quartets (a claim may span passes; some
+    cells are transposes): the same K^G as builds of one cell each.  Tolerance: sums of below 1e4
+    terms in another order."""
+    ps = inputs.periodic_sc(shells=(0, 1, 2), a=6.0, rcut=3.5, tau=1e-9)
+    P_R = inputs.periodic_density(ps, r_cells=1, seed=5)
+    h = hfx_mod.Periodic(ps).build_pairs()
+    K = {G: k.clone() for G, k in h.build_K(P_R, G_list).items()}
+    scale = max(k.abs().max().item() for k in K.values())
+    for G in G_list:
+        one = h.build_K(P_R, [G])[G]
+        assert (K[G] - one).abs().max().item() <= 1e4 * 1.2e-16 * scale, G
