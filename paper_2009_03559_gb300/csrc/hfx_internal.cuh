@@ -124,6 +124,13 @@ __device__ __forceinline__ double widen_f32(float f, int e2 = 0) {
 __device__ __forceinline__ double scale2(double x, int e) {
   return __hiloint2double(__double2hiint(x) + (e << 20), __double2loint(x));
 }
+// 2^e x, e > 0, for any x but 0 and subnormals (at most 2^e 2^-1022 comes of those); what overflows and
+// what is not finite stays not finite.
+__device__ __forceinline__ double scale_up(double x, int e) {
+  const int hi = __double2hiint(x);
+  return __hiloint2double((hi & 0x7fffffff) >= ((0x7ff - e) << 20) ? hi | 0x7ff00000 : hi + (e << 20),
+                          __double2loint(x));
+}
 // x >= 2^e... comparisons of non-negative doubles on the high word (integer units).
 __device__ __forceinline__ bool ge_hi(double x, int hi) { return __double2hiint(x) >= hi; }
 
@@ -191,6 +198,8 @@ __device__ __forceinline__ double rsqrt_nr(double x, const Fp64& op) {
 // F_L(x) and exp(-x) from row g of the table of order L: 7 FP64 instructions.
 __device__ __forceinline__ void boys_row(double x, const double* __restrict__ tabL, int g, double& F, double& e,
                                          const Fp64& op) {
+  // (no argument leads past the table: a NaN from coordinates that overflowed takes its last row)
+  g = (int)min((unsigned)g, (unsigned)(kBoysRows + kBoysTailRows - 1));
   const double2* row = reinterpret_cast<const double2*>(tabL + g * kBoysRowLen);
   const double2 r0 = __ldg(row), r1 = __ldg(row + 1), r2 = __ldg(row + 2);
   const float4 r3 = __ldg(reinterpret_cast<const float4*>(row + 3));

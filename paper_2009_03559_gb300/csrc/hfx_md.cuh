@@ -1,4 +1,6 @@
-// Hermite engine: the FP64 warp kernel (one warp evaluates and digests a stream of quartets).
+// Hermite engine: the kernel of every class launch, in FP64 and (R = float) for the FP32 pass of a
+// mixed-precision build.  A warp, or a team of 2 or 4 for the largest classes, evaluates and digests a
+// stream of quartets.
 //
 // What bounds it: the FP64 pipe, one warp instruction per 64 cycles and SM quarter whatever the
 // number of active lanes, so the algorithm with the fewest FP64 warp instructions wins and a
@@ -31,11 +33,11 @@ namespace hfx {
 template <int N>
 __device__ __forceinline__ double times(double x, const Fp64& op) {
   if constexpr (N == 1) return x;
-  if constexpr (N == 2) return scale2(x, 1);
+  if constexpr (N == 2) return scale_up(x, 1);
   if constexpr (N == 3) return op.mul(x, fp64_operand(2));
-  if constexpr (N == 4) return scale2(x, 2);
+  if constexpr (N == 4) return scale_up(x, 2);
   if constexpr (N == 5) return op.mul(x, fp64_operand(3));
-  if constexpr (N == 6) return scale2(op.mul(x, fp64_operand(2)), 1);
+  if constexpr (N == 6) return scale_up(op.mul(x, fp64_operand(2)), 1);
   if constexpr (N == 7) return op.mul(x, fp64_operand(4));
   return x;  // not reached: a chain of order L <= 8 raises with N <= 7
 }
