@@ -369,9 +369,10 @@ extern "C" int hfx_build_pairs(hfx_ctx* ctx) {
   CK(cudaStreamSynchronize(s));
   {
     EriLaunch L = base_launch(ctx);
-    int start = 0;
+    int start = n_cand;
     bool follows = false;
-    for (int pc = 0; pc < 6; ++pc) {
+    for (int pc = 5; pc >= 0; --pc) {  // the longest quartets first (see build_K_impl)
+      start -= cnt[pc];
       if (cnt[pc] > 0) {
         const int cls = pc * (pc + 1) / 2 + pc;
         L.ci = class_info_host()[cls];
@@ -383,7 +384,6 @@ extern "C" int hfx_build_pairs(hfx_ctx* ctx) {
         CK(eri_launch(L, cls, 1, grid, s, gs, 0, false, follows));
         follows = eri_overlap(gs, cnt[pc], (long long)grid * eri_groups_per_block(cls, gs));
       }
-      start += cnt[pc];
     }
   }
   // 4. pair Schwarz test and bins: sort by Q descending, then stably by bin
@@ -771,7 +771,10 @@ static int build_K_impl(hfx_ctx* ctx, const double* P, double* K, int ld, int pa
   L.Qs = ctx->d_Qs;
   if (ctx->timing) L.busy = ctx->d_busy;
   bool follows = false;  // this launch may start before the one before it has ended
-  for (int cp = 0; cp < 21; ++cp) {
+  // the classes of the longest quartets first: the end of a launch, with most SMs idle, then runs beside
+  // the next one, and the last launch, which nothing follows, ends soonest (against the other order:
+  // 3-atom diamond 0.53 -> 0.41 ms, 9-atom cluster 0.32 -> 0.27, 8-atom diamond 8.15 -> 7.92)
+  for (int cp = 20; cp >= 0; --cp) {
     ctx->class_launched[cp] = false;
     if (ctx->cls_q[cp] == 0) continue;
     int hi = 0;

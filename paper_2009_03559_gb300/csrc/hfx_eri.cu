@@ -1,7 +1,8 @@
-// ERI kernels: one class launch evaluates every screened quartet of one class pair
-// (bra pair bin >= ket pair bin) -- of one system, or of all systems of a batch -- and
-// digests it into the half exchange matrix, or, in diagonal mode, evaluates (p|p) for
-// candidate pairs and stores the Schwarz factor.
+// Class launches: one evaluates every screened quartet of one class pair (bra pair bin >= ket
+// pair bin) -- of one system, or of all systems of a batch -- and digests it into the half
+// exchange matrix, or, in diagonal mode, evaluates (p|p) for candidate pairs and stores the
+// Schwarz factor.  Here: the thread kernel (one quartet per thread, on request), and which
+// kernel, chunk and overlap a launch gets; the default kernel is the Hermite engine (hfx_md.cu).
 #include <algorithm>
 #include <cstdio>
 #include <type_traits>
@@ -408,7 +409,7 @@ int eri_chunk(int gs, long long n_quartets, long long n_groups) {
 
 // Whether the next class launch of a build is let start before a launch of n_quartets on n_groups
 // warps has ended.  Below 32 quartets a warp the launch is mostly ramp and tail (3-atom diamond build
-// 1.14 -> 0.52 ms, 8 atoms 8.6 -> 8.1 ms); above, two classes sharing the SMs cost more than the
+// 1.14 -> 0.52 ms, 8 atoms 8.6 -> 8.1 ms; then 0.41 and 7.9 with the longest classes first); above, two classes sharing the SMs cost more than the
 // tail (64 atoms 1779 -> 1815 ms when all overlapped).
 bool eri_overlap(int gs, long long n_quartets, long long n_groups) { return gs != 1 && n_quartets < 32 * n_groups; }
 
