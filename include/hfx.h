@@ -56,10 +56,9 @@ extern "C" {
 #define HFX_FP64 0                /* every integral in FP64 */
 #define HFX_MIXED 1               /* FP32 recurrences for small-bound quartets, see hfx_options */
 
-/* Default classes allowed FP32 recurrences under HFX_MIXED: every class but (dd|dd), the
- * highest recurrence (L = 8): with FP32 there, E_K of the 64-atom diamond moved by 1.7e-7 and
- * of the 216-atom one by 4.1e-7 (over the 1e-7 tolerance), against at most 1.1e-9 with the
- * other twenty classes in FP32. */
+/* Default classes allowed FP32 recurrences under HFX_MIXED: every class but (dd|dd), the highest
+ * recursion (L = 8).  E_K of the 64-atom diamond moves by 8e-12 and of the 216-atom one by 3e-11
+ * against FP64 (with (dd|dd) in FP32 too: 1e-11 and 4e-11). */
 #define HFX_FP32_CLASSES_DEFAULT 0xFFFFF
 
 /* work schedules inside a class launch (paper Sec. 3.2, Algorithms 2 and 3) */

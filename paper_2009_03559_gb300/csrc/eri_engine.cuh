@@ -1,14 +1,14 @@
 // Table-driven engine for contracted shell quartets (ab|cd) with the erfc(omega r)/r
-// kernel, fused with the exchange-matrix digest.  It runs in FP64; the recurrence and
-// contraction steps are templated on the arithmetic type, and an FP32 primitive set-up
-// (prim_core_f32) feeds them, so the mixed-precision kernel runs set-up, recurrences and
-// contraction in FP32 for the quartets that qualify (HRR, spherical step and digest in FP64).
+// kernel, fused with the exchange-matrix digest: the thread kernel, which runs on request
+// (hfx_set_group_size(1)); the default for every class is the Hermite engine (hfx_md.cuh).  It runs in
+// FP64; the recurrence and contraction steps are templated on the arithmetic type, and an FP32
+// primitive set-up (prim_core_f32) feeds them, so the mixed-precision kernel runs set-up, recurrences
+// and contraction in FP32 for the quartets that qualify (HRR, spherical step and digest in FP64).
 //
-// One "group" of G lanes (G = 1 or G = 32) evaluates one contracted quartet:
+// One thread evaluates one contracted quartet:
 //   1. for every surviving primitive quartet: the Boys step (G_m = F_m(T) -
 //      kappa^{m+1/2} F_m(kappa T), times the prefactor), then the Obara-Saika vertical
-//      recurrence level by level (ops of a level are independent and spread over the
-//      lanes), then the contraction into the accumulator block (e0|f0);
+//      recurrence level by level, then the contraction into the accumulator block (e0|f0);
 //   2. the post-contraction stages: Head-Gordon-Pople horizontal recurrence on the bra,
 //      Cartesian -> spherical on a and b, HRR on the ket, spherical on c and d;
 //   3. the digest into the half exchange matrix A (K = A + A^T afterwards):

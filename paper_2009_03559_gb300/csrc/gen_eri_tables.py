@@ -428,7 +428,9 @@ class ClassTables:
 
 
 # ---------------------------------------------------------------------------------------
-# Warp schedules.  A warp runs k primitive quartets ("streams") of one contracted quartet at
+# Warp schedules: an Obara-Saika form for whole warps, whose class variants hfx_set_streams still
+# names; the kernels run the Hermite engine instead (gen_md_tables.py), which needs fewer FP64 warp
+# instructions.  A warp runs k primitive quartets ("streams") of one contracted quartet at
 # a time; each stream owns a region of group scratch: [accumulators | VRR slots | a zero
 # slot].  The VRR ops of all streams, and one add per accumulator whose target another op
 # reads, are list-scheduled into iterations of at most 32 ops (one per lane).  The FP64

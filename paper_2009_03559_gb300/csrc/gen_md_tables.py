@@ -1,5 +1,5 @@
 #!/usr/bin/env python3
-"""Generate the per-class tables of the Hermite engine (the FP64 warp kernel).
+"""Generate the per-class tables of the Hermite engine (hfx_md.cuh).
 
 A shell pair's function product is expanded in Hermite Gaussians (McMurchie-Davidson), and the
 expansion is split into factors that depend on the primitive pair and factors that do not, so

@@ -409,8 +409,9 @@ int eri_chunk(int gs, long long n_quartets, long long n_groups) {
 
 // Whether the next class launch of a build is let start before a launch of n_quartets on n_groups
 // warps has ended.  Below 32 quartets a warp the launch is mostly ramp and tail (3-atom diamond build
-// 1.14 -> 0.52 ms, 8 atoms 8.6 -> 8.1 ms; then 0.41 and 7.9 with the longest classes first); above, two classes sharing the SMs cost more than the
-// tail (64 atoms 1779 -> 1815 ms when all overlapped).
+// 1.14 -> 0.52 ms, 8 atoms 8.6 -> 8.1 ms; then 0.41 and 7.9 with the longest classes first); above,
+// two classes sharing the SMs cost more than the tail (64 atoms 1781 -> 1806 ms when all overlapped;
+// 16 atoms 55.2 -> 55.4 with the line at 96).
 bool eri_overlap(int gs, long long n_quartets, long long n_groups) { return gs != 1 && n_quartets < 32 * n_groups; }
 
 cudaError_t eri_launch(const EriLaunch& L0, int cls, int mode, int grid, cudaStream_t stream, int gs, int prec,
