@@ -64,7 +64,8 @@ constexpr int kMatLd = kMaxUnknowns + 1;
 constexpr int kMatDoubles = kMaxUnknowns * kMatLd + kMatLd;  // matrix + right-hand side
 constexpr int kMaxNr = 1024;
 constexpr int kMaxPop = 64;
-constexpr int kWarps = 4;  // warps per block at most
+constexpr int kWarps = 4;         // warps per block at most,
+constexpr int kGeneticWarps = 8;  // in the genetic step
 constexpr size_t kMaxBlockSmem = 227 * 1024;
 
 constexpr double kRidge = 1e-12;
@@ -464,11 +465,10 @@ __device__ __forceinline__ void gene_factors(int j0, int j1, int tid, double h2,
 // gene its factors.  Which warp is first turns with the block and the generation (a warp sits on
 // one quarter of the SM, and the first has the genes to make and the odd individual to evaluate).
 // Against a restart per warp: 1280 restarts are 8.4 to an SM, which with 8 resident warps took a
-// second pass that was nearly empty, and the shared targets and populations leave room for 12
-// warps per SM instead of 8 (M = 3, 512 points, population 32).  10 functions: 46.5 -> 33.4 ms
-// of FP64 pipe time 28 ms; 20 functions x 512 restarts: 257 -> 250 ms (67 to an SM).
+// second pass that was nearly empty (M = 3, 512 points, population 32: 10 functions 46.5 -> 32.9 ms
+// of FP64 pipe time 28 ms; 20 functions x 512 restarts, 67 to an SM: 257 -> 248 ms).
 template <int M, bool STORE>
-__global__ void __launch_bounds__(kWarps * 32) nao_genetic_kernel(NaoArgs A) {
+__global__ void __launch_bounds__(kGeneticWarps * 32) nao_genetic_kernel(NaoArgs A) {
   const int lane = threadIdx.x & 31;
   const int W = blockDim.x >> 5;
   const long long q = blockIdx.x;
@@ -867,12 +867,18 @@ const void* kernel_for(int M, Which w, bool store) {
 int launch(Which w, int M, const NaoArgs& a, long long n, cudaStream_t s) {
   if (n <= 0) return HFX_OK;
   // warps per block: as many as the shared memory of a block holds, up to kWarps; in the genetic
-  // step no more than a generation has new individuals
+  // step up to 8, and of these as few as take a generation's new individuals in the same number of
+  // rounds (31 individuals, 512 points: 4 warps 33.4 ms, 6 34.0, 8 32.9, 11 32.8; 256 points: 4
+  // warps 40.9, 8 38.0, 11 38.1, 16 44.1)
   const size_t shared = (size_t)block_smem_doubles(w, M, a.npad, a.P) * sizeof(double);
   auto per_warp = [&](bool store) { return (size_t)warp_smem_doubles(w, M, a.npad, store) * sizeof(double); };
   auto warps_per_block = [&](bool store) {
     const size_t fit = shared < kMaxBlockSmem ? (kMaxBlockSmem - shared) / per_warp(store) : 0;
-    return (int)std::min<size_t>(w == kGenetic ? std::min(kWarps, a.P - 1) : kWarps, fit);
+    if (w != kGenetic) return (int)std::min<size_t>(kWarps, fit);
+    const int most = (int)std::min<size_t>(kGeneticWarps, fit);
+    if (most == 0) return 0;
+    const int rounds = (a.P - 2 + most) / most;
+    return (a.P - 2 + rounds) / rounds;
   };
   // warps an SM holds by shared memory (228 KB, 1 KB of it per block reserved)
   auto resident = [&](bool store) {

@@ -186,9 +186,9 @@ def test_largest_options(fitter):
     assert out["err"][0] == pytest.approx(ref["best"]["err"], rel=1e-6)
 
 
-@pytest.mark.parametrize("P", [2, 3, 4, 5, 33, 64])
+@pytest.mark.parametrize("P", [2, 3, 4, 5, 9, 10, 33, 64])
 def test_genetic_step_at_block_shapes(fitter, P):
-    """Populations that give blocks of one, two, three and four warps, a remainder of individuals per
+    """Populations that give blocks of one warp, of a few and of eight, a remainder of individuals per
     warp, more individuals than lanes."""
     hfx, rs, F = fitter
     r = N.grid(rs.phi.shape[1], rs.h)
