@@ -740,8 +740,8 @@ def main():
                                   "counts of the generated tables); Boys evaluations counted apart"
                                   + ("; FP32 flops counted at the FP64/FP32 peak ratio" if mixed else ""),
                          "traffic": None,
-                         "traffic_note": "not taken in this run; ncu on one 16-atom launch of this kernel "
-                                         "(dp|dp): 1.43 MB read + 0.34 MB written, L2 hit rate 99%",
+                         "traffic_note": "not taken in this run; ncu on one 24-atom launch of this kernel "
+                                         "(dp|dp): 4.1 MB read, none written back, L2 hit rate 98%",
                          "peak_source": "FP64 FMA-chain probe of this run (hfx_measure_fma_peak)",
                          "with_setup": {"achieved": achieved_all, "frac": (achieved_all / fp64_peak) if achieved_all
                                         else None, "flops": "the same plus the primitive set-up as written "
