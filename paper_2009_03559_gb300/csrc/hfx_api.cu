@@ -74,13 +74,21 @@ extern "C" int hfx_init_basis(hfx_ctx** out, int n_atoms, const double* xyz, int
   return init_basis_impl(out, n_atoms, xyz, n_shells, shell_atom, shell_l, shell_nprim, alpha, coef, opt, stream);
 }
 
-// Quartet classes whose FP32 pass stays in FP32's range.  A Hermite integral of order up to L is at
-// most C_ab C_cd (2 rho)^{L/2} / sqrt(p+q) <= f_ab f_cd with f_ab = C_ab p^{(L-1)/4} (rho <= sqrt(pq)/2)
-// and C_ab ~ w_a w_b / p, w = (8 alpha)^{(2l+3)/4} for a normalised shell; f grows with both exponents
-// (for L < 5 after p^{-z} <= (4ab)^{-z/2}), so the extremes of the shells' exponents bound it.  1e34 and 1e-22
-// leave room for contraction weights, and for integrals far below the largest of their quartet.
-// (d shells up to 7e3 in (dd|dd), p shells up to 1e8 in (pp|pp); beyond, the class runs in FP64.)
-static int fp32_range_mask(int n_shells, const int* l, const int* nprim, const double* alpha) {
+// Ranges of the Hermite integrals of a basis.  One of order up to L is at most C_ab C_cd (2 rho)^k / sqrt(p+q),
+// k = L in FP64 and L/2 in FP32 (scaled recursion), and so at most f_ab f_cd with f_ab = C_ab p^{(2k-1)/4}
+// (rho <= sqrt(pq)/2) and C_ab ~ w_a w_b / p, w = (8 alpha)^{(2l+3)/4} for a normalised shell; f grows with
+// both exponents (for 2k < 5 after p^{-z} <= (4ab)^{-z/2}), so the extremes of the shells' exponents bound it.
+struct HermiteRange {
+  // Classes whose FP32 pass stays in FP32's range: 1e34 and 1e-22 leave room for contraction weights, and for
+  // integrals far below the largest of their quartet.  (d shells up to 7e3 in (dd|dd), p shells up to 1e8 in
+  // (pp|pp); beyond, the class runs in FP64.)
+  int fp32_mask = 0;
+  // FP64: the integrals are held times 2^hexp (even; PrimPair::C), 0 unless exponents beyond 1e22 or below
+  // 1e-20 (d shells) could leave FP64's range; no FP32 pass then.
+  int hexp = 0;
+};
+
+static HermiteRange hermite_range(int n_shells, const int* l, const int* nprim, const double* alpha) {
   double lo[3] = {1e300, 1e300, 1e300}, hi[3] = {0.0, 0.0, 0.0};
   for (int s = 0, k = 0; s < n_shells; ++s)
     for (int i = 0; i < nprim[s]; ++i, ++k) {
@@ -88,12 +96,12 @@ static int fp32_range_mask(int n_shells, const int* l, const int* nprim, const d
       hi[l[s]] = std::max(hi[l[s]], alpha[k]);
     }
   const int pl[6][2] = {{0, 0}, {1, 0}, {1, 1}, {2, 0}, {2, 1}, {2, 2}};
-  int mask = 0;
+  HermiteRange range;
+  double most = 0.0, least = 0.0;  // log10, over the classes
   for (int b = 0; b < 6; ++b)
     for (int k = 0; k <= b; ++k) {
       const int L = pl[b][0] + pl[b][1] + pl[k][0] + pl[k][1];
-      const double z = (L - 5) / 4.0;
-      auto size = [&](const double* a) {  // log10 of the bound, all exponents at a[l]
+      auto size = [&](const double* a, double z) {  // log10 of the bound, all exponents at a[l]
         double v = 0.0;
         for (const int* p : {pl[b], pl[k]}) {
           const double x = a[p[0]], y = a[p[1]];
@@ -104,9 +112,18 @@ static int fp32_range_mask(int n_shells, const int* l, const int* nprim, const d
       };
       bool present = true;
       for (const int* p : {pl[b], pl[k]}) present = present && hi[p[0]] > 0.0 && hi[p[1]] > 0.0;
-      if (!present || (size(hi) < 34.0 && size(lo) > -22.0)) mask |= 1 << (b * (b + 1) / 2 + k);
+      const double z32 = (L - 5) / 4.0, z64 = (2 * L - 5) / 4.0;
+      if (!present || (size(hi, z32) < 34.0 && size(lo, z32) > -22.0)) range.fp32_mask |= 1 << (b * (b + 1) / 2 + k);
+      if (present) {
+        most = std::max(most, size(hi, z64));
+        least = std::min(least, size(lo, z64));
+      }
     }
-  return mask;
+  // decades to scale by: down to 1e285, or up to 1e-250 as far as the largest allow it
+  const double shift = most > 285.0 ? 285.0 - most : least < -250.0 ? std::min(-250.0 - least, 285.0 - most) : 0.0;
+  range.hexp = 2 * (int)std::max(-500.0, std::min(500.0, std::floor(0.5 * shift * std::log2(10.0))));
+  if (range.hexp) range.fp32_mask = 0;
+  return range;
 }
 
 static int init_basis_impl(hfx_ctx** out, int n_atoms, const double* xyz, int n_shells, const int* shell_atom,
@@ -174,7 +191,9 @@ static int init_basis_impl(hfx_ctx** out, int n_atoms, const double* xyz, int n_
   ctx->n_bf = nb;
   ctx->n_prim = np;
   ctx->h_l.assign(shell_l, shell_l + n_shells);
-  ctx->fp32_range = fp32_range_mask(n_shells, shell_l, shell_nprim, alpha);
+  const HermiteRange range = hermite_range(n_shells, shell_l, shell_nprim, alpha);
+  ctx->fp32_range = range.fp32_mask;
+  ctx->hexp = range.hexp;
   cudaDeviceGetAttribute(&ctx->n_sm, cudaDevAttrMultiProcessorCount, dev);
   auto bail = [&](int code) {
     g_init_err = ctx->err;
@@ -254,6 +273,7 @@ EriLaunch hfx::base_launch(hfx_ctx* ctx) {
   L.pa.prim = ctx->d_pp;
   L.pa.md_off = ctx->d_md_off;
   L.pa.md = ctx->d_md;
+  L.unscale = std::ldexp(1.0, -ctx->hexp);
   L.sh.bf_off = ctx->d_bf_off;
   L.sh.atom = ctx->d_atom;
   L.boys = ctx->d_boys;
@@ -349,10 +369,10 @@ extern "C" int hfx_build_pairs(hfx_ctx* ctx) {
   const long long n_pp = (long long)last[0] + last[1];
   RK(ctx->alloc(&ctx->d_pp, n_pp, true));
   CK(launch_prim_fill(n_cand, ctx->d_sa, ctx->d_sb, ctx->d_nprim, ctx->d_prim_off, ctx->d_atom, ctx->d_xyz,
-                      ctx->d_alpha, ctx->d_w, ctx->d_pp_off, ctx->opt.prim_tau, ctx->d_pp, ctx->d_pp_n, s));
+                      ctx->d_alpha, ctx->d_w, ctx->d_pp_off, ctx->opt.prim_tau, ctx->hexp, ctx->d_pp, ctx->d_pp_n, s));
   RK(ctx->alloc(&ctx->d_md, (size_t)n_md, true));
-  CK(launch_md_fill(n_cand, ctx->d_pcls, ctx->d_AB, ctx->d_pp_off, ctx->d_pp_n, ctx->d_pp, ctx->d_md_off, ctx->d_md,
-                    s));
+  CK(launch_md_fill(n_cand, ctx->d_pcls, ctx->d_AB, ctx->d_pp_off, ctx->d_pp_n, ctx->d_pp, ctx->d_md_off,
+                    ctx->hexp, ctx->d_md, s));
   // 3. group candidates by pair class, Schwarz diagonal per class
   int *d_iota, *d_ckey, *d_cidx, *d_cnt;
   RK(ctx->alloc(&d_iota, n_cand, true));

@@ -24,8 +24,9 @@ struct hfx_ctx {
   int n_atoms = 0, n_shells = 0, n_bf = 0, n_prim = 0, n_sm = 0;
   std::vector<int> h_l;
   // Classes whose quartets may take the FP32 pass: the option's mask, less the classes whose Hermite
-  // integrals could leave FP32's range for the exponents of this basis (fp32_range_mask)
+  // integrals could leave FP32's range for the exponents of this basis (hermite_range)
   int fp32_range = 0;
+  int hexp = 0;  // see PrimPair::C
   int fp32_mask() const { return opt.fp32_class_mask & fp32_range; }
   // basis (device)
   double *d_xyz = nullptr, *d_alpha = nullptr, *d_coef = nullptr, *d_w = nullptr, *d_boys = nullptr;

@@ -179,7 +179,7 @@ __device__ __forceinline__ void g1_quartet(const EriClassInfo& ci, const EriLaun
     ++t.q32;
     t.p32 += ne;
   }
-  double deg = 1.0;
+  double deg = Ls.unscale;
   if (sa == sb) deg *= 0.5;
   if (sc == sd) deg *= 0.5;
   if (bra_s == ket_s) deg *= 0.5;

@@ -35,7 +35,7 @@ cudaError_t md_launch(const EriLaunch& L, int cls, int kind, int prec, bool f32,
                       bool overlap);
 cudaError_t launch_md_size(int n, const int* pcls, const int* cap, long long* size, cudaStream_t s);
 cudaError_t launch_md_fill(int n, const int* pcls, const double* AB, const int* pp_off, const int* pp_n,
-                           const PrimPair* pp, const long long* md_off, double* md, cudaStream_t s);
+                           const PrimPair* pp, const long long* md_off, int hexp, double* md, cudaStream_t s);
 
 }  // namespace hfx
 

@@ -73,6 +73,8 @@ constexpr int kBoysTableLen = (kBoysRows + kBoysTailRows) * kBoysRowLen;   // do
 // Primitive-pair record (one per surviving primitive pair of a shell pair).
 // C = sqrt(2) pi^{5/4} w_a w_b exp(-ab/p |AB|^2) / p so that the primitive
 // quartet prefactor 2 pi^{5/2} K_ab K_cd / (p q sqrt(p+q)) = C_ab C_cd / sqrt(p+q).
+// For a basis whose Hermite integrals could leave FP64's range (hfx_ctx::hexp, 0 for any other) C is held
+// times 2^{hexp/2}; the transformation coefficients T of a pair (PairArrays::md) carry the inverse.
 // ---------------------------------------------------------------------------
 struct __align__(16) PrimPair {
   double p, inv2p;     // exponent sum and 1/(2p)
@@ -277,6 +279,7 @@ struct EriLaunch {
   int chunk;                  // schedule 2: quartets per claim
   const double* boys;         // kMaxLt + 1 tables of kBoysTableLen doubles
   double omega, omega2;
+  double unscale;             // 2^-hexp (see PrimPair::C): the thread kernel's factor for its integrals
   MdClassInfo mc;              // Hermite engine: the steps of this class
   int prec;                    // precision pass (PREC_*)
   const double* P;

@@ -1,5 +1,6 @@
 // Host side of the Hermite engine: class descriptions, launches, and the pair data it reads.
 #include <algorithm>
+#include <cmath>
 #include "hfx_md.cuh"
 #include "hfx_eri.h"
 
@@ -99,7 +100,7 @@ cudaError_t md_launch(const EriLaunch& L0, int cls, int kind, int prec, bool f32
 }
 
 // ---------------------------------------------------------------------------
-// Pair data: per candidate pair the coefficients T of its type (polynomials in AB), then the
+// Pair data: per candidate pair the coefficients T of its type (polynomials in AB, times `scale`), then the
 // factors W_s = u_b^i u_a^j (1/2p)^e of its surviving primitive pairs.
 // ---------------------------------------------------------------------------
 struct MdPairs {
@@ -124,7 +125,7 @@ __global__ void k_md_size(int n, const int* __restrict__ pcls, const int* __rest
 __global__ void k_md_fill(int n, const int* __restrict__ pcls, const double* __restrict__ AB,
                           const int* __restrict__ pp_off, const int* __restrict__ pp_n,
                           const PrimPair* __restrict__ pp, const long long* __restrict__ md_off, const MdPairs info,
-                          double* __restrict__ md) {
+                          double scale, double* __restrict__ md) {
   const int c = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (c >= n) return;
   const MdPairInfo& t = info.t[pcls[c]];
@@ -148,7 +149,7 @@ __global__ void k_md_fill(int n, const int* __restrict__ pcls, const double* __r
       for (int j = 0; j < deg - px - py; ++j) w *= x[2];
       v += w;
     }
-    out[i] = v;
+    out[i] = v * scale;
   }
   out += t.n_coef;
   const PrimPair* p = pp + pp_off[c];
@@ -168,8 +169,9 @@ cudaError_t launch_md_size(int n, const int* pcls, const int* cap, long long* si
 }
 
 cudaError_t launch_md_fill(int n, const int* pcls, const double* AB, const int* pp_off, const int* pp_n,
-                           const PrimPair* pp, const long long* md_off, double* md, cudaStream_t s) {
-  k_md_fill<<<(n + 3) / 4, 128, 0, s>>>(n, pcls, AB, pp_off, pp_n, pp, md_off, pair_infos(), md);
+                           const PrimPair* pp, const long long* md_off, int hexp, double* md, cudaStream_t s) {
+  k_md_fill<<<(n + 3) / 4, 128, 0, s>>>(n, pcls, AB, pp_off, pp_n, pp, md_off, pair_infos(),
+                                              std::ldexp(1.0, -hexp / 2), md);
   return cudaGetLastError();
 }
 

@@ -193,7 +193,7 @@ __global__ void k_prim_fill(int n_cand, const int* __restrict__ sa, const int* _
                             const int* __restrict__ nprim, const int* __restrict__ prim_off_shell,
                             const int* __restrict__ atom, const double* __restrict__ xyz,
                             const double* __restrict__ alpha, const double* __restrict__ w,
-                            const int* __restrict__ pp_off, double prim_tau, PrimPair* __restrict__ pp,
+                            const int* __restrict__ pp_off, double prim_tau, double scale, PrimPair* __restrict__ pp,
                             int* __restrict__ pp_n) {
   const int c = (blockIdx.x * blockDim.x + threadIdx.x) / G, lane = threadIdx.x % G;
   if (c >= n_cand) return;  // whole groups leave together
@@ -222,7 +222,7 @@ __global__ void k_prim_fill(int n_cand, const int* __restrict__ sa, const int* _
         r.P[i] = (ea * A[i] + eb * B[i]) / p;
         r.PA[i] = r.P[i] - A[i];
       }
-      r.C = C;
+      r.C = C * scale;
       r.inv2p3 = 1.5 / p;
       r.ua = ea / p;
       r.ub = eb / p;
@@ -682,7 +682,7 @@ cudaError_t scan_ll_inclusive(void* tmp, size_t& tmp_bytes, const long long* in,
 
 cudaError_t launch_prim_fill(int n_cand, const int* sa, const int* sb, const int* nprim, const int* prim_off_shell,
                              const int* atom, const double* xyz, const double* alpha, const double* w,
-                             const int* pp_off, double prim_tau, PrimPair* pp, int* pp_n, cudaStream_t s) {
+                             const int* pp_off, double prim_tau, int hexp, PrimPair* pp, int* pp_n, cudaStream_t s) {
   if (n_cand <= 0) return cudaSuccess;
   // 16 lanes a shell pair (9 primitive pairs at the usual 3 a shell) while these threads are all
   // resident at once (152 SMs x 2048): one round instead of nine, 45 -> 10 us for 171 pairs.  With
@@ -690,7 +690,8 @@ cudaError_t launch_prim_fill(int n_cand, const int* sa, const int* sb, const int
   constexpr int kWide = 152 * 2048 / 16;
   auto k = n_cand <= kWide ? k_prim_fill<16> : k_prim_fill<1>;
   k<<<nblk((n_cand <= kWide ? 16ll : 1ll) * n_cand, 128), 128, 0, s>>>(n_cand, sa, sb, nprim, prim_off_shell, atom, xyz,
-                                                                       alpha, w, pp_off, prim_tau, pp, pp_n);
+                                                                       alpha, w, pp_off, prim_tau,
+                                                                       std::ldexp(1.0, hexp / 2), pp, pp_n);
   return cudaGetLastError();
 }
 

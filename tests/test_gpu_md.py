@@ -72,6 +72,35 @@ def test_mixed_build_at_the_ends_of_the_fp32_range(hfx_mod, alpha):
     assert n32[0] > 0 and n32[20] == 0  # (ss|ss) within, (dd|dd) beyond
 
 
+# (2 rho)^L G leaves FP64's range beyond 4e24 and below 1e-25 in (dd|dd); 1e22 is where scaling begins.  The
+# atoms lie an orbital's width apart.  The attenuated kernel cancels at 1e-30, so Coulomb there; no primitive
+# pair is dropped by the oracle.
+@pytest.mark.parametrize("alpha,omega", [(5e21, 0.11), (2e22, 0.11), (1e25, 0.11), (1e34, 0.11), (1e-30, 0.0)])
+@pytest.mark.parametrize("mixed", [False, True])
+def test_exponents_at_the_ends_of_the_fp64_range(hfx_mod, alpha, omega, mixed):
+    xyz = np.array([[0.0, 0.0, 0.0], [0.4, 0.5, -0.3]]) / np.sqrt(alpha)
+    s = inputs.System("pair", xyz, np.repeat([0, 1], 3).astype(np.int32), np.array([0, 1, 2] * 2, np.int32),
+                      np.ones(6, np.int32), alpha * np.array([1.0, 0.7, 0.9, 0.8, 1.0, 0.6]), np.ones(6), omega=omega,
+                      tau=0.0)
+    P = np.ones((s.n_bf, s.n_bf)) + np.eye(s.n_bf)
+    kw = dict(precision=hfx_mod.HFX_MIXED, fp32_class_mask=hfx_mod.ALL_CLASS_MASK) if mixed else {}
+    h = check(hfx_mod, s, P, 1e-12, prim_tau=0.0, **kw)
+    if not mixed:
+        Ko, _ = oracle.Screen(oracle.Basis(s)).build_K(P, "sym")
+        for cls in range(6):  # ss, ps and pp pairs in the thread kernel
+            h.set_group_size(cls, 1)
+        K1 = h.build_K(torch.from_numpy(P).cuda()).cpu().numpy()
+        assert np.abs(K1 - Ko).max() <= 1e-12 * np.abs(Ko).max()
+        # the same from a batch with an ordinary system beside it
+        s2 = inputs.diamond_system(1, seed=7, tau=1e-12)
+        h2 = hfx_mod.HFX(s2).build_pairs()
+        P2 = torch.from_numpy(inputs.density_matrix(s2)).cuda()
+        K = [torch.empty_like(P2), torch.empty(P.shape, dtype=torch.float64, device="cuda")]
+        hfx_mod.Batch([h2, h]).run([P2, torch.from_numpy(P).cuda()], K)
+        torch.cuda.synchronize()
+        assert np.abs(K[1].cpu().numpy() - Ko).max() <= 1e-12 * np.abs(Ko).max()
+
+
 @pytest.mark.parametrize("mixed", [False, True])
 def test_build_inside_a_captured_graph(hfx_mod, mixed):
     """Overlapping class launches (a small system) as a captured graph, replayed for another density."""
