@@ -20,7 +20,7 @@ INCLUDE = os.path.join(ROOT, "include")
 SOURCES = ["hfx_api.cu", "hfx_eri.cu", "hfx_setup.cu", "hfx_batch.cu", "hfx_noalloc.cu", "hfx_nao.cu",
            "hfx_md_api.cu"]
 MD_SOURCE = "hfx_md.cu"  # compiled once per total angular momentum 0..8 (the slowest first)
-HEADERS = ["hfx_internal.cuh", "eri_engine.cuh", "eri_tables.inc", "eri_quartets.cuh", "eri_prim.cuh", "hfx_md.cuh",
+HEADERS = ["hfx_internal.cuh", "boys.cuh", "eri_engine.cuh", "eri_tables.inc", "eri_quartets.cuh", "eri_prim.cuh", "hfx_md.cuh",
            "gen_md_tables.py", "hfx_eri.h", "hfx_setup.h", "hfx_ctx.h"]
 ARCH = "-gencode=arch=compute_103a,code=sm_103a"
 

@@ -33,9 +33,8 @@ __device__ __forceinline__ bool prim_core(const PrimPair& b, const PrimPair& k, 
   ps.PQ[2] = op.sub(b.P[2], k.P[2]);
   const double T = op.mul(rho, fma(ps.PQ[0], ps.PQ[0], fma(ps.PQ[1], ps.PQ[1], op.mul(ps.PQ[2], ps.PQ[2]))));
   const double pref = op.mul(op.mul(b.C, k.C), y);
-  const double* tabL = tabs + Lt * kBoysTableLen;
   double F1, e1;
-  boys_any(Lt, T, tabL, F1, e1, op);
+  boys_any(Lt, T, tabs, F1, e1, op);
   const double T2 = op.add(T, T);
   if (omega2 > 0.0) {
     const double sk = op.mul(omega, rsqrt_nr(op.add(rho, omega2), op));   // sqrt(kappa)
@@ -43,7 +42,7 @@ __device__ __forceinline__ bool prim_core(const PrimPair& b, const PrimPair& k, 
     const double kT = op.mul(kap, T);
     if (ge_hi(kT, kBoysXmaxHi)) return false;
     double F2, e2;
-    boys_top(kT, tabL, F2, e2, op);
+    boys_top(Lt, kT, tabs, F2, e2, op);
     // c[m] = pref kappa^{m-1/2}, m = 1..Lt+1
     double c[kMaxLt + 2];
     c[1] = op.mul(pref, sk);

@@ -203,7 +203,7 @@ static int init_basis_impl(hfx_ctx** out, int n_atoms, const double* xyz, int n_
   int r;
   if ((r = ctx->alloc(&ctx->d_xyz, 3 * (size_t)n_atoms)) || (r = ctx->alloc(&ctx->d_alpha, np)) ||
       (r = ctx->alloc(&ctx->d_coef, np)) || (r = ctx->alloc(&ctx->d_w, np)) ||
-      (r = ctx->alloc(&ctx->d_boys, (size_t)(kMaxLt + 1) * kBoysTableLen)) || (r = ctx->alloc(&ctx->d_atom, n_shells)) ||
+      (r = ctx->alloc(&ctx->d_boys, (size_t)kBoysDoubles)) || (r = ctx->alloc(&ctx->d_atom, n_shells)) ||
       (r = ctx->alloc(&ctx->d_l, n_shells)) || (r = ctx->alloc(&ctx->d_nprim, n_shells)) ||
       (r = ctx->alloc(&ctx->d_prim_off, n_shells)) || (r = ctx->alloc(&ctx->d_bf_off, n_shells)) ||
       (r = ctx->alloc(&ctx->d_energy, 1)) || (r = ctx->alloc(&ctx->d_busy, 1024)) ||

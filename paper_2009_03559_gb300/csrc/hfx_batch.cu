@@ -39,6 +39,7 @@ struct BatchWork {
   bool mixed = false, pmax = false;
   bool fp32_class[21] = {};  // some system may run this class with FP32 recurrences
   long long total[21] = {};
+  const double* boys = nullptr;  // the Boys tables: the first system's serve all
   int gs[21] = {}, chunk[21] = {};  // lanes per quartet and dynamic chunk per class (0 = eri_chunk)
   int streams[21] = {};             // warp kernel: primitive quartets at a time (0 = default)
   EriLaunch *d_launch = nullptr, *h_launch = nullptr;
@@ -97,6 +98,7 @@ void bw_fill(BatchWork& w, hfx_ctx* const* ctxs, int n, double* const* pmax, dou
   w.pmax = false;
   for (int s = 0; s < n; ++s)
     w.pmax = w.pmax || mixed || ctxs[s]->opt.skip_zero_p || ctxs[s]->opt.density_tau > 0.0;
+  w.boys = ctxs[0]->d_boys;
   w.mixed = false;
   for (int cp = 0; cp < 21; ++cp) {
     w.fp32_class[cp] = false;
@@ -203,6 +205,7 @@ EriLaunch bw_class_launch(const BatchWork& w, int cp, int pass = 0) {
   L.work = w.d_work + cp + 21 * pass;
   L.chunk = bw_chunk(w, cp, bw_prec(w, cp, pass));
   L.n_sys = w.n;
+  L.boys = w.boys;
   L.seg = w.d_seg + (size_t)cp * (w.cap + 1);
   L.batch = w.d_launch + (size_t)cp * w.cap;
   return L;

@@ -210,7 +210,6 @@ __device__ __forceinline__ bool md_setup(const PrimPair& b, const PrimPair& k, c
   const double R2 = fma(PQ[0], PQ[0], fma(PQ[1], PQ[1], op.mul(PQ[2], PQ[2])));
   const double T = op.mul(rho, R2);
   const double pref = op.mul(op.mul(b.C, k.C), y);
-  const double* tabL = tabs + L * kBoysTableLen;
   double kap = 0.0, sk = 0.0, kT = 0.0;
   if (omega2 > 0.0) {
     sk = op.mul(omega, rsqrt_nr(op.add(rho, omega2), op));  // sqrt(kappa)
@@ -219,7 +218,7 @@ __device__ __forceinline__ bool md_setup(const PrimPair& b, const PrimPair& k, c
     if (ge_hi(kT, kBoysXmaxHi)) return false;
   }
   double F1, e1;
-  boys_any(L, T, tabL, F1, e1, op);
+  boys_any(L, T, tabs, F1, e1, op);
   const double r2 = scale2(rho, 1);
   double pL = pref;  // pref (2 rho)^L
   if constexpr (L > 0) {
@@ -237,7 +236,7 @@ __device__ __forceinline__ bool md_setup(const PrimPair& b, const PrimPair& k, c
   for (int m = 1; m < L; ++m) a[m] = op.mul(a[m - 1], r2);
   if (omega2 > 0.0) {
     double F2, e2;
-    boys_top(kT, tabL, F2, e2, op);
+    boys_top(L, kT, tabs, F2, e2, op);
     const double kr = op.mul(kap, r2);
     double c[L + 1];
     c[0] = op.mul(pref, sk);
@@ -721,7 +720,7 @@ __global__ void __launch_bounds__(md_block(LT), md_minb<R>(LT))
           }
           // (a kernel parameter is a constant operand: one product makes it a register's)
           const double om = KIND == MD_BATCH ? Ls.omega : omega, om2 = KIND == MD_BATCH ? Ls.omega2 : omega2;
-          ok = md_setup<LT>(*pb, *pk, qc, om, om2, Ls.boys, B, PQ, op);
+          ok = md_setup<LT>(*pb, *pk, qc, om, om2, L.boys, B, PQ, op);
         }
       }
       okm = __ballot_sync(0xffffffffu, ok);
@@ -763,7 +762,7 @@ __global__ void __launch_bounds__(md_block(LT), md_minb<R>(LT))
           const EriLaunch& Ls = prims(t, pb, pk);
           double G[kMaxLt + 1];
           PrimScalars ps;
-          if (prim_core(*pb, *pk, LT, Ls.omega, Ls.omega2, Ls.boys, G, ps, op)) {
+          if (prim_core(*pb, *pk, LT, Ls.omega, Ls.omega2, L.boys, G, ps, op)) {
 #pragma unroll
             for (int k = 0; k <= LT; ++k) X[(sub * NX + k) * 32 + l] = to_f32_rn(G[k]);
             atomicOr(Xok + sub, 1u << l);

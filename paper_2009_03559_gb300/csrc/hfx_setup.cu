@@ -39,62 +39,23 @@ __global__ void k_normalize(int n_shells, const int* __restrict__ l, const int* 
 }
 
 // ---------------------------------------------------------------------------
-// Boys tables: at x_g, F_15(x_g) from its series exp(-x) sum_k (2x)^k / ((31)(33)...(31+2k)),
-// lower orders by the downward recursion F_{m-1} = (2x F_m + e^{-x}) / (2m-1); then for every
-// order L = 0..kMaxLt its row; the rows of the tail from the asymptote (layout: kBoysRowLen).
+// Boys tables (layout and entries: boys.cuh).  Blocks [0, kBoysTailBlock): a thread per grid point below 60;
+// then a thread per order and tail row.  With a division per term of the series, and all orders of a tail
+// row on one thread, the table took longer than the rest of a small system's set-up.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void put_boys_row(double* row, double x, const double* f, double e) {
-  row[0] = x;
-  for (int k = 0; k < 3; ++k) row[1 + k] = f[k];
-  row[4] = e;
-  row[5] = 0.5 * e;
-  float* r = reinterpret_cast<float*>(row + 6);
-  for (int k = 0; k < 3; ++k) r[k] = (float)f[3 + k];
-  r[3] = 0.f;
-}
-
-// blocks [0, tail_block): a thread per row below 60; then a thread per order and tail row.  The series
-// multiplies by reciprocals that the block makes once: with a division per term, and all orders of a
-// tail row on one thread, the table took longer than the rest of a small system's set-up.
-constexpr int kBoysBlock = 128, kBoysTerms = 512;
+constexpr int kBoysBlock = 128;
 constexpr int kBoysTailBlock = (kBoysRows + kBoysBlock - 1) / kBoysBlock;
-__global__ void __launch_bounds__(kBoysBlock) k_boys_table(double* __restrict__ tab) {
-  double f[6];
+__global__ void __launch_bounds__(kBoysBlock) k_boys_table(double* __restrict__ tabs) {
   if (blockIdx.x >= kBoysTailBlock) {
     const int i = (blockIdx.x - kBoysTailBlock) * blockDim.x + threadIdx.x, L = i / kBoysTailRows;
-    if (L > kMaxLt) return;
-    const int g = i - L * kBoysTailRows;
-    const double t = 1.0 + (double)g / kBoysTailPerUnit;
-    double c = 0.886226925452758014;  // (2L-1)!!/2^{L+1} sqrt(pi)
-    for (int m = 0; m < L; ++m) c *= m + 0.5;
-    f[0] = c / sqrt(t);
-    for (int m = 0; m < L; ++m) f[0] /= t;
-    for (int k = 1; k < 6; ++k) f[k] = -f[k - 1] * (L + k - 0.5) / (k * t);
-    put_boys_row(tab + (size_t)L * kBoysTableLen + (size_t)(kBoysRows + g) * kBoysRowLen, t, f, 0.0);
+    if (L <= kMaxLt) boys_make_tail_row(L, i - L * kBoysTailRows, tabs);
     return;
   }
-  const int M = 15;
-  __shared__ double rcp[kBoysTerms];  // 1 / (2 M + 2 k + 1)
-  for (int k = threadIdx.x; k < kBoysTerms; k += blockDim.x) rcp[k] = 1.0 / (2 * M + 2 * k + 1);
+  __shared__ double rcp[kBoysTerms];
+  for (int k = threadIdx.x; k < kBoysTerms; k += blockDim.x) rcp[k] = 1.0 / (2 * kBoysTop + 2 * k + 1);
   __syncthreads();
   const int g = blockIdx.x * blockDim.x + threadIdx.x;
-  if (g >= kBoysRows) return;
-  const double x = (double)g / kBoysPerUnit;
-  double term = rcp[0], sum = term;
-  for (int k = 1; k < kBoysTerms; ++k) {  // (some 250 terms at x = 60)
-    term *= 2.0 * x * rcp[k];
-    sum += term;
-    if (term < 1e-18 * sum) break;
-  }
-  const double e = exp(-x);
-  double Fm[M + 1];
-  Fm[M] = e * sum;
-  for (int m = M; m >= 1; --m) Fm[m - 1] = (2.0 * x * Fm[m] + e) / (2 * m - 1);
-  const double inv_fact[6] = {1.0, -1.0, 1.0 / 2, -1.0 / 6, 1.0 / 24, -1.0 / 120};
-  for (int L = 0; L <= kMaxLt; ++L) {
-    for (int k = 0; k < 6; ++k) f[k] = inv_fact[k] * Fm[L + k];
-    put_boys_row(tab + (size_t)L * kBoysTableLen + (size_t)g * kBoysRowLen, x, f, e);
-  }
+  if (g < kBoysRows) boys_make_rows(g, rcp, tabs);
 }
 
 // ---------------------------------------------------------------------------
