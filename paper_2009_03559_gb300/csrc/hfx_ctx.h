@@ -111,8 +111,9 @@ struct hfx_ctx {
   }
   // Tables up to kSlabPiece bytes share slabs of kSlab bytes: a new context and its pair list make
   // some fifty tables, and a cudaMalloc and cudaFree for each took a fifth of a small system's
-  // first build.  A slab lives as long as its scope; own: an allocation of its own in any case.
-  static constexpr size_t kSlab = 1 << 20, kSlabPiece = 1 << 17;
+  // first build.  A slab lives as long as its scope; own: an allocation of its own in any case.  What a slab
+  // leaves unused counts as held (a server's memory budget): slabs of 1 MB were a third of a small context.
+  static constexpr size_t kSlab = 1 << 17, kSlabPiece = 1 << 15;
   struct Slab {
     char* p = nullptr;
     size_t used = 0;

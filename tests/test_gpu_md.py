@@ -121,6 +121,15 @@ def test_build_inside_a_captured_graph(hfx_mod, mixed):
         assert np.abs(K.cpu().numpy() - Ko).max() <= (1e-7 if mixed else 1e-12) * np.abs(Ko).max()
 
 
+def test_device_memory_of_a_small_context(hfx_mod):
+    """What a server's budget counts for a system of 15 shells (120 pairs): the Boys tables (2.5 MB), CUB's
+    scratch (1 MB), two slabs of 128 KB, the primitive and Hermite pair data (less than 0.3 MB)."""
+    s, _ = inputs.config1(3)
+    h = hfx_mod.HFX(s)
+    assert h.device_bytes() < 2.7e6
+    assert h.build_pairs().device_bytes() < 4.1e6
+
+
 def test_pair_records_of_few_and_many_pairs(hfx_mod):
     """Primitive-pair records are made by 16 lanes a pair for few pairs and by one for many: the same
     Schwarz factors, bit for bit, for the pairs two systems share (primitive pairs dropped among them)."""
