@@ -223,13 +223,4 @@ __device__ __forceinline__ void digest(const EriClassInfo& ci, const R* v, int s
   }
 }
 
-// Diagonal (Schwarz) epilogue: max_{a,b} |(ab|ab)|.
-__device__ __forceinline__ double diag_max(const EriClassInfo& ci, const double* v, int st) {
-  const int na = ci.dims[0], nb = ci.dims[1];
-  double mx = 0.0;
-  for (int a = 0; a < na; ++a)
-    for (int b = 0; b < nb; ++b) mx = fmax(mx, fabs(v[(((a * nb + b) * na + a) * nb + b) * st]));
-  return mx;
-}
-
 }  // namespace hfx

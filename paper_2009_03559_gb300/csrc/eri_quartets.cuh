@@ -177,45 +177,22 @@ struct Tally {
 };
 
 // The quartet ranges a warp of the thread kernel works on.  Static schedules: one range (group_range).
-// Dynamic: chunks claimed from the launch's device counter.  Batched (L.n_sys > 0): chunks
-// of the systems' concatenated quartet lists; a chunk is split at system boundaries
-// (L.seg[s] = first index of system s) and each part runs with that system's record.
-template <bool BATCH, class C, class F>
-__device__ __forceinline__ void for_each_range(const EriLaunch& L, long long wid, long long nw, C&& claim, F&& f) {
-  if (!BATCH && L.schedule != 2) {
+// Dynamic: chunks claimed from the launch's device counter.
+template <class F>
+__device__ __forceinline__ void for_each_range(const EriLaunch& L, long long wid, long long nw, int lane, F&& f) {
+  if (L.schedule != 2) {
     long long q0, q1;
     group_range(L, wid, nw, q0, q1);
-    f(L, 0, q0, q1);
+    f(q0, q1);
     return;
   }
-  const long long total = L.q_count;
   while (true) {
-    long long c0 = claim();
-    if (c0 >= total) break;
-    const long long c1 = min(c0 + L.chunk, total);
-    if constexpr (!BATCH) {
-      f(L, 0, L.q_begin + c0, L.q_begin + c1);
-    } else {
-      while (c0 < c1) {
-        int lo = 0, hi = L.n_sys - 1;  // last s with seg[s] <= c0
-        while (lo < hi) {
-          const int mid = (lo + hi + 1) >> 1;
-          if (__ldg(L.seg + mid) <= c0) lo = mid; else hi = mid - 1;
-        }
-        const long long e = min(c1, __ldg(L.seg + lo + 1));
-        const EriLaunch& Ls = L.batch[lo];
-        f(Ls, lo, Ls.q_begin + (c0 - __ldg(L.seg + lo)), Ls.q_begin + (e - __ldg(L.seg + lo)));
-        c0 = e;
-      }
-    }
+    unsigned long long c = 0;
+    if (lane == 0) c = atomicAdd(L.work, (unsigned long long)L.chunk);
+    const long long c0 = (long long)__shfl_sync(0xffffffffu, c, 0);
+    if (c0 >= L.q_count) break;
+    f(L.q_begin + c0, L.q_begin + min(c0 + L.chunk, L.q_count));
   }
-}
-
-// a warp's claim of the next L.chunk quartets
-__device__ __forceinline__ long long warp_claim(const EriLaunch& L, int lane) {
-  unsigned long long c = 0;
-  if (lane == 0) c = atomicAdd(L.work, (unsigned long long)L.chunk);
-  return (long long)__shfl_sync(0xffffffffu, c, 0);
 }
 
 __device__ __forceinline__ void flush_tally(const EriLaunch& L, const Tally& t) {

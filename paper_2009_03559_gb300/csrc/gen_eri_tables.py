@@ -706,6 +706,12 @@ def post_words_of(c):
     return p_type, p_rel, p_n, words, bases[len(c.stages)]
 
 
+def thread_kernel_fits(scratch):
+    """Whether a class's slots (64 threads of a block) and the block's two quartet queues fit a block's shared
+    memory; the op lists of the others are not written out (eri_launch refuses them)."""
+    return 8 * 64 * scratch + 2 * 64 * 16 <= 227 * 1024
+
+
 def emit(classes, f=sys.stdout):
     w = f.write
     w("// Generated by gen_eri_tables.py -- do not edit by hand.\n")
@@ -716,20 +722,23 @@ def emit(classes, f=sys.stdout):
     for c in classes:
         T, bases = c.layout()
         work_base = c.n_acc
+        fits = thread_kernel_fits(T)
         lv_off, lv_n = [], []
         for lvl in c.bra_ops + c.ket_ops:
             lv_off.append(len(vrr_words) // 4)
-            lv_n.append(len(lvl))
-            for o in lvl:
+            lv_n.append(len(lvl) if fits else 0)
+            for o in lvl if fits else ():
                 vrr_words.extend(pack_vrr(o))
         acc_off = len(acc_words)
-        acc_words.extend([(a & 0xFFFF) | ((sl & 0xFFFF) << 16) for a, sl in c.acc_src])
+        acc_words.extend([(a & 0xFFFF) | ((sl & 0xFFFF) << 16) for a, sl in (c.acc_src if fits else ())])
         p_type, p_rel, p_n, words, out_base = post_words_of(c)
         p_off = [len(post_words) // 4 + r for r in p_rel]
-        post_words.extend(words)
+        if fits:
+            post_words.extend(words)
         fl = c.flops()
         rows.append(dict(c=c, T=T, work_base=work_base, lv_off=lv_off, lv_n=lv_n, acc_off=acc_off,
-                         p_type=p_type, p_off=p_off, p_n=p_n, out_base=out_base, fl=fl))
+                         p_type=p_type, p_off=p_off, p_n=p_n, out_base=out_base, fl=fl,
+                         n_acc=len(c.acc_src) if fits else 0, n_post=len(c.stages) if fits else 0))
 
     def arr(name, words, per_line=8):
         w(f"HFX_TABLE_QUAL uint32_t {name}[{max(len(words), 4)}] = {{\n")
@@ -758,8 +767,8 @@ def emit(classes, f=sys.stdout):
             str(c.la), str(c.lb), str(c.lc), str(c.ld), str(c.E), str(c.F), str(c.Lt),
             str(c.n_acc), str(r["work_base"]), str(r["T"]),
             str(len(c.bra_ops)), str(len(c.ket_ops)),
-            lst(r["lv_off"], 8), lst(r["lv_n"], 8), str(r["acc_off"]), str(len(c.acc_src)),
-            str(len(c.stages)), lst(r["p_type"], 8), lst(r["p_off"], 8), lst(r["p_n"], 8),
+            lst(r["lv_off"], 8), lst(r["lv_n"], 8), str(r["acc_off"]), str(r["n_acc"]),
+            str(r["n_post"]), lst(r["p_type"], 8), lst(r["p_off"], 8), lst(r["p_n"], 8),
             str(r["out_base"]), lst(c.final_dims, 4),
             str(fl["vrr"] + fl["acc"]), str(fl["hrr"] + fl["sph"] + fl["digest"]), str(fl["digest"]),
         ]) + "},\n")

@@ -40,8 +40,7 @@ struct BatchWork {
   bool fp32_class[21] = {};  // some system may run this class with FP32 recurrences
   long long total[21] = {};
   const double* boys = nullptr;  // the Boys tables: the first system's serve all
-  int gs[21] = {}, chunk[21] = {};  // lanes per quartet and dynamic chunk per class (0 = eri_chunk)
-  int streams[21] = {};             // warp kernel: primitive quartets at a time (0 = default)
+  int chunk[21] = {};  // dynamic chunk per class (0 = eri_chunk)
   EriLaunch *d_launch = nullptr, *h_launch = nullptr;
   BatchSys *d_sys = nullptr, *h_sys = nullptr;
   long long *d_seg = nullptr, *h_seg = nullptr;
@@ -79,15 +78,6 @@ cudaError_t bw_alloc(BatchWork& w, int cap, int n_sm) {
   w.bytes = sizeof(EriLaunch) * nl + sizeof(BatchSys) * cap + sizeof(long long) * ns + 256 +
             sizeof(double) * 2 * kBatchPart * cap;
   return cudaSuccess;
-}
-
-// the default per-class choices (those of a single-system build)
-void bw_default_choices(BatchWork& w) {
-  for (int cp = 0; cp < 21; ++cp) {
-    w.gs[cp] = eri_group_size();
-    w.chunk[cp] = 0;
-    w.streams[cp] = 0;
-  }
 }
 
 // Fills the host mirrors for systems ctxs[0..n): launch records, segment tables and
@@ -177,23 +167,21 @@ void bw_set_buffers(BatchWork& w, const double* const* P, double* const* K, cons
 // passes: each has its own work counter)
 int bw_prec(const BatchWork& w, int cp, int pass) { return w.fp32_class[cp] ? 1 + pass : 0; }
 
-// lanes per quartet of a pass: the class's choice, except the FP32 pass, which runs on whole
-// warps in every class
-int bw_gs(const BatchWork& w, int cp, int prec) { return prec == 2 ? 32 : w.gs[cp]; }
+// batches run on whole warps in every class
+constexpr int kBatchGs = 32;
 
 int bw_grid(const BatchWork& w, int cp, long long items, int prec) {
-  const int gs = bw_gs(w, cp, prec);
-  const long long groups_per_block = eri_groups_per_block(cp, gs);
+  const long long groups_per_block = eri_groups_per_block(cp, kBatchGs);
   const long long need = (items + groups_per_block - 1) / groups_per_block;
-  const long long cap = (long long)eri_blocks_per_sm(cp, 0, gs, prec, true) * w.n_sm;
+  const long long cap = (long long)eri_blocks_per_sm(cp, 0, kBatchGs, prec, true) * w.n_sm;
   return (int)std::max(1LL, std::min(need, cap));
 }
 
-// quartets per claim of a pass: the class's choice for its own lanes per quartet, else the rule's
+// quartets per claim of a pass: the class's choice, else the rule's
 int bw_chunk(const BatchWork& w, int cp, int prec) {
-  const int gs = bw_gs(w, cp, prec);
-  if (gs == w.gs[cp] && w.chunk[cp]) return w.chunk[cp];
-  return eri_chunk(gs, w.total[cp], (long long)bw_grid(w, cp, w.total[cp], prec) * eri_groups_per_block(cp, gs));
+  if (w.chunk[cp]) return w.chunk[cp];
+  return eri_chunk(kBatchGs, w.total[cp],
+                   (long long)bw_grid(w, cp, w.total[cp], prec) * eri_groups_per_block(cp, kBatchGs));
 }
 
 EriLaunch bw_class_launch(const BatchWork& w, int cp, int pass = 0) {
@@ -268,10 +256,9 @@ cudaError_t bw_enqueue(const BatchWork& w, cudaStream_t s, const Branches* br = 
     for (int pass = 0; pass < (w.fp32_class[cp] ? 2 : 1); ++pass) {
       const EriLaunch L = bw_class_launch(w, cp, pass);
       const int prec = bw_prec(w, cp, pass);
-      const int gs = bw_gs(w, cp, prec);
       const int grid = bw_grid(w, cp, w.total[cp], prec);
-      e = eri_launch(L, cp, 0, grid, bs, gs, prec, true, follows[bi]);
-      follows[bi] = eri_overlap(gs, w.total[cp], (long long)grid * eri_groups_per_block(cp, gs));
+      e = eri_launch(L, cp, 0, grid, bs, kBatchGs, prec, true, follows[bi]);
+      follows[bi] = eri_overlap(kBatchGs, w.total[cp], (long long)grid * eri_groups_per_block(cp, kBatchGs));
       if (e != cudaSuccess) return e;
     }
   }
@@ -390,7 +377,6 @@ extern "C" int hfx_batch_create(hfx_batch** out, hfx_ctx* const* ctxs, int n, vo
     energy[s] = ctxs[s]->d_energy;
   }
   bw_fill(b->w, ctxs, n, pmax.data(), pglob.data(), energy.data(), ctxs[0]->opt.precision == HFX_MIXED);
-  bw_default_choices(b->w);
   *out = b;
   return HFX_OK;
 }
@@ -466,21 +452,6 @@ extern "C" int hfx_batch_tune(hfx_batch* b, const double* const* P, double* cons
   cudaEvent_t t0, t1;
   CKB(cudaEventCreate(&t0));
   CKB(cudaEventCreate(&t1));
-  struct Choice {
-    int gs[21], chunk[21], streams[21];
-  };
-  auto save = [&]() {
-    Choice c;
-    std::memcpy(c.gs, w.gs, sizeof(c.gs));
-    std::memcpy(c.chunk, w.chunk, sizeof(c.chunk));
-    std::memcpy(c.streams, w.streams, sizeof(c.streams));
-    return c;
-  };
-  auto restore = [&](const Choice& c) {
-    std::memcpy(w.gs, c.gs, sizeof(c.gs));
-    std::memcpy(w.chunk, c.chunk, sizeof(c.chunk));
-    std::memcpy(w.streams, c.streams, sizeof(c.streams));
-  };
   // the whole batched build with the current choices (plain launches on the branches)
   auto time_full = [&](double* ms_out) -> int {
     float ms = 0.f;
@@ -506,7 +477,7 @@ extern "C" int hfx_batch_tune(hfx_batch* b, const double* const* P, double* cons
         EriLaunch L = bw_class_launch(w, cp, pass);
         L.q_count = w1;
         const int prec = bw_prec(w, cp, pass);
-        CKB(eri_launch(L, cp, 0, bw_grid(w, cp, w1 - w0, prec), s, bw_gs(w, cp, prec), prec, true));
+        CKB(eri_launch(L, cp, 0, bw_grid(w, cp, w1 - w0, prec), s, kBatchGs, prec, true));
       }
       CKB(cudaEventRecord(t1, s));
       CKB(cudaEventSynchronize(t1));
@@ -516,7 +487,8 @@ extern "C" int hfx_batch_tune(hfx_batch* b, const double* const* P, double* cons
     return HFX_OK;
   };
   int rc = HFX_OK;
-  const Choice incumbent = save();
+  int incumbent[21];
+  std::copy(w.chunk, w.chunk + 21, incumbent);
   double full_inc = 0.0, full_new = 0.0;
   if ((rc = time_full(&full_inc)) != HFX_OK) return rc;
   CKB(bw_upload(w, s));
@@ -524,21 +496,12 @@ extern "C" int hfx_batch_tune(hfx_batch* b, const double* const* P, double* cons
   for (int cp = 0; cp < 21 && rc == HFX_OK; ++cp) {
     const long long total = w.total[cp];
     if (total == 0) continue;
-    struct Cand {
-      int gs, streams, chunk;
-    };
-    std::vector<Cand> cands;
-    for (int c : {2, 8, 32}) cands.push_back({32, 0, c});
-    // window size: grow from 16k quartets until the incumbent takes the target, and at
-    // least two claims for every resident warp of every candidate, so that a large chunk
-    // is not timed on a window that leaves most of the GPU idle
-    long long fill = 0;
-    for (const Cand& cd : cands) {
-      const int pr = bw_prec(w, cp, 0);
-      const long long groups = (long long)eri_blocks_per_sm(cp, 0, cd.gs, pr, true) * w.n_sm *
-                               eri_groups_per_block(cp, cd.gs);
-      fill = std::max(fill, 2 * groups * cd.chunk);
-    }
+    const int cands[] = {2, 8, 32};  // quartets per claim
+    // window size: grow from 16k quartets until the incumbent takes the target, and at least two
+    // claims of the largest candidate for every resident warp, so that a large chunk is not timed on
+    // a window that leaves most of the GPU idle
+    const long long fill = 2ll * 32 * eri_blocks_per_sm(cp, 0, kBatchGs, bw_prec(w, cp, 0), true) * w.n_sm *
+                           eri_groups_per_block(cp, kBatchGs);
     long long win = std::min(total, std::max(16384LL, fill));
     for (int it = 0; it < 4 && win < total && rc == HFX_OK; ++it) {
       float ms = 0.f;
@@ -551,27 +514,22 @@ extern "C" int hfx_batch_tune(hfx_batch* b, const double* const* P, double* cons
     if (rc != HFX_OK) break;
     const long long w0 = (total - win) / 2;
     // the current choice is the incumbent; a candidate must beat it by 5% to replace it
-    Cand bc = {w.gs[cp], w.streams[cp], w.chunk[cp]};
+    int bc = w.chunk[cp];
     float inc = 0.f;
     if ((rc = time_window(cp, w0, w0 + win, &inc)) != HFX_OK) break;
     double best = inc;
-    for (const Cand& cd : cands) {
+    for (int c : cands) {
       if (rc != HFX_OK) break;
-      if (cd.gs == bc.gs && cd.chunk == bc.chunk && eri_streams(cp, cd.streams) == eri_streams(cp, bc.streams))
-        continue;
-      w.gs[cp] = cd.gs;
-      w.streams[cp] = cd.streams;
-      w.chunk[cp] = cd.chunk;
+      if (c == bc) continue;
+      w.chunk[cp] = c;
       float ms = 0.f;
       if ((rc = time_window(cp, w0, w0 + win, &ms)) != HFX_OK) break;
       if (ms < best && ms < 0.95 * inc) {
         best = ms;
-        bc = cd;
+        bc = c;
       }
     }
-    w.gs[cp] = bc.gs;
-    w.streams[cp] = bc.streams;
-    w.chunk[cp] = bc.chunk;
+    w.chunk[cp] = bc;
     b->tune_ms[cp] = best * (double)total / (double)win;  // projected to the whole class
     b->tune_window[cp] = win;
   }
@@ -594,10 +552,10 @@ extern "C" int hfx_batch_tune(hfx_batch* b, const double* const* P, double* cons
     b->tune_full_tuned_ms = full_new;
     b->tune_kept = full_new < full_inc;
     b->br.n = b->tune_kept ? br_best : br_inc;
-    if (!b->tune_kept) restore(incumbent);
+    if (!b->tune_kept) std::copy(incumbent, incumbent + 21, w.chunk);
   } else {
     b->br.n = br_inc;
-    restore(incumbent);
+    std::copy(incumbent, incumbent + 21, w.chunk);
   }
   cudaEventDestroy(t0);
   cudaEventDestroy(t1);
@@ -613,9 +571,9 @@ extern "C" int hfx_batch_get_stats(hfx_batch* b, hfx_batch_stats* out) {
   std::memset(out, 0, sizeof(*out));
   for (int cp = 0; cp < 21; ++cp) {
     out->n_quartets += b->w.total[cp];
-    out->group_size_class[cp] = b->w.gs[cp];
+    out->group_size_class[cp] = kBatchGs;
     out->chunk_class[cp] = bw_chunk(b->w, cp, bw_prec(b->w, cp, 0));
-    out->streams_class[cp] = b->w.gs[cp] == 32 ? eri_streams(cp, b->w.streams[cp]) : 0;
+    out->streams_class[cp] = eri_streams(cp, 0);
     out->tune_ms_class[cp] = b->tune_ms[cp];
     out->tune_window_class[cp] = b->tune_window[cp];
   }
@@ -896,7 +854,6 @@ static cudaError_t step_enqueue(hfx_server* srv, Slot& sl, const std::vector<uin
     energy[i] = sl.d_energy + i;
   }
   bw_fill(sl.w, ctxs.data(), n, pmax.data(), pglob.data(), energy.data(), srv->opt.precision == HFX_MIXED);
-  bw_default_choices(sl.w);
   bw_set_buffers(sl.w, P.data(), K.data(), nullptr);
   if ((e = bw_enqueue(sl.w, s)) != cudaSuccess) return e;
   for (int i = 0; i < n; ++i) {

@@ -187,8 +187,8 @@ __device__ __forceinline__ void g1_quartet(const EriClassInfo& ci, const EriLaun
          __ldg(Ls.sh.bf_off + sd), deg, Ls.P, Ls.K, Ls.ld, 0, 1);
 }
 
-// Per-warp queue of the quartets that pass the density tests (64 entries: system, bra
-// position, ket position, primitive quartets).  Lanes evaluate quartets 32 at a time, the
+// Per-warp queue of the quartets that pass the density tests (64 entries: bra position, ket
+// position, primitive quartets, unused).  Lanes evaluate quartets 32 at a time, the
 // 32 with the most primitive quartets first, so that few lanes idle while the others
 // finish their primitive loops (the FP64 pipe charges a warp instruction in full whatever
 // the number of active lanes).
@@ -221,16 +221,16 @@ __device__ __forceinline__ void sort64_desc(int& k0, int& k1, int lane) {
   }
 }
 
-template <bool BATCH, typename R>
-__device__ __forceinline__ void g1_drain(const EriLaunch& L, const EriClassInfo& ci, G1Queue& Q, int lane,
-                                         double* Sd, int st, Tally& t, bool all) {
+template <typename R>
+__device__ __forceinline__ void g1_drain(const EriLaunch& L, G1Queue& Q, int lane, double* Sd, int st, Tally& t,
+                                         bool all) {
   while (Q.n >= 32 || (all && Q.n > 0)) {
     int4 e;
     int take;
     if (Q.n >= 32) {
       // the 32 entries with the most primitive quartets; the rest move to the front
-      int k0 = lane < Q.n ? ((Q.q[lane].w << 6) | lane) : -1;
-      int k1 = lane + 32 < Q.n ? ((Q.q[lane + 32].w << 6) | (lane + 32)) : -1;
+      int k0 = lane < Q.n ? ((Q.q[lane].z << 6) | lane) : -1;
+      int k1 = lane + 32 < Q.n ? ((Q.q[lane + 32].z << 6) | (lane + 32)) : -1;
       sort64_desc(k0, k1, lane);
       e = Q.q[k0 & 63];
       int4 rest = make_int4(0, 0, 0, 0);
@@ -244,46 +244,45 @@ __device__ __forceinline__ void g1_drain(const EriLaunch& L, const EriClassInfo&
     }
     __syncwarp();
     Q.n -= take;
-    if (lane < take) g1_quartet<R>(ci, BATCH ? L.batch[e.x] : L, e.y, e.z, Sd, st, t);
+    if (lane < take) g1_quartet<R>(L.ci, L, e.x, e.y, Sd, st, t);
   }
 }
 
-// Quartets [q0, q1) of the launch record Ls (system sys), one quartet per thread: the warp
-// tests 32 consecutive quartets at a time and queues the survivors.
-template <bool BATCH, int PREC, typename R>
-__device__ __forceinline__ void g1_range(const EriLaunch& L, const EriClassInfo& ci, const EriLaunch& Ls, int sys,
-                                         long long q0, long long q1, double* Sd, int st, int lane, G1Queue& Q,
-                                         Tally& t) {
-  const long long* qoff = Ls.qoff;
-  const int row_begin = Ls.row_begin, bra0 = Ls.bra_bin_start, ket0 = Ls.ket_bin_start;
-  const bool skip = Ls.skip_zero;
-  const double dens = Ls.dens_tau;
+// Quartets [q0, q1) of the list, one quartet per thread: the warp tests 32 consecutive quartets
+// at a time and queues the survivors.
+template <int PREC, typename R>
+__device__ __forceinline__ void g1_range(const EriLaunch& L, long long q0, long long q1, double* Sd, int st, int lane,
+                                         G1Queue& Q, Tally& t) {
+  const long long* qoff = L.qoff;
+  const int row_begin = L.row_begin, bra0 = L.bra_bin_start, ket0 = L.ket_bin_start;
+  const bool skip = L.skip_zero;
+  const double dens = L.dens_tau;
   int r = -1;
   for (long long base = q0; base < q1; base += 32) {
     const long long q = base + lane;
     bool keep = false;
     int bra_s = 0, ket_s = 0, npq = 0;
     if (q < q1) {
-      if (r < 0) r = find_row(qoff, row_begin, Ls.row_end, q);
+      if (r < 0) r = find_row(qoff, row_begin, L.row_end, q);
       while (__ldg(qoff + r + 1) <= q) ++r;
       bra_s = bra0 + (r - row_begin);
       ket_s = ket0 + (int)(q - __ldg(qoff + r));
-      const int bra = __ldg(Ls.sorted + bra_s), ket = __ldg(Ls.sorted + ket_s);
-      const double pm = pmax4(Ls, __ldg(Ls.pa.sa + bra), __ldg(Ls.pa.sb + bra), __ldg(Ls.pa.sa + ket),
-                              __ldg(Ls.pa.sb + ket));
-      keep = !(skip && pm == 0.0) && !(dens > 0.0 && __ldg(Ls.Qs + bra_s) * __ldg(Ls.Qs + ket_s) * pm < dens) &&
-             dist_keeps(Ls, bra_s, ket_s) && pass_takes<PREC>(Ls, bra_s, ket_s, pm);
-      npq = __ldg(Ls.pa.prim_n + bra) * __ldg(Ls.pa.prim_n + ket);
+      const int bra = __ldg(L.sorted + bra_s), ket = __ldg(L.sorted + ket_s);
+      const double pm = pmax4(L, __ldg(L.pa.sa + bra), __ldg(L.pa.sb + bra), __ldg(L.pa.sa + ket),
+                              __ldg(L.pa.sb + ket));
+      keep = !(skip && pm == 0.0) && !(dens > 0.0 && __ldg(L.Qs + bra_s) * __ldg(L.Qs + ket_s) * pm < dens) &&
+             dist_keeps(L, bra_s, ket_s) && pass_takes<PREC>(L, bra_s, ket_s, pm);
+      npq = __ldg(L.pa.prim_n + bra) * __ldg(L.pa.prim_n + ket);
     }
     const unsigned m = __ballot_sync(0xffffffffu, keep);
-    if (keep) Q.q[Q.n + __popc(m & ((1u << lane) - 1u))] = make_int4(sys, bra_s, ket_s, npq);
+    if (keep) Q.q[Q.n + __popc(m & ((1u << lane) - 1u))] = make_int4(bra_s, ket_s, npq, 0);
     Q.n += __popc(m);
     __syncwarp();
-    g1_drain<BATCH, R>(L, ci, Q, lane, Sd, st, t, false);
+    g1_drain<R>(L, Q, lane, Sd, st, t, false);
   }
 }
 
-template <int PREC, bool BATCH>
+template <int PREC>
 __global__ void __launch_bounds__(64, PREC == PREC_MIXED32 ? HFX_G1F_MINB : HFX_G1_MINB)
     eri_g1_kernel(const EriLaunch L) {
   extern __shared__ double smem[];
@@ -297,11 +296,9 @@ __global__ void __launch_bounds__(64, PREC == PREC_MIXED32 ? HFX_G1F_MINB : HFX_
   const int lane = threadIdx.x & 31;
   Tally t;
   G1Queue Q{reinterpret_cast<int4*>(smem + (size_t)L.ci.scratch * blockDim.x) + (threadIdx.x >> 5) * 64, 0};
-  for_each_range<BATCH>(L, gid >> 5, ng >> 5, [&]() { return warp_claim(L, lane); },
-                            [&](const EriLaunch& Ls, int sys, long long q0, long long q1) {
-                              g1_range<BATCH, PREC, R>(L, L.ci, Ls, sys, q0, q1, Sd, st, lane, Q, t);
-                            });
-  g1_drain<BATCH, R>(L, L.ci, Q, lane, Sd, st, t, true);
+  for_each_range(L, gid >> 5, ng >> 5, lane,
+                 [&](long long q0, long long q1) { g1_range<PREC, R>(L, q0, q1, Sd, st, lane, Q, t); });
+  g1_drain<R>(L, Q, lane, Sd, st, t, true);
   flush_tally(L, t);
   record_busy(L, t0);
 }
@@ -356,15 +353,10 @@ static int md_kind(int mode, int prec, bool batch) {
   return mode == 1 ? MD_DIAG : prec == PREC_PERIODIC ? MD_PER : batch ? MD_BATCH : MD_PLAIN;
 }
 
-template <int PREC>
-static const void* g1_ptr(bool batch) {
-  return batch ? (const void*)eri_g1_kernel<PREC, true> : (const void*)eri_g1_kernel<PREC, false>;
-}
-
-static const void* kernel_ptr(int prec, bool batch) {
-  if (prec == PREC_MIXED64) return g1_ptr<PREC_MIXED64>(batch);
-  if (prec == PREC_MIXED32) return g1_ptr<PREC_MIXED32>(batch);
-  return g1_ptr<PREC_FP64>(batch);
+static const void* g1_kernel(int prec) {
+  if (prec == PREC_MIXED64) return (const void*)eri_g1_kernel<PREC_MIXED64>;
+  if (prec == PREC_MIXED32) return (const void*)eri_g1_kernel<PREC_MIXED32>;
+  return (const void*)eri_g1_kernel<PREC_FP64>;
 }
 
 // one quartet per thread: interleaved scratch, then a 64-entry quartet queue per warp
@@ -378,18 +370,16 @@ cudaError_t eri_prepare() {
   for (int c = 0; c < HFX_N_CLASSES; ++c) mx = std::max(mx, g1_smem_bytes(c));
   if (mx > 227 * 1024) mx = 227 * 1024;
   cudaError_t e = md_prepare();
-  for (bool batch : {false, true})
-    for (int prec : {PREC_FP64, PREC_MIXED64, PREC_MIXED32})
-      if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(kernel_ptr(prec, batch), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mx);
+  for (int prec : {PREC_FP64, PREC_MIXED64, PREC_MIXED32})
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(g1_kernel(prec), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mx);
   return e;
 }
 
 int eri_blocks_per_sm(int cls, int mode, int gs, int prec, bool batch) {
   if (gs != 1) return md_blocks_per_sm(cls, md_kind(mode, prec, batch), prec == PREC_MIXED32);
   int n = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel_ptr(prec, batch), kBlock, g1_smem_bytes(cls)) !=
-      cudaSuccess)
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, g1_kernel(prec), kBlock, g1_smem_bytes(cls)) != cudaSuccess)
     return 1;
   return n > 0 ? n : 1;
 }
@@ -417,11 +407,12 @@ bool eri_overlap(int gs, long long n_quartets, long long n_groups) { return gs !
 cudaError_t eri_launch(const EriLaunch& L0, int cls, int mode, int grid, cudaStream_t stream, int gs, int prec,
                        bool batch, bool overlap) {
   if (gs != 1) return md_launch(L0, cls, md_kind(mode, prec, batch), prec, prec == PREC_MIXED32, grid, stream, overlap);
+  // the thread kernel: builds of one system, classes whose slots fit
   const size_t smem = g1_smem_bytes(cls);
-  if (smem > 227 * 1024) return cudaErrorInvalidValue;
+  if (mode != 0 || batch || prec == PREC_PERIODIC || smem > 227 * 1024) return cudaErrorInvalidValue;
   EriLaunch L = L0;
   void* args[] = {(void*)&L};
-  return cudaLaunchKernel(kernel_ptr(prec, batch), dim3(grid), dim3(kBlock), args, smem, stream);
+  return cudaLaunchKernel(g1_kernel(prec), dim3(grid), dim3(kBlock), args, smem, stream);
 }
 
 }  // namespace hfx

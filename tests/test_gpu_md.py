@@ -101,6 +101,26 @@ def test_exponents_at_the_ends_of_the_fp64_range(hfx_mod, alpha, omega, mixed):
         assert np.abs(K[1].cpu().numpy() - Ko).max() <= 1e-12 * np.abs(Ko).max()
 
 
+def test_thread_kernel_takes_the_classes_that_fit(hfx_mod):
+    """A thread's slots (at most 450 doubles: 64 threads in 227 KB) hold sixteen classes; their op lists are in
+    the generated tables, the five others are refused."""
+    s = inputs.diamond_system(3, seed=5, tau=1e-10)
+    P = torch.from_numpy(inputs.density_matrix(s)).cuda()
+    h = hfx_mod.HFX(s).build_pairs()
+    K = h.build_K(P).clone()
+    refused = []
+    for cls in range(21):
+        h.set_group_size(cls, 1)
+        try:
+            K1 = h.build_K(P)
+        except hfx_mod.HFXError:
+            refused.append(cls)
+        else:
+            assert torch.abs(K1 - K).max() <= 1e-12 * torch.abs(K).max(), cls
+        h.set_group_size(cls, 0)
+    assert refused == [14, 17, 18, 19, 20]
+
+
 @pytest.mark.parametrize("mixed", [False, True])
 def test_build_inside_a_captured_graph(hfx_mod, mixed):
     """Overlapping class launches (a small system) as a captured graph, replayed for another density."""
