@@ -369,7 +369,8 @@ extern "C" int hfx_build_pairs(hfx_ctx* ctx) {
   const long long n_pp = (long long)last[0] + last[1];
   RK(ctx->alloc(&ctx->d_pp, n_pp, true));
   CK(launch_prim_fill(n_cand, ctx->d_sa, ctx->d_sb, ctx->d_nprim, ctx->d_prim_off, ctx->d_atom, ctx->d_xyz,
-                      ctx->d_alpha, ctx->d_w, ctx->d_pp_off, ctx->opt.prim_tau, ctx->hexp, ctx->d_pp, ctx->d_pp_n, s));
+                      ctx->d_alpha, ctx->d_w, ctx->d_pp_off, ctx->opt.prim_tau, ctx->hexp, ctx->n_sm, ctx->d_pp,
+                      ctx->d_pp_n, s));
   RK(ctx->alloc(&ctx->d_md, (size_t)n_md, true));
   CK(launch_md_fill(n_cand, ctx->d_pcls, ctx->d_AB, ctx->d_pp_off, ctx->d_pp_n, ctx->d_pp, ctx->d_md_off,
                     ctx->hexp, ctx->d_md, s));

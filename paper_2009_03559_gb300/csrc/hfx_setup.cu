@@ -643,16 +643,16 @@ cudaError_t scan_ll_inclusive(void* tmp, size_t& tmp_bytes, const long long* in,
 
 cudaError_t launch_prim_fill(int n_cand, const int* sa, const int* sb, const int* nprim, const int* prim_off_shell,
                              const int* atom, const double* xyz, const double* alpha, const double* w,
-                             const int* pp_off, double prim_tau, int hexp, PrimPair* pp, int* pp_n, cudaStream_t s) {
+                             const int* pp_off, double prim_tau, int hexp, int n_sm, PrimPair* pp, int* pp_n,
+                             cudaStream_t s) {
   if (n_cand <= 0) return cudaSuccess;
   // 16 lanes a shell pair (9 primitive pairs at the usual 3 a shell) while these threads are all
-  // resident at once (152 SMs x 2048): one round instead of nine, 45 -> 10 us for 171 pairs.  With
+  // resident at once (2048 an SM): one round instead of nine, 45 -> 10 us for 171 pairs on 152 SMs.  With
   // more pairs the chip is full and idle lanes cost: a thread each.
-  constexpr int kWide = 152 * 2048 / 16;
-  auto k = n_cand <= kWide ? k_prim_fill<16> : k_prim_fill<1>;
-  k<<<nblk((n_cand <= kWide ? 16ll : 1ll) * n_cand, 128), 128, 0, s>>>(n_cand, sa, sb, nprim, prim_off_shell, atom, xyz,
-                                                                       alpha, w, pp_off, prim_tau,
-                                                                       std::ldexp(1.0, hexp / 2), pp, pp_n);
+  const bool wide = n_cand <= n_sm * (2048 / 16);
+  auto k = wide ? k_prim_fill<16> : k_prim_fill<1>;
+  k<<<nblk((wide ? 16ll : 1ll) * n_cand, 128), 128, 0, s>>>(n_cand, sa, sb, nprim, prim_off_shell, atom, xyz, alpha, w,
+                                                            pp_off, prim_tau, std::ldexp(1.0, hexp / 2), pp, pp_n);
   return cudaGetLastError();
 }
 

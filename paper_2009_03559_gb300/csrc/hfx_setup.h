@@ -49,7 +49,8 @@ cudaError_t scan_ll_inclusive(void* tmp, size_t& tmp_bytes, const long long* in,
                               cudaStream_t s);
 cudaError_t launch_prim_fill(int n_cand, const int* sa, const int* sb, const int* nprim, const int* prim_off_shell,
                              const int* atom, const double* xyz, const double* alpha, const double* w,
-                             const int* pp_off, double prim_tau, int hexp, PrimPair* pp, int* pp_n, cudaStream_t s);
+                             const int* pp_off, double prim_tau, int hexp, int n_sm, PrimPair* pp, int* pp_n,
+                             cudaStream_t s);
 // distance-aware screening: per candidate pair (centre xyz, spread, smallest exponent sum),
 // and the same gathered into sorted-pair order
 cudaError_t launch_pair_dist(int n_cand, const int* sa, const int* sb, const int* nprim, const int* prim_off_shell,

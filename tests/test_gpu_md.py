@@ -167,3 +167,24 @@ def test_pair_records_of_few_and_many_pairs(hfx_mod):
 
     many, few = factors(n), factors(99)
     assert (few > 0).sum() > 99 and np.array_equal(many[:99, :99], few[:99, :99])
+
+
+def test_pair_records_on_both_sides_of_the_line(hfx_mod):
+    """The same where 16 lanes a pair just fill the chip and where they just do not, for this chip's SMs."""
+    line = torch.cuda.get_device_properties(0).multi_processor_count * 2048 // 16
+    n = int((np.sqrt(8.0 * line + 1.0) - 1.0) / 2.0) + 1  # the first n with more than `line` pairs
+    assert (n - 1) * n // 2 <= line < n * (n + 1) // 2
+    rng = np.random.default_rng(4)
+    k = 5  # 25 primitive pairs: two rounds of 16 lanes
+    xyz, al = rng.uniform(0, 40, (n, 3)), rng.uniform(0.2, 4.0, (n, k))
+
+    def factors(m):
+        s = inputs.System("s", xyz[:m], np.arange(m, dtype=np.int32), np.zeros(m, np.int32), np.full(m, k, np.int32),
+                          al[:m].ravel(), np.ones(m * k), omega=0.11, tau=0.0)
+        a, b, q = hfx_mod.HFX(s).build_pairs().pairs()
+        out = np.zeros((n, n))
+        out[a, b] = q
+        return out
+
+    many, few = factors(n), factors(n - 1)
+    assert (few > 0).sum() > n and np.array_equal(many[:n - 1, :n - 1], few[:n - 1, :n - 1])
