@@ -121,3 +121,49 @@ def test_digest_tasks_make_the_four_blocks(ci):
     assert len(got) == sum(w.size for w in want.values())
     for (isb, isd, x, y), val in got.items():
         assert abs(val - want[isb, isd][x, y]) <= 1e-13
+
+
+def hermite_f32(Lt, G, rho, PQ):
+    """S_r as the FP32 pass makes them: the recursion on S_r / lam^|r|, lam = sqrt(2 rho), times lam^|r|."""
+    f = np.float32
+    lam = f(np.sqrt(f(2 * rho)))
+    S = {((0, 0, 0), m): f(G[m]) for m in range(Lt + 1)}
+    X = [f(v) * lam for v in PQ]
+    lp = [f(1)]
+    for _ in range(Lt):
+        lp.append(lp[-1] * lam)
+    for r in HERM[1:gen.n_herm(Lt)]:
+        ax = 0 if r[0] else (1 if r[1] else 2)
+        r1 = tuple(v - (i == ax) for i, v in enumerate(r))
+        r2 = tuple(v - 2 * (i == ax) for i, v in enumerate(r))
+        for m in range(Lt - sum(r) + 1):
+            v = X[ax] * S[r1, m + 1]
+            if r1[ax]:
+                v = v - f(r1[ax]) * S[r2, m + 1]
+            S[r, m] = v
+    return np.array([S[r, 0] * lp[sum(r)] for r in HERM[:gen.n_herm(Lt)]], dtype=f)
+
+
+@pytest.mark.parametrize("ci", range(21), ids=[c.name() for c in MD])
+def test_fp32_pass_error_by_class(ci, monkeypatch):
+    """The tables run in FP32 as the FP32 pass does (recursion and both contractions; the transformations in
+    FP64) on far-apart quartets, the kind that qualify: error relative to the quartet's largest integral.  A value
+    passes 3 roundings of 2^-24 in each of L steps and 6 around them; 4 times that for sums whose terms
+    cancel: 1.4e-6 at L = 0, 7.2e-6 at L = 8.  (Measured 5e-8 in (ss|ss), 2.6e-7 in (dd|dd): no class stands out, unlike
+    the Obara-Saika schedules' in test_schedule_emulation.py, which no kernel runs.)"""
+    c = MD[ci]
+    rng = np.random.default_rng(900 + ci)
+    worst = 0.0
+    for _ in range(4):
+        A = rng.uniform(-1, 1, 3)
+        shift = rng.normal(size=3)
+        shift *= rng.uniform(9, 12) / np.linalg.norm(shift)
+        cen = np.array([A, A + rng.uniform(-2, 2, 3), shift + rng.uniform(-1, 1, 3), shift + rng.uniform(-2, 2, 3)])
+        bra, ket = rng.uniform(0.1, 3.0, (2, 2)), rng.uniform(0.1, 3.0, (3, 2))
+        ref = run_tables(c, bra, ket, cen, 0.11)
+        with monkeypatch.context() as mk:
+            mk.setitem(globals(), "hermite", lambda Lt, G, rho, PQ, dtype: hermite_f32(Lt, G, rho, PQ))
+            got = run_tables(c, bra, ket, cen, 0.11, np.float32)
+        worst = max(worst, np.abs(got - ref).max() / np.abs(ref).max())
+    print(c.name(), worst)
+    assert 0 < worst <= 4 * (3 * c.Lt + 6) * 2.0 ** -24
