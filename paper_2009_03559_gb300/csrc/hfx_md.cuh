@@ -428,6 +428,7 @@ __global__ void __launch_bounds__(md_block(LT), md_minb<R>(LT))
   int head = 0, head_off = 0, tail = 0, waiting = 0;  // queue: entries [head, tail), primitive quartets left
   bool h_valid = false, a_valid = false;              // the head quartet's H and A hold partial sums
   int n_eval = 0;                                     // its primitive quartets evaluated so far
+  R carry = R(0);                                     // L <= 2: the partial sum of a lane's H value
   int tb_sys = -1, tb_bra = -1;                       // whose transformation is in Tb
   Tally tally;
   Fp64 op;
@@ -833,8 +834,9 @@ __global__ void __launch_bounds__(md_block(LT), md_minb<R>(LT))
       const unsigned last_k = __ballot_sync(0xffffffffu, s.ik == s.nk - 1);
       const unsigned last_q = __ballot_sync(0xffffffffu, s.ik == s.nk - 1 && s.ib == s.nb - 1);
       if constexpr (LT <= 2) {
-        // 32 / md_group runs side by side, then the bra contraction of each.  A run cut by the end
-        // of a batch needs no carry: its parts add up in A.
+        // 32 / md_group runs side by side, then the bra contraction of each.  The sum of a run cut by the end of
+        // the 32 goes on with the next ones: as two contractions the FP32 pass's roundings depended on where in
+        // the stream a quartet came (K of repeated mixed builds of 32 atoms differed by 9e-13; now by 1e-14).
         constexpr int GL = md_group(LT), G = 32 / GL;
         int* const first_row = reinterpret_cast<int*>(S + ly.Y - 18);
         const int nr = __popc(lead);
@@ -848,7 +850,7 @@ __global__ void __launch_bounds__(md_block(LT), md_minb<R>(LT))
           const int most = __reduce_max_sync(0xffffffffu, len);
           const R* r = Rb + p0 * kRow + kc_r[0];
           const R* w = Rb + p0 * kRow + kc_w[0];
-          R v = R(0);
+          R v = h_valid && t == 0 ? carry : R(0);
 #pragma unroll 4
           for (int p = 0; p < most; ++p)
             if (p < len) v = fmar(w[p * kRow], r[p * kRow], v);
@@ -861,11 +863,18 @@ __global__ void __launch_bounds__(md_block(LT), md_minb<R>(LT))
             const int l1 = lead ? __ffs(lead) - 1 : ns;
             const int np = first_row[u + 1] - first_row[u];
             const int slot = __shfl_sync(0xffffffffu, s.e, l0) & (kQ - 1), ib = __shfl_sync(0xffffffffu, s.ib, l0);
-            if (np > 0) {
+            const bool sum = np > 0 || (u == 0 && h_valid);
+            n_eval += np;
+            if (!((last_k >> (l1 - 1)) & 1)) {  // cut: the last run
+              carry = H[(u - t0) * GL + lane % GL];
+              h_valid = sum;
+              continue;
+            }
+            if (sum) {
               bra_contract(bra_factors(slot, ib), H + (u - t0) * GL);
               a_valid = true;
-              n_eval += np;
             }
+            if (u == 0) h_valid = false;
             if ((last_q >> (l1 - 1)) & 1) finish(slot);
           }
           __syncwarp();

@@ -132,3 +132,24 @@ def test_thread_kernel_fp32_pass(hfx_mod):
     st = h.stats()
     assert sum(st["quartets_fp32_class"][c] for c in (0, 1, 2, 3, 4, 6, 7, 10, 15)) > 0
     assert np.abs(K - Ko).max() <= TOL and abs(h.energy() - eo) <= TOL
+
+
+def test_mixed_K_does_not_depend_on_the_order_of_quartets(hfx_mod):
+    """Which warp takes which quartets, and after which others, changes from build to build (chunks are claimed)
+    and in a batch; only the order of the FP64 additions into K may follow.  An element is a sum of some 1e5 terms of
+    at most 3, each addition rounded to 2^-53: 3 x 1.1e-16 x sqrt(1e5) = 1e-13."""
+    s = inputs.make_system("diamond", 16, seed=9105)
+    P = torch.from_numpy(inputs.density_matrix(s, seed=550, truncate_bohr=inputs.truncation_for(s.kind))).cuda()
+    s2 = inputs.diamond_system(2, seed=3)
+    P2 = torch.from_numpy(inputs.density_matrix(s2)).cuda()
+    kw = dict(precision=hfx_mod.HFX_MIXED)
+    h, h2 = hfx_mod.HFX(s, **kw).build_pairs(), hfx_mod.HFX(s2, **kw).build_pairs()
+    Ks = [h.build_K(P).clone() for _ in range(6)]
+    b = hfx_mod.Batch([h2, h])
+    for _ in range(3):
+        K = [torch.empty_like(P2), torch.empty_like(P)]
+        b.run([P2, P], K)
+        torch.cuda.synchronize()
+        Ks.append(K[1])
+    Ks = torch.stack(Ks)
+    assert (Ks.max(0).values - Ks.min(0).values).max().item() <= 1e-13
