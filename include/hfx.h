@@ -247,9 +247,10 @@ int hfx_get_stats(hfx_ctx* ctx, hfx_stats* out);
 
 /* Lanes per quartet for class cls (0..20) in later K builds of this context: 1 (a thread
  * owns a quartet), 32 (whole warps, alone or in teams, over a stream of quartets), 0 = the
- * library's default (32).  A value set here applies to both passes of a mixed-precision class.
- * 1 needs a class whose scratch fits the thread kernel, else the build fails with
- * HFX_ERR_CUDA.  Errors: HFX_ERR_ARG. */
+ * library's default (32; 1 for long lists of the nine lowest classes in FP64 where every shell
+ * of the basis has one primitive).  A value set here applies to both passes of a mixed-precision class.
+ * 1 needs a class whose scratch fits the thread kernel (not (dp|dp), (dd|pp), (dd|ds), (dd|dp)
+ * and (dd|dd)), else the build fails with HFX_ERR_CUDA.  Errors: HFX_ERR_ARG. */
 int hfx_set_group_size(hfx_ctx* ctx, int cls, int gs);
 
 /* Enables (1) or disables (0) per-class CUDA-event timing of K builds. */

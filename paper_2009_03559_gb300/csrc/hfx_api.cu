@@ -400,7 +400,7 @@ extern "C" int hfx_build_pairs(hfx_ctx* ctx) {
         L.diag_list = d_cidx + start;
         L.diag_n = cnt[pc];
         L.diag_Q = ctx->d_Q;
-        const int gs = eri_group_size();
+        const int gs = 32;
         const int grid = grid_for(ctx, cls, 1, cnt[pc], gs);
         CK(eri_launch(L, cls, 1, grid, s, gs, 0, false, follows));
         follows = eri_overlap(gs, cnt[pc], (long long)grid * eri_groups_per_block(cls, gs));
@@ -713,7 +713,7 @@ extern "C" int hfx_build_K_periodic(hfx_ctx* ctx, int n_R, const int* R_cells, c
     L.q_begin = ctx->cls_qbegin[cp];
     L.per.n_list = ctx->cls_q[cp];
     L.q_count = ctx->cls_q[cp] * (hi > lo ? 2 * n_fwd : n_fwd);
-    const int gs = eri_group_size();
+    const int gs = 32;
     const int grid = grid_for(ctx, cp, 0, L.q_count, gs, 3);
     L.chunk = eri_chunk(gs, L.q_count, (long long)grid * eri_groups_per_block(cp, gs));
     L.work = ctx->d_work + cp;
@@ -817,7 +817,9 @@ static int build_K_impl(hfx_ctx* ctx, const double* P, double* K, int ld, int pa
     // quartets that stay FP64 then those whose recurrences run in FP32, each with a kernel
     // compiled for its precision alone (registers, hence resident warps, of its own)
     L.fp32_ok = mixed && ((ctx->fp32_mask() >> cp) & 1);
-    const int gs = ctx->gs_override[cp] ? ctx->gs_override[cp] : eri_group_size();
+    // (the FP32 recurrences of the thread kernel are the less accurate ones)
+    const bool uncontracted = ctx->n_prim == ctx->n_shells && !L.fp32_ok;
+    const int gs = ctx->gs_override[cp] ? ctx->gs_override[cp] : eri_group_size(cp, uncontracted, L.q_count, ctx->n_sm);
     ctx->gs_used[cp] = gs;
     ctx->streams_used[cp] = gs == 32 ? eri_streams(cp, ctx->streams_override[cp]) : 0;
     const long long items = ctx->opt.schedule == HFX_SCHED_PAIR ? (L.row_end - L.row_begin) : L.q_count;
@@ -827,13 +829,11 @@ static int build_K_impl(hfx_ctx* ctx, const double* P, double* K, int ld, int pa
     }
     for (int pass = 0; pass < (L.fp32_ok ? 2 : 1); ++pass) {
       const int prec = L.fp32_ok ? 1 + pass : 0;
-      // the FP32 pass runs on whole warps in every class unless the caller fixed the class's group size
-      const int gsp = (prec == 2 && !ctx->gs_override[cp]) ? 32 : gs;
-      const int grid = grid_for(ctx, cp, 0, items, gsp, prec);
-      L.chunk = eri_chunk(gsp, L.q_count, (long long)grid * eri_groups_per_block(cp, gsp));
+      const int grid = grid_for(ctx, cp, 0, items, gs, prec);
+      L.chunk = eri_chunk(gs, L.q_count, (long long)grid * eri_groups_per_block(cp, gs));
       L.work = ctx->d_work + cp + 21 * pass;
-      CK(eri_launch(L, cp, 0, grid, s, gsp, prec, false, follows));
-      follows = !ctx->timing && eri_overlap(gsp, L.q_count, (long long)grid * eri_groups_per_block(cp, gsp));
+      CK(eri_launch(L, cp, 0, grid, s, gs, prec, false, follows));
+      follows = !ctx->timing && eri_overlap(gs, L.q_count, (long long)grid * eri_groups_per_block(cp, gs));
     }
     if (ctx->timing) CK(cudaEventRecord(ctx->ev[3 + 2 * cp], s));
     ctx->class_launched[cp] = true;
@@ -892,7 +892,7 @@ extern "C" int hfx_get_stats(hfx_ctx* ctx, hfx_stats* out) {
   CK(cudaStreamSynchronize(ctx->stream));
   hfx_stats& st = ctx->stats;
   for (int cp = 0; cp < 21; ++cp) {
-    st.group_size_class[cp] = ctx->gs_used[cp] ? ctx->gs_used[cp] : eri_group_size();
+    st.group_size_class[cp] = ctx->gs_used[cp] ? ctx->gs_used[cp] : 32;
     st.streams_class[cp] = ctx->streams_used[cp];
   }
   CK(cudaMemcpy(&st.energy, ctx->d_energy, sizeof(double), cudaMemcpyDeviceToHost));

@@ -308,11 +308,18 @@ __global__ void __launch_bounds__(64, PREC == PREC_MIXED32 ? HFX_G1F_MINB : HFX_
 // ---------------------------------------------------------------------------
 static const int kBlock = 64;
 
-// Whole warps in every class.  The thread kernel was the default of the nine lowest classes
-// before the Hermite engine, which measured faster in all of them (64-atom diamond, (ss|ss)
-// 17.0 -> 11.2 ms, (pp|ps) 219 -> 129 ms, (dd|ss) 44 -> 26 ms); it runs where a caller asks for it.
-// Groups of 8 or 16 lanes were slower than either in every class.
-int eri_group_size() { return 32; }
+// Whole warps, but for long lists of uncontracted quartets in the nine classes of at most 100 slots a thread.
+// The Hermite engine's steps after the contraction cost a warp the same for 1 primitive quartet as for 81: with
+// 3 primitives a shell it is the faster in every class (64-atom diamond, (ss|ss) 17.0 -> 11.2 ms, (pp|ps)
+// 219 -> 129 ms, (dd|ss) 44 -> 26 ms), with 2 too (24 atoms, 1.3 to 4.8 times), with 1 the thread kernel
+// (64 atoms: (ss|ss) 0.92 -> 0.48 ms, (ps|ss) 3.63 -> 1.40, (pp|ps) 7.36 -> 5.81, (dd|ss) 3.87 -> 2.14; whole
+// build 306 -> 291 ms; 300 s shells 4.18 -> 1.24 ms) where a list is long enough for four quartets a thread (24
+// atoms, 260 000: (pp|ps) 0.61 -> 0.58 ms; 190 000: (ds|ps) 0.44 -> 0.47; 90 000: (ds|ss) 0.23 -> 0.27).  Groups of 8 or 16 lanes were slower than
+// either in every class.
+int eri_group_size(int cls, bool uncontracted, long long n_quartets, int n_sm) {
+  if (!uncontracted || kClassInfo[cls].scratch > HFX_G1_MAX_SCRATCH) return 32;
+  return n_quartets >= 4ll * n_sm * eri_blocks_per_sm(cls, 0, 1, PREC_FP64, false) * kBlock ? 1 : 32;
+}
 
 bool eri_group_size_valid(int gs) { return gs == 1 || gs == 32; }
 

@@ -9,7 +9,8 @@ struct EriLaunch;
 
 // Group sizes (lanes per quartet): 1 (a thread) or 32 (a warp).  Precision passes `prec`:
 // 0 every quartet in FP64; 1 and 2 the FP64 and FP32 shares of a mixed-precision class.
-int eri_group_size();  // the default: 32
+// the default of a build of one system (uncontracted: every shell has one primitive), of all others 32
+int eri_group_size(int cls, bool uncontracted, long long n_quartets, int n_sm);
 bool eri_group_size_valid(int gs);
 cudaError_t eri_prepare();
 int eri_blocks_per_sm(int cls, int mode, int gs, int prec, bool batch);

@@ -121,6 +121,37 @@ def test_thread_kernel_takes_the_classes_that_fit(hfx_mod):
     assert refused == [14, 17, 18, 19, 20]
 
 
+@pytest.mark.parametrize("kw", [{}, dict(schedule=0), dict(schedule=1), dict(density_tau=1e-8), dict(precision=1)])
+def test_long_uncontracted_lists_take_the_thread_kernel(hfx_mod, kw):
+    """48 atoms with s, p, d shells of one primitive: the long lists of the low classes go to the thread kernel
+    (in FP64), the other classes stay; against whole warps everywhere."""
+    s = inputs.diamond_system(48, seed=3, nprim=1)
+    P = torch.from_numpy(inputs.density_matrix(s)).cuda()
+    h = hfx_mod.HFX(s, **kw).build_pairs()
+    K = h.build_K(P).clone()
+    st = h.stats()
+    gs = np.array(st["group_size_class"])
+    nq = np.array(st["n_quartets_class"])
+    low = np.isin(np.arange(21), [0, 1, 2, 3, 4, 6, 7, 10, 15])
+    if kw.get("precision"):
+        assert np.all(gs[:20] == 32)  # every class but (dd|dd) may take the FP32 pass
+    else:
+        assert np.all(gs[~low] == 32) and np.all(gs[nq < 1e5] == 32) and np.all(gs[low & (nq > 5e5)] == 1)
+        assert (gs == 1).sum() >= 4
+    for cls in range(21):
+        h.set_group_size(cls, 32)
+    K32 = h.build_K(P)
+    assert torch.abs(K32 - K).max() <= 1e-12 * torch.abs(K).max()
+    if kw.get("schedule") == 1:  # whole rows: no partitions
+        return
+    parts = torch.zeros_like(K)
+    for cls in range(21):
+        h.set_group_size(cls, 0)
+    for i in range(3):  # (shorter lists)
+        parts += h.build_K(P, part=i, n_parts=3)
+    assert torch.abs(parts - K).max() <= 1e-12 * torch.abs(K).max()
+
+
 @pytest.mark.parametrize("mixed", [False, True])
 def test_build_inside_a_captured_graph(hfx_mod, mixed):
     """Overlapping class launches (a small system) as a captured graph, replayed for another density."""
