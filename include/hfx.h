@@ -57,7 +57,7 @@ extern "C" {
 #define HFX_MIXED 1               /* FP32 recurrences for small-bound quartets, see hfx_options */
 
 /* Default classes allowed FP32 recurrences under HFX_MIXED: every class but (dd|dd), the highest
- * recursion (L = 8).  E_K of the 64-atom diamond moves by 8e-12 and of the 216-atom one by 3e-11
+ * recursion (L = 8).  E_K of the 64-atom diamond moves by 9e-12 and of the 216-atom one by 3e-11
  * against FP64 (with (dd|dd) in FP32 too: 1e-11 and 4e-11). */
 #define HFX_FP32_CLASSES_DEFAULT 0xFFFFF
 

@@ -8,8 +8,8 @@
 // runs at the full rate).  The Hermite form (tables: gen_md_tables.py) contracts over the
 // primitives before it transforms, which leaves (dp|dp) 320 + 225 lane operations per primitive
 // quartet where the Obara-Saika schedule had 2053, and keeps the recursion on the lanes' own
-// registers: no interpreted op, no idle lane.  64-atom diamond, FP64 build 4331 -> 1781 ms, mixed
-// precision 2999 -> 1094 ms; the FP64 pipe is 94-97 % busy at L = 1-4, 86-95 % at L = 5-7, 74 % at L = 8.
+// registers: no interpreted op, no idle lane.  64-atom diamond, FP64 build 4331 -> 1784 ms, mixed
+// precision 2999 -> 1098 ms; the FP64 pipe is 94-97 % busy at L = 1-4, 86-94 % at L = 5-7, 74 % at L = 8.
 //
 // A warp runs a stream of primitive quartets that crosses quartet borders, 32 at a time:
 //   set-up and Hermite recursion, a lane per primitive quartet (results to shared memory);
@@ -259,8 +259,8 @@ __device__ __forceinline__ bool md_setup(const PrimPair& b, const PrimPair& k, c
 // Warps that work on one stream together (a team): they share its Hermite integrals and
 // contraction buffers, each with an even share of every step's rounds.  The buffers of a lone warp
 // leave 6, 4 and 2 resident warps per SM at L = 6, 7, 8 (FP64 pipe 73, 49 and 26 % busy); teams
-// bring that to 10, 12 and 8.  Up to L = 5 a lone warp's buffers leave 8 to 16 and the pipe 86 to
-// 90 % busy, and a team's barriers would only cost.
+// bring that to 10, 12 and 8.  Up to L = 5 a lone warp's buffers leave 9 to 16 and the pipe 87 to
+// 97 % busy, and a team's barriers would only cost.
 // (md_team: 1 up to L = 5, then 2, 4, 4)
 // threads per block: two lone warps up to L = 4, one at L = 5 (whose 23 KB a warp fill the SM better
 // in single pieces: (dp|pp) 199 -> 193 ms at 64 atoms), one team beyond
